@@ -138,6 +138,7 @@ struct Batch {
   void* d_items;              // device work list of BatchItem, longest first
   int nitems;
   int* d_n1rows;              // first global row of each instance's shock capturing (n + 1 entries)
+  unsigned ghost_blocks;      // blocks per instance of the batched ghost fill
   int n1rows;                 // rows with shock capturing over all instances (0: none)
   int graph_launches;         // kernel launches of one step's graph
   int tuning;                 // graphs for timing tile shapes: no shock-capturing stencils (they would

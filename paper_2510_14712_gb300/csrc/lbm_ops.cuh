@@ -170,7 +170,9 @@ template <int D, typename S, typename real> struct OpsImpl {
   static void ghosts(Handle& h, void* dst) {
     const Params& p = h.p;
     if (!p.periodic_x) {
-      k_ghosts<D, S><<<grid_for(2LL * p.G * p.Ny * p.Nz), kBlock, 0, h.stream>>>(p, reinterpret_cast<ST*>(dst));
+      const long long n = ghost_items<D>(p, true) + ghost_items<D>(p, false);
+      k_ghosts<D, S><<<unsigned((n + kGhostBlock - 1) / kGhostBlock), kGhostBlock, 0, h.stream>>>(
+          p, reinterpret_cast<ST*>(dst));
       h.launches += 1;
     }
   }
@@ -239,10 +241,7 @@ template <int D, typename S, typename real> struct OpsImpl {
     k_collide<D, S, real><<<grid_for((long long)p.Nx * p.Ny * p.Nz), kBlock, 0, h.stream>>>(
         p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst), M(h), W(h), h.err_dev);
     h.launches += 1;
-    if (!p.periodic_x) {
-      k_ghosts<D, S><<<grid_for(2LL * p.G * p.Ny * p.Nz), kBlock, 0, h.stream>>>(p, reinterpret_cast<ST*>(dst));
-      h.launches += 1;
-    }
+    ghosts(h, dst);
     if (p.sc_on) shock_capturing(h, M(h), W(h), W(h) + D * p.plane);
   }
 
@@ -305,6 +304,11 @@ template <int D, typename S, typename real> struct OpsImpl {
       cudaMemcpy(b.d_n1rows, rowstart.data(), sizeof(int) * (b.n + 1), cudaMemcpyHostToDevice);
       b.n1rows = rowstart[b.n];
       b.nitems = int(items.size());
+      // blocks per instance of the ghost fill: one item per thread of the instance with the most
+      long long ng = 0;
+      for (int k = 0; k < b.n; ++k)
+        if (!ti[k].p.periodic_x) ng = std::max(ng, ghost_items<D>(ti[k].p, true) + ghost_items<D>(ti[k].p, false));
+      b.ghost_blocks = unsigned(std::max(1LL, std::min((ng + 255) / 256, 4096LL)));
       const size_t smem = FG::template smem_bytes<real>();
       auto kern = k_step_fused_batch<D, S, real, TX, TY, MINB>;
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
@@ -321,8 +325,12 @@ template <int D, typename S, typename real> struct OpsImpl {
       k_step_fused_batch<D, S, real, TX, TY, MINB><<<b.grid, FG::NT, FG::template smem_bytes<real>(), b.stream>>>(
           reinterpret_cast<const BatchInstance*>(b.d_insts), reinterpret_cast<const BatchItem*>(b.d_items), b.nitems,
           parity, b.d_counter, b.d_errs);
-      k_ghosts_batch<D, S><<<b.n, 256, 0, b.stream>>>(reinterpret_cast<const BatchInstance*>(b.d_insts), parity);
-      b.launches += 2;
+      b.launches += 1;
+      for (int k0 = 0; k0 < b.n; k0 += 65535) {
+        k_ghosts_batch<D, S><<<dim3(b.ghost_blocks, unsigned(b.n - k0 < 65535 ? b.n - k0 : 65535)), 256, 0, b.stream>>>(
+            reinterpret_cast<const BatchInstance*>(b.d_insts) + k0, parity);
+        b.launches += 1;
+      }
       if (b.n1rows > 0 && !b.tuning)
         b.launches += n1_update_batch<D, real>(reinterpret_cast<const BatchInstance*>(b.d_insts), b.d_n1rows, b.n,
                                                b.n1rows, b.stream);
