@@ -269,6 +269,7 @@ void remember_cfg(const Handle& h) {
 int read_err(Handle& h) {
   CK(cudaMemcpyAsync(h.err_host, h.err_dev, sizeof(unsigned), cudaMemcpyDeviceToHost, h.stream));
   CK(cudaStreamSynchronize(h.stream));
+  if (*h.err_host & kFlagWait) return fail(LBM_ECUDA, "a shared-memory copy of the step did not complete");
   if (*h.err_host & (LBM_FLAG_NONFINITE | LBM_FLAG_NEGATIVE)) {
     h.unstable = 1;
     return fail(LBM_EUNSTABLE, "non-finite or non-positive density/temperature produced");

@@ -15,6 +15,7 @@ namespace lbm {
 
 constexpr int kGhost = 4;         // ghost layers per non-periodic x face
 constexpr int kMaxPartials = 1024;
+constexpr unsigned kFlagWait = 16u;   // status bit: a bounded wait for an asynchronous copy ran out
 constexpr int kMaxTiles = 16;     // tile candidates whose autotune times are kept
 
 // Everything a kernel needs, passed by value.

@@ -14,6 +14,7 @@
 #pragma once
 
 #include "lbm_internal.cuh"
+#include "lbm_mlp_tc.cuh"
 
 namespace lbm {
 
@@ -38,6 +39,19 @@ template <> struct Store<float> {
   template <typename real, typename I> __device__ static real ld_last(const T* p, I o, float) { return real(__ldcs(p + o)); }
   template <typename real, typename I> __device__ static void st(T* p, I o, real v, float) { p[o] = float(v); }
   template <typename real, typename I> __device__ static void st_stream(T* p, I o, real v, float) { __stcs(p + o, float(v)); }
+  // pairs of values as stored: two consecutive ones at an even offset (one
+  // 8-byte access) or two single ones; their values; the store of a pair
+  using Raw = F2;
+  __device__ static Raw raw2(const T* p) { return f2_of(__ldcs(reinterpret_cast<const float2*>(p))); }
+  __device__ static Raw raw11(const T* a, const T* b) { return F2(__ldg(a), __ldg(b)); }
+  __device__ static F2 value(Raw v, float) { return v; }
+  __device__ static void st2_stream(T* p, F2 v, float) { __stcs(reinterpret_cast<float2*>(p), f2_in(v)); }
+  // the same from shared memory, the rounded pair and its halves
+  __device__ static Raw raw2s(const T* p) { return f2_of(*reinterpret_cast<const float2*>(p)); }
+  __device__ static Raw raw11s(const T* p) { return F2(p[0], p[1]); }
+  __device__ static Raw pack(F2 v, float) { return v; }
+  __device__ static T half_of(Raw q, int k) { return k ? q.y : q.x; }
+  __device__ static void st2_raw(T* p, Raw q) { __stcs(reinterpret_cast<float2*>(p), f2_in(q)); }
   // four consecutive values p[o .. o+3], o a multiple of 4 (one 16-byte load)
   template <typename real, typename I> __device__ static void ld4(const T* p, I o, float, real* v) {
     const float4 q = __ldg(reinterpret_cast<const float4*>(p + o));
@@ -57,6 +71,31 @@ template <> struct Store<Fp16Dev> {
   }
   template <typename real, typename I> __device__ static void st_stream(T* p, I o, real v, float ref) {
     __stcs(p + o, __float2half_rn(float(v) - ref));
+  }
+  // pairs of values as stored: two consecutive ones at an even offset (one
+  // 4-byte access) or two single ones; their values; the store of a pair
+  using Raw = __half2;
+  __device__ static Raw raw2(const T* p) {
+    const unsigned q = __ldcs(reinterpret_cast<const unsigned*>(p));
+    return *reinterpret_cast<const __half2*>(&q);
+  }
+  __device__ static Raw raw11(const T* a, const T* b) { return __halves2half2(__ldg(a), __ldg(b)); }
+  __device__ static F2 value(Raw v, float ref) { return f2_of(__half22float2(v)) + F2(ref); }
+  __device__ static void st2_stream(T* p, F2 v, float ref) {
+    st2_raw(p, pack(v, ref));
+  }
+  // the same from shared memory (p odd for raw11s: the halves of two words), the
+  // rounded pair and its halves
+  __device__ static Raw raw2s(const T* p) { return *reinterpret_cast<const __half2*>(p); }
+  __device__ static Raw raw11s(const T* p) {
+    const unsigned a = *reinterpret_cast<const unsigned*>(p - 1), b = *reinterpret_cast<const unsigned*>(p + 1);
+    const unsigned q = __byte_perm(a, b, 0x5432);
+    return *reinterpret_cast<const __half2*>(&q);
+  }
+  __device__ static Raw pack(F2 v, float ref) { return __float22half2_rn(f2_in(v - F2(ref))); }
+  __device__ static T half_of(Raw q, int k) { return k ? __high2half(q) : __low2half(q); }
+  __device__ static void st2_raw(T* p, Raw q) {
+    __stcs(reinterpret_cast<unsigned*>(p), *reinterpret_cast<const unsigned*>(&q));
   }
   // four consecutive values p[o .. o+3], o a multiple of 4 (one 8-byte load)
   template <typename real, typename I> __device__ static void ld4(const T* p, I o, float ref, real* v) {
@@ -208,61 +247,169 @@ __global__ void k_init(const __grid_constant__ Params p, typename Store<S>::T* A
   }
 }
 
-// pulled populations of node (xp, y, z): 2Q values, f then g
-template <int D, typename S, typename real>
-__device__ __forceinline__ void pull(const Params& p, const typename Store<S>::T* A, int xp, int y, int z, real* fg) {
-  using L = Lattice<D>;
-#pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    const int xs = xpad(p, xp - L::c(i, 0));
-    const int ys = wrap(y - L::c(i, 1), p.Ny);
-    const int zs = D == 3 ? wrap(z - L::c(i, 2), p.Nz) : z;
-    const long long o = node_off(p, xs, ys, zs);
-    fg[i] = pop_ok(p, A, i * p.plane + o) ? Store<S>::template ld<real>(A, i * p.plane + o, p.ref[i]) : real(0);
-    fg[L::Q + i] = pop_ok(p, A, (L::Q + i) * p.plane + o)
-                       ? Store<S>::template ld<real>(A, (L::Q + i) * p.plane + o, p.ref[L::Q + i])
-                       : real(0);
+// ---------------------------------------------------------------------------
+// index arithmetic of the split step: flattened node index -> (x, y, z) by
+// multiplication (Granlund and Montgomery, "Division by invariant integers
+// using multiplication", 1994: exact for n < 2^31)
+// ---------------------------------------------------------------------------
+struct FastDiv {
+  unsigned d, m, s;
+  __host__ __device__ FastDiv() : d(1), m(1), s(0) {}
+  __host__ explicit FastDiv(unsigned d_) : d(d_), s(0) {
+    while ((1ull << s) < d) ++s;
+    m = unsigned(((1ull << 32) * ((1ull << s) - d)) / d + 1);
   }
-}
+  __device__ __forceinline__ unsigned div(unsigned n) const { return (__umulhi(n, m) + n) >> s; }
+};
 
-// x range (padded) of the moment region: radius 3 beyond the interior
+// nodes (or groups of `quad` nodes along x) of the padded-x range [lo, hi) x Ny x Nz
+struct NodeRange {
+  int lo, quad;
+  unsigned n;
+  FastDiv nx, ny;
+  __host__ NodeRange(const Params& p, int lo_, int hi_, int quad_ = 1)
+      : lo(lo_), quad(quad_), nx(unsigned((hi_ - lo_ + quad_ - 1) / quad_)), ny(unsigned(p.Ny)) {
+    n = nx.d * unsigned(p.Ny) * unsigned(p.Nz);
+  }
+  __device__ __forceinline__ bool decode(unsigned gid, int& xp, int& y, int& z) const {
+    if (gid >= n) return false;
+    const unsigned r = nx.div(gid), q = ny.div(r);
+    xp = lo + int(gid - r * nx.d) * quad;
+    y = int(r - q * ny.d);
+    z = int(q);
+    return true;
+  }
+};
+
+// x range (padded) of the moment region: radius r beyond the interior
 __host__ __device__ inline void moment_range(const Params& p, int r, int& lo, int& hi) {
   if (p.periodic_x) { lo = 0; hi = p.Nx; }
   else { lo = p.G - r; hi = p.G + p.Nx + r; }
 }
 
+// in-plane element offsets of the 3^D source nodes of one node (x - c): row
+// part per (c_y[, c_z]) and x part per c_x; a population's plane base is
+// uniform, so a load costs one addition
+template <int D> struct PullOffsets {
+  unsigned x[3], r[D == 3 ? 9 : 3];
+  __device__ __forceinline__ PullOffsets() {}
+  __device__ __forceinline__ PullOffsets(const Params& p, int xp, int y, int z) {
+    rows(p, y, z);
+#pragma unroll
+    for (int c = -1; c <= 1; ++c) x[c + 1] = unsigned(xpad(p, xp - c));
+  }
+  __device__ __forceinline__ void rows(const Params& p, int y, int z) {
+    const unsigned pitch = unsigned(p.pitch), zs = pitch * unsigned(p.Ny);
+#pragma unroll
+    for (int cz = (D == 3 ? -1 : 0); cz <= (D == 3 ? 1 : 0); ++cz)
+#pragma unroll
+      for (int cy = -1; cy <= 1; ++cy)
+        r[(D == 3 ? 3 * (cz + 1) : 0) + cy + 1] =
+            unsigned(wrap(y - cy, p.Ny)) * pitch + (D == 3 ? unsigned(wrap(z - cz, p.Nz)) * zs : 0u);
+  }
+  // row offset of direction i's source
+  __device__ __forceinline__ unsigned row(int i) const {
+    using L = Lattice<D>;
+    return r[D == 3 ? 3 * (L::c(i, D - 1) + 1) + L::c(i, 1) + 1 : L::c(i, 1) + 1];
+  }
+  __device__ __forceinline__ unsigned operator()(int i) const { return row(i) + x[Lattice<D>::c(i, 0) + 1]; }
+};
+
 // ---------------------------------------------------------------------------
-// pass 1: moments rho, j = sum c f, S = sum g (Eqs. def_h, def_u, def_E) of
-// the pulled populations, on the interior plus 3 ghost layers.
+// split step, pass 1: moments rho, j = sum c f, S = sum g (Eqs. def_h, def_u,
+// def_E) of the pulled populations, on the interior plus 3 ghost layers.
 // M planes: rho, j_0..j_{D-1}, S   (each p.plane elements, padded layout)
+// j_a is (sum over c_a = +1) minus (sum over c_a = -1), both in increasing
+// direction order: exactly zero for mirror-symmetric populations.
+// One read of every population bounds it.  QUAD (FP32 and FP16-deviation
+// storage, Nx and the ghost width multiples of 4): a thread takes four nodes,
+// one 16- (8-) byte load per direction and one scalar load for the node that a
+// +-x pull needs from outside the four.
 // ---------------------------------------------------------------------------
-template <int D, typename S, typename real>
-__global__ void k_moments(Params p, const typename Store<S>::T* A, real* M) {
+template <int D, typename S, typename real, bool QUAD>
+__global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params p, const NodeRange range,
+                                                 const typename Store<S>::T* __restrict__ A, real* __restrict__ M) {
   using L = Lattice<D>;
-  int lo, hi;
-  moment_range(p, 3, lo, hi);
+  using ST = typename Store<S>::T;
+  constexpr int N = QUAD ? 4 : 1;
   int xp, y, z;
-  if (!decode(p, blockIdx.x * (long long)blockDim.x + threadIdx.x, lo, hi, xp, y, z)) return;
-  real fg[2 * L::Q];
-  pull<D, S, real>(p, A, xp, y, z, fg);
-  real rho = 0, j[D], Se = 0;
+  if (!range.decode(blockIdx.x * blockDim.x + threadIdx.x, xp, y, z)) return;
+  PullOffsets<D> po(p, xp, y, z);
+  // QUAD: the node left of the four (c_x = +1) and right of them (c_x = -1),
+  // kept inside the row where the pulled value is not used (the outermost
+  // ghost node of a row)
+  unsigned xl = 0, xr = 0;
+  if constexpr (QUAD) {
+    xl = unsigned(p.periodic_x ? wrap(xp - 1, p.Nx) : max(xp - 1, 0));
+    xr = unsigned(p.periodic_x ? wrap(xp + 4, p.Nx) : min(xp + 4, p.Nx + 2 * p.G - 1));
+  }
+  auto pulled = [&](const int i, const int ii, real* v) {
+    const ST* Ai = A + (long long)ii * p.plane;
+    if constexpr (!QUAD) {
+      const unsigned o = po(i);
+      v[0] = pop_ok(p, Ai, o) ? Store<S>::template ld<real>(Ai, o, p.ref[ii]) : real(0);
+    } else {
+      const int cx = L::c(i, 0);
+      const unsigned r = po.row(i);
+      real w[4] = {real(0), real(0), real(0), real(0)}, e = real(0);
+      if (pop_ok(p, Ai, r + xp, 4)) Store<S>::template ld4<real>(Ai, r + unsigned(xp), p.ref[ii], w);
+      if (cx != 0 && pop_ok(p, Ai, r + (cx > 0 ? xl : xr)))
+        e = Store<S>::template ld<real>(Ai, r + (cx > 0 ? xl : xr), p.ref[ii]);
+      if (cx > 0) { v[0] = e; v[1] = w[0]; v[2] = w[1]; v[3] = w[2]; }
+      else if (cx < 0) { v[0] = w[1]; v[1] = w[2]; v[2] = w[3]; v[3] = e; }
+      else { v[0] = w[0]; v[1] = w[1]; v[2] = w[2]; v[3] = w[3]; }
+    }
+  };
+  const unsigned o = po.r[D == 3 ? 4 : 1] + unsigned(xp);
+  auto put = [&](const int k, const real* v) {
+    real* dst = M + (long long)k * p.plane + o;
+    if constexpr (QUAD) *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+    else dst[0] = v[0];
+  };
+  real acc[N], sp[D][N], sn[D][N], v[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    acc[j] = real(0);
+#pragma unroll
+    for (int a = 0; a < D; ++a) sp[a][j] = sn[a][j] = real(0);
+  }
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
-    rho += fg[i];
-    Se += fg[L::Q + i];
+    pulled(i, i, v);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      acc[j] += v[j];
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        if (L::c(i, a) == 1) sp[a][j] += v[j];
+        if (L::c(i, a) == -1) sn[a][j] += v[j];
+      }
+    }
   }
-  first_moment<D, real>(fg, j);
-  const long long o = node_off(p, xp, y, z);
-  M[o] = rho;
-  for (int a = 0; a < D; ++a) M[(1 + a) * p.plane + o] = j[a];
-  M[(1 + D) * p.plane + o] = Se;
+  put(0, acc);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = sp[a][j] - sn[a][j];
+    put(1 + a, v);
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) acc[j] = real(0);
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    pulled(i, L::Q + i, v);
+#pragma unroll
+    for (int j = 0; j < N; ++j) acc[j] += v[j];
+  }
+  put(1 + D, acc);
 }
 
 // neighbour offset along axis a by s (wrapping periodic axes)
-__device__ __forceinline__ long long nb_off(const Params& p, int xp, int y, int z, int a, int s) {
-  if (a == 0) return node_off(p, xpad(p, xp + s), y, z);
-  if (a == 1) return node_off(p, xp, wrap(y + s, p.Ny), z);
-  return node_off(p, xp, y, wrap(z + s, p.Nz));
+__device__ __forceinline__ unsigned nb_off(const Params& p, int xp, int y, int z, int a, int s) {
+  if (a == 0) xp = xpad(p, xp + s);
+  else if (a == 1) y = wrap(y + s, p.Ny);
+  else z = wrap(z + s, p.Nz);
+  return unsigned(node_off(p, xp, y, z));
 }
 
 // compact Laplacian of rho at (xp, y, z); ghost columns of a wall face read
@@ -284,96 +431,241 @@ __device__ __forceinline__ void shift(const Params& p, int& xp, int& y, int& z, 
   else z = wrap(z + s, p.Nz);
 }
 
-// ---------------------------------------------------------------------------
-// pass 2: Korteweg force and primitive fields on interior + 1 ghost layer.
-// W planes: u_0..u_{D-1}, T, h, Lam_0..Lam_{D-1}, F_0..F_{D-1}
-// ---------------------------------------------------------------------------
-template <int D, typename real>
-__global__ void k_prims(Params p, const real* M, real* W) {
-  int lo, hi;
-  moment_range(p, 1, lo, hi);
-  int xp, y, z;
-  if (!decode(p, blockIdx.x * (long long)blockDim.x + threadIdx.x, lo, hi, xp, y, z)) return;
-  Model<real> m = model_of<real>(p);
-  const long long o = node_off(p, xp, y, z);
-  const real rho = M[o];
-  real F[D];
+// Planes of the primitive fields W (split step): u_a, T, h, Lam_a, F_a and,
+// with a closure that hands them on (kExtra), P and c_s^2.
+template <int D> struct WPlanes {
+  static constexpr int U = 0, T = D, H = D + 1, LAM = D + 2, F = 2 * D + 2, P = 3 * D + 2, CS2 = 3 * D + 3;
+};
+
+// Primitive fields of one node from its moments and the Korteweg force F:
+// u, E, the closure's (T, P, c_s^2, e), then h and Lambda, stored at offset o.
+// Warp-collective closures need every lane of the warp (act: a real node).
+template <int D, typename real, class CL>
+__device__ __forceinline__ void prims_node(const Params& p, const Model<real>& m, const CL& closure, bool act,
+                                           real rho, const real* j, real S, const real* F, real* __restrict__ W,
+                                           unsigned o) {
+  using WP = WPlanes<D>;
+  real u[D], uF = real(0), u2 = real(0), E = real(0);
 #pragma unroll
-  for (int a = 0; a < D; ++a) {
-    int x1 = xp, y1 = y, z1 = z, x2 = xp, y2 = y, z2 = z;
-    shift(p, x1, y1, z1, a, 1);
-    shift(p, x2, y2, z2, a, -1);
-    F[a] = m.kappa * rho * real(0.5) * (lap_rho<D, real>(p, M, x1, y1, z1) - lap_rho<D, real>(p, M, x2, y2, z2));  // Eq. FK
-  }
-  real u[D], uF = 0, u2 = 0;
+  for (int a = 0; a < D; ++a) u[a] = real(0);
+  if (act) {
 #pragma unroll
-  for (int a = 0; a < D; ++a) {
-    u[a] = div_rn(M[(1 + a) * p.plane + o] + real(0.5) * F[a], rho);                // Eq. def_u
-    uF += u[a] * F[a];
-    u2 += u[a] * u[a];
-  }
-  const real E = div_rn(M[(1 + D) * p.plane + o] + real(0.5) * uF, rho);           // Eq. def_E
-  real T, P, h;
-  // p.t64: the temperature inversion in FP64 from the FP32 moments (as the
-  // fused step's T64 closures)
-  const bool t64 = sizeof(real) == 4 && p.t64;
-  if (m.kind == LBM_EOS_PR) {   // the caloric relation inverted for T; h = e + P/rho
-    real e;
-    if (t64) {
-      const double ed = double(E) - 0.5 * double(u2);
-      e = real(ed);
-      T = pr_temperature_q(m, rho, ed);
-    } else {
-      e = E - real(0.5) * u2;
-      T = eos_temperature(m, rho, e);
+    for (int a = 0; a < D; ++a) {
+      u[a] = div_rn(j[a] + real(0.5) * F[a], rho);                                      // Eq. def_u
+      uF += u[a] * F[a];
+      u2 += u[a] * u[a];
     }
-    P = pr_pressure(m, rho, T);
-    h = e + P / rho;
-  } else {
-    if constexpr (sizeof(real) == 4) {
-      if (t64) {
-        real e;
-        T = vdw_temperature_fp64(p.a, 1.0 / p.cv, rho, E, u2, e);
-      } else {
-        T = (E - real(0.5) * u2 + m.a * rho) / m.cv;                                // Eq. lbm_temp
-      }
-    } else {
-      T = (E - real(0.5) * u2 + m.a * rho) / m.cv;                                  // Eq. lbm_temp
-    }
-    P = vdw_pressure(m, rho, T);
-    h = vdw_energy(m, rho, T) + P / rho;                                             // Eq. enthalpy
+    E = div_rn(S + real(0.5) * uF, rho);                                                // Eq. def_E
   }
+  real T = real(0), P = real(1), cs2 = real(0), e = real(0);
+  if constexpr (CL::kWarp) closure(m, rho, E, u2, act, T, P, cs2, e);
+  else if (act) closure(m, rho, E, u2, act, T, P, cs2, e);
+  if (!act) return;
   const real theta = P / rho;
+  auto put = [&](const int k, const real v) { W[(long long)k * p.plane + o] = v; };
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    W[a * p.plane + o] = u[a];
-    W[(D + 2 + a) * p.plane + o] = rho * u[a] * u[a] * u[a] + real(3) * rho * u[a] * (theta - real(1.0 / 3.0));
-    W[(2 * D + 2 + a) * p.plane + o] = F[a];
+    put(WP::U + a, u[a]);
+    put(WP::LAM + a, rho * u[a] * u[a] * u[a] + real(3) * rho * u[a] * (theta - real(1.0 / 3.0)));
+    put(WP::F + a, F[a]);
   }
-  W[D * p.plane + o] = T;
-  W[(D + 1) * p.plane + o] = h;
+  put(WP::T, T);
+  put(WP::H, e + theta);                                                                // Eq. enthalpy
+  if constexpr (CL::kExtra > 0) {
+    put(WP::P, P);
+    put(WP::CS2, cs2);
+  }
 }
 
 // ---------------------------------------------------------------------------
-// pass 3: derivatives and collision of every interior node (Eqs. fLBGK,
-// gLBGK), written to dst at the node (pull scheme).
+// split step, pass 2: Korteweg force and primitive fields on interior + 1
+// ghost layer (2-D form: every value of the stencil read from memory).
 // ---------------------------------------------------------------------------
-template <int D, typename S, typename real>
-__global__ void k_collide(Params p, const typename Store<S>::T* A, typename Store<S>::T* B, const real* M,
-                          const real* W, unsigned* err) {
+template <int D, typename real, class CL>
+__global__ void __launch_bounds__(256) k_prims(const __grid_constant__ Params p, const NodeRange range,
+                                               const real* __restrict__ M, real* __restrict__ W) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CL closure;
+  closure.load(p, smem_raw);
+  if constexpr (CL::kSmem > 0) __syncthreads();
+  int xp = 0, y = 0, z = 0;
+  const bool act = range.decode(blockIdx.x * blockDim.x + threadIdx.x, xp, y, z);
+  if (!CL::kWarp && !act) return;
+  const Model<real> m = model_of<real>(p);
+  real rho = real(1), j[D], F[D], S = real(0);
+#pragma unroll
+  for (int a = 0; a < D; ++a) j[a] = F[a] = real(0);
+  const unsigned o = unsigned(node_off(p, xp, y, z));
+  if (act) {
+    rho = M[o];
+    S = M[(1 + D) * p.plane + o];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      int x1 = xp, y1 = y, z1 = z, x2 = xp, y2 = y, z2 = z;
+      shift(p, x1, y1, z1, a, 1);
+      shift(p, x2, y2, z2, a, -1);
+      F[a] = m.kappa * rho * real(0.5) * (lap_rho<D, real>(p, M, x1, y1, z1) - lap_rho<D, real>(p, M, x2, y2, z2));  // Eq. FK
+      j[a] = M[(1 + a) * p.plane + o];
+    }
+  }
+  prims_node<D, real, CL>(p, m, closure, act, rho, j, S, F, W, o);
+}
+
+// ---------------------------------------------------------------------------
+// split step, pass 2 in 3-D: a block of 32 x 8 threads marches z over a column
+// of nodes with the density of three planes (radius 2 in the plane) and its
+// Laplacian of three planes (radius 1) in shared memory: rho, j and S are read
+// once, the Laplacian once computed per node instead of six times from 25
+// loads.  The next plane's density and this plane's j, S are loaded before
+// they are needed; two barriers per plane.
+// ---------------------------------------------------------------------------
+constexpr int kPrimX = 32, kPrimY = 8;
+template <typename real, class CL> struct PrimsSmem {
+  real rho[3][(kPrimY + 4) * (kPrimX + 4)];
+  real lap[3][(kPrimY + 2) * (kPrimX + 2)];
+};
+template <typename real, class CL, int MINB>
+__global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_constant__ Params p, int lo, int hi, int ncolx,
+                                                           int ncoly, int nseg, const real* __restrict__ M,
+                                                           real* __restrict__ W) {
+  constexpr int NT = kPrimX * kPrimY, BX2 = kPrimX + 4, BX1 = kPrimX + 2;
+  constexpr int N2 = BX2 * (kPrimY + 4), N1 = BX1 * (kPrimY + 2), K2 = (N2 + NT - 1) / NT, K1 = (N1 + NT - 1) / NT;
+  __shared__ PrimsSmem<real, CL> sm;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CL closure;
+  closure.load(p, smem_raw);
+  const Model<real> m = model_of<real>(p);
+  const int tid = threadIdx.x, lx = tid % kPrimX, ly = tid / kPrimX;
+  int b = blockIdx.x;
+  const int x0 = lo + (b % ncolx) * kPrimX;
+  b /= ncolx;
+  const int y0 = (b % ncoly) * kPrimY, seg = b / ncoly;
+  const int mb = int((long long)p.Nz * seg / nseg), me = int((long long)p.Nz * (seg + 1) / nseg);
+  const unsigned zs = unsigned(p.Ny) * unsigned(p.pitch);
+  // in-plane offsets of the density box positions of this thread (periodic
+  // axes wrapped; on bounded x the mirror image across a wall, kept inside the
+  // row where the value is not used)
+  unsigned o2[K2];
+#pragma unroll
+  for (int k = 0; k < K2; ++k) {
+    const int q = min(tid + k * NT, N2 - 1), bx = q % BX2, by = q / BX2;
+    int x = x0 + bx - 2, y = y0 + by - 2;
+    y %= p.Ny;
+    y += y < 0 ? p.Ny : 0;
+    if (p.periodic_x) {
+      x %= p.Nx;
+      x += x < 0 ? p.Nx : 0;
+    } else {
+      x = min(max(wall_mirror(p, x - p.G) + p.G, 0), p.pitch - 1);
+    }
+    o2[k] = unsigned(y) * unsigned(p.pitch) + unsigned(x);
+  }
+  const int xp = x0 + lx, y = y0 + ly;
+  const bool node = xp < hi && y < p.Ny;
+  const real* Mn = M + (node ? unsigned(y) * unsigned(p.pitch) + unsigned(xp) : 0u);
+  real* Wn = W + (Mn - M);
+  // box position of this thread's Laplacian nodes
+  int c1[K1];
+#pragma unroll
+  for (int k = 0; k < K1; ++k) c1[k] = ((tid + k * NT) / BX1 + 1) * BX2 + (tid + k * NT) % BX1 + 1;
+  const unsigned ztop = zs * unsigned(p.Nz);
+  auto first = [&](int z) {                       // offset of plane z, any z
+    z %= p.Nz;
+    return unsigned(z < 0 ? z + p.Nz : z) * zs;
+  };
+  auto next = [&](unsigned zo) { return zo + zs == ztop ? 0u : zo + zs; };
+  unsigned zl = first(mb - 2), zo = first(mb);    // plane to load next, plane of the next output
+  real nxt[K2];
+#pragma unroll
+  for (int k = 0; k < K2; ++k) nxt[k] = __ldg(M + zl + o2[k]);
+  real *r0 = sm.rho[0], *r1 = sm.rho[2], *r2 = sm.rho[1];      // density of planes pl, pl - 1, pl - 2
+  real *l0 = sm.lap[0], *l1 = sm.lap[2], *l2 = sm.lap[1];      // Laplacian of planes pl (= pl - 3), pl - 1, pl - 2
+  for (int pl = mb - 2; pl <= me + 1; ++pl) {
+#pragma unroll
+    for (int k = 0; k < K2; ++k)
+      if (tid + k * NT < N2) r0[tid + k * NT] = nxt[k];
+    if (pl < me + 1) {
+      zl = next(zl);
+#pragma unroll
+      for (int k = 0; k < K2; ++k) nxt[k] = __ldg(M + zl + o2[k]);
+    }
+    const bool out = pl >= mb + 2, act = out && node;          // this iteration's node is on plane pl - 2
+    real rho = real(1), S = real(0), j[3] = {real(0), real(0), real(0)};
+    if (act) {
+      rho = __ldg(Mn + zo);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) j[a] = __ldg(Mn + (1 + a) * p.plane + zo);
+      S = __ldg(Mn + 4 * p.plane + zo);
+    }
+    __syncthreads();
+    // Laplacian of plane pl - 1 on radius 1
+    if (pl >= mb) {
+#pragma unroll
+      for (int k = 0; k < K1; ++k) {
+        if (tid + k * NT < N1) {
+          const int c = c1[k];
+          const real c2 = real(2) * r1[c];
+          l1[tid + k * NT] = (r1[c + 1] + r1[c - 1] - c2) + (r0[c] + r2[c] - c2) + (r1[c + BX2] + r1[c - BX2] - c2);
+        }
+      }
+    }
+    __syncthreads();
+    if (out) {
+      const int c = (ly + 1) * BX1 + lx + 1;
+      const real kr = m.kappa * rho * real(0.5);
+      const real F[3] = {kr * (l2[c + 1] - l2[c - 1]), kr * (l2[c + BX1] - l2[c - BX1]), kr * (l1[c] - l0[c])};   // Eq. FK
+      prims_node<3, real, CL>(p, m, closure, act, rho, j, S, F, Wn, zo);
+      zo = next(zo);
+    }
+    real* t = r2;
+    r2 = r1;
+    r1 = r0;
+    r0 = t;
+    t = l2;
+    l2 = l1;
+    l1 = l0;
+    l0 = t;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// split step, pass 3: derivatives and collision of every interior node (Eqs.
+// fLBGK, gLBGK), written to dst at the node (pull scheme).  EX: P and c_s^2 of
+// the node come from W (kExtra closures).
+// ---------------------------------------------------------------------------
+template <int D, typename S, typename real, bool EX, int NTB, int MINB>
+__global__ void __launch_bounds__(NTB, MINB)
+k_collide(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
+          typename Store<S>::T* __restrict__ B, const real* __restrict__ M, const real* __restrict__ W,
+          unsigned* err) {
   using L = Lattice<D>;
+  using ST = typename Store<S>::T;
+  using WP = WPlanes<D>;
   int xp, y, z;
-  if (!decode(p, blockIdx.x * (long long)blockDim.x + threadIdx.x, p.G, p.G + p.Nx, xp, y, z)) return;
-  Model<real> m = model_of<real>(p);
-  real fg[2 * L::Q];
-  pull<D, S, real>(p, A, xp, y, z, fg);
-  const long long o = node_off(p, xp, y, z);
+  if (!range.decode(blockIdx.x * NTB + threadIdx.x, xp, y, z)) return;
+  const PullOffsets<D> po(p, xp, y, z);
+  const unsigned o = po.r[D == 3 ? 4 : 1] + unsigned(xp);
+  real v[L::Q];
+  // f populations first: in flight while the fields are read
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const ST* Ai = A + (long long)i * p.plane;
+    v[i] = pop_ok(p, Ai, po(i)) ? Store<S>::template ld_last<real>(Ai, po(i), p.ref[i]) : real(0);
+  }
+  const Model<real> m = model_of<real>(p);
+  auto w = [&](const int k, const unsigned at) { return __ldg(W + (long long)k * p.plane + at); };
   NodeState<D, real> s;
-  s.rho = M[o];
-  s.T = W[D * p.plane + o];
-  s.P = eos_pressure(m, s.rho, s.T);
-  s.cs2 = eos_cs2(m, s.rho, s.T);
-  s.e = eos_energy(m, s.rho, s.T);
+  s.rho = __ldg(M + o);
+  s.T = w(WP::T, o);
+  if constexpr (EX) {
+    s.P = w(WP::P, o);
+    s.cs2 = w(WP::CS2, o);
+    s.e = w(WP::H, o) - s.P / s.rho;
+  } else {
+    s.P = vdw_pressure(m, s.rho, s.T);
+    s.cs2 = vdw_cs2(m, s.rho, s.T);
+    s.e = vdw_energy(m, s.rho, s.T);
+  }
   s.sc = p.sc_on != 0;
   s.mu_num = s.eta_num = s.k_num = real(0);
   if (s.sc) {
@@ -385,23 +677,178 @@ __global__ void k_collide(Params p, const typename Store<S>::T* A, typename Stor
   s.div_u = 0;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    s.u[a] = W[a * p.plane + o];
-    s.F[a] = W[(2 * D + 2 + a) * p.plane + o];
-    const long long op = nb_off(p, xp, y, z, a, 1), om = nb_off(p, xp, y, z, a, -1);
-    s.div_u += real(0.5) * (W[a * p.plane + op] - W[a * p.plane + om]);
-    s.gradT[a] = real(0.5) * (W[D * p.plane + op] - W[D * p.plane + om]);
-    s.gradh[a] = real(0.5) * (W[(D + 1) * p.plane + op] - W[(D + 1) * p.plane + om]);
-    const real lc = W[(D + 2 + a) * p.plane + o];
-    const real back = lc - W[(D + 2 + a) * p.plane + om];
-    const real fwd = W[(D + 2 + a) * p.plane + op] - lc;
-    // upwind-biased difference (Sec. 3.2): sgn(u) picks the side, sgn(0) = 0 averages
-    s.dLam[a] = s.u[a] > real(0) ? back : (s.u[a] < real(0) ? fwd : real(0.5) * (back + fwd));
+    s.u[a] = w(WP::U + a, o);
+    s.F[a] = w(WP::F + a, o);
+    const unsigned op = nb_off(p, xp, y, z, a, 1), om = nb_off(p, xp, y, z, a, -1);
+    s.div_u += real(0.5) * (w(WP::U + a, op) - w(WP::U + a, om));
+    s.gradT[a] = real(0.5) * (w(WP::T, op) - w(WP::T, om));
+    s.gradh[a] = real(0.5) * (w(WP::H, op) - w(WP::H, om));
+    const real lc = w(WP::LAM + a, o);
+    const real back = lc - w(WP::LAM + a, om);
+    const real fwd = w(WP::LAM + a, op) - lc;
+    s.dLam[a] = upwind(s.u[a], back, fwd);
   }
-  const unsigned fl = collide_node<D, real>(m, s, fg, fg + L::Q);
-  if (fl) atomicOr(err, fl);
+  Attractors<D, real> at;
+  at.setup(m, s);
+  if (at.flags) atomicOr(err, at.flags);
+  // f pass then g pass: one population set in flight at a time
+  auto put = [&](const int i, const real x) {
+    ST* Bi = B + (long long)i * p.plane;
+    if (pop_ok(p, Bi, o)) Store<S>::template st_stream<real>(Bi, o, x, p.ref[i]);
+  };
+  FactoredRelax<D, real>::f_pass(at, [&](int i) { return v[i]; }, put);
 #pragma unroll
-  for (int i = 0; i < 2 * L::Q; ++i)
-    if (pop_ok(p, B, i * p.plane + o)) Store<S>::template st<real>(B, i * p.plane + o, fg[i], p.ref[i]);
+  for (int i = 0; i < L::Q; ++i) {
+    const ST* Ai = A + (long long)(L::Q + i) * p.plane;
+    v[i] = pop_ok(p, Ai, po(i)) ? Store<S>::template ld_last<real>(Ai, po(i), p.ref[L::Q + i]) : real(0);
+  }
+  FactoredRelax<D, real>::g_pass(at, [&](int i) { return v[i]; }, [&](int i, real x) { put(L::Q + i, x); });
+}
+
+// ---------------------------------------------------------------------------
+// split step, pass 3 in FP32 arithmetic: two neighbouring nodes per thread
+// (x = lo + 2k and the node right of it), one register pair per value, so that
+// the collision's sums and products, the addresses and the stores cost one
+// instruction for both.  Offsets are 32-bit byte offsets onto a plane base that
+// is the same for every thread (a plane of a population is below 2^32 bytes:
+// at most 2^32 / 18 elements of up to 8 bytes).
+// Both population sets are requested before the fields are read: with 8 warps
+// per multiprocessor (255 registers) the loads of one set alone leave the
+// memory idle during the arithmetic.
+// ODD: Nx odd; past the last node of a row the pair's second node is computed
+// from in-row values and not stored.
+// ---------------------------------------------------------------------------
+template <typename T> __device__ __forceinline__ const T* at_bytes(const T* base, unsigned off) {
+  return reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
+}
+template <typename T> __device__ __forceinline__ T* at_bytes(T* base, unsigned off) {
+  return reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off);
+}
+
+template <int D, typename S, bool EX, bool ODD, int NTB, int MINB>
+__global__ void __launch_bounds__(NTB, MINB)
+k_collide2(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
+           typename Store<S>::T* __restrict__ B, const float* __restrict__ M, const float* __restrict__ W,
+           unsigned* err) {
+  using L = Lattice<D>;
+  using ST = typename Store<S>::T;
+  using WP = WPlanes<D>;
+  constexpr unsigned ES = sizeof(ST);
+  int xp, y, z;
+  if (!range.decode(blockIdx.x * NTB + threadIdx.x, xp, y, z)) return;
+  PullOffsets<D> po;                                         // rows in elements, then in bytes
+  po.rows(p, y, z);
+  const unsigned x = unsigned(xp), xm = unsigned(xpad(p, xp - 1)), x1 = unsigned(xpad(p, xp + 1)),
+                 x2 = unsigned(xpad(p, xp + 2)), r0 = po.r[D == 3 ? 4 : 1], o = r0 + x;
+  // rows of the neighbours along y and z
+  unsigned nbp[D], nbm[D];
+  nbp[0] = nbm[0] = 0;
+  nbp[1] = po.r[(D == 3 ? 3 : 0) + 0] + x;                   // source of c_y = -1: y + 1
+  nbm[1] = po.r[(D == 3 ? 3 : 0) + 2] + x;
+  if constexpr (D == 3) {
+    nbp[D - 1] = po.r[1] + x;
+    nbm[D - 1] = po.r[7] + x;
+  }
+#pragma unroll
+  for (int k = 0; k < (D == 3 ? 9 : 3); ++k) po.r[k] *= ES;
+  const unsigned bx = x * ES, bm = xm * ES, b1 = x1 * ES, b2 = x2 * ES, bo = o * ES;
+  const bool two = !ODD || xp + 1 < p.G + p.Nx;              // the second node is a node of the box
+  auto pulled = [&](const int i, const int ii) {
+    const ST* Ai = A + (long long)ii * p.plane;
+    const int cx = L::c(i, 0);
+    const unsigned r = po.row(i);
+    if (cx == 0) return pop_ok(p, at_bytes(Ai, r + bx), 0, 2) ? Store<S>::raw2(at_bytes(Ai, r + bx)) : typename Store<S>::Raw();
+    const ST *a = at_bytes(Ai, r + (cx > 0 ? bm : b1)), *b = at_bytes(Ai, r + (cx > 0 ? bx : b2));
+    return pop_ok(p, a, 0) && pop_ok(p, b, 0) ? Store<S>::raw11(a, b) : typename Store<S>::Raw();
+  };
+  typename Store<S>::Raw v[2 * L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) v[i] = pulled(i, i);
+  const Model<float> m = model_of<float>(p);
+  auto w1 = [&](const int k, const unsigned at) { return __ldg(at_bytes(W + (long long)k * p.plane, 4 * at)); };
+  auto w2 = [&](const int k, const unsigned at) {
+    return f2_of(__ldg(reinterpret_cast<const float2*>(at_bytes(W + (long long)k * p.plane, 4 * at))));
+  };
+  NodeState<D, F2> s;
+  s.rho = f2_of(__ldg(reinterpret_cast<const float2*>(at_bytes(M, 4 * o))));
+  s.T = w2(WP::T, o);
+  const F2 h = w2(WP::H, o);
+  s.sc = p.sc_on != 0;
+  s.mu_num = s.eta_num = s.k_num = F2(0.f);
+  if (s.sc) {
+    const float* V = static_cast<const float*>(p.sc_visc);
+    auto sc2 = [&](const int k) { return f2_of(__ldg(reinterpret_cast<const float2*>(V + k * p.plane + o))); };
+    s.mu_num = sc2(0);
+    s.eta_num = sc2(1);
+    s.k_num = sc2(2);
+  }
+  s.div_u = F2(0.f);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    s.u[a] = w2(WP::U + a, o);
+    s.F[a] = w2(WP::F + a, o);
+    F2 lc = w2(WP::LAM + a, o), up, um, Tp, Tm, hp, hm, lp, lm;
+    if (a == 0) {
+      // neighbours of the pair are x - 1, the pair itself and x + 2; the node
+      // right of a lone last node is read through its wrapped offset
+      float u1 = s.u[0].y, T1 = s.T.y, h1 = h.y, l1 = lc.y;
+      if (ODD && !two) {
+        u1 = w1(WP::U, r0 + x1);
+        T1 = w1(WP::T, r0 + x1);
+        h1 = w1(WP::H, r0 + x1);
+        l1 = w1(WP::LAM, r0 + x1);
+      }
+      up = F2(u1, w1(WP::U, r0 + x2));
+      um = F2(w1(WP::U, r0 + xm), s.u[0].x);
+      Tp = F2(T1, w1(WP::T, r0 + x2));
+      Tm = F2(w1(WP::T, r0 + xm), s.T.x);
+      hp = F2(h1, w1(WP::H, r0 + x2));
+      hm = F2(w1(WP::H, r0 + xm), h.x);
+      lp = F2(l1, w1(WP::LAM, r0 + x2));
+      lm = F2(w1(WP::LAM, r0 + xm), lc.x);
+    } else {
+      up = w2(WP::U + a, nbp[a]);
+      um = w2(WP::U + a, nbm[a]);
+      Tp = w2(WP::T, nbp[a]);
+      Tm = w2(WP::T, nbm[a]);
+      hp = w2(WP::H, nbp[a]);
+      hm = w2(WP::H, nbm[a]);
+      lp = w2(WP::LAM + a, nbp[a]);
+      lm = w2(WP::LAM + a, nbm[a]);
+    }
+    s.div_u = mad(F2(0.5f), up - um, s.div_u);
+    s.gradT[a] = F2(0.5f) * (Tp - Tm);
+    s.gradh[a] = F2(0.5f) * (hp - hm);
+    s.dLam[a] = upwind(s.u[a], lc - lm, lp - lc);
+  }
+  if constexpr (EX) {
+    s.P = w2(WP::P, o);
+    s.cs2 = w2(WP::CS2, o);
+    s.e = h - s.P / s.rho;
+  } else {
+    s.P = vdw_pressure(m, s.rho, s.T);
+    s.cs2 = vdw_cs2(m, s.rho, s.T);
+    s.e = vdw_energy(m, s.rho, s.T);
+  }
+  if (ODD && !two) {                                         // a lone last node: both halves are this node
+    s.rho.y = s.rho.x;
+    s.T.y = s.T.x;
+    s.P.y = s.P.x;
+  }
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) v[L::Q + i] = pulled(i, L::Q + i);
+  Attractors<D, F2> at;
+  at.setup(m, s);
+  if (at.flags) atomicOr(err, at.flags);
+  auto put = [&](const int i, const F2 val) {
+    ST* Bi = at_bytes(B + (long long)i * p.plane, bo);
+    if (!pop_ok(p, Bi, 0, 2)) return;
+    if (two) Store<S>::st2_stream(Bi, val, p.ref[i]);
+    else Store<S>::template st_stream<float>(Bi, 0, val.x, p.ref[i]);
+  };
+  FactoredRelax<D, F2>::f_pass(at, [&](int i) { return Store<S>::value(v[i], p.ref[i]); }, put);
+  FactoredRelax<D, F2>::g_pass(at, [&](int i) { return Store<S>::value(v[L::Q + i], p.ref[L::Q + i]); },
+                               [&](int i, F2 x) { put(L::Q + i, x); });
 }
 
 // ---------------------------------------------------------------------------
@@ -517,6 +964,273 @@ constexpr int kGhostBlock = 64;
 template <int D, typename S>
 __global__ void __launch_bounds__(kGhostBlock) k_ghosts(const __grid_constant__ Params p, typename Store<S>::T* B) {
   ghost_fill<D, S>(p, B, blockIdx.x * (long long)kGhostBlock + threadIdx.x, (long long)gridDim.x * kGhostBlock);
+}
+
+// ---------------------------------------------------------------------------
+// split step, pass 3 in FP32 arithmetic with the rows staged in shared memory:
+// a block owns W consecutive x of one row (y, z).  One warp requests every row
+// segment the block reads (the 2Q pulled populations and the primitive fields of
+// the row and of its neighbours along y and z) by bulk asynchronous copies, one
+// per segment, completing on one mbarrier; each thread then collides two nodes
+// from shared memory.  The loads hold no registers and no threads while they
+// are in flight, and an operand address is a base plus a compile-time offset:
+// with loads to registers a third of the instructions were 64-bit address
+// arithmetic and 8 warps per multiprocessor waited on them.
+//
+// Segments start at multiples of W elements of the padded row.  A population
+// with c_x = +1 needs the element left of the segment, one with c_x = -1 the
+// element right of it: their segments are one 16-byte unit (kA elements) longer
+// on that side.  On a periodic x the unit across the seam is a copy of its own,
+// which needs Nx to be a multiple of the unit (collide_rows_ok).
+// ---------------------------------------------------------------------------
+constexpr unsigned kWaitLimit = 1u << 22;     // polls of a copy's completion before the step gives up
+
+// Row segments of one block: element offsets in shared memory.
+template <int D, typename S, int W> struct RowsLayout {
+  using ST = typename Store<S>::T;
+  static constexpr int Q = Lattice<D>::Q, T3 = Q / 3;            // directions per c_x
+  static constexpr int kA = 16 / int(sizeof(ST)), kF = 4;        // elements per 16 bytes: populations, fields
+  // populations of one kind: T3 rows of W + kA (c_x = -1), T3 of W, T3 of W + kA
+  static constexpr int kSet = T3 * (3 * W + 2 * kA);
+  __host__ __device__ static constexpr int row(int i) {
+    return i < T3 ? i * (W + kA) : (i < 2 * T3 ? T3 * (W + kA) + (i - T3) * W : T3 * (2 * W + kA) + (i - 2 * T3) * (W + kA));
+  }
+  // index of the segment's first node in row i (the left unit of c_x = +1 rows)
+  __host__ __device__ static constexpr int lead(int i) { return i < 2 * T3 ? 0 : kA; }
+  static constexpr size_t kPopBytes = size_t(2 * kSet) * sizeof(ST);
+  // field rows: u_x, Lam_x, T, h of the row with a unit on both sides; then the
+  // row's rho, F_a, u_b, Lam_b (b > 0); then T, h, u_b, Lam_b of the two
+  // neighbours along each b > 0
+  static constexpr int kWide = W + 2 * kF, nWide = 4, nOwn = 1 + D + 2 * (D - 1), nNb = 8 * (D - 1);
+  __host__ __device__ static constexpr int wide(int k) { return k * kWide + kF; }
+  __host__ __device__ static constexpr int own(int k) { return nWide * kWide + k * W; }
+  __host__ __device__ static constexpr int nb(int b, int side, int k) {   // b in 1 .. D - 1, side 0 (minus) or 1 (plus)
+    return nWide * kWide + (nOwn + ((b - 1) * 2 + side) * 4 + k) * W;
+  }
+  static constexpr int nRows = 2 * Q + nWide + nOwn + nNb;
+  static constexpr size_t kBytes = kPopBytes + sizeof(float) * size_t(nWide * kWide + (nOwn + nNb) * W) + 16;
+};
+
+// the row form applies: every seam unit is a whole 16-byte unit
+template <typename S> inline bool collide_rows_ok(const Params& p) {
+  return !p.periodic_x || p.Nx % (16 / int(sizeof(typename Store<S>::T))) == 0;   // 4 (FP32) or 8, fields 4
+}
+
+__device__ __forceinline__ void bulk_copy(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// one thread of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+  unsigned e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0;
+}
+
+template <int D, typename S, bool EX, bool BOUNDED, int W, int MINB>
+__global__ void __launch_bounds__(W / 2, MINB)
+k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv dny,
+               const typename Store<S>::T* __restrict__ A, typename Store<S>::T* __restrict__ B,
+               const float* __restrict__ M, const float* __restrict__ Wf, unsigned* err) {
+  using L = Lattice<D>;
+  using ST = typename Store<S>::T;
+  using WP = WPlanes<D>;
+  using R = RowsLayout<D, S, W>;
+  constexpr int Q = L::Q;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  ST* sp = reinterpret_cast<ST*>(smem_raw);
+  float* sf = reinterpret_cast<float*>(smem_raw + R::kPopBytes);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + R::kBytes - 16);
+  const unsigned row = dseg.div(blockIdx.x), seg = blockIdx.x - row * unsigned(nseg);
+  const int z = D == 3 ? int(dny.div(row)) : 0, y = int(row) - z * p.Ny;
+  const int x0 = int(seg) * W, xend = BOUNDED ? p.pitch : p.Nx;        // padded x; end of the row's copied part
+  const unsigned pitch = unsigned(p.pitch), r0 = row * pitch;
+  // bytes of every segment with its side units (16 bytes each; absent at the
+  // ends of a bounded row)
+  const int n = min(W, xend - x0);                                     // elements of the segment itself
+  const bool lseam = !BOUNDED && x0 == 0, rseam = !BOUNDED && x0 + W >= p.Nx;
+  const bool lside = x0 > 0, rside = x0 + n < xend;                    // side units contiguous with the segment
+  if (threadIdx.x == 0) {
+    tc::mbar_init(bar, 1);
+    const unsigned nl = BOUNDED ? unsigned(lside) : 1u, nr = BOUNDED ? unsigned(rside) : 1u;
+    const unsigned bytes = unsigned(n) * (2u * Q * sizeof(ST) + 4u * (R::nWide + R::nOwn + R::nNb)) +
+                           16u * (nl + nr) * (2u * R::T3 + R::nWide);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_addr(bar)), "r"(bytes) : "memory");
+  }
+  __syncthreads();
+  {
+    // the warps take the segments in turn, one elected thread each: the
+    // addresses are uniform, so a request costs a few instructions
+    const unsigned s0 = tc::smem_addr(smem_raw), b0 = tc::smem_addr(bar);
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);
+    auto segment = [&](const void* rowp, const unsigned es, const unsigned dst, const bool left, const bool right) {
+      const char* src = static_cast<const char*>(rowp) + (long long)x0 * es;
+      const unsigned d = s0 + dst, nb = unsigned(n) * es;
+      const unsigned l = left && lside ? 16u : 0u, r = right && rside ? 16u : 0u;
+      bulk_copy(d - l, src - l, nb + l + r, b0);
+      if (left && lseam) bulk_copy(d - 16, static_cast<const char*>(rowp) + (long long)p.Nx * es - 16, 16, b0);
+      if (right && rseam) bulk_copy(d + nb, rowp, 16, b0);
+    };
+    if (elect_one()) {
+      constexpr int NW = W / 64;
+      const int ym = wrap(y - 1, p.Ny), yp = wrap(y + 1, p.Ny), zm = D == 3 ? wrap(z - 1, p.Nz) : 0, zp = D == 3 ? wrap(z + 1, p.Nz) : 0;
+      auto rowof = [&](const int cy, const int cz) {                   // element offset of row (y + cy, z + cz)
+        const int yy = cy < 0 ? ym : (cy > 0 ? yp : y), zz = D == 3 ? (cz < 0 ? zm : (cz > 0 ? zp : z)) : 0;
+        return (long long)(zz * p.Ny + yy) * p.pitch;
+      };
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        if (warp != w) continue;
+#pragma unroll
+        for (int k = w; k < R::nRows; k += NW) {
+          if (k < 2 * Q) {
+            const int i = k < Q ? k : k - Q, cx = L::c(i, 0);
+            const ST* rowp = A + (long long)k * p.plane + rowof(-L::c(i, 1), D == 3 ? -L::c(i, D - 1) : 0);
+            if (!pop_ok(p, rowp, x0, n)) rowp = A;                     // (bounds-check builds) counted, not read
+            segment(rowp, sizeof(ST), unsigned((k < Q ? 0 : R::kSet) + R::row(i) + R::lead(i)) * unsigned(sizeof(ST)), cx > 0, cx < 0);
+          } else {
+            int c = k - 2 * Q, f = 0, dst = 0, dy = 0, dz = 0;
+            const bool wide = c < R::nWide;
+            if (wide) {
+              f = c == 0 ? WP::U : (c == 1 ? WP::LAM : (c == 2 ? WP::T : WP::H));
+              dst = R::wide(c);
+            } else if (c < R::nWide + R::nOwn) {
+              c -= R::nWide;
+              dst = R::own(c);
+              f = c == 0 ? -1 : (c <= D ? WP::F + c - 1 : (c < 2 * D ? WP::U + c - D : WP::LAM + c - 2 * D + 1));
+            } else {
+              c -= R::nWide + R::nOwn;
+              const int bb = 1 + c / 8, side = (c / 4) & 1, q = c & 3;
+              dst = R::nb(bb, side, q);
+              f = q == 0 ? WP::T : (q == 1 ? WP::H : (q == 2 ? WP::U + bb : WP::LAM + bb));
+              (bb == 1 ? dy : dz) = side ? 1 : -1;
+            }
+            segment((f < 0 ? M : Wf + (long long)f * p.plane) + rowof(dy, dz), sizeof(float), unsigned(R::kPopBytes) + unsigned(dst) * 4u, wide, wide);
+          }
+        }
+      }
+    }
+    __syncwarp();
+  }
+  const int t = threadIdx.x, xp = x0 + 2 * t, xhi = p.G + p.Nx;
+  const bool act = xp >= p.G && xp < xhi, two = xp + 1 < xhi;
+  const unsigned o = r0 + unsigned(xp);
+  const Model<float> m = model_of<float>(p);
+  NodeState<D, F2> s;
+  s.sc = p.sc_on != 0;
+  s.mu_num = s.eta_num = s.k_num = F2(0.f);
+  auto g2 = [&](const float* base, long long k) { return f2_of(__ldg(reinterpret_cast<const float2*>(base + k * p.plane + o))); };
+  if (act) {
+    if (s.sc) {
+      const float* V = static_cast<const float*>(p.sc_visc);
+      s.mu_num = g2(V, 0);
+      s.eta_num = g2(V, 1);
+      s.k_num = g2(V, 2);
+    }
+    if constexpr (EX) {
+      s.P = g2(Wf, WP::P);
+      s.cs2 = g2(Wf, WP::CS2);
+    }
+  }
+  const bool ok = tc::mbar_wait(bar, 0, kWaitLimit);
+  if (!ok) {
+    atomicOr(err, kFlagWait);
+    tc::mbar_wait(bar, 0, kWaitLimit);                                 // the copies still in flight
+  }
+  if (ok && act) {
+  auto f2at = [&](int off) { return f2_of(*reinterpret_cast<const float2*>(sf + off + 2 * t)); };
+  auto f1at = [&](int off) { return sf[off + 2 * t]; };
+  s.rho = f2at(R::own(0));
+  s.T = f2at(R::wide(2));
+  const F2 h = f2at(R::wide(3));
+  s.div_u = F2(0.f);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    s.F[a] = f2at(R::own(1 + a));
+    F2 lc, up, um, Tp, Tm, hp, hm, lp, lm;
+    if (a == 0) {
+      s.u[0] = f2at(R::wide(0));
+      lc = f2at(R::wide(1));
+      up = F2(s.u[0].y, f1at(R::wide(0) + 2));
+      um = F2(f1at(R::wide(0) - 1), s.u[0].x);
+      lp = F2(lc.y, f1at(R::wide(1) + 2));
+      lm = F2(f1at(R::wide(1) - 1), lc.x);
+      Tp = F2(s.T.y, f1at(R::wide(2) + 2));
+      Tm = F2(f1at(R::wide(2) - 1), s.T.x);
+      hp = F2(h.y, f1at(R::wide(3) + 2));
+      hm = F2(f1at(R::wide(3) - 1), h.x);
+    } else {
+      s.u[a] = f2at(R::own(D + a));
+      lc = f2at(R::own(2 * D + a - 1));
+      Tm = f2at(R::nb(a, 0, 0));
+      hm = f2at(R::nb(a, 0, 1));
+      um = f2at(R::nb(a, 0, 2));
+      lm = f2at(R::nb(a, 0, 3));
+      Tp = f2at(R::nb(a, 1, 0));
+      hp = f2at(R::nb(a, 1, 1));
+      up = f2at(R::nb(a, 1, 2));
+      lp = f2at(R::nb(a, 1, 3));
+    }
+    s.div_u = mad(F2(0.5f), up - um, s.div_u);
+    s.gradT[a] = F2(0.5f) * (Tp - Tm);
+    s.gradh[a] = F2(0.5f) * (hp - hm);
+    s.dLam[a] = upwind(s.u[a], lc - lm, lp - lc);
+  }
+  if constexpr (EX) {
+    s.e = h - s.P / s.rho;
+  } else {
+    s.P = vdw_pressure(m, s.rho, s.T);
+    s.cs2 = vdw_cs2(m, s.rho, s.T);
+    s.e = vdw_energy(m, s.rho, s.T);
+  }
+  if (!two) {                                                          // a lone last node: both halves are this node
+    s.rho.y = s.rho.x;
+    s.T.y = s.T.x;
+    s.P.y = s.P.x;
+  }
+  Attractors<D, F2> at;
+  at.setup(m, s);
+  if (at.flags) atomicOr(err, at.flags);
+  // a row's pull of direction i: elements x - c_x of the pair
+  auto pulled = [&](const int i, const int set) {
+    const ST* q = sp + set + R::row(i) + R::lead(i) + 2 * t;
+    const int cx = L::c(i, 0);
+    return Store<S>::value(cx == 0 ? Store<S>::raw2s(q) : Store<S>::raw11s(q - cx), p.ref[set ? Q + i : i]);
+  };
+  auto put = [&](const int i, const F2 val) {
+    ST* Bi = B + (long long)i * p.plane + o;
+    if (!pop_ok(p, Bi, 0, 2)) return;
+    const typename Store<S>::Raw q = Store<S>::pack(val, p.ref[i]);
+    if (!BOUNDED || two) Store<S>::st2_raw(Bi, q);
+    else Bi[0] = Store<S>::half_of(q, 0);
+  };
+  FactoredRelax<D, F2>::f_pass(at, [&](int i) { return pulled(i, 0); }, put);
+  FactoredRelax<D, F2>::g_pass(at, [&](int i) { return pulled(i, R::kSet); }, [&](int i, F2 x) { put(Q + i, x); });
+  }
+  // ghost layers of a bounded row, by the blocks of its first and last node
+  // (their sectors have just been written; a wall's equilibrium is k_ghosts')
+  if constexpr (BOUNDED) {
+    const bool first = x0 == 0 && p.bc_lo != LBM_BC_WALL, last = xhi - 1 >= x0 && xhi - 1 < x0 + W && p.bc_hi != LBM_BC_WALL;
+    if (first || last) {
+      __syncthreads();
+      for (int i = t; i < 2 * Q; i += W / 2) {
+        ST* Br = B + (long long)i * p.plane + r0;
+        ST v;
+        if (first && pop_ok(p, Br, p.G)) {
+          if (p.bc_lo == LBM_BC_INFLOW) Store<S>::template st<double>(&v, 0, p.eq_lo[i], p.ref[i]);
+          else v = __ldcg(Br + p.G);
+          ghost_store<D, S>(p, Br, 0, v);
+        }
+        if (last && pop_ok(p, Br, xhi - 1)) {
+          if (p.bc_hi == LBM_BC_INFLOW) Store<S>::template st<double>(&v, 0, p.eq_hi[i], p.ref[i]);
+          else v = __ldcg(Br + xhi - 1);
+          ghost_store<D, S>(p, Br, xhi, v);
+        }
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------

@@ -28,16 +28,100 @@ template <int D, typename S, typename real> struct OpsImpl {
     h.launches += 1;
   }
 
-  // moments + primitive fields of `src` into scratch
-  static void fields(Handle& h, const void* src) {
+  // moments of `src` into scratch
+  static void moments(Handle& h, const void* src) {
     const Params& p = h.p;
     int lo, hi;
     moment_range(p, 3, lo, hi);
-    k_moments<D, S, real><<<grid_for((long long)(hi - lo) * p.Ny * p.Nz), kBlock, 0, h.stream>>>(
-        p, reinterpret_cast<const ST*>(src), M(h));
+    const ST* A = reinterpret_cast<const ST*>(src);
+    if constexpr (sizeof(real) == 4) {
+      // four nodes per thread: chunks of four never straddle the periodic seam
+      // and start on 16-byte boundaries
+      if (p.Nx % 4 == 0) {
+        const NodeRange r(p, lo - lo % 4, hi + (4 - hi % 4) % 4, 4);
+        k_moments<D, S, real, true><<<grid_for(r.n), kBlock, 0, h.stream>>>(p, r, A, M(h));
+        h.launches += 1;
+        return;
+      }
+    }
+    const NodeRange r(p, lo, hi);
+    k_moments<D, S, real, false><<<grid_for(r.n), kBlock, 0, h.stream>>>(p, r, A, M(h));
+    h.launches += 1;
+  }
+
+  // primitive fields from the moments in scratch (3-D: MINB blocks per
+  // multiprocessor for the register budget)
+  template <class CL, int MINB = 1> static void prims(Handle& h) {
+    const Params& p = h.p;
+    int lo, hi;
     moment_range(p, 1, lo, hi);
-    k_prims<D, real><<<grid_for((long long)(hi - lo) * p.Ny * p.Nz), kBlock, 0, h.stream>>>(p, M(h), W(h));
-    h.launches += 2;
+    if constexpr (D == 3) {
+      auto kern = k_prims3<real, CL, MINB>;
+      static const int slots = [kern] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(CL::kSmem));
+        int bps = 1, sms = 1, dev = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPrimX * kPrimY, CL::kSmem);
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        return std::max(1, bps) * sms;
+      }();
+      const int ncolx = (hi - lo + kPrimX - 1) / kPrimX, ncoly = (p.Ny + kPrimY - 1) / kPrimY;
+      // z-segments: about one round of resident blocks (a segment repeats four
+      // planes of density and two of Laplacian), at least two planes each
+      const int nseg = std::max(1, std::min(p.Nz / 2, (slots + ncolx * ncoly - 1) / (ncolx * ncoly)));
+      kern<<<unsigned(ncolx * ncoly * nseg), kPrimX * kPrimY, CL::kSmem, h.stream>>>(p, lo, hi, ncolx, ncoly, nseg,
+                                                                                      M(h), W(h));
+    } else {
+      const NodeRange r(p, lo, hi);
+      k_prims<D, real, CL><<<grid_for(r.n), kBlock, CL::kSmem, h.stream>>>(p, r, M(h), W(h));
+    }
+    h.launches += 1;
+  }
+
+  // moments + primitive fields of `src` into scratch
+  static void fields(Handle& h, const void* src) {
+    moments(h, src);
+    prims<AnyClosure<real>>(h);
+  }
+
+  // collision of every interior node; whether it filled the ghost layers too
+  template <bool EX> static bool collide(Handle& h, const void* src, void* dst) {
+    const Params& p = h.p;
+    const ST* A = reinterpret_cast<const ST*>(src);
+    ST* B = reinterpret_cast<ST*>(dst);
+    h.launches += 1;
+    if constexpr (sizeof(real) == 4) {
+      if (collide_rows_ok<S>(p)) {
+        constexpr int W128 = 128, kRowsMinB = 8;
+        using R = RowsLayout<D, S, W128>;
+        auto kern = p.periodic_x ? k_collide_rows<D, S, EX, false, W128, kRowsMinB> : k_collide_rows<D, S, EX, true, W128, kRowsMinB>;
+        static const cudaError_t ready[2] = {
+            cudaFuncSetAttribute(k_collide_rows<D, S, EX, false, W128, kRowsMinB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(R::kBytes)),
+            cudaFuncSetAttribute(k_collide_rows<D, S, EX, true, W128, kRowsMinB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(R::kBytes))};
+        (void)ready;
+        const int nseg = ((p.periodic_x ? p.Nx : p.G + p.Nx) + W128 - 1) / W128;
+        kern<<<unsigned(nseg) * unsigned(p.Ny) * unsigned(p.Nz), W128 / 2, R::kBytes, h.stream>>>(
+            p, nseg, FastDiv(unsigned(nseg)), FastDiv(unsigned(p.Ny)), A, B, M(h), W(h), h.err_dev);
+        return p.bc_lo != LBM_BC_WALL && p.bc_hi != LBM_BC_WALL;
+      }
+      constexpr int NTB = 128, MINB = 2;
+      const NodeRange r(p, p.G, p.G + p.Nx, 2);
+      auto kern = p.Nx % 2 ? k_collide2<D, S, EX, true, NTB, MINB> : k_collide2<D, S, EX, false, NTB, MINB>;
+      kern<<<unsigned((r.n + NTB - 1) / NTB), NTB, 0, h.stream>>>(p, r, A, B, M(h), W(h), h.err_dev);
+    } else {
+      constexpr int NTB = 128, MINB = 2;
+      const NodeRange r(p, p.G, p.G + p.Nx);
+      k_collide<D, S, real, EX, NTB, MINB><<<unsigned((r.n + NTB - 1) / NTB), NTB, 0, h.stream>>>(p, r, A, B, M(h),
+                                                                                                W(h), h.err_dev);
+    }
+    return false;
+  }
+
+  // One step in three passes over the box: moments, primitive fields, collision.
+  template <class CL, int MINB = 1> static void split(Handle& h, const void* src, void* dst) {
+    moments(h, src);
+    prims<CL, MINB>(h);
+    if (!collide<(CL::kExtra > 0)>(h, src, dst)) ghosts(h, dst);
   }
 
   // One tile shape of the fused kernel (TX x TY in-plane nodes, MINB CTAs
@@ -47,7 +131,7 @@ template <int D, typename S, typename real> struct OpsImpl {
     static size_t smem() { return FG::template smem_bytes<real>() + CL::kSmem; }
     struct Launch {
       int grid = 0, ncolx = 0, ncoly = 0, nseg = 1;
-      bool small = false, rows = false;
+      bool small = false;
     };
     // One CTA per (column, z-segment), never more items than resident CTA
     // slots so that all run together.  In 3-D the plane is cut into ncolx
@@ -62,10 +146,8 @@ template <int D, typename S, typename real> struct OpsImpl {
       static int blocks_per_sm = -1, sms = 0;
       if (blocks_per_sm < 0) {
         auto kern = k_step_fused<D, S, real, TX, TY, MINB, false, CL, OPT>;
-        auto kern_pos = k_step_fused<D, S, real, TX, TY, MINB, false, CL, OPT & ~kOptRows>;
-        auto kern_small = k_step_fused<D, S, real, TX, TY, MINB, true, CL, OPT & ~kOptRows>;
+        auto kern_small = k_step_fused<D, S, real, TX, TY, MINB, true, CL, OPT>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem()));
-        cudaFuncSetAttribute(kern_pos, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem()));
         cudaFuncSetAttribute(kern_small, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem()));
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kern, FG::NT, smem());
         int dev = 0;
@@ -99,53 +181,42 @@ template <int D, typename S, typename real> struct OpsImpl {
       if (g > slots) g = slots;
       l.grid = int(g);
       l.small = (p.periodic_x && p.Nx < TX + 6) || (D == 3 && p.Ny < TY + 6);
-      // row form of stage A: aligned 4-node chunks (Nx and the ghost width are
-      // multiples of 4), no wall face (mirror densities in stage A)
-      l.rows = (OPT & kOptRows) && D == 3 && sizeof(real) == 4 && !l.small && p.Nx % 4 == 0 && p.G % 4 == 0 &&
-               p.bc_lo != LBM_BC_WALL && p.bc_hi != LBM_BC_WALL;
       return l;
     }
     static void launch(Handle& h, const void* src, void* dst) {
       const Params& p = h.p;
       const Launch l = plan(p);
-      auto kern = l.small ? k_step_fused<D, S, real, TX, TY, MINB, true, CL, OPT & ~kOptRows>
-                          : (l.rows ? k_step_fused<D, S, real, TX, TY, MINB, false, CL, OPT>
-                                    : k_step_fused<D, S, real, TX, TY, MINB, false, CL, OPT & ~kOptRows>);
+      auto kern = l.small ? k_step_fused<D, S, real, TX, TY, MINB, true, CL, OPT>
+                          : k_step_fused<D, S, real, TX, TY, MINB, false, CL, OPT>;
       kern<<<l.grid, FG::NT, smem(), h.stream>>>(p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
                                                  h.err_dev, l.ncolx, l.ncoly, l.nseg);
       h.launches += 1;
+      ghosts(h, dst);
     }
   };
 
-  // Candidate tile shapes, first = default.  FP64 keeps one shape (its
-  // arithmetic, not the tile, bounds it).
+  // Candidate forms of the step, first = default.  3-D boxes take the split
+  // step: the column-marching kernel evaluated the moments on 2.1 times the
+  // nodes (radius 3 around a 32x8 tile) and held 16 warps per multiprocessor
+  // behind three barriers a plane.  Per step, before and after: 256^3 FP32 2587
+  // -> 1938 us, FP16-deviation 2072 -> 1660 us, 91x75x53 FP32 129 -> 73 us, FP64
+  // channel 100x24x20 1028 -> 117 us, 256x128x96 with a network 1326 -> 968 us.
   using LaunchFn = void (*)(Handle&, const void*, void*);
-  // The learned closure adds a register-hungry network evaluation to stage C,
-  // so its list also offers the unrestricted (MINB 1) allocation.
   template <class CL> static int candidates(const LaunchFn** fns) {
-    if constexpr (CL::kPr) {                                   // one shape: the Peng-Robinson sets compile fast
-      static const LaunchFn c[] = {D == 3 ? &Fused<32, 8, sizeof(real) == 8 ? 1 : 2, CL, kOptRows>::launch
-                                          : &Fused<256, 1, 2, CL>::launch};
+    if constexpr (D == 3 && CL::kWarp) {
+      // the network's registers: 220 and one block per multiprocessor, or 128 and
+      // two with spills (256x128x96: 970 and 1003 us per step)
+      static const LaunchFn c[] = {&split<CL, 1>, &split<CL, 2>};
+      *fns = c;
+      return 2;
+    } else if constexpr (D == 3) {
+      static const LaunchFn c[] = {&split<CL>};
       *fns = c;
       return 1;
-    } else if constexpr (D == 3) {
-      if constexpr (sizeof(real) == 8) {
-        static const LaunchFn c[] = {&Fused<32, 8, 1, CL>::launch};
-        *fns = c;
-        return 1;
-      } else if constexpr (CL::kWarp) {
-        static const LaunchFn c[] = {&Fused<32, 8, 2, CL>::launch, &Fused<32, 8, 1, CL>::launch,
-                                     &Fused<32, 16, 1, CL>::launch, &Fused<32, 8, 1, CL, kOptRows>::launch};
-        *fns = c;
-        return 4;
-      } else {
-        static const LaunchFn c[] = {&Fused<32, 8, 2, CL, kOptRows>::launch, &Fused<32, 16, 1, CL, kOptRows>::launch,
-                                     &Fused<16, 16, 2, CL, kOptRows>::launch,
-                                     &Fused<32, 8, 2, CL, kOptRows | kOptPair>::launch,
-                                     &Fused<32, 16, 1, CL, kOptRows | kOptPair>::launch};
-        *fns = c;
-        return 5;
-      }
+    } else if constexpr (CL::kPr) {                            // one shape: the Peng-Robinson sets compile fast
+      static const LaunchFn c[] = {&Fused<256, 1, 2, CL>::launch};
+      *fns = c;
+      return 1;
     } else if constexpr (sizeof(real) == 4 && !CL::kWarp) {
       // narrow tiles spread small domains (few columns) over more SMs; the
       // 2-D FP32 body also fits 80 registers without spills, so 768 threads
@@ -186,9 +257,11 @@ template <int D, typename S, typename real> struct OpsImpl {
   template <class CL> static void step_cl(Handle& h, const void* src, void* dst) {
     const LaunchFn* fns;
     const int n = candidates<CL>(&fns);
-    fns[h.tile_cfg < n ? h.tile_cfg : 0](h, src, dst);
-    ghosts(h, dst);
-    if (h.p.sc_on) {
+    const LaunchFn fn = fns[h.tile_cfg < n ? h.tile_cfg : 0];
+    fn(h, src, dst);
+    if (h.p.sc_on && D == 3) {
+      shock_capturing(h, M(h), W(h), W(h) + D * h.p.plane);
+    } else if (h.p.sc_on) {
       const real* W = static_cast<const real*>(h.p.sc_prims);
       shock_capturing(h, W, W + h.p.plane, W + (1 + D) * h.p.plane);
     }
@@ -237,11 +310,15 @@ template <int D, typename S, typename real> struct OpsImpl {
 
   static void step_multipass(Handle& h, const void* src, void* dst) {
     const Params& p = h.p;
-    fields(h, src);
-    k_collide<D, S, real><<<grid_for((long long)p.Nx * p.Ny * p.Nz), kBlock, 0, h.stream>>>(
-        p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst), M(h), W(h), h.err_dev);
-    h.launches += 1;
-    ghosts(h, dst);
+    if (p.eos_kind == LBM_EOS_PR) {
+      if constexpr (std::is_same<S, Fp16Dev>::value) return;   // refused at create
+      else if (sizeof(real) == 4 && p.t64) split<PrClosure<real, true>>(h, src, dst);
+      else split<PrClosure<real>>(h, src, dst);
+    } else if (sizeof(real) == 4 && p.t64) {
+      split<ExactClosure<real, true>>(h, src, dst);
+    } else {
+      split<ExactClosure<real>>(h, src, dst);
+    }
     if (p.sc_on) shock_capturing(h, M(h), W(h), W(h) + D * p.plane);
   }
 
@@ -262,7 +339,12 @@ template <int D, typename S, typename real> struct OpsImpl {
     }
   }
 
-  static size_t scratch_bytes(const Params& p) { return size_t(4 * D + 4) * size_t(p.plane) * sizeof(real); }
+  // moments (D + 2 planes), primitive fields (3 D + 2, and P, c_s^2 for the
+  // closures that hand them on: Peng-Robinson, or a network attached to FP32)
+  static size_t scratch_bytes(const Params& p) {
+    const int extra = p.eos_kind == LBM_EOS_PR || std::is_same<S, float>::value ? 2 : 0;
+    return size_t(4 * D + 4 + extra) * size_t(p.plane) * sizeof(real);
+  }
 
   // ---- batches -------------------------------------------------------------
   template <int TX, int TY, int MINB> struct BatchFused {
