@@ -71,6 +71,8 @@ int check_errs(Batch& b) {
   BCK(cudaMemcpyAsync(b.h_errs, b.d_errs, sizeof(unsigned) * b.n, cudaMemcpyDeviceToHost, b.stream));
   BCK(cudaStreamSynchronize(b.stream));
   for (int k = 0; k < b.n; ++k)
+    if (b.h_errs[k] & kFlagWait) return bfail(LBM_ECUDA, "a shared-memory copy of the step did not complete");
+  for (int k = 0; k < b.n; ++k)
     if (b.h_errs[k] & (LBM_FLAG_NONFINITE | LBM_FLAG_NEGATIVE)) {
       b.unstable = 1;
       return bfail(LBM_EUNSTABLE, "instance " + std::to_string(k) + ": non-finite or non-positive density/temperature");
@@ -117,8 +119,7 @@ int lbm_batch_create(lbm_batch_t* out, int lattice, int n, const int* Nx, const 
     b->inst[k] = h;
     lbm_set_stream(h, b->stream);
   }
-  if (rc == LBM_OK && (dev_malloc(&b->d_counter, sizeof(int)) != cudaSuccess ||
-                       dev_malloc(&b->d_errs, sizeof(unsigned) * n) != cudaSuccess ||
+  if (rc == LBM_OK && (dev_malloc(&b->d_errs, sizeof(unsigned) * n) != cudaSuccess ||
                        cudaMallocHost(&b->h_errs, sizeof(unsigned) * n) != cudaSuccess))
     rc = LBM_ENOMEM;
   if (rc == LBM_OK && cudaMemset(b->d_errs, 0, sizeof(unsigned) * n) != cudaSuccess) rc = LBM_ECUDA;
@@ -288,7 +289,11 @@ int lbm_batch_destroy(lbm_batch_t b) {
   if (b->d_insts) cudaFree(b->d_insts);
   if (b->d_n1rows) cudaFree(b->d_n1rows);
   if (b->d_items) cudaFree(b->d_items);
-  if (b->d_counter) cudaFree(b->d_counter);
+  for (int k = 0; k < kBatchBranches; ++k) {
+    if (b->branch[k]) cudaStreamDestroy(b->branch[k]);
+    if (b->join[k]) cudaEventDestroy(b->join[k]);
+  }
+  if (b->fork) cudaEventDestroy(b->fork);
   if (b->d_errs) cudaFree(b->d_errs);
   if (b->h_errs) cudaFreeHost(b->h_errs);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);

@@ -109,6 +109,7 @@ struct Handle {
 };
 
 struct Batch;
+constexpr int kBatchBranches = 4;
 
 // Per (D, precision) kernel set.
 struct Ops {
@@ -136,7 +137,7 @@ struct Batch {
   int n, D, Q, precision;
   Handle** inst;              // one handle per instance (own buffers and scratch)
   void* d_insts;              // device table of BatchInstance
-  void* d_items;              // device work list of BatchItem, longest first
+  void* d_items;              // device work list of BatchItem, largest instances first
   int nitems;
   int* d_n1rows;              // first global row of each instance's shock capturing (n + 1 entries)
   unsigned ghost_blocks;      // blocks per instance of the batched ghost fill
@@ -144,14 +145,14 @@ struct Batch {
   int graph_launches;         // kernel launches of one step's graph
   int tuning;                 // graphs for timing tile shapes: no shock-capturing stencils (they would
                               // overwrite the coefficients the next real step reads)
-  int* d_counter;             // work-list counter of the persistent kernel
+  cudaStream_t branch[kBatchBranches];   // 3-D batches: branches of the step's graph, with their
+  cudaEvent_t fork, join[kBatchBranches];  // fork and join events
   unsigned* d_errs;           // status word per instance
   unsigned* h_errs;           // pinned copy
   cudaStream_t stream;
   int own_stream;
   int cur;                    // parity of the current state (same for all instances)
   int tile_cfg;
-  int grid;                   // persistent CTAs
   cudaGraphExec_t graph[2];   // one step from parity 0 / 1
   int graph_ready;
   int unstable;

@@ -43,6 +43,7 @@ template <> struct Store<float> {
   // 8-byte access) or two single ones; their values; the store of a pair
   using Raw = F2;
   __device__ static Raw raw2(const T* p) { return f2_of(__ldcs(reinterpret_cast<const float2*>(p))); }
+  __device__ static Raw raw2g(const T* p) { return f2_of(__ldg(reinterpret_cast<const float2*>(p))); }
   __device__ static Raw raw11(const T* a, const T* b) { return F2(__ldg(a), __ldg(b)); }
   __device__ static F2 value(Raw v, float) { return v; }
   __device__ static void st2_stream(T* p, F2 v, float) { __stcs(reinterpret_cast<float2*>(p), f2_in(v)); }
@@ -77,6 +78,10 @@ template <> struct Store<Fp16Dev> {
   using Raw = __half2;
   __device__ static Raw raw2(const T* p) {
     const unsigned q = __ldcs(reinterpret_cast<const unsigned*>(p));
+    return *reinterpret_cast<const __half2*>(&q);
+  }
+  __device__ static Raw raw2g(const T* p) {
+    const unsigned q = __ldg(reinterpret_cast<const unsigned*>(p));
     return *reinterpret_cast<const __half2*>(&q);
   }
   __device__ static Raw raw11(const T* a, const T* b) { return __halves2half2(__ldg(a), __ldg(b)); }
@@ -924,6 +929,25 @@ __device__ inline void ghost_wall_row(const Params& p, typename Store<S>::T* B, 
   }
 }
 
+// The ghost layers of row Br of population i of a bounded box from the row's own
+// first / last node (outflow) or the face's equilibrium (inflow); `first`,
+// `last`: the ends to fill.  The nodes may have been written by this block
+// before a barrier, so they are read past L1.
+template <int D, typename S>
+__device__ __forceinline__ void ghost_row(const Params& p, typename Store<S>::T* Br, int i, bool first, bool last) {
+  typename Store<S>::T v;
+  if (first && pop_ok(p, Br, p.G)) {
+    if (p.bc_lo == LBM_BC_INFLOW) Store<S>::template st<double>(&v, 0, p.eq_lo[i], p.ref[i]);
+    else v = __ldcg(Br + p.G);
+    ghost_store<D, S>(p, Br, 0, v);
+  }
+  if (last && pop_ok(p, Br, p.G + p.Nx - 1)) {
+    if (p.bc_hi == LBM_BC_INFLOW) Store<S>::template st<double>(&v, 0, p.eq_hi[i], p.ref[i]);
+    else v = __ldcg(Br + p.G + p.Nx - 1);
+    ghost_store<D, S>(p, Br, p.G + p.Nx, v);
+  }
+}
+
 // work items of the two faces: rows of a wall face, (direction, row) pairs of another
 template <int D> __host__ __device__ inline long long ghost_items(const Params& p, bool low) {
   const long long rows = (long long)p.Ny * p.Nz;
@@ -1215,20 +1239,7 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
     const bool first = x0 == 0 && p.bc_lo != LBM_BC_WALL, last = xhi - 1 >= x0 && xhi - 1 < x0 + W && p.bc_hi != LBM_BC_WALL;
     if (first || last) {
       __syncthreads();
-      for (int i = t; i < 2 * Q; i += W / 2) {
-        ST* Br = B + (long long)i * p.plane + r0;
-        ST v;
-        if (first && pop_ok(p, Br, p.G)) {
-          if (p.bc_lo == LBM_BC_INFLOW) Store<S>::template st<double>(&v, 0, p.eq_lo[i], p.ref[i]);
-          else v = __ldcg(Br + p.G);
-          ghost_store<D, S>(p, Br, 0, v);
-        }
-        if (last && pop_ok(p, Br, xhi - 1)) {
-          if (p.bc_hi == LBM_BC_INFLOW) Store<S>::template st<double>(&v, 0, p.eq_hi[i], p.ref[i]);
-          else v = __ldcg(Br + xhi - 1);
-          ghost_store<D, S>(p, Br, xhi, v);
-        }
-      }
+      for (int i = t; i < 2 * Q; i += W / 2) ghost_row<D, S>(p, B + (long long)i * p.plane + r0, i, first, last);
     }
   }
 }

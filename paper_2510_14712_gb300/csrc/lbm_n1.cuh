@@ -16,7 +16,7 @@
 // row-mapped launches in 3-D (D + 2), and one block per row for batches.
 #pragma once
 
-#include "lbm_fused.cuh"
+#include "lbm_tile2d.cuh"
 
 namespace lbm {
 

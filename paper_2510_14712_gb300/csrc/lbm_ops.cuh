@@ -59,11 +59,9 @@ template <int D, typename S, typename real> struct OpsImpl {
       auto kern = k_prims3<real, CL, MINB>;
       static const int slots = [kern] {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(CL::kSmem));
-        int bps = 1, sms = 1, dev = 0;
+        int bps = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPrimX * kPrimY, CL::kSmem);
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        return std::max(1, bps) * sms;
+        return std::max(1, bps) * multiprocessors();
       }();
       const int ncolx = (hi - lo + kPrimX - 1) / kPrimX, ncoly = (p.Ny + kPrimY - 1) / kPrimY;
       // z-segments: about one round of resident blocks (a segment repeats four
@@ -124,83 +122,54 @@ template <int D, typename S, typename real> struct OpsImpl {
     if (!collide<(CL::kExtra > 0)>(h, src, dst)) ghosts(h, dst);
   }
 
-  // One tile shape of the fused kernel (TX x TY in-plane nodes, MINB CTAs
-  // per SM for the register budget) with thermodynamic closure CL.
-  template <int TX, int TY, int MINB, class CL, int OPT = 0> struct Fused {
-    using FG = FusedGeom<D, TX, TY, CL::kExtra, planes_per_interval<OPT>()>;
-    static size_t smem() { return FG::template smem_bytes<real>() + CL::kSmem; }
-    struct Launch {
-      int grid = 0, ncolx = 0, ncoly = 0, nseg = 1;
-      bool small = false;
-    };
-    // One CTA per (column, z-segment), never more items than resident CTA
-    // slots so that all run together.  In 3-D the plane is cut into ncolx
-    // columns along x and ncoly bands along y (at least ceil(Ny / TY) bands,
-    // at most TY rows each); the number of bands and of z-segments (each at
-    // least 16 planes long: a segment repeats 6 warm-up planes) is the one that
-    // minimises the modelled time rounds x (rows per band + 1.5) x (planes per
-    // segment + 6): with 256 x 256 planes and 304 slots, 38 bands of 6-7 rows
-    // give every slot one column, where 32 bands of 8 rows would leave 48 slots
-    // without work.
-    static Launch plan(const Params& p) {
-      static int blocks_per_sm = -1, sms = 0;
-      if (blocks_per_sm < 0) {
-        auto kern = k_step_fused<D, S, real, TX, TY, MINB, false, CL, OPT>;
-        auto kern_small = k_step_fused<D, S, real, TX, TY, MINB, true, CL, OPT>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem()));
-        cudaFuncSetAttribute(kern_small, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem()));
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kern, FG::NT, smem());
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (blocks_per_sm < 1) blocks_per_sm = 1;
-      }
-      Launch l;
-      l.ncolx = (p.Nx + TX - 1) / TX;
-      const int Nm = D == 3 ? p.Nz : p.Ny;
-      const long long slots = (long long)blocks_per_sm * sms;
-      const int nb0 = D == 3 ? (p.Ny + TY - 1) / TY : 1;
-      const int nb1 = D == 3 ? std::min(p.Ny, 2 * nb0) : 1;
-      double best = 1e300;
-      for (int nb = nb0; nb <= nb1; ++nb) {
-        const long long ncol = (long long)l.ncolx * nb;
-        long long nseg = slots / ncol;
-        if (nseg > Nm / 16) nseg = Nm / 16;
-        if (nseg < 1) nseg = 1;
-        const long long items = ncol * nseg;
-        const double rounds = double((items + slots - 1) / slots);
-        const double rows = D == 3 ? double((p.Ny + nb - 1) / nb) : 1.0;
-        const double cost = rounds * (rows + 1.5) * (double((Nm + nseg - 1) / nseg) + 6.0);
-        if (cost < best * (1.0 - 1e-9)) {
-          best = cost;
-          l.ncoly = nb;
-          l.nseg = int(nseg);
-        }
-      }
-      long long g = (long long)l.ncolx * l.ncoly * l.nseg;
-      if (g > slots) g = slots;
-      l.grid = int(g);
-      l.small = (p.periodic_x && p.Nx < TX + 6) || (D == 3 && p.Ny < TY + 6);
-      return l;
+  static int multiprocessors() {
+    static const int sms = [] {
+      int n = 1, dev = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+      return n;
+    }();
+    return sms;
+  }
+
+  // wall ghosts after a step whose kernel filled the other faces' layers
+  static void wall_ghosts(Handle& h, void* dst) {
+    if (h.p.bc_lo == LBM_BC_WALL || h.p.bc_hi == LBM_BC_WALL) ghosts(h, dst);
+  }
+
+  // One tile shape of the 2-D step (TX x TY nodes per block, MINB blocks per
+  // multiprocessor for the register budget) with thermodynamic closure CL.
+  template <int TX, int TY, int MINB, class CL> struct Tile {
+    using G = TileGeom<real, Unit<S, real>::N, TX, TY>;
+    static constexpr size_t kSmem = G::kBytes + CL::kSmem;
+    static long long tiles(const Params& p) {
+      return (long long)((p.Nx + TX - 1) / TX) * ((p.Ny + TY - 1) / TY);
     }
+    // work of a block in units of one population sum: density of the radius-3
+    // box, primitive fields of the radius-1 box, collision of the tile
+    static double work() { return G::P3 * G::H3 * 1.0 + G::P1 * G::H1 * 6.0 + TX * TY * 20.0; }
     static void launch(Handle& h, const void* src, void* dst) {
       const Params& p = h.p;
-      const Launch l = plan(p);
-      auto kern = l.small ? k_step_fused<D, S, real, TX, TY, MINB, true, CL, OPT>
-                          : k_step_fused<D, S, real, TX, TY, MINB, false, CL, OPT>;
-      kern<<<l.grid, FG::NT, smem(), h.stream>>>(p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
-                                                 h.err_dev, l.ncolx, l.ncoly, l.nseg);
+      auto kern = k_step2d<S, real, CL, TX, TY, MINB>;
+      static const cudaError_t ready = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
+      (void)ready;
+      kern<<<unsigned(tiles(p)), G::NT, kSmem, h.stream>>>(p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
+                                                          h.err_dev, (p.Nx + TX - 1) / TX);
       h.launches += 1;
-      ghosts(h, dst);
+      wall_ghosts(h, dst);
     }
   };
 
-  // Candidate forms of the step, first = default.  3-D boxes take the split
-  // step: the column-marching kernel evaluated the moments on 2.1 times the
-  // nodes (radius 3 around a 32x8 tile) and held 16 warps per multiprocessor
-  // behind three barriers a plane.  Per step, before and after: 256^3 FP32 2587
-  // -> 1938 us, FP16-deviation 2072 -> 1660 us, 91x75x53 FP32 129 -> 73 us, FP64
-  // channel 100x24x20 1028 -> 117 us, 256x128x96 with a network 1326 -> 968 us.
+  // Candidate forms of the step, first = default.
+  //
+  // 3-D boxes take the split step: the column-marching kernel evaluated the
+  // moments on 2.1 times the nodes (radius 3 around a 32x8 tile) and held 16
+  // warps per multiprocessor behind three barriers a plane.  Per step, before
+  // and after: 256^3 FP32 2587 -> 1938 us, FP16-deviation 2072 -> 1660 us,
+  // 91x75x53 FP32 129 -> 73 us, FP64 channel 100x24x20 1028 -> 117 us,
+  // 256x128x96 with a network 1326 -> 968 us.
+  //
+  // 2-D planes take one tile per block; the default picks the shape.
   using LaunchFn = void (*)(Handle&, const void*, void*);
   template <class CL> static int candidates(const LaunchFn** fns) {
     if constexpr (D == 3 && CL::kWarp) {
@@ -213,30 +182,43 @@ template <int D, typename S, typename real> struct OpsImpl {
       static const LaunchFn c[] = {&split<CL>};
       *fns = c;
       return 1;
-    } else if constexpr (CL::kPr) {                            // one shape: the Peng-Robinson sets compile fast
-      static const LaunchFn c[] = {&Fused<256, 1, 2, CL>::launch};
-      *fns = c;
-      return 1;
-    } else if constexpr (sizeof(real) == 4 && !CL::kWarp) {
-      // narrow tiles spread small domains (few columns) over more SMs; the
-      // 2-D FP32 body also fits 80 registers without spills, so 768 threads
-      // per SM (3 x 256, 6 x 128) can hide more of the latency of its short
-      // per-row stages
-      static const LaunchFn c[] = {&Fused<256, 1, 2, CL>::launch, &Fused<128, 1, 4, CL>::launch,
-                                   &Fused<512, 1, 1, CL>::launch, &Fused<64, 1, 8, CL>::launch,
-                                   &Fused<32, 1, 16, CL>::launch, &Fused<256, 1, 3, CL>::launch,
-                                   &Fused<128, 1, 6, CL>::launch, &Fused<128, 1, 6, CL, kOptPair>::launch,
-                                   &Fused<256, 1, 3, CL, kOptPair>::launch};
-      *fns = c;
-      return 9;
     } else {
-      static const LaunchFn c[] = {&Fused<256, 1, 2, CL>::launch, &Fused<128, 1, 4, CL>::launch,
-                                   &Fused<512, 1, 1, CL>::launch, &Fused<64, 1, 8, CL>::launch,
-                                   &Fused<32, 1, 16, CL>::launch};
-      *fns = c;
-      return 5;
+      return Tiles<CL>::list(fns);
     }
   }
+
+  // The shapes of the 2-D step and the rule among them: blocks run in rounds of
+  // one per multiprocessor, so the shape with the smallest rounds x work per
+  // block is taken; large tiles (least halo) where there are many, small ones
+  // where large ones would leave multiprocessors without a tile.
+  template <class CL, class... T> struct TileSet {
+    static constexpr int n = int(sizeof...(T));
+    static void rule(Handle& h, const void* src, void* dst) {
+      static const LaunchFn fn[] = {&T::launch...};
+      const double work[] = {T::work()...};
+      const long long tiles[] = {T::tiles(h.p)...};
+      int best = 0;
+      double bt = 1e300;
+      for (int k = 0; k < n; ++k) {
+        const double t = double((tiles[k] + multiprocessors() - 1) / multiprocessors()) * work[k];
+        if (t < bt) {
+          bt = t;
+          best = k;
+        }
+      }
+      fn[best](h, src, dst);
+    }
+    static int list(const LaunchFn** fns) {
+      static const LaunchFn c[] = {&rule, &T::launch...};
+      *fns = c;
+      return n + 1;
+    }
+  };
+  template <class CL, bool F64 = sizeof(real) == 8> struct Tiles
+      : TileSet<CL, Tile<64, 8, CL::kWarp ? 1 : 2, CL>, Tile<64, 4, 4, CL>, Tile<32, 8, 4, CL>,
+                Tile<16, 8, 8, CL>> {};
+  template <class CL> struct Tiles<CL, true>
+      : TileSet<CL, Tile<32, 8, 1, CL>, Tile<32, 4, 2, CL>, Tile<16, 4, 4, CL>, Tile<16, 2, 4, CL>, Tile<8, 4, 4, CL>> {};
 
   static void ghosts(Handle& h, void* dst) {
     const Params& p = h.p;
@@ -257,13 +239,12 @@ template <int D, typename S, typename real> struct OpsImpl {
   template <class CL> static void step_cl(Handle& h, const void* src, void* dst) {
     const LaunchFn* fns;
     const int n = candidates<CL>(&fns);
-    const LaunchFn fn = fns[h.tile_cfg < n ? h.tile_cfg : 0];
-    fn(h, src, dst);
+    fns[h.tile_cfg < n ? h.tile_cfg : 0](h, src, dst);
     if (h.p.sc_on && D == 3) {
       shock_capturing(h, M(h), W(h), W(h) + D * h.p.plane);
     } else if (h.p.sc_on) {
-      const real* W = static_cast<const real*>(h.p.sc_prims);
-      shock_capturing(h, W, W + h.p.plane, W + (1 + D) * h.p.plane);
+      const real* P = static_cast<const real*>(h.p.sc_prims);
+      shock_capturing(h, P, P + h.p.plane, P + (1 + D) * h.p.plane);
     }
   }
   static void step(Handle& h, const void* src, void* dst) { step_cl<ExactClosure<real>>(h, src, dst); }
@@ -347,32 +328,27 @@ template <int D, typename S, typename real> struct OpsImpl {
   }
 
   // ---- batches -------------------------------------------------------------
-  template <int TX, int TY, int MINB> struct BatchFused {
-    using FG = FusedGeom<D, TX, TY>;
+  // 2-D: one launch over the tiles of every instance
+  template <int TX, int TY, int MINB> struct BatchTiles {
+    using G = TileGeom<real, Unit<S, real>::N, TX, TY>;
     static int prepare(Batch& b) {
       std::vector<BatchInstance> ti(b.n);
       std::vector<BatchItem> items;
-      const int seg_len = 128;                                // planes per work item (long columns split)
+      std::vector<int> order(b.n), rowstart(b.n + 1, 0);      // rows of the batched shock-capturing kernels
       for (int k = 0; k < b.n; ++k) {
         const Handle& h = *b.inst[k];
-        BatchInstance& bi = ti[k];
-        bi.p = h.p;
-        bi.pop[0] = h.pop[0];
-        bi.pop[1] = h.pop[1];
-        bi.ncolx = (h.p.Nx + TX - 1) / TX;
-        bi.ncoly = D == 3 ? (h.p.Ny + TY - 1) / TY : 1;
-        const int Nm = D == 3 ? h.p.Nz : h.p.Ny;
-        const int nseg = Nm > seg_len ? (Nm + seg_len - 1) / seg_len : 1;
-        for (int c = 0; c < bi.ncolx * bi.ncoly; ++c)
-          for (int sg = 0; sg < nseg; ++sg)
-            items.push_back({k, c, int((long long)Nm * sg / nseg), int((long long)Nm * (sg + 1) / nseg)});
+        ti[k].p = h.p;
+        ti[k].pop[0] = h.pop[0];
+        ti[k].pop[1] = h.pop[1];
+        order[k] = k;
+        rowstart[k + 1] = rowstart[k] + (h.p.sc_on ? h.p.Ny * h.p.Nz : 0);
       }
-      std::stable_sort(items.begin(), items.end(),
-                       [](const BatchItem& a, const BatchItem& c) { return a.me - a.mb > c.me - c.mb; });
-      // rows of the batched shock-capturing kernels: instances with it on
-      std::vector<int> rowstart(b.n + 1, 0);
-      for (int k = 0; k < b.n; ++k)
-        rowstart[k + 1] = rowstart[k] + (ti[k].p.sc_on ? ti[k].p.Ny * ti[k].p.Nz : 0);
+      std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
+        return (long long)ti[a].p.Nx * ti[a].p.Ny > (long long)ti[c].p.Nx * ti[c].p.Ny;
+      });
+      for (int k : order)
+        for (int y = 0; y < ti[k].p.Ny; y += TY)
+          for (int x = 0; x < ti[k].p.Nx; x += TX) items.push_back({k, x, y});
       if (b.d_insts) cudaFree(b.d_insts);
       if (b.d_items) cudaFree(b.d_items);
       if (b.d_n1rows) cudaFree(b.d_n1rows);
@@ -386,71 +362,76 @@ template <int D, typename S, typename real> struct OpsImpl {
       cudaMemcpy(b.d_n1rows, rowstart.data(), sizeof(int) * (b.n + 1), cudaMemcpyHostToDevice);
       b.n1rows = rowstart[b.n];
       b.nitems = int(items.size());
-      // blocks per instance of the ghost fill: one item per thread of the instance with the most
+      // blocks per instance of the wall fill: one item per thread of the instance with the most
       long long ng = 0;
       for (int k = 0; k < b.n; ++k)
-        if (!ti[k].p.periodic_x) ng = std::max(ng, ghost_items<D>(ti[k].p, true) + ghost_items<D>(ti[k].p, false));
+        if (ti[k].p.bc_lo == LBM_BC_WALL || ti[k].p.bc_hi == LBM_BC_WALL)
+          ng = std::max(ng, ghost_items<D>(ti[k].p, true) + ghost_items<D>(ti[k].p, false));
       b.ghost_blocks = unsigned(std::max(1LL, std::min((ng + 255) / 256, 4096LL)));
-      const size_t smem = FG::template smem_bytes<real>();
-      auto kern = k_step_fused_batch<D, S, real, TX, TY, MINB>;
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-      int bps = 1, sms = 1, dev = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, FG::NT, smem);
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      b.grid = (bps < 1 ? 1 : bps) * sms;
-      if (b.grid > b.nitems) b.grid = b.nitems;
+      cudaFuncSetAttribute(k_step2d_batch<S, real, TX, TY, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(G::kBytes));
       return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ECUDA;
     }
     static void enqueue(Batch& b, int parity) {
-      cudaMemsetAsync(b.d_counter, 0, sizeof(int), b.stream);
-      k_step_fused_batch<D, S, real, TX, TY, MINB><<<b.grid, FG::NT, FG::template smem_bytes<real>(), b.stream>>>(
-          reinterpret_cast<const BatchInstance*>(b.d_insts), reinterpret_cast<const BatchItem*>(b.d_items), b.nitems,
-          parity, b.d_counter, b.d_errs);
+      const BatchInstance* insts = reinterpret_cast<const BatchInstance*>(b.d_insts);
+      k_step2d_batch<S, real, TX, TY, MINB><<<unsigned(b.nitems), G::NT, G::kBytes, b.stream>>>(
+          insts, reinterpret_cast<const BatchItem*>(b.d_items), parity, b.d_errs);
       b.launches += 1;
       for (int k0 = 0; k0 < b.n; k0 += 65535) {
         k_ghosts_batch<D, S><<<dim3(b.ghost_blocks, unsigned(b.n - k0 < 65535 ? b.n - k0 : 65535)), 256, 0, b.stream>>>(
-            reinterpret_cast<const BatchInstance*>(b.d_insts) + k0, parity);
+            insts + k0, parity);
         b.launches += 1;
       }
-      if (b.n1rows > 0 && !b.tuning)
-        b.launches += n1_update_batch<D, real>(reinterpret_cast<const BatchInstance*>(b.d_insts), b.d_n1rows, b.n,
-                                               b.n1rows, b.stream);
+      if (b.n1rows > 0 && !b.tuning) b.launches += n1_update_batch<D, real>(insts, b.d_n1rows, b.n, b.n1rows, b.stream);
+    }
+  };
+
+  // 3-D: the split step of every instance, the instances dealt to branches of
+  // the step's graph that run side by side
+  struct BatchSplit {
+    static int prepare(Batch& b) {
+      if (b.fork) return LBM_OK;
+      if (cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming) != cudaSuccess) return LBM_ECUDA;
+      for (int k = 0; k < kBatchBranches; ++k)
+        if (cudaStreamCreateWithFlags(&b.branch[k], cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&b.join[k], cudaEventDisableTiming) != cudaSuccess)
+          return LBM_ECUDA;
+      return LBM_OK;
+    }
+    static void enqueue(Batch& b, int parity) {
+      const int nb = std::min(b.n, kBatchBranches);
+      cudaEventRecord(b.fork, b.stream);
+      for (int k = 0; k < nb; ++k) cudaStreamWaitEvent(b.branch[k], b.fork, 0);
+      for (int k = 0; k < b.n; ++k) {
+        Handle& h = *b.inst[k];
+        const Handle saved = h;
+        h.stream = b.branch[k % nb];
+        h.err_dev = b.d_errs + k;
+        split<ExactClosure<real>>(h, h.pop[parity], h.pop[parity ^ 1]);
+        if (h.p.sc_on && !b.tuning) shock_capturing(h, M(h), W(h), W(h) + D * h.p.plane);
+        b.launches += h.launches - saved.launches;
+        h = saved;
+      }
+      for (int k = 0; k < nb; ++k) {
+        cudaEventRecord(b.join[k], b.branch[k]);
+        cudaStreamWaitEvent(b.stream, b.join[k], 0);
+      }
     }
   };
 
   using PrepFn = int (*)(Batch&);
   using EnqFn = void (*)(Batch&, int);
+  template <class... T> static int batch_list(const PrepFn** pf, const EnqFn** ef) {
+    static const PrepFn p[] = {&T::prepare...};
+    static const EnqFn e[] = {&T::enqueue...};
+    *pf = p;
+    *ef = e;
+    return int(sizeof...(T));
+  }
   static int batch_cands(const PrepFn** pf, const EnqFn** ef) {
-    if constexpr (D == 3) {
-      if constexpr (sizeof(real) == 8) {
-        static const PrepFn p[] = {&BatchFused<32, 8, 1>::prepare};
-        static const EnqFn e[] = {&BatchFused<32, 8, 1>::enqueue};
-        *pf = p; *ef = e;
-        return 1;
-      } else {
-        static const PrepFn p[] = {&BatchFused<32, 8, 2>::prepare, &BatchFused<16, 16, 2>::prepare};
-        static const EnqFn e[] = {&BatchFused<32, 8, 2>::enqueue, &BatchFused<16, 16, 2>::enqueue};
-        *pf = p; *ef = e;
-        return 2;
-      }
-    } else if constexpr (sizeof(real) == 4) {
-      static const PrepFn p[] = {&BatchFused<256, 1, 2>::prepare, &BatchFused<128, 1, 4>::prepare,
-                                 &BatchFused<64, 1, 8>::prepare, &BatchFused<256, 1, 3>::prepare,
-                                 &BatchFused<128, 1, 6>::prepare};
-      static const EnqFn e[] = {&BatchFused<256, 1, 2>::enqueue, &BatchFused<128, 1, 4>::enqueue,
-                                &BatchFused<64, 1, 8>::enqueue, &BatchFused<256, 1, 3>::enqueue,
-                                &BatchFused<128, 1, 6>::enqueue};
-      *pf = p; *ef = e;
-      return 5;
-    } else {
-      static const PrepFn p[] = {&BatchFused<256, 1, 2>::prepare, &BatchFused<128, 1, 4>::prepare,
-                                 &BatchFused<64, 1, 8>::prepare};
-      static const EnqFn e[] = {&BatchFused<256, 1, 2>::enqueue, &BatchFused<128, 1, 4>::enqueue,
-                                &BatchFused<64, 1, 8>::enqueue};
-      *pf = p; *ef = e;
-      return 3;
-    }
+    if constexpr (D == 3) return batch_list<BatchSplit>(pf, ef);
+    else if constexpr (sizeof(real) == 4)
+      return batch_list<BatchTiles<64, 8, 2>, BatchTiles<32, 8, 4>>(pf, ef);
+    else return batch_list<BatchTiles<32, 8, 1>, BatchTiles<16, 4, 4>>(pf, ef);
   }
   static int batch_ncfg() {
     const PrepFn* pf;

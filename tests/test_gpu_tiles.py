@@ -1,0 +1,101 @@
+"""GPU parity of the 2-D tile step at the sizes where a tile can go wrong: planes
+narrower than a tile's halo, one node more or less than a tile, odd widths (a
+pair of nodes across the edge), one- and two-row planes, inflow / outflow and
+wall ends, in every storage form and with every tile shape; and 3-D batches
+(one graph branch per group of instances) against single handles.
+
+Three steps from a noisy drifting state against the FP64 oracle, with the
+suite's tolerances: FP64 1e-12, FP32 1e-5, FP16-deviation 1e-3 on rho and T.
+"""
+import numpy as np
+import pytest
+
+import inputs
+from parity_util import oracle_run, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+P = pytest.importorskip("paper_2510_14712_gb300")
+
+TOL = {"fp64": 1e-12, "fp32": 1e-5, "fp16dev": 1e-3}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_14712_gb300 import build
+    build.build()
+    P.load()
+
+
+def _plane(shape, faces, seed=1):
+    sc = inputs.scenario("tgv_d3q27")
+    D = len(shape)
+    c = inputs.Case(name="tgv_d3q27", D=D, shape=shape, eos=dict(sc["eos"]), tau=0.15, Pr=0.71, cv=sc["cv"])
+    arr, n = tuple(reversed(shape)), int(np.prod(shape))
+    drift = (0.07, -0.05, 0.04)[:D]
+    c.rho = sc["rho0"] * (1 + 0.01 * inputs.uniform(seed, n).reshape(arr))
+    c.T = sc["T0"] * (1 + 0.01 * inputs.uniform(seed + 1, n).reshape(arr))
+    c.u = [drift[a] + 0.01 * inputs.uniform(seed + 2 + a, n).reshape(arr) for a in range(D)]
+    wall = ("wall", (([0.0, -0.05, 0.04])[:D], sc["T0"]))
+    if faces == "tube":
+        c.x_low, c.x_high = ("inflow", (1.02 * sc["rho0"], list(drift), sc["T0"])), "outflow"
+    elif faces in ("walls", "mixed"):
+        c.x_low, c.x_high = wall, (wall if faces == "walls" else "outflow")
+        c.u[0] = 0.01 * inputs.uniform(seed + 2, n).reshape(arr)
+    return c
+
+
+CASES = (
+    [(s, "periodic", "fp32") for s in ((1, 1), (2, 3), (3, 2), (6, 4), (15, 9), (16, 8), (33, 7), (63, 17), (64, 8), (65, 16),
+                                       (130, 5))]
+    + [(s, "periodic", "fp16dev") for s in ((5, 3), (32, 9), (67, 8))]
+    + [(s, "periodic", "fp64") for s in ((1, 2), (9, 5), (33, 9))]
+    + [(s, "tube", "fp32") for s in ((5, 1), (60, 4), (63, 9), (64, 8), (65, 3), (128, 17))]
+    + [(s, "tube", p) for s in ((31, 5), (66, 8)) for p in ("fp16dev", "fp64")]
+    + [(s, "walls", p) for s in ((4, 1), (61, 3), (64, 9), (66, 2)) for p in ("fp32", "fp64")]
+    + [((63, 5), "mixed", "fp32"), ((40, 9), "mixed", "fp64")]
+)
+
+
+@pytest.mark.parametrize("shape,faces,precision", CASES, ids=["x".join(map(str, c[0])) + "-%s-%s" % c[1:] for c in CASES])
+def test_tile_step_matches_oracle(shape, faces, precision):
+    c = _plane(shape, faces)
+    want = oracle_run(c, 3)
+    s = P.Solver(c, precision=precision)
+    try:
+        for k in range(P.lbm_tile_count(s.h)):
+            s.init()
+            P.lbm_set_tile(s.h, k)
+            got = s.step(3).fields()
+            for q in ("rho", "T") + (() if precision == "fp16dev" else ("u",)):
+                err = rel_l2(got[q], want[q])
+                assert err <= TOL[precision], "tile %d %s: relative L2 %.2e" % (k, q, err)
+    finally:
+        s.close()
+
+
+def test_batch_3d_matches_single_handles():
+    """A 3-D batch (periodic and tube instances, shock capturing on one) steps each
+    instance as a single handle does."""
+    cases = [_plane((24, 9, 5), "periodic", 11), _plane((40, 6, 7), "tube", 21), _plane((13, 5, 4), "periodic", 31),
+             _plane((130, 3, 2), "tube", 41), _plane((16, 8, 8), "periodic", 51)]
+    b = P.Batch(cases, precision="fp32")
+    try:
+        b.set_shock_capturing(0.1, 0.0, 0.1, k=1)
+        b.init().step(7)
+        got = [b.fields(k) for k in range(len(cases))]
+    finally:
+        b.close()
+    for k, c in enumerate(cases):
+        s = P.Solver(c, precision="fp32")
+        try:
+            if k == 1:
+                P.lbm_set_shock_capturing(s.h, 0.1, 0.0, 0.1)
+            want = s.init().step(7).fields()
+        finally:
+            s.close()
+        for q in ("rho", "u", "T"):
+            assert np.array_equal(got[k][q], want[q]), (k, q)
