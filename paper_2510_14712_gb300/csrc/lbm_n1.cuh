@@ -12,8 +12,9 @@
 // on periodic axes and are clamped to the nearest interior node on
 // non-periodic x faces.  Fields live on the padded plane layout of the handle
 // (offset (z Ny + y) pitch + x + G, one plane per component).  Three forms
-// share the per-node arithmetic: 2-D tiles in shared memory (two launches),
-// row-mapped launches in 3-D (D + 2), and one block per row for batches.
+// share the per-node arithmetic: in 2-D the step itself leaves S and |grad s|
+// (its block holds the neighbours' u, T and rho) and one launch over tiles does
+// the rest; in 3-D row-mapped launches (D + 2); one block per row for batches.
 #pragma once
 
 #include "lbm_tile2d.cuh"
@@ -83,21 +84,25 @@ template <typename real> __device__ __forceinline__ real n1_ld(const real* q) { 
 
 // five-point fourth difference and binomial (1, 4, 6, 4, 1)/16 of the values at
 // offsets -2 .. +2 along one axis, and the coefficients from the filtered norms
-// (one definition for the row-mapped and the tiled forms)
-template <typename real>
-__device__ __forceinline__ real n1_fourth(real vm2, real vm1, real v0, real vp1, real vp2) {
-  return vp2 - real(4) * vp1 + real(6) * v0 - real(4) * vm1 + vm2;
+// (one definition for every form; V: a scalar or a packed pair, multiply-adds
+// written out, so that the forms give the same bits)
+template <typename V> __device__ __forceinline__ V n1_fourth(V vm2, V vm1, V v0, V vp1, V vp2) {
+  return mad(V(-4), vp1 + vm1, mad(V(6), v0, vp2 + vm2));
 }
-template <typename real>
-__device__ __forceinline__ real n1_binom5(real vm2, real vm1, real v0, real vp1, real vp2) {
-  return (vm2 + real(4) * vm1 + real(6) * v0 + real(4) * vp1 + vp2) / real(16);
+template <typename V> __device__ __forceinline__ V n1_binom5(V vm2, V vm1, V v0, V vp1, V vp2) {
+  return mad(V(4), vp1 + vm1, mad(V(6), v0, vp2 + vm2)) * V(0.0625f);
 }
-template <typename real>
-__device__ __forceinline__ N1Vals<real, 3> n1_coefs(const Params& p, const Model<real>& m, real r, real t, real s4,
-                                                    real g4) {
-  const real cs2 = eos_cs2(m, r, t);
-  const real cs = sqrt(cs2 > real(0) ? cs2 : real(0));
-  return {{r * real(p.sc_c[0]) * s4, r * real(p.sc_c[1]) * s4, r * cs * real(p.sc_c[2]) * g4}};
+// c_s of k^num
+template <typename real> __device__ __forceinline__ real n1_sound(const Model<real>& m, real r, real t) {
+  return root(positive(eos_cs2(m, r, t)));
+}
+__device__ __forceinline__ F2 n1_sound(const Model<float>& m, F2 r, F2 t) {
+  return m.kind == LBM_EOS_PR ? F2(n1_sound(m, r.x, t.x), n1_sound(m, r.y, t.y)) : root(positive(vdw_cs2(m, r, t)));
+}
+template <typename real, typename V>
+__device__ __forceinline__ N1Vals<V, 3> n1_coefs(const Params& p, const Model<real>& m, V r, V t, V s4, V g4) {
+  const V cs = n1_sound(m, r, t);
+  return {{r * V(real(p.sc_c[0])) * s4, r * V(real(p.sc_c[1])) * s4, r * cs * V(real(p.sc_c[2])) * g4}};
 }
 
 // S and |grad s| at the node
@@ -117,29 +122,15 @@ __device__ __forceinline__ N1Vals<real, 2> n1_strain_at(const Params& p, const r
 #pragma unroll
     for (int b = 0; b < D; ++b)
       g[a][b] = real(0.5) * (n1_ld(u + b * p.plane + op[a]) - n1_ld(u + b * p.plane + om[a]));
-  real acc = real(0);
-#pragma unroll
-  for (int a = 0; a < D; ++a)
-#pragma unroll
-    for (int b = 0; b < D; ++b) acc += (g[a][b] + g[b][a]) * (g[a][b] + g[b][a]);
-  const real S = real(0.5) * sqrt(acc);
-  const real r = n1_ld(rho + o), t = n1_ld(T + o);
-  real cT, cR;
-  if (p.eos_kind == LBM_EOS_PR) {
-    eos_entropy_coefs(model_of<real>(p), r, t, cT, cR);
-  } else {
-    cR = real(p.R) / (r * (real(1) - real(p.b) * r));
-    cT = real(p.cv) / t;
-  }
-  real gs2 = real(0);
+  real gT[D], gr[D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    const real gT = real(0.5) * (n1_ld(T + op[a]) - n1_ld(T + om[a]));
-    const real gr = real(0.5) * (n1_ld(rho + op[a]) - n1_ld(rho + om[a]));
-    const real gs = cT * gT - cR * gr;
-    gs2 += gs * gs;
+    gT[a] = real(0.5) * (n1_ld(T + op[a]) - n1_ld(T + om[a]));
+    gr[a] = real(0.5) * (n1_ld(rho + op[a]) - n1_ld(rho + om[a]));
   }
-  return {{S, sqrt(gs2)}};
+  N1Vals<real, 2> v;
+  n1_norms<D>(model_of<real>(p), g, gT, gr, n1_ld(rho + o), n1_ld(T + o), v.v[0], v.v[1]);
+  return v;
 }
 
 // norm of the per-axis fourth differences of the two fields of `in` at the node
@@ -163,9 +154,9 @@ __device__ __forceinline__ N1Vals<real, 2> n1_d4_at(const Params& p, const real*
     for (int a = 0; a < D; ++a) {
       const real d4 = n1_fourth(n1_ld(v + nb[a][0]), n1_ld(v + nb[a][1]), n1_ld(v + o), n1_ld(v + nb[a][2]),
                                 n1_ld(v + nb[a][3]));
-      acc += d4 * d4;
+      acc = mad(d4, d4, acc);
     }
-    res.v[f] = sqrt(acc);
+    res.v[f] = root(acc);
   }
   return res;
 }
@@ -249,107 +240,127 @@ __global__ void k_n1_filter_coef(Params p, const real* __restrict__ rho, const r
   });
 }
 
-// ---- 2-D single-instance form: two launches over tiles of the plane ----
-// A block owns kN1TileX x kN1TileY nodes (threads along x) and walks tiles
-// gridDim.y apart along y.  The strain launch evaluates S and |grad s| on the
-// tile and a two-node halo into shared memory and takes the fourth
-// differences there; the filter launch runs the x pass on the tile's columns
-// and a two-row halo, then the y pass with the coefficients.  Halo positions
-// take the values of the node the row-mapped stencils read there: x wrapped
-// on a periodic x, clamped to the nearest interior node otherwise; y wrapped.
-// The arithmetic of every value is that of the per-node stages above.
-constexpr int kN1TileX = 128, kN1TileY = 16;
-constexpr int kN1HX = kN1TileX + 4, kN1HY = kN1TileY + 4;
+// ---- 2-D single-instance form: one launch over tiles of the plane ----
+// The step's blocks leave S and |grad s| in w0 (n1_norms on the fields they hold
+// in shared memory), rho and T in sc_prims.  A block here owns 64 x 16 nodes (one
+// unit of Unit<> per thread and step): S and |grad s| of the tile and a four-node
+// halo, the norm of their fourth differences on a two-node halo, the x pass on
+// the tile's columns and a two-row halo, the y pass with the coefficients.  Halo
+// positions take the values of the node the row-mapped stencils read there:
+// wrapped on a periodic axis, clamped to the nearest interior node otherwise.
+// Two tiled launches that read the fields again (strain with fourth differences,
+// filter with coefficients; 48 registers, one node per thread and pass, 572
+// instructions per node) took 137 + 107 us at 4096x2048.
+constexpr int kN1TileX = 64, kN1TileY = 16, kN1Threads = 256;
 
-// x of the node whose values a stencil reads at x (any integer)
-__device__ __forceinline__ int n1_xsrc(const Params& p, int x) {
-  return p.periodic_x ? modp(x, p.Nx) : (x < 0 ? 0 : (x >= p.Nx ? p.Nx - 1 : x));
-}
-
-template <typename real>
-__global__ void __launch_bounds__(kN1TileX)
-k_n1_strain_d4_2d(Params p, const real* __restrict__ rho, const real* __restrict__ u, const real* __restrict__ T) {
-  __shared__ real sv[2][kN1HY][kN1HX];             // S, |grad s| on the tile and its halo
-  const N1Buffers<2, real> b(p, rho, u, T);
-  const unsigned pitch = unsigned(p.pitch);
-  const int x0 = blockIdx.x * kN1TileX, tx = threadIdx.x;
-  const int ntile = (p.Ny + kN1TileY - 1) / kN1TileY;
-  for (int ty = blockIdx.y; ty < ntile; ty += gridDim.y) {
-    const int y0 = ty * kN1TileY;
-#pragma unroll 4
-    for (int k = tx; k < kN1HX * kN1HY; k += kN1TileX) {
-      const int hx = k % kN1HX, hy = k / kN1HX;
-      const int xs = n1_xsrc(p, x0 + hx - 2), ys = modp(y0 + hy - 2, p.Ny);
-      const N1Vals<real, 2> v =
-          n1_strain_at<2, real>(p, b.rho, b.u, b.T, xs, ys, 0, unsigned(ys) * pitch + unsigned(xs + p.G));
-      sv[0][hy][hx] = v.v[0];
-      sv[1][hy][hx] = v.v[1];
-    }
-    __syncthreads();
-    const int x = x0 + tx, hx = tx + 2;
-    if (x < p.Nx) {
-      for (int r = 0; r < kN1TileY && y0 + r < p.Ny; ++r) {
-        const int hy = r + 2;
-        N1Vals<real, 2> res;
-#pragma unroll
-        for (int f = 0; f < 2; ++f) {
-          const real(*v)[kN1HX] = sv[f];
-          real acc = real(0);                        // axis x, then y (n1_d4_at)
-          const real dx = n1_fourth(v[hy][hx - 2], v[hy][hx - 1], v[hy][hx], v[hy][hx + 1], v[hy][hx + 2]);
-          acc += dx * dx;
-          const real dy = n1_fourth(v[hy - 2][hx], v[hy - 1][hx], v[hy][hx], v[hy + 1][hx], v[hy + 2][hx]);
-          acc += dy * dy;
-          res.v[f] = sqrt(acc);
-        }
-        n1_store(p, b.w1, unsigned(y0 + r) * pitch + unsigned(x + p.G), res);
-      }
-    }
-    __syncthreads();                                 // the next tile overwrites sv
-  }
-}
-
-template <typename real>
-__global__ void __launch_bounds__(kN1TileX)
-k_n1_filter_coef_2d(Params p, const real* __restrict__ rho, const real* __restrict__ T) {
-  __shared__ real sf[2][kN1HY][kN1TileX];          // x-filtered norms; each thread reads only its own column
-  const N1Buffers<2, real> b(p, rho, nullptr, T);
+template <typename S, typename real>
+__global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant__ Params p, int ntx) {
+  using U = Unit<S, real>;
+  using V = typename U::V;
+  constexpr int N = U::N, HX = 4, P4 = kN1TileX + 2 * HX, H4 = kN1TileY + 8, P2 = kN1TileX + 4, H2 = kN1TileY + 4;
+  constexpr int PX = kN1TileX;
+  __shared__ __align__(16) real s4[2][H4 * P4];          // S, |grad s|; later the x-filtered norms
+  __shared__ __align__(16) real s2[2][H2 * P2];          // norms of the fourth differences
+  const N1Buffers<2, real> b(p);
   const Model<real> m = model_of<real>(p);
+  const int tid = threadIdx.x;
+  const int x0 = int(blockIdx.x % unsigned(ntx)) * kN1TileX, y0 = int(blockIdx.x / unsigned(ntx)) * kN1TileY;
   const unsigned pitch = unsigned(p.pitch);
-  const int tx = threadIdx.x, x = blockIdx.x * kN1TileX + tx;
-  if (x >= p.Nx) return;
-  const int ntile = (p.Ny + kN1TileY - 1) / kN1TileY;
-  for (int ty = blockIdx.y; ty < ntile; ty += gridDim.y) {
-    const int y0 = ty * kN1TileY;
-#pragma unroll 4
-    for (int hy = 0; hy < kN1HY; ++hy) {
-      const int ys = modp(y0 + hy - 2, p.Ny);
-      const N1Vals<real, 2> v = n1_filter_at<real>(p, 0, b.w1, x, ys, 0, unsigned(ys) * pitch + unsigned(x + p.G));
-      sf[0][hy][tx] = v.v[0];
-      sf[1][hy][tx] = v.v[1];
+  // node that a stencil reads at x: wrapped, or clamped to the box
+  auto src = [&](int x) { return p.periodic_x ? n1_wrap(x, p.Nx) : min(max(x, 0), p.Nx - 1); };
+  // units of the box whose nodes are not neighbours in memory, or whose halo is clamped
+  const bool edge = x0 < HX || x0 + kN1TileX + HX > p.Nx;
+  for (int k = tid; k < P4 / N * H4; k += kN1Threads) {
+    const int r = k / (P4 / N), u = k - r * (P4 / N), x = x0 + N * u - HX;
+    const unsigned row = unsigned(n1_wrap(y0 + r - 4, p.Ny)) * pitch + unsigned(p.G);
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const real* w = b.w0 + f * p.plane + row;
+      V v;
+      if (!edge) {
+        v = U::ld_field(w + x);
+      } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) U::set(v, q, __ldg(w + src(x + q)));
+      }
+      U::st(s4[f] + r * P4 + N * u, v);
     }
-    for (int r = 0; r < kN1TileY && y0 + r < p.Ny; ++r) {
-      const int hy = r + 2;
-      // y pass, then the coefficients (as n1_filter_coef_at)
-      const real s4 =
-          n1_binom5(sf[0][hy - 2][tx], sf[0][hy - 1][tx], sf[0][hy][tx], sf[0][hy + 1][tx], sf[0][hy + 2][tx]);
-      const real g4 =
-          n1_binom5(sf[1][hy - 2][tx], sf[1][hy - 1][tx], sf[1][hy][tx], sf[1][hy + 1][tx], sf[1][hy + 2][tx]);
-      const unsigned o = unsigned(y0 + r) * pitch + unsigned(x + p.G);
-      n1_store(p, b.visc, o, n1_coefs(p, m, n1_ld(b.rho + o), n1_ld(b.T + o), s4, g4));
+  }
+  __syncthreads();
+  for (int k = tid; k < P2 / N * H2; k += kN1Threads) {
+    const int r = k / (P2 / N), u = k - r * (P2 / N), x = x0 + N * u - 2;
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      V v;
+      if (!edge || p.periodic_x) {
+        const real* c = s4[f] + (r + 2) * P4 + N * u + 2;
+        const V c0 = U::ld(c);
+        const V dx = n1_fourth(U::at(c, -2), U::at(c, -1), c0, U::at(c, 1), U::at(c, 2));
+        const V dy = n1_fourth(U::ld(c - 2 * P4), U::ld(c - P4), c0, U::ld(c + P4), U::ld(c + 2 * P4));
+        v = root(mad(dy, dy, dx * dx));
+      } else {                                            // the norm of the clamped node, one node at a time
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+          const real* c = s4[f] + (r + 2) * P4 + min(max(src(x + q) - x0 + HX, 2), P4 - 3);
+          const real dx = n1_fourth(c[-2], c[-1], c[0], c[1], c[2]);
+          const real dy = n1_fourth(c[-2 * P4], c[-P4], c[0], c[P4], c[2 * P4]);
+          U::set(v, q, root(mad(dy, dy, dx * dx)));
+        }
+      }
+      U::st(s2[f] + r * P2 + N * u, v);
     }
+  }
+  __syncthreads();
+  for (int k = tid; k < PX / N * H2; k += kN1Threads) {
+    const int r = k / (PX / N), u = k - r * (PX / N);
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const real* c = s2[f] + r * P2 + N * u + 2;
+      U::st(s4[f] + r * PX + N * u, n1_binom5(U::at(c, -2), U::at(c, -1), U::ld(c), U::at(c, 1), U::at(c, 2)));
+    }
+  }
+  __syncthreads();
+  for (int k = tid; k < PX / N * kN1TileY; k += kN1Threads) {
+    const int r = k / (PX / N), u = k - r * (PX / N), x = x0 + N * u, y = y0 + r;
+    if (x >= p.Nx || y >= p.Ny) continue;
+    V q[2];
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const real* c = s4[f] + r * PX + N * u;
+      q[f] = n1_binom5(U::ld(c), U::ld(c + PX), U::ld(c + 2 * PX), U::ld(c + 3 * PX), U::ld(c + 4 * PX));
+    }
+    const unsigned o = unsigned(y) * pitch + unsigned(x + p.G);
+    const N1Vals<V, 3> res = n1_coefs<real, V>(p, m, U::ld_field(b.rho + o), U::ld_field(b.T + o), q[0], q[1]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) U::store_field(b.visc + j * p.plane + o, res.v[j], x + N - 1 < p.Nx);
   }
 }
 
-// The whole update of a handle's coefficients from the step's rho, u (D planes),
-// T (padded plane layout): 2 launches in 2-D, D + 2 in 3-D.
-template <int D, typename real>
+// S and |grad s| of a plane from its rho, u, T, which also go to sc_prims (the
+// multi-pass step keeps them in its scratch area)
+template <typename real>
+__global__ void __launch_bounds__(256) k_n1_norms_2d(const __grid_constant__ Params p, const real* __restrict__ rho,
+                                                     const real* __restrict__ u, const real* __restrict__ T) {
+  const long long n = blockIdx.x * 256LL + threadIdx.x;
+  if (n >= (long long)p.Nx * p.Ny) return;
+  const int y = int(n / p.Nx), x = int(n - (long long)y * p.Nx);
+  const unsigned o = unsigned(y) * unsigned(p.pitch) + unsigned(x + p.G);
+  const N1Buffers<2, real> b(p);
+  n1_store(p, b.w0, o, n1_strain_at<2, real>(p, rho, u, T, x, y, 0, o));
+  const_cast<real*>(b.rho)[o] = rho[o];
+  const_cast<real*>(b.T)[o] = T[o];
+}
+
+// The whole update of a handle's coefficients.  2-D: one launch after a step that
+// left S and |grad s| (`rho` null), two after one that left rho, u (D planes) and
+// T; 3-D: D + 2 launches from rho, u, T (padded plane layout).
+template <int D, typename S, typename real>
 inline int n1_update(const Params& p, cudaStream_t st, const real* rho, const real* u, const real* T) {
   if constexpr (D == 2) {
-    const int ntile = (p.Ny + kN1TileY - 1) / kN1TileY;
-    const dim3 grid(unsigned((p.Nx + kN1TileX - 1) / kN1TileX), unsigned(ntile < 65535 ? ntile : 65535));
-    k_n1_strain_d4_2d<real><<<grid, kN1TileX, 0, st>>>(p, rho, u, T);
-    k_n1_filter_coef_2d<real><<<grid, kN1TileX, 0, st>>>(p, rho, T);
-    return 2;
+    if (rho) k_n1_norms_2d<real><<<unsigned(((long long)p.Nx * p.Ny + 255) / 256), 256, 0, st>>>(p, rho, u, T);
+    const int ntx = (p.Nx + kN1TileX - 1) / kN1TileX, nty = (p.Ny + kN1TileY - 1) / kN1TileY;
+    k_n1_coef_2d<S, real><<<unsigned(ntx) * unsigned(nty), kN1Threads, 0, st>>>(p, ntx);
+    return rho ? 2 : 1;
   } else {
     const int groups = (p.Ny * p.Nz + kN1Rows - 1) / kN1Rows;
     const dim3 block(128), grid(unsigned((p.Nx + 127) / 128), unsigned(groups < 65535 ? groups : 65535));

@@ -23,6 +23,28 @@
 
 namespace lbm {
 
+// S = |grad u + grad u^T| / 2 and |grad s| of shock capturing (lbm_n1.cuh) from
+// the central differences g[a][b] = d_a u_b, d_a T, d_a rho and rho, T
+template <int D, typename C, typename V>
+__device__ __forceinline__ void n1_norms(const Model<C>& m, const V (&g)[D][D], const V (&gT)[D], const V (&gr)[D],
+                                         V rho, V T, V& S, V& gs) {
+  V acc = V(0);
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll
+    for (int b = 0; b < D; ++b) acc = mad(g[a][b] + g[b][a], g[a][b] + g[b][a], acc);
+  S = V(C(0.5)) * root(acc);
+  V cT, cR;
+  entropy_coefs(m, rho, T, cT, cR);
+  V s2 = V(0);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const V d = mad(cT, gT[a], V(-1) * (cR * gr[a]));
+    s2 = mad(d, d, s2);
+  }
+  gs = root(s2);
+}
+
 // One unit of nodes along x and its arithmetic.
 template <typename S, typename real> struct Unit;
 template <typename S> struct Unit<S, float> {          // two nodes, packed
@@ -59,6 +81,9 @@ template <typename S> struct Unit<S, float> {          // two nodes, packed
     if (two) Store<S>::st2_raw(p, q);
     else p[0] = Store<S>::half_of(q, 0);
   }
+  // values at x + d of the nodes of the unit at s
+  __device__ static V at(const float* s, int d) { return F2(s[d], s[d + 1]); }
+  __device__ static V ld_field(const float* p) { return f2_of(__ldg(reinterpret_cast<const float2*>(p))); }
   __device__ static void store_field(float* p, V v, bool two) {
     if (two) *reinterpret_cast<float2*>(p) = f2_in(v);
     else p[0] = v.x;
@@ -85,6 +110,8 @@ template <typename S> struct Unit<S, double> {         // one node
   __device__ static double get(V v, int) { return v; }
   __device__ static void set(V& v, int, double a) { v = a; }
   __device__ static void store(ST* p, V v, float ref, bool) { Store<S>::template st_stream<double>(p, 0, v, ref); }
+  __device__ static V at(const double* s, int d) { return s[d]; }
+  __device__ static V ld_field(const double* p) { return __ldg(p); }
   __device__ static void store_field(double* p, V v, bool) { *p = v; }
 };
 
@@ -122,7 +149,8 @@ struct Ring {
   }
 };
 
-template <typename S, typename real, class CL, int TX, int TY>
+// kNorms: with shock capturing on, leave S and |grad s| for k_n1_coef_2d
+template <typename S, typename real, class CL, int TX, int TY, bool kNorms>
 __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>::T* __restrict__ A,
                                        typename Store<S>::T* __restrict__ B, const int x0, const int y0, real* sm,
                                        unsigned& flags, const CL& closure) {
@@ -351,15 +379,46 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
       s.mu_num = U::ld(Vc);
       s.eta_num = U::ld(Vc + p.plane);
       s.k_num = U::ld(Vc + 2 * p.plane);
-      // this step's rho, u, T for the shock-capturing coefficients of the next step
-      real* W = static_cast<real*>(p.sc_prims) + o;
-      U::store_field(W, s.rho, two);
-#pragma unroll
-      for (int a = 0; a < 2; ++a) U::store_field(W + (1 + a) * p.plane, s.u[a], two);
-      U::store_field(W + 3 * p.plane, s.T, two);
     }
     const real* d = s_prm + (uy + 1) * G::P1 + N * (ux + G::U1);
     auto fld = [&](int k) { return d + k * G::P1 * G::H1; };
+    if (s.sc) {
+      // this step's fields for the shock-capturing coefficients of the next step:
+      // rho and T with S and |grad s| (kNorms), or with u for the batched stencils
+      const V half = V(real(0.5));
+      real* W = static_cast<real*>(p.sc_prims) + o;
+      U::store_field(W, s.rho, two);
+      U::store_field(W + 3 * p.plane, s.T, two);
+      if constexpr (kNorms) {
+        // differences at the box ends are one-sided sums over the clamped node
+        const bool lo = !p.periodic_x && gx == 0;
+        auto diff = [&](const real* c, V v, int pitch, V gu[2]) {
+          V r = U::right(c, v), l = U::left(c, v);
+          if (lo) U::set(l, 0, U::get(v, 0));
+#pragma unroll
+          for (int q = 0; q < N; ++q)
+            if (!p.periodic_x && gx + q == p.Nx - 1) U::set(r, q, U::get(v, q));
+          gu[0] = half * (r - l);
+          gu[1] = half * (U::ld(c + pitch) - U::ld(c - pitch));
+        };
+        V gu[2][2], gT[2], gr[2], t[2], Sn, gn;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          diff(fld(G::PU + b), s.u[b], G::P1, t);
+          gu[0][b] = t[0];
+          gu[1][b] = t[1];
+        }
+        diff(fld(G::PT), s.T, G::P1, gT);
+        diff(s_rho + (uy + 3) * G::P3 + N * (ux + G::U3), s.rho, G::P3, gr);
+        n1_norms<2>(m, gu, gT, gr, s.rho, s.T, Sn, gn);
+        real* w0 = static_cast<real*>(const_cast<void*>(p.sc_visc)) + 3 * p.plane + o;
+        U::store_field(w0, Sn, two);
+        U::store_field(w0 + p.plane, gn, two);
+      } else {
+#pragma unroll
+        for (int a = 0; a < 2; ++a) U::store_field(W + (1 + a) * p.plane, s.u[a], two);
+      }
+    }
     const V h = U::ld(fld(G::PH));
     if constexpr (CL::kExtra > 0) s.e = h - s.P / s.rho;
     else s.e = vdw_energy(m, s.rho, s.T);
@@ -414,7 +473,7 @@ k_step2d(const __grid_constant__ Params p, const typename Store<S>::T* __restric
   CL closure;
   closure.load(p, smem_raw + G::kBytes);                // (stage A's barrier covers it)
   unsigned flags = 0;
-  tile2d<S, real, CL, TX, TY>(p, A, B, int(blockIdx.x % unsigned(ntx)) * TX, int(blockIdx.x / unsigned(ntx)) * TY,
+  tile2d<S, real, CL, TX, TY, true>(p, A, B, int(blockIdx.x % unsigned(ntx)) * TX, int(blockIdx.x / unsigned(ntx)) * TY,
                               reinterpret_cast<real*>(smem_raw), flags, closure);
   if (flags) atomicOr(err, flags);
 }
@@ -441,7 +500,7 @@ k_step2d_batch(const BatchInstance* __restrict__ insts, const BatchItem* __restr
   const BatchItem it = items[blockIdx.x];
   const BatchInstance& bi = insts[it.inst];
   unsigned flags = 0;
-  tile2d<S, real, ExactClosure<real>, TX, TY>(bi.p, reinterpret_cast<const ST*>(bi.pop[parity]),
+  tile2d<S, real, ExactClosure<real>, TX, TY, false>(bi.p, reinterpret_cast<const ST*>(bi.pop[parity]),
                                               reinterpret_cast<ST*>(bi.pop[parity ^ 1]), it.x0, it.y0,
                                               reinterpret_cast<real*>(smem_raw), flags, ExactClosure<real>{});
   if (flags) atomicOr(errs + it.inst, flags);

@@ -99,3 +99,31 @@ def test_batch_3d_matches_single_handles():
             s.close()
         for q in ("rho", "u", "T"):
             assert np.array_equal(got[k][q], want[q]), (k, q)
+
+
+SC_TOL = {"fp64": 1e-12, "fp32": 5e-5}            # the suite's bounds with shock capturing
+SC_CASES = ([(s, "periodic") for s in ((1, 1), (3, 2), (7, 5), (63, 17), (64, 16), (65, 33), (130, 3))]
+            + [(s, "tube") for s in ((4, 1), (61, 15), (64, 17), (66, 4), (129, 18))] + [((62, 5), "walls")])
+
+
+@pytest.mark.parametrize("step_kernel", [0, 1])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("shape,faces", SC_CASES, ids=["x".join(map(str, c[0])) + "-" + c[1] for c in SC_CASES])
+def test_shock_capturing_tiles_match_oracle(shape, faces, precision, step_kernel):
+    """The coefficient tiles (64 x 16 nodes, four-node halo, wrapped or clamped) at their
+    edges, after the tile step and after the multi-pass step."""
+    from oracle import lbm as olbm
+    c = _plane(shape, faces)
+    coef = (0.5, 0.2, 0.4)
+    m = olbm.Model(c.D, c.shape, c.eos, c.tau, c.Pr, c.cv, c.x_low, c.x_high)
+    m.shock_capturing = coef
+    want = olbm.Sim(m, c.rho, c.u, c.T).step(4).fields()
+    s = P.Solver(c, precision=precision, step_kernel=step_kernel)
+    try:
+        P.lbm_set_shock_capturing(s.h, *coef)
+        got = s.init().step(4).fields()
+    finally:
+        s.close()
+    for q, w in (("rho", want["rho"]), ("u", np.stack(want["u"])), ("T", want["T"])):
+        err = rel_l2(got[q], w)
+        assert err <= SC_TOL[precision], "%s: relative L2 %.2e" % (q, err)
