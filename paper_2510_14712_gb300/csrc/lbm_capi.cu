@@ -224,8 +224,8 @@ void set_face_eq(Handle& h, int face) {
   double* eq = face == 0 ? p.eq_lo : p.eq_hi;
   Model<double> m = host_model(h);
   double feq[27], geq[27], u[3] = {st[1], st[2], st[3]};
-  if (h.D == 2) equilibria<2, double>(m, st[0], u, st[4], feq, geq);
-  else equilibria<3, double>(m, st[0], u, st[4], feq, geq);
+  if (h.D == 2) equilibria<2>(m, st[0], u, st[4], feq, geq);
+  else equilibria<3>(m, st[0], u, st[4], feq, geq);
   for (int i = 0; i < h.Q; ++i) {
     eq[i] = feq[i];
     eq[h.Q + i] = geq[i];
@@ -387,8 +387,8 @@ int lbm_create(lbm_t* out, int lattice, int Nx, int Ny, int Nz, const lbm_eos* e
   m = host_model(*h);
   if (h->precision == LBM_FP16DEV) {
     double feq[27], geq[27], u0[3] = {0, 0, 0};
-    if (D == 2) equilibria<2, double>(m, eos->rho_ref, u0, eos->T_ref, feq, geq);
-    else equilibria<3, double>(m, eos->rho_ref, u0, eos->T_ref, feq, geq);
+    if (D == 2) equilibria<2>(m, eos->rho_ref, u0, eos->T_ref, feq, geq);
+    else equilibria<3>(m, eos->rho_ref, u0, eos->T_ref, feq, geq);
     for (int i = 0; i < h->Q; ++i) {
       p.ref[i] = float(feq[i]);
       p.ref[h->Q + i] = float(geq[i]);

@@ -217,43 +217,7 @@ __device__ inline void prim_ext(const Params& p, const double* rho, const double
 }
 
 // ---------------------------------------------------------------------------
-// initialisation: pulled value at every node used by a step = equilibrium of
-// the (extended) initial primitive state there (Fig. FlowChart, Initialize).
-// Thread per source node x in [-G-1, Nx+G] (bounded) or [0, Nx) (periodic);
-// writes A_i(x - c_i) = eq_i(x), which is what node x - c_i + c_i = x pulls.
-// ---------------------------------------------------------------------------
-// (Params as a grid constant: prim_ext takes the address of its inflow state,
-// which would otherwise copy the whole parameter block to local memory)
-template <int D, typename S>
-__global__ void k_init(const __grid_constant__ Params p, typename Store<S>::T* A, const double* rho, const double* u,
-                       const double* T) {
-  using L = Lattice<D>;
-  const int xlo = p.periodic_x ? 0 : -p.G - 1;
-  const int xhi = p.periodic_x ? p.Nx : p.Nx + p.G + 1;
-  int x, y, z;
-  if (!decode(p, blockIdx.x * (long long)blockDim.x + threadIdx.x, xlo, xhi, x, y, z)) return;
-  double r, uu[D], t;
-  prim_ext<D>(p, rho, u, T, x, y, z, r, uu, t);
-  Model<double> m = model_of<double>(p);
-  double feq[L::Q], geq[L::Q];
-  equilibria<D, double>(m, r, uu, t, feq, geq);
-  const int NxP = p.Nx + 2 * p.G;
-#pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    int xs = x - L::c(i, 0) + p.G;
-    if (p.periodic_x) xs = wrap(xs, p.Nx);
-    else if (xs < 0 || xs >= NxP) continue;
-    const int ys = wrap(y - L::c(i, 1), p.Ny);
-    const int zs = D == 3 ? wrap(z - L::c(i, 2), p.Nz) : z;
-    const long long o = node_off(p, xs, ys, zs);
-    if (pop_ok(p, A, i * p.plane + o)) Store<S>::template st<double>(A, i * p.plane + o, feq[i], p.ref[i]);
-    if (pop_ok(p, A, (L::Q + i) * p.plane + o))
-      Store<S>::template st<double>(A, (L::Q + i) * p.plane + o, geq[i], p.ref[L::Q + i]);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// index arithmetic of the split step: flattened node index -> (x, y, z) by
+// index arithmetic: flattened node index -> (x, y, z) by
 // multiplication (Granlund and Montgomery, "Division by invariant integers
 // using multiplication", 1994: exact for n < 2^31)
 // ---------------------------------------------------------------------------
@@ -319,6 +283,116 @@ template <int D> struct PullOffsets {
   }
   __device__ __forceinline__ unsigned operator()(int i) const { return row(i) + x[Lattice<D>::c(i, 0) + 1]; }
 };
+
+// ---------------------------------------------------------------------------
+// initialisation: pulled value at every node used by a step = equilibrium of
+// the (extended) initial primitive state there (Fig. FlowChart, Initialize).
+// Thread per source node x in [-G-1, Nx+G] (bounded) or [0, Nx) (periodic);
+// writes A_i(x - c_i) = eq_i(x), which is what node x - c_i + c_i = x pulls.
+// ---------------------------------------------------------------------------
+// (Params as a grid constant: prim_ext takes the address of its inflow state,
+// which would otherwise copy the whole parameter block to local memory)
+template <int D, typename S>
+__global__ void __launch_bounds__(128) k_init(const __grid_constant__ Params p, typename Store<S>::T* A,
+                                              const double* rho, const double* u, const double* T) {
+  using L = Lattice<D>;
+  const int xlo = p.periodic_x ? 0 : -p.G - 1;
+  const int xhi = p.periodic_x ? p.Nx : p.Nx + p.G + 1;
+  int x, y, z;
+  if (!decode(p, blockIdx.x * (long long)blockDim.x + threadIdx.x, xlo, xhi, x, y, z)) return;
+  double r, uu[D], t;
+  prim_ext<D>(p, rho, u, T, x, y, z, r, uu, t);
+  Model<double> m = model_of<double>(p);
+  const int NxP = p.Nx + 2 * p.G;
+  auto put = [&](int i, int ii, double v) {
+    int xs = x - L::c(i, 0) + p.G;
+    if (p.periodic_x) xs = wrap(xs, p.Nx);
+    else if (xs < 0 || xs >= NxP) return;
+    const int ys = wrap(y - L::c(i, 1), p.Ny);
+    const int zs = D == 3 ? wrap(z - L::c(i, 2), p.Nz) : z;
+    const long long o = ii * p.plane + node_off(p, xs, ys, zs);
+    if (pop_ok(p, A, o)) Store<S>::template st<double>(A, o, v, p.ref[ii]);
+  };
+  equilibria_of<D>(r, uu, eos_pressure(m, r, t) / r, eos_energy(m, r, t), [&](int i, double v) { put(i, i, v); },
+                   [&](int i, double v) { put(i, L::Q + i, v); });
+}
+
+// The same for populations stored in FP32 or less, in packed double-float
+// arithmetic: two nodes per thread, 32 apart, so that every store of a warp is
+// a full line.  The FP64 form is bound by the FP64 pipe (425 instructions per
+// node, 11.4 ms at 256^3 against 0.6 ms of memory traffic); its values, rounded
+// to FP32, are these except where a value lies within 2^-45 of the middle
+// between two FP32 numbers.
+struct InitConsts {
+  float a[2], b[2], R[2], cv[2];             // model constants as high and low parts
+  __host__ explicit InitConsts(const Params& p) {
+    auto split = [](double v, float* s) {
+      s[0] = float(v);
+      s[1] = float(v - double(s[0]));
+    };
+    split(p.a, a);
+    split(p.b, b);
+    split(p.R, R);
+    split(p.cv, cv);
+  }
+};
+
+template <int D, typename S>
+__global__ void __launch_bounds__(128) k_init_df(const __grid_constant__ Params p, const InitConsts c,
+                                                 const NodeRange range, typename Store<S>::T* A, const double* rho,
+                                                 const double* u, const double* T) {
+  using L = Lattice<D>;
+  using ST = typename Store<S>::T;
+  const unsigned gid = blockIdx.x * 256u + (threadIdx.x >> 5) * 64u + (threadIdx.x & 31u);
+  int x[2], y[2], z[2];
+  bool act[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) act[k] = range.decode(gid + 32u * k, x[k], y[k], z[k]);
+  if (!act[0]) return;
+  if (!act[1]) { x[1] = x[0]; y[1] = y[0]; z[1] = z[0]; }
+  double r[2], uu[2][D], t[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) prim_ext<D>(p, rho, u, T, x[k], y[k], z[k], r[k], uu[k], t[k]);
+  DF2 theta, e, ud[D];
+  const DF2 rd = df_of(r[0], r[1]);
+#pragma unroll
+  for (int a = 0; a < D; ++a) ud[a] = df_of(uu[0][a], uu[1][a]);
+  if (p.eos_kind == LBM_EOS_PR) {
+    const Model<double> m = model_of<double>(p);
+    theta = df_of(pr_pressure(m, r[0], t[0]) / r[0], pr_pressure(m, r[1], t[1]) / r[1]);
+    e = df_of(pr_energy(m, r[0], t[0]), pr_energy(m, r[1], t[1]));
+  } else {
+    auto cst = [](const float* v) { return DF2(F2(v[0]), F2(v[1])); };
+    const DF2 td = df_of(t[0], t[1]), ar = cst(c.a) * rd;
+    theta = cst(c.R) * td * df_inverse(DF2(1.f) - cst(c.b) * rd) - ar;         // P / rho of Eq. Pvdw
+    e = cst(c.cv) * td - ar;
+  }
+  // destinations: row offsets and x of both nodes (dropped past the ends of a bounded row)
+  unsigned ro[2][D == 3 ? 9 : 3], xo[2][3];
+  bool in[2][3];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    PullOffsets<D> po;
+    po.rows(p, y[k], z[k]);
+#pragma unroll
+    for (int q = 0; q < (D == 3 ? 9 : 3); ++q) ro[k][q] = po.r[q];
+#pragma unroll
+    for (int cx = -1; cx <= 1; ++cx) {
+      const int xs = p.periodic_x ? wrap(x[k] - cx, p.Nx) : x[k] - cx + p.G;
+      in[k][cx + 1] = act[k] && (p.periodic_x || (xs >= 0 && xs < p.Nx + 2 * p.G));
+      xo[k][cx + 1] = unsigned(xs);
+    }
+  }
+  auto put = [&](int i, int ii, F2 v) {
+    ST* Ai = A + (long long)ii * p.plane;
+    const int q = D == 3 ? 3 * (L::c(i, D - 1) + 1) + L::c(i, 1) + 1 : L::c(i, 1) + 1, cx = L::c(i, 0) + 1;
+    const auto w = Store<S>::pack(v, p.ref[ii]);
+    const unsigned o0 = ro[0][q] + xo[0][cx], o1 = ro[1][q] + xo[1][cx];
+    if (in[0][cx] && pop_ok(p, Ai, o0)) Ai[o0] = Store<S>::half_of(w, 0);
+    if (in[1][cx] && pop_ok(p, Ai, o1)) Ai[o1] = Store<S>::half_of(w, 1);
+  };
+  equilibria_of<D>(rd, ud, theta, e, [&](int i, F2 v) { put(i, i, v); }, [&](int i, F2 v) { put(i, L::Q + i, v); });
+}
 
 // ---------------------------------------------------------------------------
 // split step, pass 1: moments rho, j = sum c f, S = sum g (Eqs. def_h, def_u,
@@ -913,7 +987,7 @@ __device__ inline void ghost_wall_row(const Params& p, typename Store<S>::T* B, 
   double uw[D], feq[L::Q], geq[L::Q];
 #pragma unroll
   for (int a = 0; a < D; ++a) uw[a] = st[1 + a];
-  equilibria<D, double>(model_of<double>(p), rho_e, uw, st[4], feq, geq);
+  equilibria<D>(model_of<double>(p), rho_e, uw, st[4], feq, geq);
   double out = 0.0;
 #pragma unroll
   for (int i = 0; i < L::Q; ++i)
@@ -1297,15 +1371,18 @@ __global__ void k_totals(Params p, const real* M, const real* W, double* partial
   }
 }
 
-// fixed-order sum of the block partials (one thread per component)
+// sum of the block partials in a fixed order: one warp per component, 32 strided
+// partial sums and a butterfly (one thread per component took 57 us for 1024
+// blocks, a chain of dependent loads; 3 us now)
 template <int D>
-__global__ void k_totals_final(const double* partials, int nblocks, double* totals) {
+__global__ void __launch_bounds__(32 * (D + 2)) k_totals_final(const double* partials, int nblocks, double* totals) {
   constexpr int K = D + 2;
-  const int k = threadIdx.x;
-  if (k >= K) return;
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double v = 0.0;
-  for (int b = 0; b < nblocks; ++b) v += partials[b * K + k];
-  totals[k] = v;
+  for (int b = lane; b < nblocks; b += 32) v += partials[b * K + k];
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  if (lane == 0) totals[k] = v;
 }
 
 }  // namespace lbm

@@ -23,8 +23,14 @@ template <int D, typename S, typename real> struct OpsImpl {
 
   static void init(Handle& h, const double* rho, const double* u, const double* T) {
     const Params& p = h.p;
-    const long long n = (long long)(p.periodic_x ? p.Nx : p.Nx + 2 * p.G + 2) * p.Ny * p.Nz;
-    k_init<D, S><<<grid_for(n), kBlock, 0, h.stream>>>(p, reinterpret_cast<ST*>(h.pop[h.cur]), rho, u, T);
+    ST* A = reinterpret_cast<ST*>(h.pop[h.cur]);
+    if constexpr (sizeof(real) == 4) {
+      const NodeRange r = p.periodic_x ? NodeRange(p, 0, p.Nx) : NodeRange(p, -p.G - 1, p.Nx + p.G + 1);
+      k_init_df<D, S><<<unsigned((r.n + 255u) / 256u), 128, 0, h.stream>>>(p, InitConsts(p), r, A, rho, u, T);
+    } else {
+      const long long n = (long long)(p.periodic_x ? p.Nx : p.Nx + 2 * p.G + 2) * p.Ny * p.Nz;
+      k_init<D, S><<<unsigned((n + 127) / 128), 128, 0, h.stream>>>(p, A, rho, u, T);
+    }
     h.launches += 1;
   }
 
@@ -49,9 +55,12 @@ template <int D, typename S, typename real> struct OpsImpl {
     h.launches += 1;
   }
 
+  // blocks of k_prims3 per multiprocessor: 40 registers without a network
+  template <class CL> static constexpr int kPrimsMinB = CL::kWarp ? 1 : (sizeof(real) == 8 ? 3 : 6);
+
   // primitive fields from the moments in scratch (3-D: MINB blocks per
   // multiprocessor for the register budget)
-  template <class CL, int MINB = 1> static void prims(Handle& h) {
+  template <class CL, int MINB = kPrimsMinB<CL>> static void prims(Handle& h) {
     const Params& p = h.p;
     int lo, hi;
     moment_range(p, 1, lo, hi);
@@ -116,7 +125,7 @@ template <int D, typename S, typename real> struct OpsImpl {
   }
 
   // One step in three passes over the box: moments, primitive fields, collision.
-  template <class CL, int MINB = 1> static void split(Handle& h, const void* src, void* dst) {
+  template <class CL, int MINB = kPrimsMinB<CL>> static void split(Handle& h, const void* src, void* dst) {
     moments(h, src);
     prims<CL, MINB>(h);
     if (!collide<(CL::kExtra > 0)>(h, src, dst)) ghosts(h, dst);
@@ -314,7 +323,7 @@ template <int D, typename S, typename real> struct OpsImpl {
       int nb = int((n + kBlock - 1) / kBlock);
       if (nb > kMaxPartials) nb = kMaxPartials;
       k_totals<D, real><<<nb, kBlock, 0, h.stream>>>(p, M(h), W(h), h.partials);
-      k_totals_final<D><<<1, 32, 0, h.stream>>>(h.partials, nb, totals);
+      k_totals_final<D><<<1, 32 * (D + 2), 0, h.stream>>>(h.partials, nb, totals);
       h.launches += 2;
     }
   }

@@ -127,3 +127,25 @@ def test_shock_capturing_tiles_match_oracle(shape, faces, precision, step_kernel
     for q, w in (("rho", want["rho"]), ("u", np.stack(want["u"])), ("T", want["T"])):
         err = rel_l2(got[q], w)
         assert err <= SC_TOL[precision], "%s: relative L2 %.2e" % (q, err)
+
+
+@pytest.mark.parametrize("shape,faces", [((70, 9), "periodic"), ((61, 5), "tube"), ((33, 7, 5), "periodic"), ((40, 3, 6), "tube"),
+                                         ((1, 1), "periodic")])
+def test_initial_populations_round_the_fp64_equilibria(shape, faces):
+    """FP32 handles evaluate the initial equilibria in double-float arithmetic (2^-45 relative): every
+    stored value is the FP64 handle's rounded to FP32, at most one ulp off where it lies that close to
+    the middle of two FP32 numbers (2^-20 of all values; 1e-4 allowed)."""
+    c = _plane(shape, faces)
+    c.rho = c.rho * (1 + 0.3 * np.sin(np.arange(c.rho.size)).reshape(c.rho.shape))
+    pops = {}
+    for prec, dt in (("fp64", np.float64), ("fp32", np.float32)):
+        s = P.Solver(c, precision=prec)
+        try:
+            s.init()
+            pops[prec] = P.lbm_get_populations(s.h).view(dt).copy()
+        finally:
+            s.close()
+    want = pops["fp64"].astype(np.float32)
+    off = pops["fp32"] != want
+    assert off.mean() <= 1e-4
+    assert np.all(np.abs(pops["fp32"] - want) <= np.spacing(np.abs(want)))
