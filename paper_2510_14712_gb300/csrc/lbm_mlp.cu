@@ -1,16 +1,17 @@
 // lbm_mlp.cu - training and standalone evaluation of the learned closure and
 // the lbm_mlp_* interface of include/lbm_mlp.h.
 //
-// One training step is five launches on the network's stream:
-//   k_mlp_batch     draw the minibatch (SplitMix64 indices), exact FP64 labels
+// One training step is two launches on the network's stream:
 //   k_mlp_train_tc  forward pass, backward pass and every weight gradient of
 //                   the minibatch on the fifth-generation tensor cores
 //                   (tcgen05.mma, BF16 hi + lo operands, FP32 accumulators in
 //                   tensor memory): one partial gradient per block
-//   k_mlp_sum       fixed-order sum of the partials (deterministic)
-//   k_mlp_adamw     AdamW update of the FP32 master weights
-//   k_mlp_image     bfloat16 weights, mma fragments and operand images for the
-//                   next forward
+//   k_mlp_update    fixed-order sum of the partials (deterministic), AdamW
+//                   update of the FP32 master weights, their entries of the
+//                   operand images for the next forward; further blocks draw the
+//                   next minibatch (SplitMix64 indices, exact FP64 labels)
+// (k_mlp_batch draws the first one.  With a launch for each part a step took
+// 37 us for 25 us of device time: the launches were the bound.)
 // lbm_mlp_set_mma(LBM_MLP_MMA_WARP) selects the warp-level form instead:
 //   k_mlp_fwd_bwd   per-sample forward and backward pass (mma.sync for the
 //                   64 x 64 products), per-sample factors to memory
@@ -119,11 +120,10 @@ __global__ void k_mlp_image(const float* __restrict__ th, Scale sc, TrainImage* 
   }
 }
 
-__global__ void k_mlp_batch(const double* __restrict__ rho, const double* __restrict__ e, long long n, uint64_t seed,
-                            unsigned long long base, int B, Scale sc, Eos q, float* __restrict__ X,
-                            float* __restrict__ Y) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B) return;
+// sample i of the minibatch starting at draw `base`: its normalised inputs and exact labels
+__device__ __forceinline__ void draw_sample(const double* __restrict__ rho, const double* __restrict__ e, long long n,
+                                            uint64_t seed, unsigned long long base, int i, const Scale& sc, const Eos& q,
+                                            float* __restrict__ X, float* __restrict__ Y) {
   const long long idx = (long long)(splitmix(seed, base + i) % (unsigned long long)n);
   const double r = rho[idx], ee = e[idx];
   double T, P, c2;
@@ -133,6 +133,13 @@ __global__ void k_mlp_batch(const double* __restrict__ rho, const double* __rest
   Y[3 * i] = float((T - sc.v[4]) / sc.v[5]);
   Y[3 * i + 1] = float((P - sc.v[6]) / sc.v[7]);
   Y[3 * i + 2] = float((c2 - sc.v[8]) / sc.v[9]);
+}
+
+__global__ void k_mlp_batch(const double* __restrict__ rho, const double* __restrict__ e, long long n, uint64_t seed,
+                            unsigned long long base, int B, const __grid_constant__ Scale sc, Eos q,
+                            float* __restrict__ X, float* __restrict__ Y) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < B) draw_sample(rho, e, n, seed, base, i, sc, q, X, Y);
 }
 
 // Per-sample forward and backward pass (4 warps per block, 32 samples per
@@ -697,12 +704,11 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ X,
 // record and eight slices of the partials; each thread adds its slice in
 // order, then the slices are added in order.
 constexpr int kSumCols = 32, kSumSlices = 8, kSumBlocks = (kPart + kSumCols - 1) / kSumCols;
-__global__ void __launch_bounds__(kSumCols * kSumSlices)
-    k_mlp_sum(const float* __restrict__ partial, int nchunk, float loss_scale, float* __restrict__ grad,
-              float* __restrict__ loss) {
-  __shared__ double s[kSumSlices][kSumCols + 1];
+// the sum of entry p = 32 blockIdx.x + column, in the threads of slice 0
+__device__ __forceinline__ double sum_partials(const float* __restrict__ partial, int nchunk,
+                                               double (*s)[kSumCols + 1], int& p) {
   const int col = threadIdx.x % kSumCols, sl = threadIdx.x / kSumCols;
-  const int p = blockIdx.x * kSumCols + col;
+  p = blockIdx.x * kSumCols + col;
   double acc = 0.0;
   if (p < kPart) {
     const int per = (nchunk + kSumSlices - 1) / kSumSlices;
@@ -719,26 +725,94 @@ __global__ void __launch_bounds__(kSumCols * kSumSlices)
   }
   s[sl][col] = acc;
   __syncthreads();
-  if (sl == 0 && p < kPart) {
-    double t = 0.0;
+  double t = 0.0;
+  if (sl == 0)
 #pragma unroll
     for (int k = 0; k < kSumSlices; ++k) t += s[k][col];
-    if (p < NPARAM) grad[p] = float(t);
-    else *loss = float(t * loss_scale);
+  return t;
+}
+__global__ void __launch_bounds__(kSumCols * kSumSlices)
+    k_mlp_sum(const float* __restrict__ partial, int nchunk, float loss_scale, float* __restrict__ grad,
+              float* __restrict__ loss) {
+  __shared__ double s[kSumSlices][kSumCols + 1];
+  int p;
+  const double t = sum_partials(partial, nchunk, s, p);
+  if (threadIdx.x >= kSumCols || p >= kPart) return;
+  if (p < NPARAM) grad[p] = float(t);
+  else *loss = float(t * loss_scale);
+}
+
+// The entries of the operand images that hold parameter p (k_mlp_image writes the
+// same from all parameters at once).
+__device__ __forceinline__ void image_entry(int p, float v, TrainImage* img, uint4* w2k) {
+  Image& f = img->fwd;
+  const __nv_bfloat16 hb = __float2bfloat16_rn(v);
+  const float bv = __bfloat162float(hb);
+  if (p < OB1) {
+    reinterpret_cast<float*>(&f.l1[(p - OW1) >> 1])[(p - OW1) & 1] = bv;
+  } else if (p < OW2) {
+    f.l1[p - OB1].z = v;
+  } else if (p < OB2) {
+    const int n = (p - OW2) / H, k = (p - OW2) % H;                  // W2[n][k]
+    // fragment half-word of element (k, n) of a B operand
+    auto frag = [](int k, int n) {
+      return ((((k >> 4) * 8 + (n >> 3)) * 32 + 4 * (n & 7) + ((k & 7) >> 1)) * 2 + ((k >> 3) & 1)) * 2 + (k & 1);
+    };
+    reinterpret_cast<__nv_bfloat16*>(&f.w2f[0][0][0][0])[frag(k, n)] = hb;      // B[k][n] = W2[n][k]
+    reinterpret_cast<__nv_bfloat16*>(&img->w2b[0][0][0][0])[frag(n, k)] = hb;   // B[k][n] = W2[k][n]
+    __nv_bfloat16* w = reinterpret_cast<__nv_bfloat16*>(w2k);
+    w[tc::kmajor_offset(n, k, H) / 2] = hb;
+    w[H * H + tc::kmajor_offset(k, n, H) / 2] = hb;
+  } else if (p < OW3) {
+    f.b2[p - OB2] = v;
+  } else if (p < OB3) {
+    f.w3[(p - OW3) / H][(p - OW3) % H] = bv;
+  } else {
+    f.b3[p - OB3] = v;
   }
 }
 
-// AdamW (Loshchilov and Hutter): bias-corrected moments, decoupled decay
-__global__ void k_mlp_adamw(float* __restrict__ th, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, float lr, float bc1, float bc2, float wd) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= NPARAM) return;
-  const float gi = g[p];
+// One optimiser step: blocks 0 .. kSumBlocks - 1 sum 32 entries of the partial
+// records each (as k_mlp_sum), apply AdamW (Loshchilov and Hutter: bias-corrected
+// moments, decoupled decay) and write the parameters' image entries; the blocks
+// after them draw the next minibatch (kUpdateDraw samples each: the FP64 labels
+// are spread over the multiprocessors).
+constexpr int kUpdateDraw = 64;
+struct Draw {
+  const double *rho, *e;
+  long long n;
+  uint64_t seed;
+  unsigned long long base;
+  int B;                                     // 0: none
+  Eos q;
+};
+__global__ void __launch_bounds__(kSumCols * kSumSlices)
+    k_mlp_update(const float* __restrict__ partial, int nchunk, float loss_scale, float* __restrict__ loss,
+                 float* __restrict__ th, float* __restrict__ m, float* __restrict__ v, float lr, float bc1, float bc2,
+                 float wd, TrainImage* __restrict__ img, uint4* __restrict__ w2k, const __grid_constant__ Draw d,
+                 const __grid_constant__ Scale sc, float* __restrict__ X, float* __restrict__ Y) {
+  __shared__ double s[kSumSlices][kSumCols + 1];
+  if (blockIdx.x >= kSumBlocks) {
+    const int i = (blockIdx.x - kSumBlocks) * kUpdateDraw + threadIdx.x;
+    if (threadIdx.x < kUpdateDraw && i < d.B) draw_sample(d.rho, d.e, d.n, d.seed, d.base, i, sc, d.q, X, Y);
+    return;
+  }
+  int p;
+  const double t = sum_partials(partial, nchunk, s, p);
+  if (threadIdx.x >= kSumCols || p >= kPart) return;
+  if (p == NPARAM) {
+    *loss = float(t * loss_scale);
+    return;
+  }
+  const float gi = float(t);
   const float mi = 0.9f * m[p] + 0.1f * gi;
   const float vi = 0.999f * v[p] + 0.001f * gi * gi;
   m[p] = mi;
   v[p] = vi;
-  th[p] -= lr * ((mi / bc1) / (sqrtf(vi / bc2) + 1e-8f) + wd * th[p]);
+  float w = th[p];
+  w -= lr * ((mi / bc1) / (sqrtf(vi / bc2) + 1e-8f) + wd * w);
+  th[p] = w;
+  image_entry(p, w, img, w2k);
 }
 
 __global__ void k_mlp_minmax(const double* __restrict__ rho, const double* __restrict__ e, long long n, Eos q,
@@ -867,8 +941,8 @@ void launch_image(lbm_mlp_s& n) {
   k_mlp_image<<<(kImageThreads + 255) / 256, 256, 0, n.stream>>>(n.theta, scale_of(n), n.img, n.w2k);
 }
 
-// loss (written to loss_dev) and gradient (n.grad) on the B samples in n.X, n.Y
-int launch_grad(lbm_mlp_s& n, int B, float* loss_dev) {
+// the partial gradient records of the B samples in n.X, n.Y; their number in nchunk
+int launch_partials(lbm_mlp_s& n, int B, int& nchunk) {
   const int ngrp = (B + 31) / 32;
   int blocks = (ngrp + 3) / 4;
   if (blocks > 152 * 8) blocks = 152 * 8;
@@ -885,13 +959,21 @@ int launch_grad(lbm_mlp_s& n, int B, float* loss_dev) {
     const int groups = (B + tcl::kRows - 1) / tcl::kRows;
     const int grid = groups < n.sms ? groups : n.sms;
     k_mlp_train_tc<<<grid, tcl::kThreads, tcl::kSmem, n.stream>>>(n.img, n.w2k, n.X, n.Y, B, n.partial, n.status);
-    k_mlp_sum<<<kSumBlocks, kSumCols * kSumSlices, 0, n.stream>>>(n.partial, grid, inv3B, n.grad, loss_dev);
+    nchunk = grid;
     return LBM_OK;
   }
   k_mlp_fwd_bwd<<<blocks, 128, 0, n.stream>>>(n.img, n.X, n.Y, B, inv3B, n.dY, n.H1, n.dZ1, n.dZ2, n.H2);
-  const int nchunk = (B + kChunk - 1) / kChunk;
+  nchunk = (B + kChunk - 1) / kChunk;
   k_mlp_reduce<<<nchunk, 256, 0, n.stream>>>(n.X, n.H1, n.dZ1, n.dZ2, n.H2, n.dY, B, n.partial);
-  k_mlp_sum<<<kSumBlocks, kSumCols * kSumSlices, 0, n.stream>>>(n.partial, nchunk, inv3B, n.grad, loss_dev);
+  return LBM_OK;
+}
+
+// loss (written to loss_dev) and gradient (n.grad) on the B samples in n.X, n.Y
+int launch_grad(lbm_mlp_s& n, int B, float* loss_dev) {
+  int nchunk = 0;
+  const int rc = launch_partials(n, B, nchunk);
+  if (rc != LBM_OK) return rc;
+  k_mlp_sum<<<kSumBlocks, kSumCols * kSumSlices, 0, n.stream>>>(n.partial, nchunk, float(1.0 / (3.0 * B)), n.grad, loss_dev);
   return LBM_OK;
 }
 
@@ -1117,17 +1199,19 @@ int lbm_mlp_train(lbm_mlp_t net, const double* d_rho, const double* d_e, long lo
     net->loss_cap = steps;
   }
   const Scale sc = scale_of(*net);
+  if (steps > 0)
+    k_mlp_batch<<<(batch + 63) / 64, 64, 0, net->stream>>>(d_rho, d_e, n, seed, 0ull, batch, sc, net->q, net->X, net->Y);
   for (int k = 0; k < steps; ++k) {
     const double lr = lr1 + 0.5 * (lr0 - lr1) * (1.0 + std::cos(M_PI * k / steps));
-    k_mlp_batch<<<(batch + 63) / 64, 64, 0, net->stream>>>(d_rho, d_e, n, seed, (unsigned long long)k * batch,
-                                                                batch, sc, net->q, net->X, net->Y);
-    rc = launch_grad(*net, batch, net->losses + k);
+    int nchunk = 0;
+    rc = launch_partials(*net, batch, nchunk);
     if (rc != LBM_OK) return rc;
     net->t += 1;
     const double bc1 = 1.0 - std::pow(0.9, double(net->t)), bc2 = 1.0 - std::pow(0.999, double(net->t));
-    k_mlp_adamw<<<(NPARAM + 255) / 256, 256, 0, net->stream>>>(net->theta, net->m, net->v, net->grad, float(lr),
-                                                               float(bc1), float(bc2), float(wd));
-    launch_image(*net);
+    const Draw next = {d_rho, d_e, n, seed, (unsigned long long)(k + 1) * batch, k + 1 < steps ? batch : 0, net->q};
+    k_mlp_update<<<kSumBlocks + (next.B + kUpdateDraw - 1) / kUpdateDraw, kSumCols * kSumSlices, 0, net->stream>>>(
+        net->partial, nchunk, float(1.0 / (3.0 * batch)), net->losses + k, net->theta, net->m, net->v, float(lr),
+        float(bc1), float(bc2), float(wd), net->img, net->w2k, next, sc, net->X, net->Y);
   }
   CKM(cudaGetLastError());
   if (losses && steps > 0)
