@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(128) k_mlp_fwd_bwd(const TrainImage* __restric
     const bool valid = s < B;
     const float x0 = valid ? X[2 * s] : 0.f, x1 = valid ? X[2 * s + 1] : 0.f;
     float y[3];
-    forward_warp(w, x0, x1, y);
+    forward_warp<true>(w, x0, x1, y);
     float dy[3], l2 = 0.f;
 #pragma unroll
     for (int o = 0; o < 3; ++o) {

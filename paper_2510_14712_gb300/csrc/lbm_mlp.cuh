@@ -71,6 +71,19 @@ __device__ __forceinline__ float gelu(float z) {
   return __fdividef(z, 1.f + __expf(-2.f * u));
 }
 
+// The same for the fused closure: exp(-2u) as one base-2 exponential with the
+// constants folded and no handling of subnormal results (1 + exp(-2u) lies in
+// [1, 2^116]: below the clamp the exponential is at most 2^115.4): 9 instructions
+// against 19.
+__device__ __forceinline__ float gelu_inf(float z) {
+  constexpr float c0 = -2.f * 1.4426950408889634f * kG0, c1 = c0 * kG1;
+  const float x = fminf(z * fmaf(c1 * z, z, c0), 115.4f);
+  float e, r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
+  return z * r;
+}
+
 // gelu and its derivative: s = sigma(2u), gelu = z s,
 // gelu' = s + z s (1 - s) 2 k0 (1 + 3 k1 z^2)
 __device__ __forceinline__ void gelu_d(float z, float& g, float& dg) {
@@ -105,6 +118,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 // Layer 1 of m-tile rows (g, g+8) in A-operand layout, split into hi / lo.
 // xr[h][i]: input i of row g + 8h.  Register r of k-step ks holds columns
 // 16 ks + 8 (r >> 1) + 2t, +1 of row g + 8 (r & 1).
+template <bool TRAIN>
 __device__ __forceinline__ void layer1_frag(const Image& w, const float (&xr)[2][2], uint32_t (&ah)[4][4],
                                             uint32_t (&al)[4][4]) {
   const int t = threadIdx.x & 3;
@@ -118,7 +132,8 @@ __device__ __forceinline__ void layer1_frag(const Image& w, const float (&xr)[2]
       for (int h = 0; h < 2; ++h) {
         const float za = fmaf(wa.x, xr[h][0], fmaf(wa.y, xr[h][1], wa.z));
         const float zb = fmaf(wb.x, xr[h][0], fmaf(wb.y, xr[h][1], wb.z));
-        split_bf16(gelu(za), gelu(zb), ah[ks][h + 2 * half], al[ks][h + 2 * half]);
+        split_bf16(TRAIN ? gelu(za) : gelu_inf(za), TRAIN ? gelu(zb) : gelu_inf(zb), ah[ks][h + 2 * half],
+                   al[ks][h + 2 * half]);
       }
     }
 }
@@ -126,6 +141,8 @@ __device__ __forceinline__ void layer1_frag(const Image& w, const float (&xr)[2]
 // Network outputs for the 32 nodes of a warp.  Every lane of the warp must
 // call this (mma.sync is warp-collective); (x0, x1) are the lane's own
 // normalised inputs, y its three normalised outputs.
+// TRAIN: the form of gelu whose derivative the training kernels take.
+template <bool TRAIN>
 __device__ __forceinline__ void forward_warp(const Image& w, float x0, float x1, float (&y)[3]) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -139,7 +156,7 @@ __device__ __forceinline__ void forward_warp(const Image& w, float x0, float x1,
       xr[h][1] = __shfl_sync(full, x1, 16 * mt + 8 * h + g);
     }
     uint32_t ah[4][4], al[4][4];
-    layer1_frag(w, xr, ah, al);
+    layer1_frag<TRAIN>(w, xr, ah, al);
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -155,7 +172,7 @@ __device__ __forceinline__ void forward_warp(const Image& w, float x0, float x1,
         mma_bf16(d, al[ks], b.x, b.y);
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) d[q] = gelu(d[q]);
+      for (int q = 0; q < 4; ++q) d[q] = TRAIN ? gelu(d[q]) : gelu_inf(d[q]);
 #pragma unroll
       for (int o = 0; o < 3; ++o) {
         const float w0 = w.w3[o][c], w1 = w.w3[o][c + 1];
@@ -203,7 +220,7 @@ __device__ __forceinline__ bool closure_warp(const Image& w, const Model<float>&
   if (!inr) x0 = x1 = 0.f;
   if (__any_sync(0xffffffffu, inr)) {
     float y[3];
-    forward_warp(w, x0, x1, y);
+    forward_warp<false>(w, x0, x1, y);
     if (inr) {
       T = fmaf(w.norm[5], y[0], w.norm[4]);
       P = fmaf(w.norm[7], y[1], w.norm[6]);
