@@ -120,6 +120,13 @@ __global__ void k_mlp_image(const float* __restrict__ th, Scale sc, TrainImage* 
   }
 }
 
+// The training kernels are launched with programmatic serialisation: a kernel's
+// blocks may start while the launch before it drains, and wait here for that
+// launch's results before their first use.  (On other launches both return at
+// once.)
+__device__ __forceinline__ void wait_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // sample i of the minibatch starting at draw `base`: its normalised inputs and exact labels
 __device__ __forceinline__ void draw_sample(const double* __restrict__ rho, const double* __restrict__ e, long long n,
                                             uint64_t seed, unsigned long long base, int i, const Scale& sc, const Eos& q,
@@ -367,6 +374,16 @@ __global__ void __launch_bounds__(tcl::kThreads, 1)
   const int quad = warp & 3, cp = warp >> 2;
   const int row = 32 * quad + lane, f0 = kFeat * cp;
   const float inv3B = float(1.0 / (3.0 * double(B)));
+  // what needs nothing of the launch before: barrier, tensor memory, the constant
+  // columns of HB: 1 (bfloat16 0x3F80) at column 128, zeros to 143
+  if (tid == 0) tc::mbar_init(bar, 1);
+  if (warp == 0) tc::tmem_alloc(tslot, kCols);
+  if (cp == 0) {
+    *reinterpret_cast<uint4*>(hb + tc::kmajor_offset(row, 128, kCH)) = make_uint4(0x3F80u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(hb + tc::kmajor_offset(row, 136, kCH)) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  wait_previous_launch();
+  allow_next_launch();
   // W2 in both operand layouts (16 KB, consecutive in w2k and in shared memory)
   for (int i = tid; i < 2 * H * H * 2 / 16; i += kThreads) reinterpret_cast<uint4*>(sm + oWF)[i] = __ldg(&w2k[i]);
   // layers 1 and 3 and the biases (read by every thread in every group)
@@ -378,13 +395,6 @@ __global__ void __launch_bounds__(tcl::kThreads, 1)
   } else if (tid < H + 4) {
     ws.b3[tid - H] = w.b3[tid - H];
   }
-  // the constant columns of HB: 1 (bfloat16 0x3F80) at column 128, zeros to 143
-  if (cp == 0) {
-    *reinterpret_cast<uint4*>(hb + tc::kmajor_offset(row, 128, kCH)) = make_uint4(0x3F80u, 0u, 0u, 0u);
-    *reinterpret_cast<uint4*>(hb + tc::kmajor_offset(row, 136, kCH)) = make_uint4(0u, 0u, 0u, 0u);
-  }
-  if (tid == 0) tc::mbar_init(bar, 1);
-  if (warp == 0) tc::tmem_alloc(tslot, kCols);
   tc::fence_smem_to_async();
   tc::fence_before_sync();
   __syncthreads();
@@ -792,6 +802,8 @@ __global__ void __launch_bounds__(kSumCols * kSumSlices)
                  float wd, TrainImage* __restrict__ img, uint4* __restrict__ w2k, const __grid_constant__ Draw d,
                  const __grid_constant__ Scale sc, float* __restrict__ X, float* __restrict__ Y) {
   __shared__ double s[kSumSlices][kSumCols + 1];
+  wait_previous_launch();
+  allow_next_launch();
   if (blockIdx.x >= kSumBlocks) {
     const int i = (blockIdx.x - kSumBlocks) * kUpdateDraw + threadIdx.x;
     if (threadIdx.x < kUpdateDraw && i < d.B) draw_sample(d.rho, d.e, d.n, d.seed, d.base, i, sc, d.q, X, Y);
@@ -941,6 +953,23 @@ void launch_image(lbm_mlp_s& n) {
   k_mlp_image<<<(kImageThreads + 255) / 256, 256, 0, n.stream>>>(n.theta, scale_of(n), n.img, n.w2k);
 }
 
+// a launch that may overlap the end of the one before it on the stream (its kernel
+// calls wait_previous_launch before it reads or writes what that one touches)
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // the partial gradient records of the B samples in n.X, n.Y; their number in nchunk
 int launch_partials(lbm_mlp_s& n, int B, int& nchunk) {
   const int ngrp = (B + 31) / 32;
@@ -958,7 +987,8 @@ int launch_partials(lbm_mlp_s& n, int B, int& nchunk) {
     // one block per SM (all 512 TMEM columns), every block at least one group
     const int groups = (B + tcl::kRows - 1) / tcl::kRows;
     const int grid = groups < n.sms ? groups : n.sms;
-    k_mlp_train_tc<<<grid, tcl::kThreads, tcl::kSmem, n.stream>>>(n.img, n.w2k, n.X, n.Y, B, n.partial, n.status);
+    CKM(launch_overlapped(k_mlp_train_tc, grid, tcl::kThreads, tcl::kSmem, n.stream, n.img, n.w2k, n.X, n.Y, B, n.partial,
+                          n.status));
     nchunk = grid;
     return LBM_OK;
   }
@@ -1209,9 +1239,10 @@ int lbm_mlp_train(lbm_mlp_t net, const double* d_rho, const double* d_e, long lo
     net->t += 1;
     const double bc1 = 1.0 - std::pow(0.9, double(net->t)), bc2 = 1.0 - std::pow(0.999, double(net->t));
     const Draw next = {d_rho, d_e, n, seed, (unsigned long long)(k + 1) * batch, k + 1 < steps ? batch : 0, net->q};
-    k_mlp_update<<<kSumBlocks + (next.B + kUpdateDraw - 1) / kUpdateDraw, kSumCols * kSumSlices, 0, net->stream>>>(
-        net->partial, nchunk, float(1.0 / (3.0 * batch)), net->losses + k, net->theta, net->m, net->v, float(lr),
-        float(bc1), float(bc2), float(wd), net->img, net->w2k, next, sc, net->X, net->Y);
+    CKM(launch_overlapped(k_mlp_update, kSumBlocks + (next.B + kUpdateDraw - 1) / kUpdateDraw, kSumCols * kSumSlices, 0,
+                          net->stream, net->partial, nchunk, float(1.0 / (3.0 * batch)), net->losses + k, net->theta,
+                          net->m, net->v, float(lr), float(bc1), float(bc2), float(wd), net->img, net->w2k, next, sc,
+                          net->X, net->Y));
   }
   CKM(cudaGetLastError());
   if (losses && steps > 0)
