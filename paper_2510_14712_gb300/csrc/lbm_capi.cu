@@ -393,6 +393,11 @@ int lbm_create(lbm_t* out, int lattice, int Nx, int Ny, int Nz, const lbm_eos* e
       p.ref[i] = float(feq[i]);
       p.ref[h->Q + i] = float(geq[i]);
     }
+    for (int k = 0; k < 2; ++k) {
+      double sum = 0.0;
+      for (int i = 0; i < h->Q; ++i) sum += double(p.ref[k * h->Q + i]);
+      p.refsum[k] = float(sum);
+    }
   }
   int rc;
   cudaError_t ae = dev_malloc(&h->partials, kMaxPartials * 5 * sizeof(double));

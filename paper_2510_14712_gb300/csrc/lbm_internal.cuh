@@ -35,6 +35,7 @@ struct Params {
   double eq_lo[54], eq_hi[54];   // f then g
   // FP16-deviation reference populations (f then g)
   float ref[54];
+  float refsum[2];               // their sums over f and over g
   // learned closure: device inference image (mlp::Image), NULL for the exact closure
   const void* mlp;
   // shock capturing (Sec. 4.4): on/off, coefficients C_mu, C_eta, C_k; the step

@@ -53,11 +53,13 @@ template <> struct Store<float> {
   __device__ static Raw pack(F2 v, float) { return v; }
   __device__ static T half_of(Raw q, int k) { return k ? q.y : q.x; }
   __device__ static void st2_raw(T* p, Raw q) { __stcs(reinterpret_cast<float2*>(p), f2_in(q)); }
-  // four consecutive values p[o .. o+3], o a multiple of 4 (one 16-byte load)
-  template <typename real, typename I> __device__ static void ld4(const T* p, I o, float, real* v) {
-    const float4 q = __ldg(reinterpret_cast<const float4*>(p + o));
-    v[0] = real(q.x); v[1] = real(q.y); v[2] = real(q.z); v[3] = real(q.w);
+  // the values of one 16-byte load, as stored; one value
+  static constexpr int kGroup = 4;
+  __device__ static void group(const T* p, float* v) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
   }
+  __device__ static float deviation(const T* p) { return __ldg(p); }
 };
 template <> struct Store<Fp16Dev> {
   using T = __half;
@@ -102,13 +104,19 @@ template <> struct Store<Fp16Dev> {
   __device__ static void st2_raw(T* p, Raw q) {
     __stcs(reinterpret_cast<unsigned*>(p), *reinterpret_cast<const unsigned*>(&q));
   }
-  // four consecutive values p[o .. o+3], o a multiple of 4 (one 8-byte load)
-  template <typename real, typename I> __device__ static void ld4(const T* p, I o, float ref, real* v) {
-    const uint2 q = __ldg(reinterpret_cast<const uint2*>(p + o));
-    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q.x));
-    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&q.y));
-    v[0] = real(a.x + ref); v[1] = real(a.y + ref); v[2] = real(b.x + ref); v[3] = real(b.y + ref);
+  // the deviations of one 16-byte load, without the reference; one deviation
+  static constexpr int kGroup = 8;
+  __device__ static void group(const T* p, float* v) {
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(p));
+    const unsigned w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[k]));
+      v[2 * k] = f.x;
+      v[2 * k + 1] = f.y;
+    }
   }
+  __device__ static float deviation(const T* p) { return __half2float(__ldg(p)); }
 };
 
 // ---------------------------------------------------------------------------
@@ -398,89 +406,147 @@ __global__ void __launch_bounds__(128) k_init_df(const __grid_constant__ Params 
 // split step, pass 1: moments rho, j = sum c f, S = sum g (Eqs. def_h, def_u,
 // def_E) of the pulled populations, on the interior plus 3 ghost layers.
 // M planes: rho, j_0..j_{D-1}, S   (each p.plane elements, padded layout)
-// j_a is (sum over c_a = +1) minus (sum over c_a = -1), both in increasing
-// direction order: exactly zero for mirror-symmetric populations.
-// One read of every population bounds it.  QUAD (FP32 and FP16-deviation
-// storage, Nx and the ghost width multiples of 4): a thread takes four nodes,
-// one 16- (8-) byte load per direction and one scalar load for the node that a
-// +-x pull needs from outside the four.
+// Each component of j is (sum over c_a = +1) minus (sum over c_a = -1), the two
+// summed in the same order: exactly zero for mirror-symmetric populations.
+// One read of every population bounds it.
 // ---------------------------------------------------------------------------
-template <int D, typename S, typename real, bool QUAD>
+// FP64: one node per thread
+template <int D>
 __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params p, const NodeRange range,
-                                                 const typename Store<S>::T* __restrict__ A, real* __restrict__ M) {
+                                                 const double* __restrict__ A, double* __restrict__ M) {
   using L = Lattice<D>;
-  using ST = typename Store<S>::T;
-  constexpr int N = QUAD ? 4 : 1;
   int xp, y, z;
   if (!range.decode(blockIdx.x * blockDim.x + threadIdx.x, xp, y, z)) return;
-  PullOffsets<D> po(p, xp, y, z);
-  // QUAD: the node left of the four (c_x = +1) and right of them (c_x = -1),
-  // kept inside the row where the pulled value is not used (the outermost
-  // ghost node of a row)
-  unsigned xl = 0, xr = 0;
-  if constexpr (QUAD) {
-    xl = unsigned(p.periodic_x ? wrap(xp - 1, p.Nx) : max(xp - 1, 0));
-    xr = unsigned(p.periodic_x ? wrap(xp + 4, p.Nx) : min(xp + 4, p.Nx + 2 * p.G - 1));
-  }
-  auto pulled = [&](const int i, const int ii, real* v) {
-    const ST* Ai = A + (long long)ii * p.plane;
-    if constexpr (!QUAD) {
-      const unsigned o = po(i);
-      v[0] = pop_ok(p, Ai, o) ? Store<S>::template ld<real>(Ai, o, p.ref[ii]) : real(0);
-    } else {
-      const int cx = L::c(i, 0);
-      const unsigned r = po.row(i);
-      real w[4] = {real(0), real(0), real(0), real(0)}, e = real(0);
-      if (pop_ok(p, Ai, r + xp, 4)) Store<S>::template ld4<real>(Ai, r + unsigned(xp), p.ref[ii], w);
-      if (cx != 0 && pop_ok(p, Ai, r + (cx > 0 ? xl : xr)))
-        e = Store<S>::template ld<real>(Ai, r + (cx > 0 ? xl : xr), p.ref[ii]);
-      if (cx > 0) { v[0] = e; v[1] = w[0]; v[2] = w[1]; v[3] = w[2]; }
-      else if (cx < 0) { v[0] = w[1]; v[1] = w[2]; v[2] = w[3]; v[3] = e; }
-      else { v[0] = w[0]; v[1] = w[1]; v[2] = w[2]; v[3] = w[3]; }
-    }
+  const PullOffsets<D> po(p, xp, y, z);
+  auto pulled = [&](const int i, const int ii) {
+    const double* Ai = A + (long long)ii * p.plane;
+    return pop_ok(p, Ai, po(i)) ? __ldg(Ai + po(i)) : 0.0;
   };
   const unsigned o = po.r[D == 3 ? 4 : 1] + unsigned(xp);
-  auto put = [&](const int k, const real* v) {
-    real* dst = M + (long long)k * p.plane + o;
-    if constexpr (QUAD) *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-    else dst[0] = v[0];
-  };
-  real acc[N], sp[D][N], sn[D][N], v[N];
+  double rho = 0.0, S = 0.0, sp[D], sn[D];
 #pragma unroll
-  for (int j = 0; j < N; ++j) {
-    acc[j] = real(0);
-#pragma unroll
-    for (int a = 0; a < D; ++a) sp[a][j] = sn[a][j] = real(0);
-  }
+  for (int a = 0; a < D; ++a) sp[a] = sn[a] = 0.0;
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
-    pulled(i, i, v);
+    const double v = pulled(i, i);
+    rho += v;
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-      acc[j] += v[j];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        if (L::c(i, a) == 1) sp[a][j] += v[j];
-        if (L::c(i, a) == -1) sn[a][j] += v[j];
-      }
+    for (int a = 0; a < D; ++a) {
+      if (L::c(i, a) == 1) sp[a] += v;
+      if (L::c(i, a) == -1) sn[a] += v;
     }
   }
-  put(0, acc);
 #pragma unroll
-  for (int a = 0; a < D; ++a) {
+  for (int i = 0; i < L::Q; ++i) S += pulled(i, L::Q + i);
+  M[o] = rho;
 #pragma unroll
-    for (int j = 0; j < N; ++j) v[j] = sp[a][j] - sn[a][j];
-    put(1 + a, v);
+  for (int a = 0; a < D; ++a) M[(1 + a) * p.plane + o] = sp[a] - sn[a];
+  M[(1 + D) * p.plane + o] = S;
+}
+
+// FP32 arithmetic: the nodes of one 16-byte load (4 FP32, 8 FP16-deviation
+// values) per thread, packed sums; a direction with c_x != 0 takes one scalar
+// load for the node pulled from outside the group.  FP16-deviation: the stored
+// deviations are summed and the reference populations' sum added once (in j the
+// references of mirrored directions cancel).  RAGGED: a row's last group holds
+// fewer nodes, its last one pulls across the seam.  With four nodes (8-byte
+// loads) FP16-deviation issued as many loads as FP32 for half the bytes: 584 us
+// at 256^3, against FP32's 560 (7 TB/s).
+template <int D, typename S, bool RAGGED>
+__global__ void __launch_bounds__(128) k_moments_row(const __grid_constant__ Params p, const NodeRange range,
+                                                     const typename Store<S>::T* __restrict__ A,
+                                                     float* __restrict__ M) {
+  using L = Lattice<D>;
+  using ST = typename Store<S>::T;
+  constexpr int N = Store<S>::kGroup, H = N / 2, T3 = L::Q / 3;
+  int xp, y, z;
+  if (!range.decode(blockIdx.x * blockDim.x + threadIdx.x, xp, y, z)) return;
+  PullOffsets<D> po;
+  po.rows(p, y, z);
+  // the node that pulls from right of the group, and the sources left and right
+  // (kept inside the row where the pulled value is not used)
+  const int last = RAGGED && p.periodic_x ? min(N, p.Nx - xp) - 1 : N - 1;
+  const unsigned xl = unsigned(p.periodic_x ? wrap(xp - 1, p.Nx) : max(xp - 1, 0));
+  const unsigned xr = unsigned(p.periodic_x ? wrap(xp + last + 1, p.Nx) : min(xp + N, p.pitch - 1));
+  const unsigned o = po.r[D == 3 ? 4 : 1] + unsigned(xp);
+  auto put = [&](const int k, const F2* v) {
+    float* dst = M + (long long)k * p.plane + o;
+#pragma unroll
+    for (int q = 0; q < H; q += 2) *reinterpret_cast<float4*>(dst + 2 * q) = make_float4(v[q].x, v[q].y, v[q + 1].x, v[q + 1].y);
+  };
+  // the group's values of direction i, as pulled
+  auto pulled = [&](const int i, const int ii, F2* v) {
+    const int cx = L::c(i, 0);
+    const ST* Ai = A + (long long)ii * p.plane + po.row(i);
+    float w[N], e = 0.f;
+    if (pop_ok(p, Ai, xp, N)) Store<S>::group(Ai + xp, w);
+    else
+#pragma unroll
+      for (int j = 0; j < N; ++j) w[j] = 0.f;
+    if (cx != 0 && pop_ok(p, Ai, cx > 0 ? xl : xr)) e = Store<S>::deviation(Ai + (cx > 0 ? xl : xr));
+    float q[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      if (cx > 0) q[j] = j == 0 ? e : w[j - (j > 0)];
+      else if (cx < 0) q[j] = j == N - 1 ? e : (RAGGED && j == last ? e : w[j + (j < N - 1)]);
+      else q[j] = w[j];
+    }
+#pragma unroll
+    for (int j = 0; j < H; ++j) v[j] = F2(q[2 * j], q[2 * j + 1]);
+  };
+  F2 rho[H], jx[H], sp[2][H], sn[2][H], b[H], v[H];
+#pragma unroll
+  for (int j = 0; j < H; ++j) {
+    rho[j] = jx[j] = F2(0.f);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) sp[a][j] = sn[a][j] = F2(0.f);
   }
 #pragma unroll
-  for (int j = 0; j < N; ++j) acc[j] = real(0);
+  for (int c = 0; c < 3; ++c) {                              // the directions of one c_x
+#pragma unroll
+    for (int j = 0; j < H; ++j) b[j] = F2(0.f);
+#pragma unroll
+    for (int k = 0; k < T3; ++k) {
+      const int i = c * T3 + k;
+      pulled(i, i, v);
+#pragma unroll
+      for (int j = 0; j < H; ++j) {
+        b[j] += v[j];
+#pragma unroll
+        for (int a = 1; a < D; ++a) {
+          if (L::c(i, a) == 1) sp[a - 1][j] += v[j];
+          if (L::c(i, a) == -1) sn[a - 1][j] += v[j];
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      rho[j] += b[j];
+      if (c == 0) jx[j] = b[j];                              // c_x = -1
+      if (c == 2) jx[j] = b[j] - jx[j];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < H; ++j) {
+    rho[j] += F2(p.refsum[0]);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) sp[a][j] = sp[a][j] - sn[a][j];
+  }
+  put(0, rho);
+  put(1, jx);
+#pragma unroll
+  for (int a = 1; a < D; ++a) put(1 + a, sp[a - 1]);
+#pragma unroll
+  for (int j = 0; j < H; ++j) rho[j] = F2(0.f);
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
     pulled(i, L::Q + i, v);
 #pragma unroll
-    for (int j = 0; j < N; ++j) acc[j] += v[j];
+    for (int j = 0; j < H; ++j) rho[j] += v[j];
   }
-  put(1 + D, acc);
+#pragma unroll
+  for (int j = 0; j < H; ++j) rho[j] += F2(p.refsum[1]);
+  put(1 + D, rho);
 }
 
 // neighbour offset along axis a by s (wrapping periodic axes)
@@ -563,7 +629,7 @@ __device__ __forceinline__ void prims_node(const Params& p, const Model<real>& m
 template <int D, typename real, class CL>
 __global__ void __launch_bounds__(256) k_prims(const __grid_constant__ Params p, const NodeRange range,
                                                const real* __restrict__ M, real* __restrict__ W) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   CL closure;
   closure.load(p, smem_raw);
   if constexpr (CL::kSmem > 0) __syncthreads();
@@ -610,7 +676,7 @@ __global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_c
   constexpr int NT = kPrimX * kPrimY, BX2 = kPrimX + 4, BX1 = kPrimX + 2;
   constexpr int N2 = BX2 * (kPrimY + 4), N1 = BX1 * (kPrimY + 2), K2 = (N2 + NT - 1) / NT, K1 = (N1 + NT - 1) / NT;
   __shared__ PrimsSmem<real, CL> sm;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   CL closure;
   closure.load(p, smem_raw);
   const Model<real> m = model_of<real>(p);

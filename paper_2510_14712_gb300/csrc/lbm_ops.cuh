@@ -41,17 +41,15 @@ template <int D, typename S, typename real> struct OpsImpl {
     moment_range(p, 3, lo, hi);
     const ST* A = reinterpret_cast<const ST*>(src);
     if constexpr (sizeof(real) == 4) {
-      // four nodes per thread: chunks of four never straddle the periodic seam
-      // and start on 16-byte boundaries
-      if (p.Nx % 4 == 0) {
-        const NodeRange r(p, lo - lo % 4, hi + (4 - hi % 4) % 4, 4);
-        k_moments<D, S, real, true><<<grid_for(r.n), kBlock, 0, h.stream>>>(p, r, A, M(h));
-        h.launches += 1;
-        return;
-      }
+      // groups start at multiples of 16 bytes of the padded row
+      constexpr int N = Store<S>::kGroup;
+      const NodeRange r(p, 0, p.Nx + 2 * p.G, N);
+      auto kern = p.Nx % N ? k_moments_row<D, S, true> : k_moments_row<D, S, false>;
+      kern<<<unsigned((r.n + 127u) / 128u), 128, 0, h.stream>>>(p, r, A, M(h));
+    } else {
+      const NodeRange r(p, lo, hi);
+      k_moments<D><<<grid_for(r.n), kBlock, 0, h.stream>>>(p, r, A, M(h));
     }
-    const NodeRange r(p, lo, hi);
-    k_moments<D, S, real, false><<<grid_for(r.n), kBlock, 0, h.stream>>>(p, r, A, M(h));
     h.launches += 1;
   }
 

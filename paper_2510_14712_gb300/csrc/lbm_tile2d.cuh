@@ -301,7 +301,7 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
   // ---------------- C: force and primitive fields on radius 1 ------------------
   // unit (bu, br) of the radius-1 box with its moments; returns rho-independent
   // results through F, T (and P, c_s^2 of closures that hand them on)
-  auto prims = [&](int bu, int br, V rho, const V* j, V S, bool act, V* F, V* u, V& T, V& P, V& cs2) {
+  auto prims = [&](int bu, int br, V rho, const V* j, V Sg, bool act, V* F, V* u, V& T, V& P, V& cs2) {
     const real* l = s_lap + (br + 1) * G::P2 + N * (bu + G::U2 - G::U1);
     const V kr = V(m.kappa) * rho * V(real(0.5)), lc = U::ld(l);
     F[0] = kr * (U::right(l, lc) - U::left(l, lc));                                      // Eq. FK
@@ -315,7 +315,7 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
       uF = mad(u[a], F[a], uF);
       u2 = mad(u[a], u[a], u2);
     }
-    const V n = mad(V(real(0.5)), uF, S);
+    const V n = mad(V(real(0.5)), uF, Sg);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       U::set(E, k, div_rn(U::get(n, k), U::get(rho, k)));                                // Eq. def_E
@@ -468,7 +468,7 @@ template <typename S, typename real, class CL, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(TX / Unit<S, real>::N * TY, MINB)
 k_step2d(const __grid_constant__ Params p, const typename Store<S>::T* __restrict__ A,
          typename Store<S>::T* __restrict__ B, unsigned* err, int ntx) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   using G = TileGeom<real, Unit<S, real>::N, TX, TY>;
   CL closure;
   closure.load(p, smem_raw + G::kBytes);                // (stage A's barrier covers it)
@@ -495,7 +495,7 @@ template <typename S, typename real, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(TX / Unit<S, real>::N * TY, MINB)
 k_step2d_batch(const BatchInstance* __restrict__ insts, const BatchItem* __restrict__ items, int parity,
                unsigned* errs) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   using ST = typename Store<S>::T;
   const BatchItem it = items[blockIdx.x];
   const BatchInstance& bi = insts[it.inst];
