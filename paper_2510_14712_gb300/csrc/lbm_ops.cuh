@@ -145,8 +145,9 @@ template <int D, typename S, typename real> struct OpsImpl {
   }
 
   // One tile shape of the 2-D step (TX x TY nodes per block, MINB blocks per
-  // multiprocessor for the register budget) with thermodynamic closure CL.
-  template <int TX, int TY, int MINB, class CL> struct Tile {
+  // multiprocessor for the register budget, HELP threads beyond the tile's units)
+  // with thermodynamic closure CL.
+  template <int TX, int TY, int MINB, class CL, int HELP = 0> struct Tile {
     using G = TileGeom<real, Unit<S, real>::N, TX, TY>;
     static constexpr size_t kSmem = G::kBytes + CL::kSmem;
     static long long tiles(const Params& p) {
@@ -157,10 +158,10 @@ template <int D, typename S, typename real> struct OpsImpl {
     static double work() { return G::P3 * G::H3 * 1.0 + G::P1 * G::H1 * 6.0 + TX * TY * 20.0; }
     static void launch(Handle& h, const void* src, void* dst) {
       const Params& p = h.p;
-      auto kern = k_step2d<S, real, CL, TX, TY, MINB>;
+      auto kern = k_step2d<S, real, CL, TX, TY, HELP, MINB>;
       static const cudaError_t ready = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
       (void)ready;
-      kern<<<unsigned(tiles(p)), G::NT, kSmem, h.stream>>>(p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
+      kern<<<unsigned(tiles(p)), G::NT + HELP, kSmem, h.stream>>>(p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
                                                           h.err_dev, (p.Nx + TX - 1) / TX);
       h.launches += 1;
       wall_ghosts(h, dst);
@@ -225,7 +226,8 @@ template <int D, typename S, typename real> struct OpsImpl {
       : TileSet<CL, Tile<64, 8, CL::kWarp ? 1 : 2, CL>, Tile<64, 4, 4, CL>, Tile<32, 8, 4, CL>,
                 Tile<16, 8, 8, CL>> {};
   template <class CL> struct Tiles<CL, true>
-      : TileSet<CL, Tile<32, 8, 1, CL>, Tile<32, 4, 2, CL>, Tile<16, 4, 4, CL>, Tile<16, 2, 4, CL>, Tile<8, 4, 4, CL>> {};
+      : TileSet<CL, Tile<32, 8, 1, CL>, Tile<32, 4, 2, CL>, Tile<16, 4, 2, CL, 64>, Tile<16, 2, 2, CL, 96>,
+                Tile<8, 4, 2, CL, 96>> {};
 
   static void ghosts(Handle& h, void* dst) {
     const Params& p = h.p;

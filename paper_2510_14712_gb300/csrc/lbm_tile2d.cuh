@@ -150,7 +150,12 @@ struct Ring {
 };
 
 // kNorms: with shock capturing on, leave S and |grad s| for k_n1_coef_2d
-template <typename S, typename real, class CL, int TX, int TY, bool kNorms>
+// HELP: threads of the block beyond the tile's units.  They take the halo first,
+// next to the warps that own the units: where a small plane leaves a block a
+// multiprocessor of its own, its time is the chain of loads and divisions of a
+// unit, not their number (FP64 1000x4: 26 us with the owners doing the halo
+// after their own units).
+template <typename S, typename real, class CL, int TX, int TY, int HELP, bool kNorms>
 __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>::T* __restrict__ A,
                                        typename Store<S>::T* __restrict__ B, const int x0, const int y0, real* sm,
                                        unsigned& flags, const CL& closure) {
@@ -161,7 +166,10 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
   constexpr int N = U::N, Q = L::Q;
   using G = TileGeom<real, N, TX, TY>;
   real *s_rho = sm, *s_lap = sm + G::oLap, *s_prm = sm + G::oPrm, *s_own = sm + G::oOwn;
+  constexpr int NTB = G::NT + HELP;
   const int tid = threadIdx.x, ux = tid % (TX / N), uy = tid / (TX / N);
+  const bool own = HELP == 0 || tid < G::NT;
+  const int rank = HELP == 0 ? tid : (own ? tid + HELP : tid - G::NT);       // order in which the halo is taken
   const Model<real> m = model_of<real>(p);
   const bool wtile = (p.bc_lo == LBM_BC_WALL && x0 < 4) || (p.bc_hi == LBM_BC_WALL && x0 + TX + 4 > p.Nx);
   // padded x of any box coordinate: wrapped (images past the seam are the nodes
@@ -255,10 +263,12 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
   unsigned ro[3];
   rows3(gy, ro);
   typename U::Raw f[Q], g[Q];
-  pull_set(xo, ro, 0, f);
-  pull_set(xo, ro, Q, g);
+  if (own) {
+    pull_set(xo, ro, 0, f);
+    pull_set(xo, ro, Q, g);
+  }
   const Ring ring3{G::P3 / N, G::H3, G::U3, 3};
-  for (int k = tid; k < ring3.count(); k += G::NT) {
+  for (int k = rank; k < ring3.count(); k += NTB) {
     int bu, br;
     ring3.at(k, bu, br);
     const int hx = x0 + N * (bu - G::U3), hy = y0 + br - 3;
@@ -282,14 +292,16 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
       U::st(d + 2 * G::P1 * G::H1, energy(v));
     }
   }
-  V rho, j[2];
-  sums(f, rho, j);
-  const V Se = energy(g);
-  U::st(s_rho + (uy + 3) * G::P3 + N * (ux + G::U3), wtile ? capillary(rho, gx, gy, uy + 1) : rho);
+  V rho, j[2], Se = V(0);
+  if (own) {
+    sums(f, rho, j);
+    Se = energy(g);
+    U::st(s_rho + (uy + 3) * G::P3 + N * (ux + G::U3), wtile ? capillary(rho, gx, gy, uy + 1) : rho);
+  }
   __syncthreads();
 
   // ---------------- B: Laplacian of rho on radius 2 ----------------------------
-  for (int k = tid; k < G::P2 / N * G::H2; k += G::NT) {
+  for (int k = tid; k < G::P2 / N * G::H2; k += NTB) {
     const int br = k / (G::P2 / N), bu = k - br * (G::P2 / N);
     const real* r = s_rho + (br + 1) * G::P3 + N * (bu + G::U3 - G::U2);
     const V c = U::ld(r), c2 = c + c;
@@ -340,7 +352,7 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
     put(G::PH, e + theta);                                                               // Eq. enthalpy
   };
   const Ring ring1{G::P1 / N, G::H1, G::U1, 1};
-  for (int k = tid; CL::kWarp ? k - (tid & 31) < ring1.count() : k < ring1.count(); k += G::NT) {
+  for (int k = rank; CL::kWarp ? k - (tid & 31) < ring1.count() : k < ring1.count(); k += NTB) {
     int bu = 0, br = 0;
     if (k < ring1.count()) ring1.at(k, bu, br);
     const bool corner = (br == 0 || br == G::H1 - 1) && (bu == 0 || bu == G::P1 / N - 1);
@@ -365,11 +377,11 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
   }
   NodeState<2, V> s;
   s.rho = rho;
-  prims(ux + G::U1, uy + 1, rho, j, Se, true, s.F, s.u, s.T, s.P, s.cs2);
+  if (own) prims(ux + G::U1, uy + 1, rho, j, Se, true, s.F, s.u, s.T, s.P, s.cs2);
   __syncthreads();
 
   // ---------------- D: derivatives and collision -------------------------------
-  const bool act = gx < p.Nx && gy < p.Ny, two = gx + N - 1 < p.Nx;
+  const bool act = own && gx < p.Nx && gy < p.Ny, two = gx + N - 1 < p.Nx;
   if (act) {
     const unsigned o = unsigned(gy) * unsigned(p.pitch) + unsigned(gx + p.G);
     s.sc = p.sc_on != 0;
@@ -456,7 +468,7 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
     const bool first = x0 == 0 && p.bc_lo != LBM_BC_WALL, last = x0 <= p.Nx - 1 && p.Nx - 1 < x0 + TX && p.bc_hi != LBM_BC_WALL;
     if (first || last) {
       __syncthreads();                                  // the tile's new populations are written
-      for (int k = tid; k < 2 * Q * TY; k += G::NT) {
+      for (int k = tid; k < 2 * Q * TY; k += NTB) {
         const int i = k / TY, y = y0 + k - i * TY;
         if (y < p.Ny) ghost_row<2, S>(p, B + (long long)i * p.plane + (long long)y * p.pitch, i, first, last);
       }
@@ -464,8 +476,8 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
   }
 }
 
-template <typename S, typename real, class CL, int TX, int TY, int MINB>
-__global__ void __launch_bounds__(TX / Unit<S, real>::N * TY, MINB)
+template <typename S, typename real, class CL, int TX, int TY, int HELP, int MINB>
+__global__ void __launch_bounds__(TX / Unit<S, real>::N * TY + HELP, MINB)
 k_step2d(const __grid_constant__ Params p, const typename Store<S>::T* __restrict__ A,
          typename Store<S>::T* __restrict__ B, unsigned* err, int ntx) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -473,7 +485,7 @@ k_step2d(const __grid_constant__ Params p, const typename Store<S>::T* __restric
   CL closure;
   closure.load(p, smem_raw + G::kBytes);                // (stage A's barrier covers it)
   unsigned flags = 0;
-  tile2d<S, real, CL, TX, TY, true>(p, A, B, int(blockIdx.x % unsigned(ntx)) * TX, int(blockIdx.x / unsigned(ntx)) * TY,
+  tile2d<S, real, CL, TX, TY, HELP, true>(p, A, B, int(blockIdx.x % unsigned(ntx)) * TX, int(blockIdx.x / unsigned(ntx)) * TY,
                               reinterpret_cast<real*>(smem_raw), flags, closure);
   if (flags) atomicOr(err, flags);
 }
@@ -500,7 +512,7 @@ k_step2d_batch(const BatchInstance* __restrict__ insts, const BatchItem* __restr
   const BatchItem it = items[blockIdx.x];
   const BatchInstance& bi = insts[it.inst];
   unsigned flags = 0;
-  tile2d<S, real, ExactClosure<real>, TX, TY, false>(bi.p, reinterpret_cast<const ST*>(bi.pop[parity]),
+  tile2d<S, real, ExactClosure<real>, TX, TY, 0, false>(bi.p, reinterpret_cast<const ST*>(bi.pop[parity]),
                                               reinterpret_cast<ST*>(bi.pop[parity ^ 1]), it.x0, it.y0,
                                               reinterpret_cast<real*>(smem_raw), flags, ExactClosure<real>{});
   if (flags) atomicOr(errs + it.inst, flags);
