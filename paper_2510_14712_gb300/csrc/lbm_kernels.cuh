@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(128) k_init_df(const __grid_constant__ Params 
 template <int D>
 __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params p, const NodeRange range,
                                                  const double* __restrict__ A, double* __restrict__ M) {
+  wait_previous_launch();
   using L = Lattice<D>;
   int xp, y, z;
   if (!range.decode(blockIdx.x * blockDim.x + threadIdx.x, xp, y, z)) return;
@@ -456,6 +457,7 @@ template <int D, typename S, bool RAGGED>
 __global__ void __launch_bounds__(128) k_moments_row(const __grid_constant__ Params p, const NodeRange range,
                                                      const typename Store<S>::T* __restrict__ A,
                                                      float* __restrict__ M) {
+  wait_previous_launch();
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   constexpr int N = Store<S>::kGroup, H = N / 2, T3 = L::Q / 3;
@@ -629,6 +631,7 @@ __device__ __forceinline__ void prims_node(const Params& p, const Model<real>& m
 template <int D, typename real, class CL>
 __global__ void __launch_bounds__(256) k_prims(const __grid_constant__ Params p, const NodeRange range,
                                                const real* __restrict__ M, real* __restrict__ W) {
+  wait_previous_launch();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   CL closure;
   closure.load(p, smem_raw);
@@ -673,6 +676,7 @@ template <typename real, class CL, int MINB>
 __global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_constant__ Params p, int lo, int hi, int ncolx,
                                                            int ncoly, int nseg, const real* __restrict__ M,
                                                            real* __restrict__ W) {
+  wait_previous_launch();
   constexpr int NT = kPrimX * kPrimY, BX2 = kPrimX + 4, BX1 = kPrimX + 2;
   constexpr int N2 = BX2 * (kPrimY + 4), N1 = BX1 * (kPrimY + 2), K2 = (N2 + NT - 1) / NT, K1 = (N1 + NT - 1) / NT;
   __shared__ PrimsSmem<real, CL> sm;
@@ -783,6 +787,7 @@ __global__ void __launch_bounds__(NTB, MINB)
 k_collide(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
           typename Store<S>::T* __restrict__ B, const real* __restrict__ M, const real* __restrict__ W,
           unsigned* err) {
+  wait_previous_launch();
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   using WP = WPlanes<D>;
@@ -875,6 +880,7 @@ __global__ void __launch_bounds__(NTB, MINB)
 k_collide2(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
            typename Store<S>::T* __restrict__ B, const float* __restrict__ M, const float* __restrict__ W,
            unsigned* err) {
+  wait_previous_launch();
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   using WP = WPlanes<D>;
@@ -1127,6 +1133,7 @@ __device__ __forceinline__ void ghost_fill(const Params& p, typename Store<S>::T
 constexpr int kGhostBlock = 64;
 template <int D, typename S>
 __global__ void __launch_bounds__(kGhostBlock) k_ghosts(const __grid_constant__ Params p, typename Store<S>::T* B) {
+  wait_previous_launch();
   ghost_fill<D, S>(p, B, blockIdx.x * (long long)kGhostBlock + threadIdx.x, (long long)gridDim.x * kGhostBlock);
 }
 
@@ -1198,6 +1205,7 @@ __global__ void __launch_bounds__(W / 2, MINB)
 k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv dny,
                const typename Store<S>::T* __restrict__ A, typename Store<S>::T* __restrict__ B,
                const float* __restrict__ M, const float* __restrict__ Wf, unsigned* err) {
+  wait_previous_launch();
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   using WP = WPlanes<D>;

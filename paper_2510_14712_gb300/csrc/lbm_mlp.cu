@@ -120,13 +120,6 @@ __global__ void k_mlp_image(const float* __restrict__ th, Scale sc, TrainImage* 
   }
 }
 
-// The training kernels are launched with programmatic serialisation: a kernel's
-// blocks may start while the launch before it drains, and wait here for that
-// launch's results before their first use.  (On other launches both return at
-// once.)
-__device__ __forceinline__ void wait_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void allow_next_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // sample i of the minibatch starting at draw `base`: its normalised inputs and exact labels
 __device__ __forceinline__ void draw_sample(const double* __restrict__ rho, const double* __restrict__ e, long long n,
                                             uint64_t seed, unsigned long long base, int i, const Scale& sc, const Eos& q,
@@ -953,23 +946,6 @@ void launch_image(lbm_mlp_s& n) {
   k_mlp_image<<<(kImageThreads + 255) / 256, 256, 0, n.stream>>>(n.theta, scale_of(n), n.img, n.w2k);
 }
 
-// a launch that may overlap the end of the one before it on the stream (its kernel
-// calls wait_previous_launch before it reads or writes what that one touches)
-template <class... P, class... A>
-cudaError_t launch_overlapped(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
-}
-
 // the partial gradient records of the B samples in n.X, n.Y; their number in nchunk
 int launch_partials(lbm_mlp_s& n, int B, int& nchunk) {
   const int ngrp = (B + 31) / 32;
@@ -987,7 +963,7 @@ int launch_partials(lbm_mlp_s& n, int B, int& nchunk) {
     // one block per SM (all 512 TMEM columns), every block at least one group
     const int groups = (B + tcl::kRows - 1) / tcl::kRows;
     const int grid = groups < n.sms ? groups : n.sms;
-    CKM(launch_overlapped(k_mlp_train_tc, grid, tcl::kThreads, tcl::kSmem, n.stream, n.img, n.w2k, n.X, n.Y, B, n.partial,
+    CKM(launch_overlapped(k_mlp_train_tc, dim3(grid), tcl::kThreads, tcl::kSmem, n.stream, n.img, n.w2k, n.X, n.Y, B, n.partial,
                           n.status));
     nchunk = grid;
     return LBM_OK;
@@ -1239,7 +1215,7 @@ int lbm_mlp_train(lbm_mlp_t net, const double* d_rho, const double* d_e, long lo
     net->t += 1;
     const double bc1 = 1.0 - std::pow(0.9, double(net->t)), bc2 = 1.0 - std::pow(0.999, double(net->t));
     const Draw next = {d_rho, d_e, n, seed, (unsigned long long)(k + 1) * batch, k + 1 < steps ? batch : 0, net->q};
-    CKM(launch_overlapped(k_mlp_update, kSumBlocks + (next.B + kUpdateDraw - 1) / kUpdateDraw, kSumCols * kSumSlices, 0,
+    CKM(launch_overlapped(k_mlp_update, dim3(kSumBlocks + (next.B + kUpdateDraw - 1) / kUpdateDraw), kSumCols * kSumSlices, 0,
                           net->stream, net->partial, nchunk, float(1.0 / (3.0 * batch)), net->losses + k, net->theta,
                           net->m, net->v, float(lr), float(bc1), float(bc2), float(wd), net->img, net->w2k, next, sc,
                           net->X, net->Y));

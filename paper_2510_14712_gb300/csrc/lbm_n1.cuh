@@ -215,17 +215,20 @@ template <int D, typename real> struct N1Buffers {
 template <int D, typename real>
 __global__ void k_n1_strain(Params p, const real* __restrict__ rho, const real* __restrict__ u,
                             const real* __restrict__ T) {
+  wait_previous_launch();
   const N1Buffers<D, real> b(p, rho, u, T);
   n1_rows<2>(p, b.w0,
              [&](int x, int y, int z, unsigned o) { return n1_strain_at<D, real>(p, b.rho, b.u, b.T, x, y, z, o); });
 }
 
 template <int D, typename real> __global__ void k_n1_d4(Params p) {
+  wait_previous_launch();
   const N1Buffers<D, real> b(p);
   n1_rows<2>(p, b.w1, [&](int x, int y, int z, unsigned o) { return n1_d4_at<D, real>(p, b.w0, x, y, z, o); });
 }
 
 template <int D, typename real> __global__ void k_n1_filter(Params p, int a) {
+  wait_previous_launch();
   const N1Buffers<D, real> b(p);
   n1_rows<2>(p, b.filter_out(a),
              [&](int x, int y, int z, unsigned o) { return n1_filter_at<real>(p, a, b.filter_in(a), x, y, z, o); });
@@ -233,6 +236,7 @@ template <int D, typename real> __global__ void k_n1_filter(Params p, int a) {
 
 template <int D, typename real>
 __global__ void k_n1_filter_coef(Params p, const real* __restrict__ rho, const real* __restrict__ T) {
+  wait_previous_launch();
   const N1Buffers<D, real> b(p, rho, nullptr, T);
   const Model<real> m = model_of<real>(p);
   n1_rows<3>(p, b.visc, [&](int x, int y, int z, unsigned o) {
@@ -255,6 +259,7 @@ constexpr int kN1TileX = 64, kN1TileY = 16, kN1Threads = 256;
 
 template <typename S, typename real>
 __global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant__ Params p, int ntx) {
+  wait_previous_launch();
   using U = Unit<S, real>;
   using V = typename U::V;
   constexpr int N = U::N, HX = 4, P4 = kN1TileX + 2 * HX, H4 = kN1TileY + 8, P2 = kN1TileX + 4, H2 = kN1TileY + 4;
@@ -341,6 +346,7 @@ __global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant
 template <typename real>
 __global__ void __launch_bounds__(256) k_n1_norms_2d(const __grid_constant__ Params p, const real* __restrict__ rho,
                                                      const real* __restrict__ u, const real* __restrict__ T) {
+  wait_previous_launch();
   const long long n = blockIdx.x * 256LL + threadIdx.x;
   if (n >= (long long)p.Nx * p.Ny) return;
   const int y = int(n / p.Nx), x = int(n - (long long)y * p.Nx);
@@ -357,17 +363,17 @@ __global__ void __launch_bounds__(256) k_n1_norms_2d(const __grid_constant__ Par
 template <int D, typename S, typename real>
 inline int n1_update(const Params& p, cudaStream_t st, const real* rho, const real* u, const real* T) {
   if constexpr (D == 2) {
-    if (rho) k_n1_norms_2d<real><<<unsigned(((long long)p.Nx * p.Ny + 255) / 256), 256, 0, st>>>(p, rho, u, T);
+    if (rho) launch_overlapped(k_n1_norms_2d<real>, dim3(unsigned(((long long)p.Nx * p.Ny + 255) / 256)), 256, 0, st, p, rho, u, T);
     const int ntx = (p.Nx + kN1TileX - 1) / kN1TileX, nty = (p.Ny + kN1TileY - 1) / kN1TileY;
-    k_n1_coef_2d<S, real><<<unsigned(ntx) * unsigned(nty), kN1Threads, 0, st>>>(p, ntx);
+    launch_overlapped(k_n1_coef_2d<S, real>, dim3(unsigned(ntx) * unsigned(nty)), kN1Threads, 0, st, p, ntx);
     return rho ? 2 : 1;
   } else {
     const int groups = (p.Ny * p.Nz + kN1Rows - 1) / kN1Rows;
     const dim3 block(128), grid(unsigned((p.Nx + 127) / 128), unsigned(groups < 65535 ? groups : 65535));
-    k_n1_strain<D, real><<<grid, block, 0, st>>>(p, rho, u, T);
-    k_n1_d4<D, real><<<grid, block, 0, st>>>(p);
-    for (int a = 0; a + 1 < D; ++a) k_n1_filter<D, real><<<grid, block, 0, st>>>(p, a);
-    k_n1_filter_coef<D, real><<<grid, block, 0, st>>>(p, rho, T);
+    launch_overlapped(k_n1_strain<D, real>, grid, block.x, 0, st, p, rho, u, T);
+    launch_overlapped(k_n1_d4<D, real>, grid, block.x, 0, st, p);
+    for (int a = 0; a + 1 < D; ++a) launch_overlapped(k_n1_filter<D, real>, grid, block.x, 0, st, p, a);
+    launch_overlapped(k_n1_filter_coef<D, real>, grid, block.x, 0, st, p, rho, T);
     return D + 2;
   }
 }
@@ -389,6 +395,7 @@ __device__ __forceinline__ int n1_instance(const int* __restrict__ rowstart, int
 // stage 0: strain, 1: fourth differences, 2: filter pass a, 3: last pass + coefficients
 template <int D, typename real, int STAGE>
 __global__ void k_n1_batch(const BatchInstance* __restrict__ insts, const int* __restrict__ rowstart, int n, int a) {
+  wait_previous_launch();
   const int k = n1_instance(rowstart, n, blockIdx.x);
   const Params& p = insts[k].p;
   const N1Buffers<D, real> b(p);
@@ -409,10 +416,10 @@ __global__ void k_n1_batch(const BatchInstance* __restrict__ insts, const int* _
 // `rows` global rows
 template <int D, typename real>
 inline int n1_update_batch(const BatchInstance* insts, const int* rowstart, int n, int rows, cudaStream_t st) {
-  k_n1_batch<D, real, 0><<<rows, 128, 0, st>>>(insts, rowstart, n, 0);
-  k_n1_batch<D, real, 1><<<rows, 128, 0, st>>>(insts, rowstart, n, 0);
-  for (int a = 0; a + 1 < D; ++a) k_n1_batch<D, real, 2><<<rows, 128, 0, st>>>(insts, rowstart, n, a);
-  k_n1_batch<D, real, 3><<<rows, 128, 0, st>>>(insts, rowstart, n, D - 1);
+  launch_overlapped(k_n1_batch<D, real, 0>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, 0);
+  launch_overlapped(k_n1_batch<D, real, 1>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, 0);
+  for (int a = 0; a + 1 < D; ++a) launch_overlapped(k_n1_batch<D, real, 2>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, a);
+  launch_overlapped(k_n1_batch<D, real, 3>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, D - 1);
   return D + 2;
 }
 

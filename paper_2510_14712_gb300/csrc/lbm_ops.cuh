@@ -45,16 +45,16 @@ template <int D, typename S, typename real> struct OpsImpl {
       constexpr int N = Store<S>::kGroup;
       const NodeRange r(p, 0, p.Nx + 2 * p.G, N);
       auto kern = p.Nx % N ? k_moments_row<D, S, true> : k_moments_row<D, S, false>;
-      kern<<<unsigned((r.n + 127u) / 128u), 128, 0, h.stream>>>(p, r, A, M(h));
+      launch_overlapped(kern, dim3(unsigned((r.n + 127u) / 128u)), 128, 0, h.stream, p, r, A, M(h));
     } else {
       const NodeRange r(p, lo, hi);
-      k_moments<D><<<grid_for(r.n), kBlock, 0, h.stream>>>(p, r, A, M(h));
+      launch_overlapped(k_moments<D>, dim3(grid_for(r.n)), kBlock, 0, h.stream, p, r, A, M(h));
     }
     h.launches += 1;
   }
 
   // blocks of k_prims3 per multiprocessor: 40 registers without a network
-  template <class CL> static constexpr int kPrimsMinB = CL::kWarp ? 1 : (sizeof(real) == 8 ? 3 : 6);
+  template <class CL> static constexpr int kPrimsMinB = CL::kWarp ? 2 : (sizeof(real) == 8 ? 3 : 6);
 
   // primitive fields from the moments in scratch (3-D: MINB blocks per
   // multiprocessor for the register budget)
@@ -74,11 +74,11 @@ template <int D, typename S, typename real> struct OpsImpl {
       // z-segments: about one round of resident blocks (a segment repeats four
       // planes of density and two of Laplacian), at least two planes each
       const int nseg = std::max(1, std::min(p.Nz / 2, (slots + ncolx * ncoly - 1) / (ncolx * ncoly)));
-      kern<<<unsigned(ncolx * ncoly * nseg), kPrimX * kPrimY, CL::kSmem, h.stream>>>(p, lo, hi, ncolx, ncoly, nseg,
+      launch_overlapped(kern, dim3(unsigned(ncolx * ncoly * nseg)), kPrimX * kPrimY, CL::kSmem, h.stream, p, lo, hi, ncolx, ncoly, nseg,
                                                                                       M(h), W(h));
     } else {
       const NodeRange r(p, lo, hi);
-      k_prims<D, real, CL><<<grid_for(r.n), kBlock, CL::kSmem, h.stream>>>(p, r, M(h), W(h));
+      launch_overlapped(k_prims<D, real, CL>, dim3(grid_for(r.n)), kBlock, CL::kSmem, h.stream, p, r, M(h), W(h));
     }
     h.launches += 1;
   }
@@ -105,18 +105,18 @@ template <int D, typename S, typename real> struct OpsImpl {
             cudaFuncSetAttribute(k_collide_rows<D, S, EX, true, W128, kRowsMinB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(R::kBytes))};
         (void)ready;
         const int nseg = ((p.periodic_x ? p.Nx : p.G + p.Nx) + W128 - 1) / W128;
-        kern<<<unsigned(nseg) * unsigned(p.Ny) * unsigned(p.Nz), W128 / 2, R::kBytes, h.stream>>>(
+        launch_overlapped(kern, dim3(unsigned(nseg) * unsigned(p.Ny) * unsigned(p.Nz)), W128 / 2, R::kBytes, h.stream,
             p, nseg, FastDiv(unsigned(nseg)), FastDiv(unsigned(p.Ny)), A, B, M(h), W(h), h.err_dev);
         return p.bc_lo != LBM_BC_WALL && p.bc_hi != LBM_BC_WALL;
       }
       constexpr int NTB = 128, MINB = 2;
       const NodeRange r(p, p.G, p.G + p.Nx, 2);
       auto kern = p.Nx % 2 ? k_collide2<D, S, EX, true, NTB, MINB> : k_collide2<D, S, EX, false, NTB, MINB>;
-      kern<<<unsigned((r.n + NTB - 1) / NTB), NTB, 0, h.stream>>>(p, r, A, B, M(h), W(h), h.err_dev);
+      launch_overlapped(kern, dim3(unsigned((r.n + NTB - 1) / NTB)), NTB, 0, h.stream, p, r, A, B, M(h), W(h), h.err_dev);
     } else {
       constexpr int NTB = 128, MINB = 2;
       const NodeRange r(p, p.G, p.G + p.Nx);
-      k_collide<D, S, real, EX, NTB, MINB><<<unsigned((r.n + NTB - 1) / NTB), NTB, 0, h.stream>>>(p, r, A, B, M(h),
+      launch_overlapped(k_collide<D, S, real, EX, NTB, MINB>, dim3(unsigned((r.n + NTB - 1) / NTB)), NTB, 0, h.stream, p, r, A, B, M(h),
                                                                                                 W(h), h.err_dev);
     }
     return false;
@@ -161,7 +161,7 @@ template <int D, typename S, typename real> struct OpsImpl {
       auto kern = k_step2d<S, real, CL, TX, TY, HELP, MINB>;
       static const cudaError_t ready = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
       (void)ready;
-      kern<<<unsigned(tiles(p)), G::NT + HELP, kSmem, h.stream>>>(p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
+      launch_overlapped(kern, dim3(unsigned(tiles(p))), G::NT + HELP, kSmem, h.stream, p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
                                                           h.err_dev, (p.Nx + TX - 1) / TX);
       h.launches += 1;
       wall_ghosts(h, dst);
@@ -181,9 +181,9 @@ template <int D, typename S, typename real> struct OpsImpl {
   using LaunchFn = void (*)(Handle&, const void*, void*);
   template <class CL> static int candidates(const LaunchFn** fns) {
     if constexpr (D == 3 && CL::kWarp) {
-      // the network's registers: 220 and one block per multiprocessor, or 128 and
-      // two with spills (256x128x96: 970 and 1003 us per step)
-      static const LaunchFn c[] = {&split<CL, 1>, &split<CL, 2>};
+      // the network's registers: 128 and two blocks per multiprocessor, or one block
+      // without spills (256x128x96: 819 and 864 us per step)
+      static const LaunchFn c[] = {&split<CL, 2>, &split<CL, 1>};
       *fns = c;
       return 2;
     } else if constexpr (D == 3) {
@@ -233,7 +233,7 @@ template <int D, typename S, typename real> struct OpsImpl {
     const Params& p = h.p;
     if (!p.periodic_x) {
       const long long n = ghost_items<D>(p, true) + ghost_items<D>(p, false);
-      k_ghosts<D, S><<<unsigned((n + kGhostBlock - 1) / kGhostBlock), kGhostBlock, 0, h.stream>>>(
+      launch_overlapped(k_ghosts<D, S>, dim3(unsigned((n + kGhostBlock - 1) / kGhostBlock)), kGhostBlock, 0, h.stream,
           p, reinterpret_cast<ST*>(dst));
       h.launches += 1;
     }
@@ -381,11 +381,11 @@ template <int D, typename S, typename real> struct OpsImpl {
     }
     static void enqueue(Batch& b, int parity) {
       const BatchInstance* insts = reinterpret_cast<const BatchInstance*>(b.d_insts);
-      k_step2d_batch<S, real, TX, TY, MINB><<<unsigned(b.nitems), G::NT, G::kBytes, b.stream>>>(
+      launch_overlapped(k_step2d_batch<S, real, TX, TY, MINB>, dim3(unsigned(b.nitems)), G::NT, G::kBytes, b.stream,
           insts, reinterpret_cast<const BatchItem*>(b.d_items), parity, b.d_errs);
       b.launches += 1;
       for (int k0 = 0; k0 < b.n; k0 += 65535) {
-        k_ghosts_batch<D, S><<<dim3(b.ghost_blocks, unsigned(b.n - k0 < 65535 ? b.n - k0 : 65535)), 256, 0, b.stream>>>(
+        launch_overlapped(k_ghosts_batch<D, S>, dim3(b.ghost_blocks, unsigned(b.n - k0 < 65535 ? b.n - k0 : 65535)), 256, 0, b.stream,
             insts + k0, parity);
         b.launches += 1;
       }

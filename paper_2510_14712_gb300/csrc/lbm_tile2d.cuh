@@ -480,6 +480,7 @@ template <typename S, typename real, class CL, int TX, int TY, int HELP, int MIN
 __global__ void __launch_bounds__(TX / Unit<S, real>::N * TY + HELP, MINB)
 k_step2d(const __grid_constant__ Params p, const typename Store<S>::T* __restrict__ A,
          typename Store<S>::T* __restrict__ B, unsigned* err, int ntx) {
+  wait_previous_launch();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using G = TileGeom<real, Unit<S, real>::N, TX, TY>;
   CL closure;
@@ -507,6 +508,7 @@ template <typename S, typename real, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(TX / Unit<S, real>::N * TY, MINB)
 k_step2d_batch(const BatchInstance* __restrict__ insts, const BatchItem* __restrict__ items, int parity,
                unsigned* errs) {
+  wait_previous_launch();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using ST = typename Store<S>::T;
   const BatchItem it = items[blockIdx.x];
@@ -522,6 +524,7 @@ k_step2d_batch(const BatchInstance* __restrict__ insts, const BatchItem* __restr
 // instance k, as k_ghosts does for one handle (other faces: the step itself).
 template <int D, typename S>
 __global__ void k_ghosts_batch(const BatchInstance* __restrict__ insts, int parity) {
+  wait_previous_launch();
   using ST = typename Store<S>::T;
   const BatchInstance& bi = insts[blockIdx.y];
   const Params& p = bi.p;
