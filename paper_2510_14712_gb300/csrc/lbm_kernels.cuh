@@ -596,13 +596,14 @@ __device__ __forceinline__ void prims_node(const Params& p, const Model<real>& m
 #pragma unroll
   for (int a = 0; a < D; ++a) u[a] = real(0);
   if (act) {
+    const Divider<real> over_rho(rho);
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-      u[a] = div_rn(j[a] + real(0.5) * F[a], rho);                                      // Eq. def_u
-      uF += u[a] * F[a];
-      u2 += u[a] * u[a];
+      u[a] = over_rho(mad(real(0.5), F[a], j[a]));                                      // Eq. def_u
+      uF = mad(u[a], F[a], uF);
+      u2 = mad(u[a], u[a], u2);
     }
-    E = div_rn(S + real(0.5) * uF, rho);                                                // Eq. def_E
+    E = over_rho(mad(real(0.5), uF, S));                                                // Eq. def_E
   }
   real T = real(0), P = real(1), cs2 = real(0), e = real(0);
   if constexpr (CL::kWarp) closure(m, rho, E, u2, act, T, P, cs2, e);

@@ -318,19 +318,17 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
     const V kr = V(m.kappa) * rho * V(real(0.5)), lc = U::ld(l);
     F[0] = kr * (U::right(l, lc) - U::left(l, lc));                                      // Eq. FK
     F[1] = kr * (U::ld(l + G::P2) - U::ld(l - G::P2));
-    V uF = V(0), u2 = V(0), E, e = V(0);
+    V uF = V(0), u2 = V(0), e = V(0);
+    const Divider<V> over_rho(rho);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-      const V n = mad(V(real(0.5)), F[a], j[a]);
-#pragma unroll
-      for (int k = 0; k < N; ++k) U::set(u[a], k, div_rn(U::get(n, k), U::get(rho, k)));  // Eq. def_u
+      u[a] = over_rho(mad(V(real(0.5)), F[a], j[a]));                                    // Eq. def_u
       uF = mad(u[a], F[a], uF);
       u2 = mad(u[a], u[a], u2);
     }
-    const V n = mad(V(real(0.5)), uF, Sg);
+    const V E = over_rho(mad(V(real(0.5)), uF, Sg));                                     // Eq. def_E
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      U::set(E, k, div_rn(U::get(n, k), U::get(rho, k)));                                // Eq. def_E
       real t = real(0), pp = real(1), c = real(0), ee = real(0);
       if (CL::kWarp || act) closure(m, U::get(rho, k), U::get(E, k), U::get(u2, k), act, t, pp, c, ee);
       U::set(T, k, t);
