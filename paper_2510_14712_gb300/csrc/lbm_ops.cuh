@@ -98,7 +98,7 @@ template <int D, typename S, typename real> struct OpsImpl {
     if constexpr (sizeof(real) == 4) {
       if (collide_rows_ok<S>(p)) {
         constexpr int W128 = 128, kRowsMinB = 8;
-        using R = RowsLayout<D, S, W128>;
+        using R = RowsLayout<D, S, EX, W128>;
         auto kern = p.periodic_x ? k_collide_rows<D, S, EX, false, W128, kRowsMinB> : k_collide_rows<D, S, EX, true, W128, kRowsMinB>;
         static const cudaError_t ready[2] = {
             cudaFuncSetAttribute(k_collide_rows<D, S, EX, false, W128, kRowsMinB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(R::kBytes)),
