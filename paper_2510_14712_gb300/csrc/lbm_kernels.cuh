@@ -592,13 +592,18 @@ template <int D> struct WPlanes {
 // on they have no such form.
 template <typename real, bool EX> constexpr bool derives_fields() { return sizeof(real) == 4 && !EX; }
 
+// The Korteweg force of a 3-D node is the difference of the density's Laplacian
+// across it: FP32 steps hand the Laplacian on, one plane (in F's place) for three
+// (256^3: 1838 -> 1807 us per step in FP32, 1260 -> 1240 with FP16 deviations).
+template <int D, typename real> constexpr bool hands_laplacian() { return D == 3 && sizeof(real) == 4; }
+
 // Primitive fields of one node from its moments and the Korteweg force F:
 // u, E, the closure's (T, P, c_s^2, e), then h and Lambda, stored at offset o.
 // Warp-collective closures need every lane of the warp (act: a real node).
 template <int D, typename real, class CL>
 __device__ __forceinline__ void prims_node(const Params& p, const Model<real>& m, const CL& closure, bool act,
-                                           real rho, const real* j, real S, const real* F, real* __restrict__ W,
-                                           unsigned o) {
+                                           real rho, const real* j, real S, const real* F, real lap,
+                                           real* __restrict__ W, unsigned o) {
   using WP = WPlanes<D>;
   real u[D], uF = real(0), u2 = real(0), E = real(0);
 #pragma unroll
@@ -618,14 +623,16 @@ __device__ __forceinline__ void prims_node(const Params& p, const Model<real>& m
   else if (act) closure(m, rho, E, u2, act, T, P, cs2, e);
   if (!act) return;
   constexpr bool kDerived = !CL::kOutput && !derives_fields<real, (CL::kExtra > 0)>();
+  constexpr bool kLap = !CL::kOutput && hands_laplacian<D, real>();
   const real theta = P / rho;
   auto put = [&](const int k, const real v) { W[(long long)k * p.plane + o] = v; };
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     put(WP::U + a, u[a]);
     if constexpr (kDerived) put(WP::LAM + a, rho * u[a] * u[a] * u[a] + real(3) * rho * u[a] * (theta - real(1.0 / 3.0)));
-    put(WP::F + a, F[a]);
+    if constexpr (!kLap) put(WP::F + a, F[a]);
   }
+  if constexpr (kLap) put(WP::F, lap);
   put(WP::T, T);
   if constexpr (kDerived) put(WP::H, e + theta);                                        // Eq. enthalpy
   if constexpr (CL::kExtra > 0) {
@@ -666,7 +673,7 @@ __global__ void __launch_bounds__(256) k_prims(const __grid_constant__ Params p,
       j[a] = M[(1 + a) * p.plane + o];
     }
   }
-  prims_node<D, real, CL>(p, m, closure, act, rho, j, S, F, W, o);
+  prims_node<D, real, CL>(p, m, closure, act, rho, j, S, F, real(0), W, o);
 }
 
 // ---------------------------------------------------------------------------
@@ -773,7 +780,7 @@ __global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_c
       const int c = (ly + 1) * BX1 + lx + 1;
       const real kr = m.kappa * rho * real(0.5);
       const real F[3] = {kr * (l2[c + 1] - l2[c - 1]), kr * (l2[c + BX1] - l2[c - BX1]), kr * (l1[c] - l0[c])};   // Eq. FK
-      prims_node<3, real, CL>(p, m, closure, act, rho, j, S, F, Wn, zo);
+      prims_node<3, real, CL>(p, m, closure, act, rho, j, S, F, l2[c], Wn, zo);
       zo = next(zo);
     }
     real* t = r2;
@@ -933,8 +940,10 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
   NodeState<D, F2> s;
   s.rho = f2_of(__ldg(reinterpret_cast<const float2*>(at_bytes(M, 4 * o))));
   s.T = w2(WP::T, o);
-  constexpr bool DER = derives_fields<float, EX>();
-  F2 h, theta;
+  constexpr bool DER = derives_fields<float, EX>(), LAP = hands_laplacian<D, float>();
+  const F2 kr = F2(m.kappa) * s.rho * F2(0.5f);
+  F2 h, theta, lap;
+  if constexpr (LAP) lap = w2(WP::F, o);
   if constexpr (DER) h = vdw_enthalpy(m, s.rho, s.T, theta);
   else h = w2(WP::H, o);
   s.sc = p.sc_on != 0;
@@ -950,7 +959,7 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     s.u[a] = w2(WP::U + a, o);
-    s.F[a] = w2(WP::F + a, o);
+    if constexpr (!LAP) s.F[a] = w2(WP::F + a, o);
     F2 lc, up, um, Tp, Tm, hp, hm, lp, lm;
     if constexpr (DER) lc = lambda_of(s.rho, s.u[a], theta);
     else lc = w2(WP::LAM + a, o);
@@ -971,6 +980,10 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
         ho = F2(w1(WP::H, outm), w1(WP::H, out2));
         lo = F2(w1(WP::LAM, outm), w1(WP::LAM, out2));
       }
+      if constexpr (LAP) {
+        const F2 po2 = F2(w1(WP::F, outm), w1(WP::F, out2));
+        s.F[0] = kr * (F2(lone ? po2.y : lap.y, po2.y) - F2(po2.x, lap.x));                  // Eq. FK
+      }
       up = F2(lone ? uo.y : s.u[0].y, uo.y);
       um = F2(uo.x, s.u[0].x);
       Tp = F2(lone ? To.y : s.T.y, To.y);
@@ -980,6 +993,7 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
       lp = F2(lone ? lo.y : lc.y, lo.y);
       lm = F2(lo.x, lc.x);
     } else {
+      if constexpr (LAP) s.F[a] = kr * (w2(WP::F, nbp[a]) - w2(WP::F, nbm[a]));
       up = w2(WP::U + a, nbp[a]);
       um = w2(WP::U + a, nbm[a]);
       Tp = w2(WP::T, nbp[a]);
@@ -1201,21 +1215,27 @@ template <int D, typename S, bool EX, int W> struct RowsLayout {
   // index of the segment's first node in row i (the left unit of c_x = +1 rows)
   __host__ __device__ static constexpr int lead(int i) { return i < 2 * T3 ? 0 : kA; }
   static constexpr size_t kPopBytes = size_t(2 * kSet) * sizeof(ST);
-  // field rows (planes of plane()): kWide of the row with a unit on both sides; then
-  // the row's nOwn; then nSide of the two neighbours along each b > 0
+  // field rows (planes of W): nWide of the row with a unit on both sides; then the
+  // row's nOwn; then nSide of the two neighbours along each b > 0
   static constexpr bool DER = derives_fields<float, EX>();       // h, Lam_a from rho, u_a, T; else read
+  static constexpr bool LAP = hands_laplacian<D, float>();       // F from the Laplacian; else read
   static constexpr int RHO = -1;                                 // the density, a plane of M
-  static constexpr int nSide = DER ? 3 : 4, nOwn = DER ? D + D - 1 : 1 + D + 2 * (D - 1);
+  static constexpr int nF = LAP ? 0 : D;
+  static constexpr int nSide = (DER ? 3 : 4) + LAP, nOwn = nF + D - 1 + (DER ? 0 : D);
   static constexpr int kWide = W + 2 * kF, nWide = nSide, nNb = 2 * nSide * (D - 1);
-  // wide and side fields of axis a: u_a, T, then rho, or h and Lam_a
+  // wide and side fields of axis a: u_a, T, then rho, or h and Lam_a; the Laplacian
+  static constexpr int kU = 0, kT = 1, kRho = 2, kH = 2, kLam = 3, kLap = DER ? 3 : 4;
   __host__ __device__ static constexpr int field(int a, int k) {
     using WP = WPlanes<D>;
-    return k == 0 ? WP::U + a : (k == 1 ? WP::T : (DER ? RHO : (k == 2 ? WP::H : WP::LAM + a)));
+    return k == kU ? WP::U + a : (k == kT ? WP::T : (k == kLap ? WP::F : (DER ? RHO : (k == kH ? WP::H : WP::LAM + a))));
   }
   // own rows: F_a, u_b (b > 0), then, if read, Lam_b (b > 0) and rho
+  static constexpr int ownRho = nF + 2 * (D - 1);
+  __host__ __device__ static constexpr int ownU(int b) { return nF + b - 1; }
+  __host__ __device__ static constexpr int ownLam(int b) { return nF + D - 1 + b - 1; }
   __host__ __device__ static constexpr int own_field(int k) {
     using WP = WPlanes<D>;
-    return k < D ? WP::F + k : (k < 2 * D - 1 ? WP::U + k - D + 1 : (k < 3 * D - 2 ? WP::LAM + k - 2 * D + 2 : RHO));
+    return k < nF ? WP::F + k : (k < ownLam(1) ? WP::U + 1 + k - nF : (k < ownRho ? WP::LAM + 1 + k - ownLam(1) : RHO));
   }
   __host__ __device__ static constexpr int wide(int k) { return k * kWide + kF; }
   __host__ __device__ static constexpr int own(int k) { return nWide * kWide + k * W; }
@@ -1357,32 +1377,37 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
   if (ok && act) {
   auto f2at = [&](int off) { return f2_of(*reinterpret_cast<const float2*>(sf + off + 2 * t)); };
   auto f1at = [&](int off) { return sf[off + 2 * t]; };
-  s.rho = f2at(R::DER ? R::wide(2) : R::own(3 * D - 2));
-  s.T = f2at(R::wide(1));
+  s.rho = f2at(R::DER ? R::wide(R::kRho) : R::own(R::ownRho));
+  s.T = f2at(R::wide(R::kT));
   F2 h, theta;
   if constexpr (R::DER) h = vdw_enthalpy(m, s.rho, s.T, theta);
-  else h = f2at(R::wide(2));
+  else h = f2at(R::wide(R::kH));
+  const F2 kr = F2(m.kappa) * s.rho * F2(0.5f);
   s.div_u = F2(0.f);
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    s.F[a] = f2at(R::own(a));
-    s.u[a] = f2at(a == 0 ? R::wide(0) : R::own(D + a - 1));
+    s.u[a] = f2at(a == 0 ? R::wide(R::kU) : R::own(R::ownU(a)));
+    if constexpr (!R::LAP) s.F[a] = f2at(R::own(a));
     F2 lc, up, um, Tp, Tm, hp, hm, lp, lm;
     if constexpr (R::DER) lc = lambda_of(s.rho, s.u[a], theta);
-    else lc = f2at(a == 0 ? R::wide(R::nSide - 1) : R::own(2 * D + a - 2));
+    else lc = f2at(a == 0 ? R::wide(R::kLam) : R::own(R::ownLam(a)));
     if (a == 0) {
       // outer neighbours of the pair: x - 1 and x + 2
       auto outer = [&](const int k) { return F2(f1at(R::wide(k) - 1), f1at(R::wide(k) + 2)); };
-      const F2 uo = outer(0), To = outer(1);
+      const F2 uo = outer(R::kU), To = outer(R::kT);
       F2 ho, lo;
       if constexpr (R::DER) {
-        const F2 ro = outer(2);
+        const F2 ro = outer(R::kRho);
         F2 tho;
         ho = vdw_enthalpy(m, ro, To, tho);
         lo = lambda_of(ro, uo, tho);
       } else {
-        ho = outer(2);
-        lo = outer(R::nSide - 1);
+        ho = outer(R::kH);
+        lo = outer(R::kLam);
+      }
+      if constexpr (R::LAP) {
+        const F2 c = f2at(R::wide(R::kLap)), n2 = outer(R::kLap);
+        s.F[0] = kr * (F2(c.y, n2.y) - F2(n2.x, c.x));                                     // Eq. FK
       }
       up = F2(s.u[0].y, uo.y);
       um = F2(uo.x, s.u[0].x);
@@ -1393,23 +1418,25 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
       lp = F2(lc.y, lo.y);
       lm = F2(lo.x, lc.x);
     } else {
-      um = f2at(R::nb(a, 0, 0));
-      Tm = f2at(R::nb(a, 0, 1));
-      up = f2at(R::nb(a, 1, 0));
-      Tp = f2at(R::nb(a, 1, 1));
+      auto side = [&](const int d, const int k) { return f2at(R::nb(a, d, k)); };
+      um = side(0, R::kU);
+      up = side(1, R::kU);
+      Tm = side(0, R::kT);
+      Tp = side(1, R::kT);
       if constexpr (R::DER) {
-        const F2 rm = f2at(R::nb(a, 0, 2)), rp = f2at(R::nb(a, 1, 2));
+        const F2 rm = side(0, R::kRho), rp = side(1, R::kRho);
         F2 th;
         hm = vdw_enthalpy(m, rm, Tm, th);
         lm = lambda_of(rm, um, th);
         hp = vdw_enthalpy(m, rp, Tp, th);
         lp = lambda_of(rp, up, th);
       } else {
-        hm = f2at(R::nb(a, 0, 2));
-        lm = f2at(R::nb(a, 0, R::nSide - 1));
-        hp = f2at(R::nb(a, 1, 2));
-        lp = f2at(R::nb(a, 1, R::nSide - 1));
+        hm = side(0, R::kH);
+        hp = side(1, R::kH);
+        lm = side(0, R::kLam);
+        lp = side(1, R::kLam);
       }
+      if constexpr (R::LAP) s.F[a] = kr * (side(1, R::kLap) - side(0, R::kLap));
     }
     s.div_u = mad(F2(0.5f), up - um, s.div_u);
     s.gradT[a] = F2(0.5f) * (Tp - Tm);
