@@ -139,6 +139,22 @@ inline cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, unsigned blo
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 
+// Dynamic shared memory of a kernel that may pass 48 KB, and the blocks of it that
+// the device holds at once, found on first use.  Internal linkage, as the kernel
+// template's own launch stub has it: each translation unit prepares the kernel it
+// launches (one prepared flag for all of them left the others' copies at 48 KB).
+template <auto kern> static int prepared_blocks(int threads, size_t smem) {
+  static const int blocks = [threads, smem] {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    int n = 1, dev = 0, sms = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem);
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return (n > 1 ? n : 1) * sms;
+  }();
+  return blocks;
+}
+
 struct Batch;
 constexpr int kBatchBranches = 4;
 

@@ -14,7 +14,8 @@
 // (offset (z Ny + y) pitch + x + G, one plane per component).  Three forms
 // share the per-node arithmetic: in 2-D the step itself leaves S and |grad s|
 // (its block holds the neighbours' u, T and rho) and one launch over tiles does
-// the rest; in 3-D row-mapped launches (D + 2); one block per row for batches.
+// the rest; in 3-D one row-mapped launch for S and |grad s| and one over columns of
+// the box; one block per row for the 2-D batches.
 #pragma once
 
 #include "lbm_tile2d.cuh"
@@ -221,29 +222,6 @@ __global__ void k_n1_strain(Params p, const real* __restrict__ rho, const real* 
              [&](int x, int y, int z, unsigned o) { return n1_strain_at<D, real>(p, b.rho, b.u, b.T, x, y, z, o); });
 }
 
-template <int D, typename real> __global__ void k_n1_d4(Params p) {
-  wait_previous_launch();
-  const N1Buffers<D, real> b(p);
-  n1_rows<2>(p, b.w1, [&](int x, int y, int z, unsigned o) { return n1_d4_at<D, real>(p, b.w0, x, y, z, o); });
-}
-
-template <int D, typename real> __global__ void k_n1_filter(Params p, int a) {
-  wait_previous_launch();
-  const N1Buffers<D, real> b(p);
-  n1_rows<2>(p, b.filter_out(a),
-             [&](int x, int y, int z, unsigned o) { return n1_filter_at<real>(p, a, b.filter_in(a), x, y, z, o); });
-}
-
-template <int D, typename real>
-__global__ void k_n1_filter_coef(Params p, const real* __restrict__ rho, const real* __restrict__ T) {
-  wait_previous_launch();
-  const N1Buffers<D, real> b(p, rho, nullptr, T);
-  const Model<real> m = model_of<real>(p);
-  n1_rows<3>(p, b.visc, [&](int x, int y, int z, unsigned o) {
-    return n1_filter_coef_at<D, real>(p, m, b.filter_in(D - 1), b.rho, b.T, x, y, z, o);
-  });
-}
-
 // ---- 2-D single-instance form: one launch over tiles of the plane ----
 // The step's blocks leave S and |grad s| in w0 (n1_norms on the fields they hold
 // in shared memory), rho and T in sc_prims.  A block here owns 64 x 16 nodes (one
@@ -299,9 +277,10 @@ __global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant
       V v;
       if (!edge || p.periodic_x) {
         const real* c = s4[f] + (r + 2) * P4 + N * u + 2;
-        const V c0 = U::ld(c);
-        const V dx = n1_fourth(U::at(c, -2), U::at(c, -1), c0, U::at(c, 1), U::at(c, 2));
-        const V dy = n1_fourth(U::ld(c - 2 * P4), U::ld(c - P4), c0, U::ld(c + P4), U::ld(c + 2 * P4));
+        V w[5];
+        U::five(c, w);
+        const V dx = n1_fourth(w[0], w[1], w[2], w[3], w[4]);
+        const V dy = n1_fourth(U::ld(c - 2 * P4), U::ld(c - P4), w[2], U::ld(c + P4), U::ld(c + 2 * P4));
         v = root(mad(dy, dy, dx * dx));
       } else {                                            // the norm of the clamped node, one node at a time
 #pragma unroll
@@ -321,7 +300,9 @@ __global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant
 #pragma unroll
     for (int f = 0; f < 2; ++f) {
       const real* c = s2[f] + r * P2 + N * u + 2;
-      U::st(s4[f] + r * PX + N * u, n1_binom5(U::at(c, -2), U::at(c, -1), U::ld(c), U::at(c, 1), U::at(c, 2)));
+      V w[5];
+      U::five(c, w);
+      U::st(s4[f] + r * PX + N * u, n1_binom5(w[0], w[1], w[2], w[3], w[4]));
     }
   }
   __syncthreads();
@@ -338,6 +319,167 @@ __global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant
     const N1Vals<V, 3> res = n1_coefs<real, V>(p, m, U::ld_field(b.rho + o), U::ld_field(b.T + o), q[0], q[1]);
 #pragma unroll
     for (int j = 0; j < 3; ++j) U::store_field(b.visc + j * p.plane + o, res.v[j], x + N - 1 < p.Nx);
+  }
+}
+
+// ---- 3-D single-instance form: one launch from S and |grad s| to the coefficients ----
+// A block marches z over a column of TX x TY nodes: S and |grad s| of five planes
+// with a four-node halo in the plane, in a ring of shared memory; the norm of the
+// fourth differences of the ring's middle plane on a two-node halo, its x pass, its
+// y pass at the nodes, and the z pass over five planes held in registers.  The next
+// plane is requested before this one is worked on; three barriers per plane.  Halo
+// positions as in the 2-D form, which gives the bits of the row-mapped stages.
+// Those (fourth differences, two filter passes, last pass with the coefficients:
+// four launches with a pass over memory each) took 193 us at 384x128x128 in FP32, this
+// launch 151.
+template <typename S, typename real> struct N1Column {
+  using U = Unit<S, real>;
+  static constexpr int N = U::N, TX = 32 * N, TY = sizeof(real) == 4 ? 8 : 8, HX = 4;
+  static constexpr int P4 = TX + 2 * HX, H4 = TY + 8, P2 = TX + 4, H2 = TY + 4, NU = TY * 32 / kN1Threads;
+  static constexpr int kPlane = H4 * P4;                         // one field of one plane
+  static constexpr size_t kBytes = sizeof(real) * 2 * (5 * kPlane + H2 * P2 + H2 * TX);
+};
+template <typename S, typename real>
+__global__ void __launch_bounds__(kN1Threads)
+k_n1_coef_3d(const __grid_constant__ Params p, const real* __restrict__ rho, const real* __restrict__ T, int ntx, int nty,
+             int nseg) {
+  wait_previous_launch();
+  using C = N1Column<S, real>;
+  using U = typename C::U;
+  using V = typename U::V;
+  constexpr int N = U::N, P4 = C::P4, P2 = C::P2, H2 = C::H2, TX = C::TX, HX = C::HX, NU = C::NU;
+  constexpr int U4 = P4 / N, K4 = (U4 * C::H4 + kN1Threads - 1) / kN1Threads;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  real* ring = reinterpret_cast<real*>(smem_raw);
+  real* s2 = ring + 10 * C::kPlane;                              // norms of the fourth differences
+  real* sx = s2 + 2 * H2 * P2;                                   // the same after the x pass
+  const N1Buffers<3, real> b(p, rho, nullptr, T);
+  const Model<real> m = model_of<real>(p);
+  const int tid = threadIdx.x;
+  int blk = blockIdx.x;
+  const int x0 = (blk % ntx) * TX;
+  blk /= ntx;
+  const int y0 = (blk % nty) * C::TY, seg = blk / nty;
+  const int mb = int((long long)p.Nz * seg / nseg), me = int((long long)p.Nz * (seg + 1) / nseg);
+  const unsigned pitch = unsigned(p.pitch), zs = unsigned(p.Ny) * pitch, ztop = zs * unsigned(p.Nz);
+  // node that a stencil reads at x: wrapped, or clamped to the box
+  auto src = [&](int x) { return p.periodic_x ? n1_wrap(x, p.Nx) : min(max(x, 0), p.Nx - 1); };
+  const bool edge = x0 < HX || x0 + TX + HX > p.Nx;
+  unsigned at[K4][N];                                            // in-plane offsets of this thread's box units
+#pragma unroll
+  for (int k = 0; k < K4; ++k) {
+    const int q = min(tid + k * kN1Threads, U4 * C::H4 - 1), r = q / U4, x = x0 + N * (q - r * U4) - HX;
+    const unsigned row = unsigned(n1_wrap(y0 + r - 4, p.Ny)) * pitch + unsigned(p.G);
+#pragma unroll
+    for (int j = 0; j < N; ++j) at[k][j] = row + unsigned(src(x + j));
+  }
+  unsigned zl = unsigned(n1_wrap(mb - 4, p.Nz)) * zs;            // plane to load next
+  V nxt[2][K4];
+  auto load = [&] {
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const real* w = b.w0 + f * p.plane + zl;
+#pragma unroll
+      for (int k = 0; k < K4; ++k) {
+        if (!edge) {
+          nxt[f][k] = U::ld_field(w + at[k][0]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < N; ++j) U::set(nxt[f][k], j, __ldg(w + at[k][j]));
+        }
+      }
+    }
+    zl = zl + zs == ztop ? 0u : zl + zs;
+  };
+  load();
+  const int ux = tid % 32, uy = tid / 32, x = x0 + N * ux;
+  V zr[NU][2][5];                                                // x- and y-filtered norms of five planes
+#pragma unroll
+  for (int i = 0; i < NU; ++i)
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) zr[i][f][k] = V(0);
+  unsigned zo = unsigned(mb) * zs;                               // plane of the next output
+  int slot = 0;                                                  // ring slot of plane pl
+  for (int pl = mb - 4; pl <= me + 3; ++pl) {
+    real* now = ring + slot * 2 * C::kPlane;
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+      for (int k = 0; k < K4; ++k)
+        if (tid + k * kN1Threads < U4 * C::H4) U::st(now + f * C::kPlane + N * (tid + k * kN1Threads), nxt[f][k]);
+    if (pl < me + 3) load();
+    __syncthreads();
+    const int cur = slot;
+    slot = slot == 4 ? 0 : slot + 1;
+    if (pl < mb) continue;
+    auto plane = [&](const int d) {                              // ring slot of plane pl - 2 + d
+      const int q = cur + 3 + d;                                 // cur - 2 + d + 5
+      return ring + (q >= 5 ? q - 5 : q) * 2 * C::kPlane;
+    };
+    const real *cm2 = plane(-2), *cm1 = plane(-1), *c0 = plane(0), *cp1 = plane(1), *cp2 = plane(2);
+    for (int k = tid; k < P2 / N * H2; k += kN1Threads) {
+      const int r = k / (P2 / N), u = k - r * (P2 / N);
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        V v;
+        if (!edge || p.periodic_x) {
+          const int c = f * C::kPlane + (r + 2) * P4 + N * u + 2;
+          const real* q = c0 + c;
+          V w[5];
+          U::five(q, w);
+          const V dx = n1_fourth(w[0], w[1], w[2], w[3], w[4]);
+          const V dy = n1_fourth(U::ld(q - 2 * P4), U::ld(q - P4), w[2], U::ld(q + P4), U::ld(q + 2 * P4));
+          const V dz = n1_fourth(U::ld(cm2 + c), U::ld(cm1 + c), w[2], U::ld(cp1 + c), U::ld(cp2 + c));
+          v = root(mad(dz, dz, mad(dy, dy, dx * dx)));
+        } else {                                                 // the norm of the clamped node, one node at a time
+#pragma unroll
+          for (int j = 0; j < N; ++j) {
+            const int xc = min(max(src(x0 + N * u - 2 + j) - x0 + HX, 2), P4 - 3);
+            const int c = f * C::kPlane + (r + 2) * P4 + xc;
+            const real* q = c0 + c;
+            const real dx = n1_fourth(q[-2], q[-1], q[0], q[1], q[2]);
+            const real dy = n1_fourth(q[-2 * P4], q[-P4], q[0], q[P4], q[2 * P4]);
+            const real dz = n1_fourth(cm2[c], cm1[c], q[0], cp1[c], cp2[c]);
+            U::set(v, j, root(mad(dz, dz, mad(dy, dy, dx * dx))));
+          }
+        }
+        U::st(s2 + f * H2 * P2 + r * P2 + N * u, v);
+      }
+    }
+    __syncthreads();
+    for (int k = tid; k < 32 * H2; k += kN1Threads) {
+      const int r = k / 32, u = k % 32;
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        const real* c = s2 + f * H2 * P2 + r * P2 + N * u + 2;
+        V w[5];
+        U::five(c, w);
+        U::st(sx + f * H2 * TX + r * TX + N * u, n1_binom5(w[0], w[1], w[2], w[3], w[4]));
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const int r = uy + i * (kN1Threads / 32), y = y0 + r;
+      V q[2];
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        const real* c = sx + f * H2 * TX + r * TX + N * ux;
+        V* z = zr[i][f];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) z[k] = z[k + 1];
+        z[4] = n1_binom5(U::ld(c), U::ld(c + TX), U::ld(c + 2 * TX), U::ld(c + 3 * TX), U::ld(c + 4 * TX));
+        q[f] = n1_binom5(z[0], z[1], z[2], z[3], z[4]);
+      }
+      if (pl < mb + 4 || x >= p.Nx || y >= p.Ny) continue;
+      const unsigned o = zo + unsigned(y) * pitch + unsigned(x + p.G);
+      const N1Vals<V, 3> res = n1_coefs<real, V>(p, m, U::ld_field(b.rho + o), U::ld_field(b.T + o), q[0], q[1]);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) U::store_field(b.visc + j * p.plane + o, res.v[j], x + N - 1 < p.Nx);
+    }
+    if (pl >= mb + 4) zo += zs;
   }
 }
 
@@ -359,7 +501,7 @@ __global__ void __launch_bounds__(256) k_n1_norms_2d(const __grid_constant__ Par
 
 // The whole update of a handle's coefficients.  2-D: one launch after a step that
 // left S and |grad s| (`rho` null), two after one that left rho, u (D planes) and
-// T; 3-D: D + 2 launches from rho, u, T (padded plane layout).
+// T; 3-D: two from rho, u, T (padded plane layout).
 template <int D, typename S, typename real>
 inline int n1_update(const Params& p, cudaStream_t st, const real* rho, const real* u, const real* T) {
   if constexpr (D == 2) {
@@ -371,10 +513,24 @@ inline int n1_update(const Params& p, cudaStream_t st, const real* rho, const re
     const int groups = (p.Ny * p.Nz + kN1Rows - 1) / kN1Rows;
     const dim3 block(128), grid(unsigned((p.Nx + 127) / 128), unsigned(groups < 65535 ? groups : 65535));
     launch_overlapped(k_n1_strain<D, real>, grid, block.x, 0, st, p, rho, u, T);
-    launch_overlapped(k_n1_d4<D, real>, grid, block.x, 0, st, p);
-    for (int a = 0; a + 1 < D; ++a) launch_overlapped(k_n1_filter<D, real>, grid, block.x, 0, st, p, a);
-    launch_overlapped(k_n1_filter_coef<D, real>, grid, block.x, 0, st, p, rho, T);
-    return D + 2;
+    using C = N1Column<S, real>;
+    auto kern = k_n1_coef_3d<S, real>;
+    const int slots = prepared_blocks<k_n1_coef_3d<S, real>>(kN1Threads, C::kBytes);
+    // z-segments: whole rounds of resident blocks against the eight planes (two
+    // thirds of a plane's work) that each segment repeats
+    const int ntx = (p.Nx + C::TX - 1) / C::TX, nty = (p.Ny + C::TY - 1) / C::TY;
+    int nseg = 1;
+    long long least = -1;
+    for (int n = 1; n <= std::min(p.Nz, 32); ++n) {
+      const long long cost = ((long long)ntx * nty * n + slots - 1) / slots * ((p.Nz + n - 1) / n + 5);
+      if (least < 0 || cost < least) {
+        least = cost;
+        nseg = n;
+      }
+    }
+    launch_overlapped(kern, dim3(unsigned(ntx) * unsigned(nty) * unsigned(nseg)), kN1Threads, C::kBytes, st, p, rho, T, ntx,
+                      nty, nseg);
+    return 2;
   }
 }
 

@@ -64,12 +64,7 @@ template <int D, typename S, typename real> struct OpsImpl {
     moment_range(p, 1, lo, hi);
     if constexpr (D == 3) {
       auto kern = k_prims3<real, CL, MINB>;
-      static const int slots = [kern] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(CL::kSmem));
-        int bps = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPrimX * kPrimY, CL::kSmem);
-        return std::max(1, bps) * multiprocessors();
-      }();
+      const int slots = prepared_blocks<k_prims3<real, CL, MINB>>(kPrimX * kPrimY, CL::kSmem);
       const int ncolx = (hi - lo + kPrimX - 1) / kPrimX, ncoly = (p.Ny + kPrimY - 1) / kPrimY;
       // z-segments: about one round of resident blocks (a segment repeats four
       // planes of density and two of Laplacian), at least two planes each
@@ -100,10 +95,8 @@ template <int D, typename S, typename real> struct OpsImpl {
         constexpr int W128 = 128, kRowsMinB = 8;
         using R = RowsLayout<D, S, EX, W128>;
         auto kern = p.periodic_x ? k_collide_rows<D, S, EX, false, W128, kRowsMinB> : k_collide_rows<D, S, EX, true, W128, kRowsMinB>;
-        static const cudaError_t ready[2] = {
-            cudaFuncSetAttribute(k_collide_rows<D, S, EX, false, W128, kRowsMinB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(R::kBytes)),
-            cudaFuncSetAttribute(k_collide_rows<D, S, EX, true, W128, kRowsMinB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(R::kBytes))};
-        (void)ready;
+        if (p.periodic_x) prepared_blocks<k_collide_rows<D, S, EX, false, W128, kRowsMinB>>(W128 / 2, R::kBytes);
+        else prepared_blocks<k_collide_rows<D, S, EX, true, W128, kRowsMinB>>(W128 / 2, R::kBytes);
         const int nseg = ((p.periodic_x ? p.Nx : p.G + p.Nx) + W128 - 1) / W128;
         launch_overlapped(kern, dim3(unsigned(nseg) * unsigned(p.Ny) * unsigned(p.Nz)), W128 / 2, R::kBytes, h.stream,
             p, nseg, FastDiv(unsigned(nseg)), FastDiv(unsigned(p.Ny)), A, B, M(h), W(h), h.err_dev);
@@ -159,8 +152,7 @@ template <int D, typename S, typename real> struct OpsImpl {
     static void launch(Handle& h, const void* src, void* dst) {
       const Params& p = h.p;
       auto kern = k_step2d<S, real, CL, TX, TY, HELP, MINB>;
-      static const cudaError_t ready = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
-      (void)ready;
+      prepared_blocks<k_step2d<S, real, CL, TX, TY, HELP, MINB>>(G::NT + HELP, kSmem);
       launch_overlapped(kern, dim3(unsigned(tiles(p))), G::NT + HELP, kSmem, h.stream, p, reinterpret_cast<const ST*>(src), reinterpret_cast<ST*>(dst),
                                                           h.err_dev, (p.Nx + TX - 1) / TX);
       h.launches += 1;

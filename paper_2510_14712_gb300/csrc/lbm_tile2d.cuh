@@ -81,8 +81,14 @@ template <typename S> struct Unit<S, float> {          // two nodes, packed
     if (two) Store<S>::st2_raw(p, q);
     else p[0] = Store<S>::half_of(q, 0);
   }
-  // values at x + d of the nodes of the unit at s
-  __device__ static V at(const float* s, int d) { return F2(s[d], s[d + 1]); }
+  // values at x - 2 .. x + 2 of the nodes of the unit at s
+  __device__ static void five(const float* s, V (&w)[5]) {
+    w[0] = ld(s - 2);
+    w[2] = ld(s);
+    w[4] = ld(s + 2);
+    w[1] = F2(w[0].y, w[2].x);
+    w[3] = F2(w[2].y, w[4].x);
+  }
   __device__ static V ld_field(const float* p) { return f2_of(__ldg(reinterpret_cast<const float2*>(p))); }
   __device__ static void store_field(float* p, V v, bool two) {
     if (two) *reinterpret_cast<float2*>(p) = f2_in(v);
@@ -110,7 +116,10 @@ template <typename S> struct Unit<S, double> {         // one node
   __device__ static double get(V v, int) { return v; }
   __device__ static void set(V& v, int, double a) { v = a; }
   __device__ static void store(ST* p, V v, float ref, bool) { Store<S>::template st_stream<double>(p, 0, v, ref); }
-  __device__ static V at(const double* s, int d) { return s[d]; }
+  __device__ static void five(const double* s, V (&w)[5]) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) w[k] = s[k - 2];
+  }
   __device__ static V ld_field(const double* p) { return __ldg(p); }
   __device__ static void store_field(double* p, V v, bool) { *p = v; }
 };

@@ -129,6 +129,32 @@ def test_shock_capturing_tiles_match_oracle(shape, faces, precision, step_kernel
         assert err <= SC_TOL[precision], "%s: relative L2 %.2e" % (q, err)
 
 
+SC3_CASES = ([(s, "periodic") for s in ((1, 1, 1), (3, 2, 5), (7, 9, 3), (33, 8, 6), (64, 5, 9), (66, 17, 4), (9, 8, 37))]
+             + [(s, "tube") for s in ((4, 1, 2), (61, 9, 5), (64, 8, 7), (67, 3, 11))] + [((34, 6, 5), "walls")])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("shape,faces", SC3_CASES, ids=["x".join(map(str, c[0])) + "-" + c[1] for c in SC3_CASES])
+def test_shock_capturing_columns_match_oracle(shape, faces, precision):
+    """The 3-D coefficient columns (64 or 32 x 8 nodes marching z, four-node halo, wrapped
+    or clamped) at the edges of the columns and of their z-segments."""
+    from oracle import lbm as olbm
+    c = _plane(shape, faces)
+    coef = (0.5, 0.2, 0.4)
+    m = olbm.Model(c.D, c.shape, c.eos, c.tau, c.Pr, c.cv, c.x_low, c.x_high)
+    m.shock_capturing = coef
+    want = olbm.Sim(m, c.rho, c.u, c.T).step(4).fields()
+    s = P.Solver(c, precision=precision)
+    try:
+        P.lbm_set_shock_capturing(s.h, *coef)
+        got = s.init().step(4).fields()
+    finally:
+        s.close()
+    for q, w in (("rho", want["rho"]), ("u", np.stack(want["u"])), ("T", want["T"])):
+        err = rel_l2(got[q], w)
+        assert err <= SC_TOL[precision], "%s: relative L2 %.2e" % (q, err)
+
+
 @pytest.mark.parametrize("shape,faces", [((70, 9), "periodic"), ((61, 5), "tube"), ((33, 7, 5), "periodic"), ((40, 3, 6), "tube"),
                                          ((1, 1), "periodic")])
 def test_initial_populations_round_the_fp64_equilibria(shape, faces):
