@@ -14,7 +14,7 @@
 // (offset (z Ny + y) pitch + x + G, one plane per component).  Three forms
 // share the per-node arithmetic: in 2-D the step itself leaves S and |grad s|
 // (its block holds the neighbours' u, T and rho) and one launch over tiles does
-// the rest; in 3-D one row-mapped launch for S and |grad s| and one over columns of
+// the rest; in 3-D one launch for S and |grad s| and one over columns of
 // the box; one block per row for the 2-D batches.
 #pragma once
 
@@ -34,34 +34,6 @@ template <typename real, int K>
 __device__ __forceinline__ void n1_store(const Params& p, real* out, unsigned o, const N1Vals<real, K>& r) {
 #pragma unroll
   for (int k = 0; k < K; ++k) out[k * p.plane + o] = r.v[k];
-}
-
-// Thread layout of the stencil kernels: threads along x, blocks along x and over
-// groups of kN1Rows consecutive rows (y, z), each block walking groups gridDim.y
-// apart.  f(x, y, z, o) computes the values of every interior node of the
-// thread, o its element offset in a plane (a plane holds fewer than 2^31
-// elements: the buffers of a handle stay below 2^32 elements, checked at
-// create).  The values of a whole group are computed before any is stored, so
-// that the loads of its rows can all be in flight together (the compiler
-// cannot move a load across a store to a pointer it cannot tell apart).
-constexpr int kN1Rows = 4;
-template <int K, typename real, class F>
-__device__ __forceinline__ void n1_rows(const Params& p, real* out, F&& f) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= p.Nx) return;
-  const int rows = p.Ny * p.Nz;
-  auto off = [&](const int row) { return unsigned(row) * unsigned(p.pitch) + unsigned(x + p.G); };
-  for (int r0 = blockIdx.y * kN1Rows; r0 < rows; r0 += gridDim.y * kN1Rows) {
-    if (r0 + kN1Rows <= rows) {
-      N1Vals<real, K> res[kN1Rows];
-#pragma unroll
-      for (int r = 0; r < kN1Rows; ++r) res[r] = f(x, (r0 + r) % p.Ny, (r0 + r) / p.Ny, off(r0 + r));
-#pragma unroll
-      for (int r = 0; r < kN1Rows; ++r) n1_store(p, out, off(r0 + r), res[r]);
-    } else {
-      for (int row = r0; row < rows; ++row) n1_store(p, out, off(row), f(x, row % p.Ny, row / p.Ny, off(row)));
-    }
-  }
 }
 
 // offset of the interior neighbour (x, y, z) + s e_a of the node at offset o:
@@ -213,13 +185,49 @@ template <int D, typename real> struct N1Buffers {
 
 // ---- single-instance kernels ----
 
-template <int D, typename real>
-__global__ void k_n1_strain(Params p, const real* __restrict__ rho, const real* __restrict__ u,
-                            const real* __restrict__ T) {
+// 3-D: S and |grad s|, one unit of nodes per thread: the loads along y and z and the
+// arithmetic serve both nodes of an FP32 unit (one node per thread, 64 scalar loads
+// for two nodes: 84 us at 384x128x128, now 53 us).
+template <typename S, typename real>
+__global__ void __launch_bounds__(128)
+k_n1_strain_3d(const __grid_constant__ Params p, unsigned n, FastDiv dnx, FastDiv dny, const real* __restrict__ rho,
+               const real* __restrict__ u, const real* __restrict__ T) {
   wait_previous_launch();
-  const N1Buffers<D, real> b(p, rho, u, T);
-  n1_rows<2>(p, b.w0,
-             [&](int x, int y, int z, unsigned o) { return n1_strain_at<D, real>(p, b.rho, b.u, b.T, x, y, z, o); });
+  using U = Unit<S, real>;
+  using V = typename U::V;
+  constexpr int N = U::N;
+  const unsigned gid = blockIdx.x * 128u + threadIdx.x;
+  if (gid >= n) return;
+  const unsigned row = dnx.div(gid), z = dny.div(row);
+  const int y = int(row - z * unsigned(p.Ny)), x = N * int(gid - row * unsigned((p.Nx + N - 1) / N));
+  const bool whole = x + N <= p.Nx;                              // every node of the unit is one of the box
+  const unsigned o = row * unsigned(p.pitch) + unsigned(x + p.G);
+  const unsigned xm = n1_nb(p, x, y, int(z), o, 0, -1), xp = n1_nb(p, x, y, int(z), o, 0, whole ? N : 1);
+  const unsigned nb[2][2] = {{n1_nb(p, x, y, int(z), o, 1, -1), n1_nb(p, x, y, int(z), o, 1, 1)},
+                             {n1_nb(p, x, y, int(z), o, 2, -1), n1_nb(p, x, y, int(z), o, 2, 1)}};
+  auto differences = [&](const real* f, V& c, V& dx, V& dy, V& dz) {
+    const V half = V(real(0.5));
+    c = U::ld_field(f + o);
+    const real l = n1_ld(f + xm), r = n1_ld(f + xp);
+    V up, um;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      U::set(up, k, whole && k + 1 < N ? U::get(c, (k + 1) % N) : r);
+      U::set(um, k, k > 0 ? U::get(c, k > 0 ? k - 1 : 0) : l);
+    }
+    dx = half * (up - um);
+    dy = half * (U::ld_field(f + nb[0][1]) - U::ld_field(f + nb[0][0]));
+    dz = half * (U::ld_field(f + nb[1][1]) - U::ld_field(f + nb[1][0]));
+  };
+  V g[3][3], gT[3], gr[3], r, t, c, Sn, gn;
+#pragma unroll
+  for (int b = 0; b < 3; ++b) differences(u + b * p.plane, c, g[0][b], g[1][b], g[2][b]);
+  differences(T, t, gT[0], gT[1], gT[2]);
+  differences(rho, r, gr[0], gr[1], gr[2]);
+  n1_norms<3>(model_of<real>(p), g, gT, gr, r, t, Sn, gn);
+  const N1Buffers<3, real> b(p);
+  U::store_field(b.w0 + o, Sn, whole);
+  U::store_field(b.w0 + p.plane + o, gn, whole);
 }
 
 // ---- 2-D single-instance form: one launch over tiles of the plane ----
@@ -510,22 +518,22 @@ inline int n1_update(const Params& p, cudaStream_t st, const real* rho, const re
     launch_overlapped(k_n1_coef_2d<S, real>, dim3(unsigned(ntx) * unsigned(nty)), kN1Threads, 0, st, p, ntx);
     return rho ? 2 : 1;
   } else {
-    const int groups = (p.Ny * p.Nz + kN1Rows - 1) / kN1Rows;
-    const dim3 block(128), grid(unsigned((p.Nx + 127) / 128), unsigned(groups < 65535 ? groups : 65535));
-    launch_overlapped(k_n1_strain<D, real>, grid, block.x, 0, st, p, rho, u, T);
     using C = N1Column<S, real>;
     auto kern = k_n1_coef_3d<S, real>;
     const int slots = prepared_blocks<k_n1_coef_3d<S, real>>(kN1Threads, C::kBytes);
+    const unsigned nx = unsigned((p.Nx + C::N - 1) / C::N), n = nx * unsigned(p.Ny) * unsigned(p.Nz);
+    launch_overlapped(k_n1_strain_3d<S, real>, dim3((n + 127u) / 128u), 128, 0, st, p, n, FastDiv(nx),
+                      FastDiv(unsigned(p.Ny)), rho, u, T);
     // z-segments: whole rounds of resident blocks against the eight planes (two
     // thirds of a plane's work) that each segment repeats
     const int ntx = (p.Nx + C::TX - 1) / C::TX, nty = (p.Ny + C::TY - 1) / C::TY;
     int nseg = 1;
     long long least = -1;
-    for (int n = 1; n <= std::min(p.Nz, 32); ++n) {
-      const long long cost = ((long long)ntx * nty * n + slots - 1) / slots * ((p.Nz + n - 1) / n + 5);
+    for (int k = 1; k <= std::min(p.Nz, 32); ++k) {
+      const long long cost = ((long long)ntx * nty * k + slots - 1) / slots * ((p.Nz + k - 1) / k + 5);
       if (least < 0 || cost < least) {
         least = cost;
-        nseg = n;
+        nseg = k;
       }
     }
     launch_overlapped(kern, dim3(unsigned(ntx) * unsigned(nty) * unsigned(nseg)), kN1Threads, C::kBytes, st, p, rho, T, ntx,
