@@ -1,4 +1,4 @@
-"""Throughput benchmark of the fused non-ideal LBM step on GB300.
+"""Throughput benchmark of the non-ideal LBM step on GB300.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                     [--workload tgv256|tgv256-fp64|tgv256-fp16dev|riemann|shockdrop2d|column2d|
@@ -49,7 +49,7 @@ WORKLOADS = {
                     "D3Q27 shock-drop 512x256x256: saturated liquid sphere radius 32 at T_r 0.9, Ma 1.47 shock "
                     "(U^2 = 35), shock capturing C_mu = C_k = 0.3, FP32"),
     "batched": ("batch", dict(), "fp32",
-                "256 uneven D2Q9 shock tubes (128x64 .. 1024x512, Ma 1.1-1.3), one persistent launch per step, FP32"),
+                "256 uneven D2Q9 shock tubes (128x64 .. 1024x512, Ma 1.1-1.3), one graph launch per step, FP32"),
     "batched-drops": ("batch_columns", dict(), "fp32",
                       "256 uneven D2Q9 instances (128x64 .. 1024x512), about half with a liquid column (radius 9-64), "
                       "Ma 1.1-1.5 shocks, saturated liquid/vapour at T_r 0.9 (U^2 = 35), shock capturing C_mu = C_k "
@@ -467,7 +467,7 @@ def run_batched(args):
                        "tile_shape": tile[0], "graph_captured": True, "shock_capturing": sc_coef,
                        "timed_chunk_steps": min(chunk, args.steps)},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                         "traffic": None, "kernel": "batched step (persistent fused kernel + ghost fill%s)"
+                         "traffic": None, "kernel": "batched step (tile kernel + ghost fill%s)"
                          % (" + batched shock-capturing stencils" if sc_coef else ""),
                          "algorithmic_bytes_per_step": alg, "peak_source": peak_kind},
             "e2e": None, "gpu_launches": launches}

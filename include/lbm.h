@@ -104,8 +104,8 @@ enum { LBM_EOS_VDW = 0, LBM_EOS_PR = 1 };
  * (the identity e = c_v T + int_0^rho (P - T dP/dT)/rho'^2 drho', c_v the
  * ideal-gas part); T(rho, e) is the positive root of a quadratic in sqrt(T),
  * taken in a form without cancellation in the arithmetic precision.
- * Peng-Robinson handles step with the exact closure in FP32 or FP64 (fused
- * or multipass); FP16-deviation storage, the learned closure and batches are
+ * Peng-Robinson handles step with the exact closure in FP32 or FP64 (either
+ * step kernel); FP16-deviation storage, the learned closure and batches are
  * van der Waals only.
  * kappa: Korteweg capillarity coefficient, F = kappa rho grad lap rho (Eq. FK).
  * eta_over_mu: bulk to shear viscosity ratio entering alpha (Eq. corr_bulk).
@@ -215,14 +215,15 @@ int lbm_set_populations(lbm_t h, const void* host, size_t bytes);
 /* step implementations (lbm_set_step_kernel) */
 enum { LBM_STEP_FUSED = 0, LBM_STEP_MULTIPASS = 1 };
 
-/* Select how lbm_step runs one time step: LBM_STEP_FUSED (default) is one
- * single-pass kernel per step (plus the ghost fill when x is not periodic);
- * LBM_STEP_MULTIPASS runs moments, primitive fields and collision as three
- * kernels through FP-typed scratch fields.  Both compute the same update.
+/* Select how lbm_step runs one time step: LBM_STEP_FUSED (default) is the
+ * fastest form of the lattice: D2Q9 one kernel per step, D3Q27 moments, primitive
+ * fields and collision as three kernels through scratch fields (plus the ghost
+ * fill at walls); LBM_STEP_MULTIPASS runs the three kernels in either case.
+ * Both compute the same update.
  * Errors: LBM_EINVAL (NULL handle or unknown kind). */
 int lbm_set_step_kernel(lbm_t h, int kind);
 
-/* Time each tile shape of the fused step kernel for `reps` steps from the
+/* Time each form (D2Q9: tile shape) of the step for `reps` steps from the
  * current state (writing only the spare buffer: the state does not advance)
  * and use the fastest from then on.  *chosen (may be NULL) receives the index
  * of the shape (0 is the default), *ms_per_step (may be NULL) its time.
@@ -246,10 +247,9 @@ int lbm_autotune(lbm_t h, int reps, int* chosen, float* ms_per_step);
  * C_mu = C_k = 0.1 a D3Q27 Ma 1.2 shock 32 x 32 nodes wide stays stable,
  * Ma 1.25 needs 0.3 (without: blow-up within 100-200 steps).  C_eta > 0
  * enlarges the explicit bulk shift alpha (Eq. corr_bulk) and can
- * destabilise.  Costs D+2 planes written by the step and extra launches per
- * step: 2 in 2-D (strain with fourth differences over shared-memory tiles;
- * both filter passes with the coefficients), D+2 in 3-D (the last filter pass
- * fused with the coefficients).
+ * destabilise.  Costs four planes written by the step and one launch per step in
+ * 2-D (two with the multi-pass step), two launches in 3-D (S and |grad s|; fourth
+ * differences, filter and coefficients).
  * Errors: LBM_EINVAL (NULL handle, negative or non-finite C), LBM_ENOMEM. */
 int lbm_set_shock_capturing(lbm_t h, double C_mu, double C_eta, double C_k);
 
@@ -270,7 +270,7 @@ int lbm_set_graphs(lbm_t h, int on);
  * a NULL handle. */
 int lbm_autotune_times(lbm_t h, float* ms_per_step, int n);
 
-/* Number of tile shapes of the fused step kernel for this handle's lattice,
+/* Number of forms (tile shapes) of the step for this handle's lattice,
  * precision and closure (the candidates lbm_autotune times, in its order).
  * Returns the count (>= 1), or LBM_EINVAL for a NULL handle. */
 int lbm_tile_count(lbm_t h);
@@ -288,8 +288,8 @@ int lbm_tile_count(lbm_t h);
  * trajectory error of FP32 runs is set by rounding throughout the step, not
  * by the inversion alone.  FP64 handles ignore the setting (their arithmetic
  * is FP64), and so do the learned closure (its network replaces the
- * inversion) and the batched step (FP32 inversion).  Applies to the fused
- * and multi-pass steps from the next step on; does not synchronise.
+ * inversion) and the batched step (FP32 inversion).  Applies to both
+ * step kernels from the next step on; does not synchronise.
  * Errors: LBM_EINVAL (NULL handle). */
 int lbm_set_temperature_fp64(lbm_t h, int on);
 /* 1 while the FP64 temperature inversion is in use (FP32 / FP16-deviation
@@ -297,7 +297,7 @@ int lbm_set_temperature_fp64(lbm_t h, int on);
 int lbm_get_temperature_fp64(lbm_t h);
 
 /* Use tile shape `index` (0 <= index < lbm_tile_count(h); 0 is the default)
- * for the fused step from now on, instead of the autotuner's choice.  Every
+ * for the step from now on, instead of the autotuner's choice.  Every
  * shape computes the same step.  The setting lasts until the next lbm_init,
  * lbm_autotune or closure change (those re-select the remembered or default
  * shape).  Does not synchronise.
@@ -309,11 +309,10 @@ long long lbm_launch_count(lbm_t h);
 
 /* ---- batches ------------------------------------------------------------
  * Many independent instances of one lattice, fluid and precision, each with
- * its own size and x faces, advanced together: every step is one launch of a
- * persistent fused kernel over a work list of (instance, column, plane range)
- * items sorted longest first and taken from an atomic counter, followed by one
- * batched ghost fill; the two launches of a step are captured in a CUDA graph
- * (one per buffer parity).  Results are bit-identical to stepping each
+ * its own size and x faces, advanced together by one graph launch per step (one
+ * graph per buffer parity): D2Q9 one kernel over a work list of (instance, tile)
+ * items and one batched ghost fill, D3Q27 the split step of every instance on
+ * parallel branches of the graph.  Results are bit-identical to stepping each
  * instance alone.  Instances are numbered 0..n-1; all per-instance calls take
  * that index.  The batch uses its own non-blocking stream unless
  * lbm_batch_set_stream gives one (the default stream cannot be captured). */
@@ -406,7 +405,7 @@ int lbm_destroy(lbm_t h);
  * reason to call it.  Errors: LBM_EINVAL (k < 0). */
 int lbm_debug_fail_alloc(int k);
 
-/* Population accesses of the step kernels (fused, multi-pass, ghost fill,
+/* Population accesses of the step kernels (both step kernels, ghost fill,
  * initialisation) that fell outside the handle's population buffers since the
  * library was loaded, in a library built with -DLBM_BOUNDS_CHECK (each such
  * access is skipped: a load gives 0, a store is dropped); -1 in other builds,

@@ -20,7 +20,7 @@
  * fixed-order gradient reduction and AdamW, all in this library's kernels.
  *
  * Once attached to an FP32 solver handle (lbm_mlp_attach) the network is
- * evaluated inside the fused step for every node whose normalised input lies
+ * evaluated inside the step for every node whose normalised input lies
  * in the training box |x0| <= 1, |x1| <= 1; other nodes use the exact closure
  * (range gate).  The exact closure remains the reference: lbm_moments reports
  * T from the exact caloric relation whatever the closure of the step.
@@ -118,7 +118,7 @@ int lbm_mlp_get_mma(lbm_mlp_t net);
 int lbm_mlp_train(lbm_mlp_t net, const double* d_rho, const double* d_e, long long n, int batch, int steps,
                   double lr0, double lr1, double wd, uint64_t seed, float* losses);
 
-/* The closure as the fused step evaluates it, for n device samples:
+/* The closure as the step evaluates it, for n device samples:
  * d_out[4k .. 4k+3] = T, P, c_s^2 and 1 if the network was used (the sample
  * is inside the box) else 0 (exact van der Waals values). */
 int lbm_mlp_predict(lbm_mlp_t net, const double* d_rho, const double* d_e, long long n, double* d_out);

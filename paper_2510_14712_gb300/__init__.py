@@ -284,7 +284,7 @@ def lbm_set_step_kernel(h, kind):
 
 
 def lbm_autotune(h, reps=3):
-    """Pick the fastest fused-kernel tile shape; returns (index, ms per step)."""
+    """Pick the fastest form of the step; returns (index, ms per step)."""
     c, ms = ctypes.c_int(), ctypes.c_float()
     _check(load().lbm_autotune(h, reps, ctypes.byref(c), ctypes.byref(ms)))
     return c.value, ms.value
@@ -318,7 +318,7 @@ def lbm_debug_bounds_violations():
 
 
 def lbm_tile_count(h):
-    """Number of tile shapes of the fused step for this handle."""
+    """Number of forms (tile shapes) of the step for this handle."""
     n = load().lbm_tile_count(h)
     if n < 0:
         _check(n)
@@ -326,7 +326,7 @@ def lbm_tile_count(h):
 
 
 def lbm_set_tile(h, index):
-    """Use tile shape `index` of the fused step until the next init / autotune."""
+    """Use form `index` of the step until the next init / autotune."""
     _check(load().lbm_set_tile(h, int(index)))
 
 

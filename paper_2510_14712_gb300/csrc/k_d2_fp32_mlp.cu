@@ -1,4 +1,4 @@
-// Fused step with the learned closure: D = 2, storage float, arithmetic float.
+// Step with the learned closure: D = 2, storage float, arithmetic float.
 #include "lbm_ops.cuh"
 
 namespace lbm {

@@ -1,4 +1,4 @@
-// Fused step with the exact Peng-Robinson closure: D = 2, FP32 and FP64 storage
+// Step with the exact Peng-Robinson closure: D = 2, FP32 and FP64 storage
 // and arithmetic, FP32 also with the FP64 temperature inversion.
 #include "lbm_ops.cuh"
 

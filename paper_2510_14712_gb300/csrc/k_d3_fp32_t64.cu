@@ -1,4 +1,4 @@
-// Fused step with the FP64 temperature inversion (exact van der Waals
+// Step with the FP64 temperature inversion (exact van der Waals
 // closure): D = 3, storage float, arithmetic float.
 #include "lbm_ops.cuh"
 

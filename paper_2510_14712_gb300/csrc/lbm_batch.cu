@@ -1,10 +1,10 @@
-// lbm_batch.cu - batches of instances stepped by one persistent launch per
+// lbm_batch.cu - batches of instances stepped together by one graph launch per
 // step (include/lbm.h, lbm_batch_*).  Each instance is an ordinary handle
 // (own buffers, boundaries, moments); the batch adds a device table of the
-// instances, a work list of (instance, column, plane range) items sorted
-// longest first, and one CUDA graph per buffer parity holding a step:
-// counter reset, the persistent fused kernel, the batched ghost fill and, when
-// any instance has shock capturing on, the batched shock-capturing stencils.
+// instances and one CUDA graph per buffer parity holding a step.  2-D: a work list
+// of (instance, tile) items, one block each, the batched ghost fill and, when any
+// instance has shock capturing on, the batched shock-capturing stencils.  3-D: the
+// split step of every instance on one of four parallel branches of the graph.
 #include <cstring>
 #include <new>
 #include <string>

@@ -43,7 +43,7 @@ int cuda_fail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call); \
   } while (0)
 
-// Exact-closure table with the fused step and the autotuner swapped for the
+// Exact-closure table with the step and the autotuner swapped for the
 // learned-closure ones (multi-pass and batched steps are exact-only).
 Ops with_mlp(const Ops* base, void (*step)(Handle&, const void*, void*), int (*tune)(Handle&, int, float*),
               int (*ntiles)()) {
@@ -58,7 +58,7 @@ Ops with_mlp(const Ops* base, void (*step)(Handle&, const void*, void*), int (*t
   return o;
 }
 
-// Exact-closure table with the fused step and the autotuner of the Peng-Robinson
+// Exact-closure table with the step and the autotuner of the Peng-Robinson
 // closure (the multi-pass step is EOS-generic; batches are van der Waals only).
 Ops with_pr(const Ops* base, void (*step)(Handle&, const void*, void*), int (*tune)(Handle&, int, float*),
              int (*ntiles)()) {
@@ -72,7 +72,7 @@ Ops with_pr(const Ops* base, void (*step)(Handle&, const void*, void*), int (*tu
   return o;
 }
 
-// Exact-closure table with the fused step and the autotuner of the FP64
+// Exact-closure table with the step and the autotuner of the FP64
 // temperature inversion (the multi-pass step reads Params::t64; batches keep
 // the FP32 inversion).
 Ops with_t64(const Ops* base, void (*step)(Handle&, const void*, void*), int (*tune)(Handle&, int, float*),

@@ -46,8 +46,8 @@ template <typename real, bool T64 = false> struct ExactClosure {
 };
 
 // Exact Peng-Robinson closure: T from the quadratic in sqrt(T) of its caloric
-// relation, then P and c_s^2 of the fluid; stage D reads P and c_s^2 from the
-// centre ring (kExtra = 2) and e = h - P/rho.  T64 (FP32 arithmetic only):
+// relation, then P and c_s^2 of the fluid, handed on to the collision with
+// e = h - P/rho (kExtra = 2).  T64 (FP32 arithmetic only):
 // e = E - |u|^2/2 and the root's argument e - B0 in FP64, rounded once; the
 // root itself has only positive terms and stays in FP32.
 template <typename real, bool T64 = false> struct PrClosure {

@@ -47,7 +47,7 @@ struct Params {
   void* sc_prims;
   const void* sc_visc;
   // FP64 temperature inversion in FP32 arithmetic (lbm_set_temperature_fp64);
-  // read by the multi-pass step (the fused step selects its closure instead)
+  // read by AnyClosure (the steps select their closure instead)
   int t64;
   // the handle's two population buffers (2 Q plane elements each): the
   // bounds of every population access in bounds-check builds
@@ -86,7 +86,7 @@ struct Handle {
   size_t elem_bytes;          // bytes per stored population value
   void* pop[2];               // ping-pong population buffers
   int cur;                    // index of the buffer holding the current state
-  void* scratch;              // moment / primitive fields of the multi-pass path
+  void* scratch;              // moment / primitive fields of the split step and the reported fields
   size_t scratch_bytes;
   double* partials;           // kMaxPartials*(D+2) reduction partials
   double* totals_dev;         // D+2
@@ -97,7 +97,7 @@ struct Handle {
   cudaStream_t stream;
   int initialized, unstable;
   int step_kernel;            // LBM_STEP_FUSED | LBM_STEP_MULTIPASS
-  int tile_cfg;               // index of the fused kernel's tile shape (lbm_autotune)
+  int tile_cfg;               // index of the step's candidate (lbm_autotune)
   long long launches;
   int closure;                // LBM_CLOSURE_EXACT | LBM_CLOSURE_MLP
   void* mlp_img;              // device copy of the attached network's inference image
@@ -168,14 +168,14 @@ struct Ops {
   // macroscopic FP64 fields of pop[cur] into device outputs (any may be NULL);
   // totals (device, D+2 doubles) when non-NULL
   void (*macro)(Handle& h, const void* src, double* rho, double* u, double* T, double* totals);
-  // time the fused kernel's tile shapes, keep the fastest; returns its index
+  // time the step's candidates, keep the fastest; returns its index
   int (*autotune)(Handle& h, int reps, float* best_ms);
   // batches: number of tile shapes; build the device instance table and the
   // sorted work list of shape cfg; enqueue one batched step from `parity`
   int (*batch_ncfg)();
   int (*batch_prepare)(Batch& b, int cfg);
   void (*batch_enqueue)(Batch& b, int parity);
-  // number of tile shapes of the fused step (indices of lbm_set_tile / lbm_autotune)
+  // number of candidates of the step (indices of lbm_set_tile / lbm_autotune)
   int (*ntiles)();
 };
 
@@ -232,10 +232,10 @@ const Ops* ops_d3_fp64();
 const Ops* ops_d3_fp32();
 const Ops* ops_d2_fp16();
 const Ops* ops_d3_fp16();
-// fused step and tile autotuner with the learned closure (FP32 storage)
+// step and autotuner with the learned closure (FP32 storage)
 void step_d2_fp32_mlp(Handle& h, const void* src, void* dst);
 void step_d3_fp32_mlp(Handle& h, const void* src, void* dst);
-// exact Peng-Robinson closure (lbm_eos.kind LBM_EOS_PR): fused step and its autotuner
+// exact Peng-Robinson closure (lbm_eos.kind LBM_EOS_PR): step and its autotuner
 void step_d2_fp32_pr(Handle& h, const void* src, void* dst);
 void step_d3_fp32_pr(Handle& h, const void* src, void* dst);
 void step_d2_fp64_pr(Handle& h, const void* src, void* dst);
@@ -253,7 +253,7 @@ int ntiles_d3_fp64_pr();
 int ntiles_d2_fp32_mlp();
 int ntiles_d3_fp32_mlp();
 // FP32 arithmetic with the FP64 temperature inversion (exact closures):
-// fused step, autotuner and tile count of FP32 and FP16-deviation storage,
+// step, autotuner and candidate count of FP32 and FP16-deviation storage,
 // van der Waals and Peng-Robinson
 void step_d2_fp32_t64(Handle& h, const void* src, void* dst);
 void step_d3_fp32_t64(Handle& h, const void* src, void* dst);

@@ -857,7 +857,7 @@ __global__ void k_mlp_minmax(const double* __restrict__ rho, const double* __res
   }
 }
 
-// The closure of the fused step for standalone samples (4 warps per block).
+// The closure of the step for standalone samples (4 warps per block).
 __global__ void __launch_bounds__(128) k_mlp_predict(const Image* __restrict__ img, Model<float> m,
                                                      const double* __restrict__ rho, const double* __restrict__ e,
                                                      long long n, double* __restrict__ out) {

@@ -162,10 +162,11 @@ __device__ __forceinline__ N1Vals<real, 3> n1_filter_coef_at(const Params& p, co
 }
 
 // Buffers of one handle's shock capturing: the step's rho, u (D planes), T (by
-// default the fused step's copy in sc_prims), the coefficients (3 planes)
-// followed by the work planes w0, w1 (2 each).  The stages run strain -> w0,
-// fourth differences w0 -> w1, filter passes alternating w1 -> w0 -> w1 ...,
-// the last pass with the coefficients.
+// default the 2-D step's copy in sc_prims), the coefficients (3 planes) followed by
+// the work planes w0, w1 (2 each).  S and |grad s| go to w0; the single-instance
+// forms go from there to the coefficients, the batched stages run fourth differences
+// w0 -> w1, filter passes alternating w1 -> w0 -> w1 ..., the last pass with the
+// coefficients.
 template <int D, typename real> struct N1Buffers {
   const real *rho, *u, *T;
   real *visc, *w0, *w1;
@@ -178,7 +179,7 @@ template <int D, typename real> struct N1Buffers {
   __host__ __device__ explicit N1Buffers(const Params& p)
       : N1Buffers(p, static_cast<const real*>(p.sc_prims), static_cast<const real*>(p.sc_prims) + p.plane,
                   static_cast<const real*>(p.sc_prims) + (1 + D) * p.plane) {}
-  // input of filter pass a (a = D - 1: the pass fused with the coefficients)
+  // input of filter pass a (a = D - 1: the pass with the coefficients)
   __host__ __device__ const real* filter_in(int a) const { return a % 2 == 0 ? w1 : w0; }
   __host__ __device__ real* filter_out(int a) const { return a % 2 == 0 ? w0 : w1; }
 };
