@@ -165,19 +165,19 @@ template <int D, typename S, typename real> struct OpsImpl {
 
   // Candidate forms of the step, first = default.
   //
-  // 3-D boxes take the split step: the column-marching kernel evaluated the
-  // moments on 2.1 times the nodes (radius 3 around a 32x8 tile) and held 16
-  // warps per multiprocessor behind three barriers a plane.  Per step, before
-  // and after: 256^3 FP32 2587 -> 1938 us, FP16-deviation 2072 -> 1660 us,
-  // 91x75x53 FP32 129 -> 73 us, FP64 channel 100x24x20 1028 -> 117 us,
-  // 256x128x96 with a network 1326 -> 968 us.
+  // 3-D boxes take the split step: a kernel that marched columns with everything in
+  // one pass evaluated the moments on 2.1 times the nodes (radius 3 around a 32x8
+  // tile) and held 16 warps per multiprocessor behind three barriers a plane.  Per
+  // step, that form and now: 256^3 FP32 2587 and 1808 us, FP16 deviations 2072 and
+  // 1235 us, 91x75x53 FP32 129 and 67 us, Peng-Robinson 128^3 449 and 275 us, FP64
+  // channel 100x24x20 1061 and 128 us, 256x128x96 with a network 1441 and 778 us.
   //
   // 2-D planes take one tile per block; the default picks the shape.
   using LaunchFn = void (*)(Handle&, const void*, void*);
   template <class CL> static int candidates(const LaunchFn** fns) {
     if constexpr (D == 3 && CL::kWarp) {
       // the network's registers: 128 and two blocks per multiprocessor, or one block
-      // without spills (256x128x96: 819 and 864 us per step)
+      // without spills (256x128x96: 778 and 785 us per step)
       static const LaunchFn c[] = {&split<CL, 2>, &split<CL, 1>};
       *fns = c;
       return 2;
@@ -315,9 +315,15 @@ template <int D, typename S, typename real> struct OpsImpl {
       h.launches += 1;
     }
     if (totals) {
-      int nb = int((n + kBlock - 1) / kBlock);
-      if (nb > kMaxPartials) nb = kMaxPartials;
-      k_totals<D, real><<<nb, kBlock, 0, h.stream>>>(p, M(h), W(h), h.partials);
+      int nb;
+      if constexpr (sizeof(real) == 4) {
+        const NodeRange r(p, 0, p.Nx + 2 * p.G, 4);
+        nb = std::min(int((r.n + kBlock - 1) / kBlock), kMaxPartials);
+        k_totals_row<D><<<nb, kBlock, 0, h.stream>>>(p, r, M(h), W(h), h.partials);
+      } else {
+        nb = int(std::min((n + kBlock - 1) / kBlock, (long long)kMaxPartials));
+        k_totals<D, real><<<nb, kBlock, 0, h.stream>>>(p, M(h), W(h), h.partials);
+      }
       k_totals_final<D><<<1, 32 * (D + 2), 0, h.stream>>>(h.partials, nb, totals);
       h.launches += 2;
     }

@@ -7,6 +7,8 @@ wall ends, in every storage form and with every tile shape; and 3-D batches
 Three steps from a noisy drifting state against the FP64 oracle, with the
 suite's tolerances: FP64 1e-12, FP32 1e-5, FP16-deviation 1e-3 on rho and T.
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -175,3 +177,26 @@ def test_initial_populations_round_the_fp64_equilibria(shape, faces):
     off = pops["fp32"] != want
     assert off.mean() <= 1e-4
     assert np.all(np.abs(pops["fp32"] - want) <= np.spacing(np.abs(want)))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16dev", "fp64"])
+@pytest.mark.parametrize("shape,faces", [((1, 1), "periodic"), ((70, 9), "periodic"), ((61, 5), "tube"), ((33, 7, 5), "periodic"),
+                                         ((40, 3, 6), "tube"), ((515, 300), "periodic")])
+def test_totals_are_the_sums_of_the_fields(shape, faces, precision):
+    """lbm_totals by groups of four nodes (rows of any length, ghost columns left out): the
+    mass is the sum of the reported rho up to FP64's rounding; momentum and energy are the
+    sums of rho u and rho (c_v T - a rho + u^2 / 2) up to the fields' FP32 rounding (6e-8
+    each, a few of them per term)."""
+    c = _plane(shape, faces)
+    s = P.Solver(c, precision=precision)
+    try:
+        f = s.init().step(2).fields()
+    finally:
+        s.close()
+    rho, u, T, tot = f["rho"], f["u"], f["T"], f["totals"]
+    assert abs(tot[0] - math.fsum(rho.ravel())) <= 1e-14 * np.abs(rho).sum()
+    tol = 1e-12 if precision == "fp64" else 2e-6
+    for a in range(c.D):
+        assert abs(tot[1 + a] - (rho * u[a]).sum()) <= tol * np.abs(rho * u[a]).sum() + 1e-300
+    e = [rho * c.cv * T, -c.eos["a"] * rho * rho, 0.5 * rho * (u * u).sum(0)]
+    assert abs(tot[1 + c.D] - sum(x.sum() for x in e)) <= tol * sum(np.abs(x).sum() for x in e)
