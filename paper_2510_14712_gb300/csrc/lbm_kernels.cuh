@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params 
 // references of mirrored directions cancel).  RAGGED: a row's last group holds
 // fewer nodes, its last one pulls across the seam.  With four nodes (8-byte
 // loads) FP16-deviation issued as many loads as FP32 for half the bytes: 584 us
-// at 256^3, against FP32's 560 (7 TB/s).
+// at 256^3, against FP32's 560 (7 TB/s); with whole groups 314 and 550 us.
 template <int D, typename S, bool RAGGED>
 __global__ void __launch_bounds__(128) k_moments_row(const __grid_constant__ Params p, const NodeRange range,
                                                      const typename Store<S>::T* __restrict__ A,
@@ -590,8 +590,9 @@ template <int D> struct WPlanes {
 // h and Lambda of a van der Waals node are functions of rho, u_a and T alone: in FP32
 // arithmetic the collision, bound by memory, evaluates them at the node and its
 // neighbours instead of reading four more planes that the pass before wrote
-// (256^3: 1917 -> 1838 us per step in FP32, 1382 -> 1263 with FP16 deviations).  In FP64, bound by the FP64 units, they stay planes; with P and c_s^2 handed
-// on they have no such form.
+// (256^3: 1917 -> 1838 us per step in FP32, 1382 -> 1263 with FP16 deviations).  In
+// FP64, bound by the FP64 units, they stay planes; with P and c_s^2 handed on they
+// have no such form.
 template <typename real, bool EX> constexpr bool derives_fields() { return sizeof(real) == 4 && !EX; }
 
 // The Korteweg force of a 3-D node is the difference of the density's Laplacian
@@ -684,7 +685,9 @@ __global__ void __launch_bounds__(256) k_prims(const __grid_constant__ Params p,
 // Laplacian of three planes (radius 1) in shared memory: rho, j and S are read
 // once, the Laplacian once computed per node instead of six times from 25
 // loads.  The next plane's density and this plane's j, S are loaded before
-// they are needed; two barriers per plane.
+// they are needed; two barriers per plane.  256^3 FP32: 711 us with every value of
+// the stencil read from memory, 217 us in this form, 155 us (5.1 TB/s) since it hands
+// on seven planes fewer.
 // ---------------------------------------------------------------------------
 constexpr int kPrimX = 32, kPrimY = 8;
 template <typename real, class CL> struct PrimsSmem {
@@ -1187,14 +1190,17 @@ __global__ void __launch_bounds__(kGhostBlock) k_ghosts(const __grid_constant__ 
 
 // ---------------------------------------------------------------------------
 // split step, pass 3 in FP32 arithmetic with the rows staged in shared memory:
-// a block owns W consecutive x of one row (y, z).  One warp requests every row
+// a block owns W consecutive x of one row (y, z).  Its warps request every row
 // segment the block reads (the 2Q pulled populations and the primitive fields of
 // the row and of its neighbours along y and z) by bulk asynchronous copies, one
 // per segment, completing on one mbarrier; each thread then collides two nodes
 // from shared memory.  The loads hold no registers and no threads while they
 // are in flight, and an operand address is a base plus a compile-time offset:
 // with loads to registers a third of the instructions were 64-bit address
-// arithmetic and 8 warps per multiprocessor waited on them.
+// arithmetic and 8 warps per multiprocessor waited on them.  256^3: 1437 us with
+// loads to registers, 1619 us with copies issued lane by lane, 1158 us in this form
+// and 1102 us (7.0 TB/s, the copy rate) since it reads fewer fields; FP16 deviations
+// 873 and 790 us, bound by the issue of the conversions.
 //
 // Segments start at multiples of W elements of the padded row; in FP32 storage of a
 // bounded row from its first node on (the G elements before it are a 16-byte unit),

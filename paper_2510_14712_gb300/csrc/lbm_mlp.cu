@@ -11,7 +11,7 @@
 //                   operand images for the next forward; further blocks draw the
 //                   next minibatch (SplitMix64 indices, exact FP64 labels)
 // (k_mlp_batch draws the first one.  With a launch for each part a step took
-// 37 us for 25 us of device time: the launches were the bound.)
+// 37 us for 25 us of device time: the launches were the bound; now 19.8 us.)
 // lbm_mlp_set_mma(LBM_MLP_MMA_WARP) selects the warp-level form instead:
 //   k_mlp_fwd_bwd   per-sample forward and backward pass (mma.sync for the
 //                   64 x 64 products), per-sample factors to memory

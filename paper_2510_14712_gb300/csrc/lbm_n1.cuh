@@ -241,7 +241,7 @@ k_n1_strain_3d(const __grid_constant__ Params p, unsigned n, FastDiv dnx, FastDi
 // wrapped on a periodic axis, clamped to the nearest interior node otherwise.
 // Two tiled launches that read the fields again (strain with fourth differences,
 // filter with coefficients; 48 registers, one node per thread and pass, 572
-// instructions per node) took 137 + 107 us at 4096x2048.
+// instructions per node) took 137 + 107 us at 4096x2048; this launch 85 us.
 constexpr int kN1TileX = 64, kN1TileY = 16, kN1Threads = 256;
 
 template <typename S, typename real>
