@@ -241,7 +241,8 @@ k_n1_strain_3d(const __grid_constant__ Params p, unsigned n, FastDiv dnx, FastDi
 // wrapped on a periodic axis, clamped to the nearest interior node otherwise.
 // Two tiled launches that read the fields again (strain with fourth differences,
 // filter with coefficients; 48 registers, one node per thread and pass, 572
-// instructions per node) took 137 + 107 us at 4096x2048; this launch 85 us.
+// instructions per node) took 137 + 107 us at 4096x2048; this launch 67 us (85 with
+// each load of the box followed by its store).
 constexpr int kN1TileX = 64, kN1TileY = 16, kN1Threads = 256;
 
 template <typename S, typename real>
@@ -262,22 +263,29 @@ __global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant
   auto src = [&](int x) { return p.periodic_x ? n1_wrap(x, p.Nx) : min(max(x, 0), p.Nx - 1); };
   // units of the box whose nodes are not neighbours in memory, or whose halo is clamped
   const bool edge = x0 < HX || x0 + kN1TileX + HX > p.Nx;
-  for (int k = tid; k < P4 / N * H4; k += kN1Threads) {
-    const int r = k / (P4 / N), u = k - r * (P4 / N), x = x0 + N * u - HX;
+  // every load of the box in flight before the first store
+  constexpr int K4 = (P4 / N * H4 + kN1Threads - 1) / kN1Threads;
+  V box[2][K4];
+#pragma unroll
+  for (int i = 0; i < K4; ++i) {
+    const int k = min(tid + i * kN1Threads, P4 / N * H4 - 1), r = k / (P4 / N), x = x0 + N * (k - r * (P4 / N)) - HX;
     const unsigned row = unsigned(n1_wrap(y0 + r - 4, p.Ny)) * pitch + unsigned(p.G);
 #pragma unroll
     for (int f = 0; f < 2; ++f) {
       const real* w = b.w0 + f * p.plane + row;
-      V v;
       if (!edge) {
-        v = U::ld_field(w + x);
+        box[f][i] = U::ld_field(w + x);
       } else {
 #pragma unroll
-        for (int q = 0; q < N; ++q) U::set(v, q, __ldg(w + src(x + q)));
+        for (int q = 0; q < N; ++q) U::set(box[f][i], q, __ldg(w + src(x + q)));
       }
-      U::st(s4[f] + r * P4 + N * u, v);
     }
   }
+#pragma unroll
+  for (int i = 0; i < K4; ++i)
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+      if (tid + i * kN1Threads < P4 / N * H4) U::st(s4[f] + N * (tid + i * kN1Threads), box[f][i]);
   __syncthreads();
   for (int k = tid; k < P2 / N * H2; k += kN1Threads) {
     const int r = k / (P2 / N), u = k - r * (P2 / N), x = x0 + N * u - 2;
