@@ -193,8 +193,14 @@ int sc_alloc(Handle& h) {
   return LBM_OK;
 }
 
-// geometry of the padded layout and the device allocations that depend on it
+// geometry of the padded layout and the device allocations that depend on it.
+// Step graphs hold the addresses of the populations and of the scratch planes,
+// and the allocator may hand out some of the old addresses again: they go first.
 int layout(Handle& h) {
+  if (h.graphs) {
+    CK(cudaDeviceSynchronize());
+    drop_graphs(h);
+  }
   free_state(h);
   Params& p = h.p;
   p.G = p.periodic_x ? 0 : kGhost;
