@@ -196,12 +196,22 @@ int sc_alloc(Handle& h) {
 // geometry of the padded layout and the device allocations that depend on it.
 // Step graphs hold the addresses of the populations and of the scratch planes,
 // and the allocator may hand out some of the old addresses again: they go first.
+// After a failure the handle holds no buffers and is uninitialised; the next
+// lbm_init or lbm_set_populations tries again (ensure_layout).
+int allocate(Handle& h);
 int layout(Handle& h) {
   if (h.graphs) {
     CK(cudaDeviceSynchronize());
     drop_graphs(h);
   }
   free_state(h);
+  h.initialized = 0;
+  const int rc = allocate(h);
+  if (rc != LBM_OK) free_state(h);
+  return rc;
+}
+int ensure_layout(Handle& h) { return h.io_dev ? LBM_OK : layout(h); }
+int allocate(Handle& h) {
   Params& p = h.p;
   p.G = p.periodic_x ? 0 : kGhost;
   const int nxp = p.Nx + 2 * p.G;
@@ -220,7 +230,6 @@ int layout(Handle& h) {
   h.io_bytes = size_t(h.D + 2) * size_t(h.Nx) * h.Ny * h.Nz * sizeof(double);
   CK(dev_malloc(&h.io_dev, h.io_bytes));
   h.cur = 0;
-  h.initialized = 0;
   return sc_alloc(h);
 }
 
@@ -488,6 +497,8 @@ static int init_common(lbm_t h, const double* d_rho, const double* d_u, const do
 
 int lbm_init(lbm_t h, const double* rho, const double* u, const double* T) {
   if (!h || !rho || !u || !T) return fail(LBM_EINVAL, "NULL argument");
+  const int rc = ensure_layout(*h);
+  if (rc != LBM_OK) return rc;
   const size_t N = size_t(h->Nx) * h->Ny * h->Nz;
   double* d = h->io_dev;
   CK(cudaMemcpyAsync(d, rho, N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
@@ -498,6 +509,8 @@ int lbm_init(lbm_t h, const double* rho, const double* u, const double* T) {
 
 int lbm_init_device(lbm_t h, const double* d_rho, const double* d_u, const double* d_T) {
   if (!h || !d_rho || !d_u || !d_T) return fail(LBM_EINVAL, "NULL argument");
+  const int rc = ensure_layout(*h);
+  if (rc != LBM_OK) return rc;
   return init_common(h, d_rho, d_u, d_T);
 }
 
@@ -627,6 +640,8 @@ int lbm_get_populations(lbm_t h, void* host, size_t bytes) {
 int lbm_set_populations(lbm_t h, const void* host, size_t bytes) {
   if (!h || !host) return fail(LBM_EINVAL, "NULL argument");
   if (bytes != lbm_population_bytes(h)) return fail(LBM_EINVAL, "size mismatch");
+  const int rc = ensure_layout(*h);
+  if (rc != LBM_OK) return rc;
   CK(cudaMemcpyAsync(h->pop[h->cur], host, bytes, cudaMemcpyHostToDevice, h->stream));
   CK(cudaMemsetAsync(h->err_dev, 0, sizeof(unsigned), h->stream));
   CK(cudaStreamSynchronize(h->stream));
