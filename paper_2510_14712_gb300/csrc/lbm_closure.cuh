@@ -38,7 +38,7 @@ template <typename real, bool T64 = false> struct ExactClosure {
       T = vdw_temperature_fp64(a64, inv_cv64, rho, E, u2, e);
     } else {
       e = E - real(0.5) * u2;
-      T = (e + m.a * rho) / m.cv;
+      T = vdw_temperature(m, rho, e);
     }
     P = vdw_pressure(m, rho, T);
     cs2 = vdw_cs2(m, rho, T);

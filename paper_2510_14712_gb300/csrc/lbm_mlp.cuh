@@ -228,7 +228,7 @@ __device__ __forceinline__ bool closure_warp(const Image& w, const Model<float>&
     }
   }
   if (!inr) {
-    T = (e + m.a * rho) / m.cv;
+    T = vdw_temperature(m, rho, e);
     P = vdw_pressure(m, rho, T);
     cs2 = vdw_cs2(m, rho, T);
   }
