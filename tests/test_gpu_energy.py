@@ -35,6 +35,12 @@ def vdw(U2, rho, T):
 FLUIDS = {"a3_7": vdw(7.0, 0.6, 0.15), "a3_10": vdw(10.0, 0.65, 0.115), "a3_10_light": vdw(10.0, 0.3, 0.11),
           "a3_35_vapour": vdw(35.0, 0.7385, 0.0326), "a3_35_liquid": vdw(35.0, 1.657, 0.9 / 35.0)}
 
+# Peng-Robinson: h and P handed from the closure to the collision
+PR_EOS = dict(kind="pr", a=0.4032248593772784, b=0.2530765865415995, R=3.253076586541602, kappa=0.01, eta_over_mu=0.0,
+              rho_ref=0.4, T_ref=0.0875, Tc=1.0 / 12.0, m=0.43163854590719997)
+for _r in (0.3, 0.4, 0.45):
+    FLUIDS["pr_%g" % _r] = dict(eos=PR_EOS, cv=8.132691466354006, rho=_r, T=0.0875 if _r < 0.45 else 0.09, u=0.05)
+
 
 def box(fluid, shape):
     f = FLUIDS[fluid]
