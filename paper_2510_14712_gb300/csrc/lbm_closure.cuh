@@ -14,6 +14,7 @@ namespace lbm {
 // `act` says whether the lane's node is real).  kExtra: fields the closure
 // adds to the primitive ring.  kSmem: shared-memory table bytes it loads.
 // kOutput: its fields are reported, not stepped with (no h, no Lambda).
+// kEnergy: the collision takes e as the closure found it, not from T.
 // load() runs once per CTA before the first work item.
 
 // Exact van der Waals closure: Eqs. lbm_temp, Pvdw, vdW_speed_of_sound.
@@ -22,7 +23,7 @@ namespace lbm {
 // FP16-deviation builds.
 template <typename real, bool T64 = false> struct ExactClosure {
   static constexpr bool kPr = false;
-  static constexpr bool kWarp = false, kOutput = false;
+  static constexpr bool kWarp = false, kOutput = false, kEnergy = T64 && sizeof(real) == 4;
   static constexpr int kExtra = 0;
   static constexpr size_t kSmem = 0;
   double a64 = 0.0, inv_cv64 = 0.0;
@@ -52,7 +53,7 @@ template <typename real, bool T64 = false> struct ExactClosure {
 // root itself has only positive terms and stays in FP32.
 template <typename real, bool T64 = false> struct PrClosure {
   static constexpr bool kPr = true;
-  static constexpr bool kWarp = false, kOutput = false;
+  static constexpr bool kWarp = false, kOutput = false, kEnergy = false;
   static constexpr int kExtra = 2;
   static constexpr size_t kSmem = 0;
   __device__ __forceinline__ void load(const Params&, unsigned char*) {}
@@ -75,7 +76,7 @@ template <typename real, bool T64 = false> struct PrClosure {
 // time (Model::kind, Params::t64): the fields that lbm_moments reports and the
 // multi-pass step.
 template <typename real> struct AnyClosure {
-  static constexpr bool kWarp = false, kOutput = true;
+  static constexpr bool kWarp = false, kOutput = true, kEnergy = false;
   static constexpr int kExtra = 0;
   static constexpr size_t kSmem = 0;
   ExactClosure<real, true> vdw64;
@@ -101,7 +102,7 @@ template <typename real> struct AnyClosure {
 // exact closure outside it (range gate).  FP32 arithmetic only.
 struct MlpClosure {
   static constexpr bool kPr = false;
-  static constexpr bool kWarp = true, kOutput = false;
+  static constexpr bool kWarp = true, kOutput = false, kEnergy = false;
   static constexpr int kExtra = 2;
   static constexpr size_t kSmem = sizeof(mlp::Image);
   const mlp::Image* w;

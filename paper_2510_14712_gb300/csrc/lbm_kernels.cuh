@@ -580,11 +580,20 @@ __device__ __forceinline__ void shift(const Params& p, int& xp, int& y, int& z, 
   else z = wrap(z + s, p.Nz);
 }
 
+// What a closure hands on to the collision besides T: nothing (h, Lambda and e of a van
+// der Waals node follow from rho, u and T); P and c_s^2 with h and Lambda (kExtra
+// closures); or e (kEnergy closures: T inverted in FP64, where T rounded to FP32 would
+// not give e back).
+enum Handed { kHandNothing, kHandState, kHandEnergy };
+template <class CL> constexpr Handed handed() {
+  return CL::kExtra > 0 ? kHandState : (CL::kEnergy ? kHandEnergy : kHandNothing);
+}
+
 // Planes of the primitive fields W (split step): u_a, T, F_a; h and Lam_a, unless
-// the collision takes them from rho, u and T (derives_fields); with a closure that
-// hands them on (kExtra), P and c_s^2.
+// the collision takes them from rho, u and T (derives_fields), where e may stand in
+// h's place; with a closure that hands them on, P and c_s^2.
 template <int D> struct WPlanes {
-  static constexpr int U = 0, T = D, H = D + 1, LAM = D + 2, F = 2 * D + 2, P = 3 * D + 2, CS2 = 3 * D + 3;
+  static constexpr int U = 0, T = D, H = D + 1, E = H, LAM = D + 2, F = 2 * D + 2, P = 3 * D + 2, CS2 = 3 * D + 3;
 };
 
 // h and Lambda of a van der Waals node are functions of rho, u_a and T alone: in FP32
@@ -593,7 +602,7 @@ template <int D> struct WPlanes {
 // (256^3: 1917 -> 1838 us per step in FP32, 1382 -> 1263 with FP16 deviations).  In
 // FP64, bound by the FP64 units, they stay planes; with P and c_s^2 handed on they
 // have no such form.
-template <typename real, bool EX> constexpr bool derives_fields() { return sizeof(real) == 4 && !EX; }
+template <typename real, Handed HD> constexpr bool derives_fields() { return sizeof(real) == 4 && HD != kHandState; }
 
 // The Korteweg force of a 3-D node is the difference of the density's Laplacian
 // across it: FP32 steps hand the Laplacian on, one plane (in F's place) for three
@@ -631,19 +640,20 @@ __device__ __forceinline__ void prims_node(const Params& p, const Model<real>& m
   if constexpr (CL::kWarp) closure(m, rho, E, u2, act, T, P, cs2, e);
   else if (act) closure(m, rho, E, u2, act, T, P, cs2, e);
   if (!act) return;
-  constexpr bool kDerived = !CL::kOutput && !derives_fields<real, (CL::kExtra > 0)>();
+  constexpr bool kPlanes = !CL::kOutput && !derives_fields<real, handed<CL>()>();     // h and Lambda
   constexpr bool kLap = !CL::kOutput && hands_laplacian<D, real>();
   const real theta = over_rho(P);                                                       // rounded as handed_energy's
   auto put = [&](const int k, const real v) { W[(long long)k * p.plane + o] = v; };
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     put(WP::U + a, u[a]);
-    if constexpr (kDerived) put(WP::LAM + a, rho * u[a] * u[a] * u[a] + real(3) * rho * u[a] * (theta - real(1.0 / 3.0)));
+    if constexpr (kPlanes) put(WP::LAM + a, rho * u[a] * u[a] * u[a] + real(3) * rho * u[a] * (theta - real(1.0 / 3.0)));
     if constexpr (!kLap) put(WP::F + a, F[a]);
   }
   if constexpr (kLap) put(WP::F, lap);
   put(WP::T, T);
-  if constexpr (kDerived) put(WP::H, e + theta);                                        // Eq. enthalpy
+  if constexpr (kPlanes) put(WP::H, e + theta);                                         // Eq. enthalpy
+  if constexpr (!CL::kOutput && handed<CL>() == kHandEnergy) put(WP::E, e);
   if constexpr (CL::kExtra > 0) {
     put(WP::P, P);
     put(WP::CS2, cs2);
@@ -807,10 +817,10 @@ __global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_c
 
 // ---------------------------------------------------------------------------
 // split step, pass 3: derivatives and collision of every interior node (Eqs.
-// fLBGK, gLBGK), written to dst at the node (pull scheme).  EX: P and c_s^2 of
-// the node come from W (kExtra closures).
+// fLBGK, gLBGK), written to dst at the node (pull scheme).  HD: what the closure
+// handed on.
 // ---------------------------------------------------------------------------
-template <int D, typename S, typename real, bool EX, int NTB, int MINB>
+template <int D, typename S, typename real, Handed HD, int NTB, int MINB>
 __global__ void __launch_bounds__(NTB, MINB)
 k_collide(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
           typename Store<S>::T* __restrict__ B, const real* __restrict__ M, const real* __restrict__ W,
@@ -835,7 +845,7 @@ k_collide(const __grid_constant__ Params p, const NodeRange range, const typenam
   NodeState<D, real> s;
   s.rho = __ldg(M + o);
   s.T = w(WP::T, o);
-  if constexpr (EX) {
+  if constexpr (HD == kHandState) {
     s.P = w(WP::P, o);
     s.cs2 = w(WP::CS2, o);
     s.e = handed_energy(w(WP::H, o), s.P, s.rho);
@@ -903,7 +913,7 @@ template <typename T> __device__ __forceinline__ T* at_bytes(T* base, unsigned o
   return reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off);
 }
 
-template <int D, typename S, bool EX, bool ODD, int NTB, int MINB>
+template <int D, typename S, Handed HD, bool ODD, int NTB, int MINB>
 __global__ void __launch_bounds__(NTB, MINB)
 k_collide2(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
            typename Store<S>::T* __restrict__ B, const float* __restrict__ M, const float* __restrict__ W,
@@ -951,11 +961,19 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
   NodeState<D, F2> s;
   s.rho = f2_of(__ldg(reinterpret_cast<const float2*>(at_bytes(M, 4 * o))));
   s.T = w2(WP::T, o);
-  constexpr bool DER = derives_fields<float, EX>(), LAP = hands_laplacian<D, float>();
+  constexpr bool DER = derives_fields<float, HD>(), LAP = hands_laplacian<D, float>();
   const F2 kr = F2(m.kappa) * s.rho * F2(0.5f);
   F2 h, theta, lap;
   if constexpr (LAP) lap = w2(WP::F, o);
-  if constexpr (DER) h = vdw_enthalpy(m, s.rho, s.T, theta);
+  constexpr bool EN = HD == kHandEnergy;
+  // h and theta = P / rho of a node pair from rho and T, and e where it is handed on
+  auto enthalpy = [&](const F2 rho, const F2 T, const F2 e, F2& th) {
+    const F2 hd = vdw_enthalpy(m, rho, T, th);
+    return EN ? e + th : hd;
+  };
+  F2 e0(0.f), e1(0.f);
+  if constexpr (EN) e0 = w2(WP::E, o);
+  if constexpr (DER) h = enthalpy(s.rho, s.T, e0, theta);
   else h = w2(WP::H, o);
   s.sc = p.sc_on != 0;
   s.mu_num = s.eta_num = s.k_num = F2(0.f);
@@ -985,7 +1003,8 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
       if constexpr (DER) {
         const F2 ro = F2(__ldg(at_bytes(M, 4 * outm)), __ldg(at_bytes(M, 4 * out2)));
         F2 tho;
-        ho = vdw_enthalpy(m, ro, To, tho);
+        if constexpr (EN) e1 = F2(w1(WP::E, outm), w1(WP::E, out2));
+        ho = enthalpy(ro, To, e1, tho);
         lo = lambda_of(ro, uo, tho);
       } else {
         ho = F2(w1(WP::H, outm), w1(WP::H, out2));
@@ -1013,9 +1032,11 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
         const F2 rp = f2_of(__ldg(reinterpret_cast<const float2*>(at_bytes(M, 4 * nbp[a])))),
                  rm = f2_of(__ldg(reinterpret_cast<const float2*>(at_bytes(M, 4 * nbm[a]))));
         F2 th;
-        hp = vdw_enthalpy(m, rp, Tp, th);
+        if constexpr (EN) e1 = w2(WP::E, nbp[a]);
+        hp = enthalpy(rp, Tp, e1, th);
         lp = lambda_of(rp, up, th);
-        hm = vdw_enthalpy(m, rm, Tm, th);
+        if constexpr (EN) e1 = w2(WP::E, nbm[a]);
+        hm = enthalpy(rm, Tm, e1, th);
         lm = lambda_of(rm, um, th);
       } else {
         hp = w2(WP::H, nbp[a]);
@@ -1029,14 +1050,14 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
     s.gradh[a] = F2(0.5f) * (hp - hm);
     s.dLam[a] = upwind(s.u[a], lc - lm, lp - lc);
   }
-  if constexpr (EX) {
+  if constexpr (HD == kHandState) {
     s.P = w2(WP::P, o);
     s.cs2 = w2(WP::CS2, o);
     s.e = handed_energy(h, s.P, s.rho);
   } else {
     s.P = vdw_pressure(m, s.rho, s.T);
     s.cs2 = vdw_cs2(m, s.rho, s.T);
-    s.e = vdw_energy(m, s.rho, s.T);
+    s.e = EN ? e0 : vdw_energy(m, s.rho, s.T);
   }
   if (ODD && !two) {                                         // a lone last node: both halves are this node
     s.rho.y = s.rho.x;
@@ -1220,7 +1241,7 @@ __global__ void __launch_bounds__(kGhostBlock) k_ghosts(const __grid_constant__ 
 constexpr unsigned kWaitLimit = 1u << 22;     // polls of a copy's completion before the step gives up
 
 // Row segments of one block: element offsets in shared memory.
-template <int D, typename S, bool EX, int W> struct RowsLayout {
+template <int D, typename S, Handed HD, int W> struct RowsLayout {
   using ST = typename Store<S>::T;
   static constexpr int Q = Lattice<D>::Q, T3 = Q / 3;            // directions per c_x
   static constexpr int kA = 16 / int(sizeof(ST)), kF = 4;        // elements per 16 bytes: populations, fields
@@ -1236,17 +1257,18 @@ template <int D, typename S, bool EX, int W> struct RowsLayout {
   static constexpr size_t kPopBytes = size_t(2 * kSet) * sizeof(ST);
   // field rows (planes of W): nWide of the row with a unit on both sides; then the
   // row's nOwn; then nSide of the two neighbours along each b > 0
-  static constexpr bool DER = derives_fields<float, EX>();       // h, Lam_a from rho, u_a, T; else read
+  static constexpr bool DER = derives_fields<float, HD>();       // h, Lam_a from rho, u_a, T; else read
+  static constexpr bool EN = HD == kHandEnergy;                  // e of every node read, for h
   static constexpr bool LAP = hands_laplacian<D, float>();       // F from the Laplacian; else read
   static constexpr int RHO = -1;                                 // the density, a plane of M
   static constexpr int nF = LAP ? 0 : D;
-  static constexpr int nSide = (DER ? 3 : 4) + LAP, nOwn = nF + D - 1 + (DER ? 0 : D);
+  static constexpr int nSide = (DER ? 3 : 4) + EN + LAP, nOwn = nF + D - 1 + (DER ? 0 : D);
   static constexpr int kWide = W + 2 * kF, nWide = nSide, nNb = 2 * nSide * (D - 1);
-  // wide and side fields of axis a: u_a, T, then rho, or h and Lam_a; the Laplacian
-  static constexpr int kU = 0, kT = 1, kRho = 2, kH = 2, kLam = 3, kLap = DER ? 3 : 4;
+  // wide and side fields of axis a: u_a, T, then rho (and e), or h and Lam_a; the Laplacian
+  static constexpr int kU = 0, kT = 1, kRho = 2, kEn = 3, kH = 2, kLam = 3, kLap = (DER ? 3 : 4) + EN;
   __host__ __device__ static constexpr int field(int a, int k) {
     using WP = WPlanes<D>;
-    return k == kU ? WP::U + a : (k == kT ? WP::T : (k == kLap ? WP::F : (DER ? RHO : (k == kH ? WP::H : WP::LAM + a))));
+    return k == kU ? WP::U + a : (k == kT ? WP::T : (k == kLap ? WP::F : (DER ? (k == kRho ? RHO : WP::E) : (k == kH ? WP::H : WP::LAM + a))));
   }
   // own rows: F_a, u_b (b > 0), then, if read, Lam_b (b > 0) and rho
   static constexpr int ownRho = nF + 2 * (D - 1);
@@ -1283,7 +1305,7 @@ __device__ __forceinline__ bool elect_one() {
   return e != 0;
 }
 
-template <int D, typename S, bool EX, bool BOUNDED, int W, int MINB>
+template <int D, typename S, Handed HD, bool BOUNDED, int W, int MINB>
 __global__ void __launch_bounds__(W / 2, MINB)
 k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv dny,
                const typename Store<S>::T* __restrict__ A, typename Store<S>::T* __restrict__ B,
@@ -1292,7 +1314,7 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   using WP = WPlanes<D>;
-  using R = RowsLayout<D, S, EX, W>;
+  using R = RowsLayout<D, S, HD, W>;
   constexpr int Q = L::Q;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   ST* sp = reinterpret_cast<ST*>(smem_raw);
@@ -1383,7 +1405,7 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
       s.eta_num = g2(V, 1);
       s.k_num = g2(V, 2);
     }
-    if constexpr (EX) {
+    if constexpr (HD == kHandState) {
       s.P = g2(Wf, WP::P);
       s.cs2 = g2(Wf, WP::CS2);
     }
@@ -1398,8 +1420,14 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
   auto f1at = [&](int off) { return sf[off + 2 * t]; };
   s.rho = f2at(R::DER ? R::wide(R::kRho) : R::own(R::ownRho));
   s.T = f2at(R::wide(R::kT));
-  F2 h, theta;
-  if constexpr (R::DER) h = vdw_enthalpy(m, s.rho, s.T, theta);
+  // h and theta = P / rho of a node pair from rho and T, and e where it is handed on
+  auto enthalpy = [&](const F2 rho, const F2 T, const F2 e, F2& th) {
+    const F2 hd = vdw_enthalpy(m, rho, T, th);
+    return R::EN ? e + th : hd;
+  };
+  F2 h, theta, e0(0.f), e1(0.f);
+  if constexpr (R::EN) e0 = f2at(R::wide(R::kEn));
+  if constexpr (R::DER) h = enthalpy(s.rho, s.T, e0, theta);
   else h = f2at(R::wide(R::kH));
   const F2 kr = F2(m.kappa) * s.rho * F2(0.5f);
   s.div_u = F2(0.f);
@@ -1418,7 +1446,8 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
       if constexpr (R::DER) {
         const F2 ro = outer(R::kRho);
         F2 tho;
-        ho = vdw_enthalpy(m, ro, To, tho);
+        if constexpr (R::EN) e1 = outer(R::kEn);
+        ho = enthalpy(ro, To, e1, tho);
         lo = lambda_of(ro, uo, tho);
       } else {
         ho = outer(R::kH);
@@ -1445,9 +1474,11 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
       if constexpr (R::DER) {
         const F2 rm = side(0, R::kRho), rp = side(1, R::kRho);
         F2 th;
-        hm = vdw_enthalpy(m, rm, Tm, th);
+        if constexpr (R::EN) e1 = side(0, R::kEn);
+        hm = enthalpy(rm, Tm, e1, th);
         lm = lambda_of(rm, um, th);
-        hp = vdw_enthalpy(m, rp, Tp, th);
+        if constexpr (R::EN) e1 = side(1, R::kEn);
+        hp = enthalpy(rp, Tp, e1, th);
         lp = lambda_of(rp, up, th);
       } else {
         hm = side(0, R::kH);
@@ -1462,12 +1493,12 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
     s.gradh[a] = F2(0.5f) * (hp - hm);
     s.dLam[a] = upwind(s.u[a], lc - lm, lp - lc);
   }
-  if constexpr (EX) {
+  if constexpr (HD == kHandState) {
     s.e = handed_energy(h, s.P, s.rho);
   } else {
     s.P = vdw_pressure(m, s.rho, s.T);
     s.cs2 = vdw_cs2(m, s.rho, s.T);
-    s.e = vdw_energy(m, s.rho, s.T);
+    s.e = R::EN ? e0 : vdw_energy(m, s.rho, s.T);
   }
   if (!two) {                                                          // a lone last node: both halves are this node
     s.rho.y = s.rho.x;

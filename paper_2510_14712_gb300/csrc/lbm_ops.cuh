@@ -85,7 +85,7 @@ template <int D, typename S, typename real> struct OpsImpl {
   }
 
   // collision of every interior node; whether it filled the ghost layers too
-  template <bool EX> static bool collide(Handle& h, const void* src, void* dst) {
+  template <Handed HD> static bool collide(Handle& h, const void* src, void* dst) {
     const Params& p = h.p;
     const ST* A = reinterpret_cast<const ST*>(src);
     ST* B = reinterpret_cast<ST*>(dst);
@@ -96,10 +96,10 @@ template <int D, typename S, typename real> struct OpsImpl {
         // of 40 KB, 1013 -> 990 us at 384x128x128 against the bound of 128 registers, which
         // spilled; FP16 deviations: eight of 25 KB, 1234 us at 256^3, with seven 1247)
         constexpr int W128 = 128, kRowsMinB = sizeof(ST) == 4 ? 5 : 8;
-        using R = RowsLayout<D, S, EX, W128>;
-        auto kern = p.periodic_x ? k_collide_rows<D, S, EX, false, W128, kRowsMinB> : k_collide_rows<D, S, EX, true, W128, kRowsMinB>;
-        if (p.periodic_x) prepared_blocks<k_collide_rows<D, S, EX, false, W128, kRowsMinB>>(W128 / 2, R::kBytes);
-        else prepared_blocks<k_collide_rows<D, S, EX, true, W128, kRowsMinB>>(W128 / 2, R::kBytes);
+        using R = RowsLayout<D, S, HD, W128>;
+        auto kern = p.periodic_x ? k_collide_rows<D, S, HD, false, W128, kRowsMinB> : k_collide_rows<D, S, HD, true, W128, kRowsMinB>;
+        if (p.periodic_x) prepared_blocks<k_collide_rows<D, S, HD, false, W128, kRowsMinB>>(W128 / 2, R::kBytes);
+        else prepared_blocks<k_collide_rows<D, S, HD, true, W128, kRowsMinB>>(W128 / 2, R::kBytes);
         const int nseg = (p.G + p.Nx - R::first(p.G, !p.periodic_x) + W128 - 1) / W128;
         launch_overlapped(kern, dim3(unsigned(nseg) * unsigned(p.Ny) * unsigned(p.Nz)), W128 / 2, R::kBytes, h.stream,
             p, nseg, FastDiv(unsigned(nseg)), FastDiv(unsigned(p.Ny)), A, B, M(h), W(h), h.err_dev);
@@ -107,12 +107,12 @@ template <int D, typename S, typename real> struct OpsImpl {
       }
       constexpr int NTB = 128, MINB = 2;
       const NodeRange r(p, p.G, p.G + p.Nx, 2);
-      auto kern = p.Nx % 2 ? k_collide2<D, S, EX, true, NTB, MINB> : k_collide2<D, S, EX, false, NTB, MINB>;
+      auto kern = p.Nx % 2 ? k_collide2<D, S, HD, true, NTB, MINB> : k_collide2<D, S, HD, false, NTB, MINB>;
       launch_overlapped(kern, dim3(unsigned((r.n + NTB - 1) / NTB)), NTB, 0, h.stream, p, r, A, B, M(h), W(h), h.err_dev);
     } else {
       constexpr int NTB = 128, MINB = 2;
       const NodeRange r(p, p.G, p.G + p.Nx);
-      launch_overlapped(k_collide<D, S, real, EX, NTB, MINB>, dim3(unsigned((r.n + NTB - 1) / NTB)), NTB, 0, h.stream, p, r, A, B, M(h),
+      launch_overlapped(k_collide<D, S, real, HD, NTB, MINB>, dim3(unsigned((r.n + NTB - 1) / NTB)), NTB, 0, h.stream, p, r, A, B, M(h),
                                                                                                 W(h), h.err_dev);
     }
     return false;
@@ -122,7 +122,7 @@ template <int D, typename S, typename real> struct OpsImpl {
   template <class CL, int MINB = kPrimsMinB<CL>> static void split(Handle& h, const void* src, void* dst) {
     moments(h, src);
     prims<CL, MINB>(h);
-    if (!collide<(CL::kExtra > 0)>(h, src, dst)) ghosts(h, dst);
+    if (!collide<handed<CL>()>(h, src, dst)) ghosts(h, dst);
   }
 
   static int multiprocessors() {

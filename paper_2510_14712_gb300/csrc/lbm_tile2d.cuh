@@ -324,12 +324,13 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
   // ---------------- C: force and primitive fields on radius 1 ------------------
   // unit (bu, br) of the radius-1 box with its moments; returns rho-independent
   // results through F, T (and P, c_s^2 of closures that hand them on)
-  auto prims = [&](int bu, int br, V rho, const V* j, V Sg, bool act, V* F, V* u, V& T, V& P, V& cs2) {
+  auto prims = [&](int bu, int br, V rho, const V* j, V Sg, bool act, V* F, V* u, V& T, V& P, V& cs2, V& e) {
     const real* l = s_lap + (br + 1) * G::P2 + N * (bu + G::U2 - G::U1);
     const V kr = V(m.kappa) * rho * V(real(0.5)), lc = U::ld(l);
     F[0] = kr * (U::right(l, lc) - U::left(l, lc));                                      // Eq. FK
     F[1] = kr * (U::ld(l + G::P2) - U::ld(l - G::P2));
-    V uF = V(0), u2 = V(0), e = V(0);
+    V uF = V(0), u2 = V(0);
+    e = V(0);
     const Divider<V> over_rho(rho);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
@@ -367,7 +368,7 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
     const bool corner = (br == 0 || br == G::H1 - 1) && (bu == 0 || bu == G::P1 / N - 1);
     const bool act = k < ring1.count() && !corner;
     if (!CL::kWarp && !act) continue;
-    V hr = V(1), hj[2] = {V(0), V(0)}, hS = V(0), F[2], u[2], T, P, cs2;
+    V hr = V(1), hj[2] = {V(0), V(0)}, hS = V(0), F[2], u[2], T, P, cs2, e;
     if (act) {
       hr = U::ld(s_rho + (br + 2) * G::P3 + N * (bu + G::U3 - G::U1));
       if (wtile) {
@@ -382,11 +383,12 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
       hj[1] = U::ld(d + G::P1 * G::H1);
       hS = U::ld(d + 2 * G::P1 * G::H1);
     }
-    prims(bu, br, hr, hj, hS, act, F, u, T, P, cs2);
+    prims(bu, br, hr, hj, hS, act, F, u, T, P, cs2, e);
   }
   NodeState<2, V> s;
   s.rho = rho;
-  if (own) prims(ux + G::U1, uy + 1, rho, j, Se, true, s.F, s.u, s.T, s.P, s.cs2);
+  V e0 = V(0);
+  if (own) prims(ux + G::U1, uy + 1, rho, j, Se, true, s.F, s.u, s.T, s.P, s.cs2, e0);
   __syncthreads();
 
   // ---------------- D: derivatives and collision -------------------------------
@@ -442,7 +444,7 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
     }
     const V h = U::ld(fld(G::PH));
     if constexpr (CL::kExtra > 0) s.e = h - s.P / s.rho;
-    else s.e = vdw_energy(m, s.rho, s.T);
+    else s.e = CL::kEnergy ? e0 : vdw_energy(m, s.rho, s.T);
     s.div_u = V(0);
     const V half = V(real(0.5));
 #pragma unroll

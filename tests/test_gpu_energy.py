@@ -68,9 +68,9 @@ def drift(c, **form):
     return (e1 / r1 - e0 / r0) / STEPS
 
 
-@pytest.mark.parametrize("step_kernel", [0, 1])
+@pytest.mark.parametrize("step_kernel,t_fp64", [(0, None), (1, None), (0, True), (1, True)])
 @pytest.mark.parametrize("shape", [(64, 40, 24), (45, 31, 20), (200, 100)], ids=str)
 @pytest.mark.parametrize("fluid", sorted(FLUIDS))
-def test_total_energy_does_not_drift(fluid, shape, step_kernel):
-    d = drift(box(fluid, shape), step_kernel=step_kernel)
+def test_total_energy_does_not_drift(fluid, shape, step_kernel, t_fp64):
+    d = drift(box(fluid, shape), step_kernel=step_kernel, t_fp64=t_fp64)
     assert abs(d) <= BOUND, "%.2e of the total energy per step" % d
