@@ -1287,9 +1287,28 @@ template <int D, typename S, Handed HD, int W> struct RowsLayout {
   static constexpr size_t kBytes = kPopBytes + sizeof(float) * size_t(nWide * kWide + (nOwn + nNb) * W) + 16;
 };
 
-// the row form applies: every seam unit is a whole 16-byte unit
+constexpr int kRowW = 128;                    // nodes of a block's segment
+
+// segments of a row
+template <typename S> inline int collide_segments(const Params& p) {
+  constexpr int kA = 16 / int(sizeof(typename Store<S>::T));
+  const int first = !p.periodic_x && p.G % kA == 0 ? p.G : 0;              // RowsLayout::first
+  return (p.G + p.Nx - first + kRowW - 1) / kRowW;
+}
+
+// The row form applies when every seam unit is a whole 16-byte unit (4 FP32, 8
+// FP16-deviation values), and is taken when the segments are full enough: its cost is
+// per segment, k_collide2's per node.  Periodic rows cross at 9/16 (2 million nodes, us
+// per step, rows and pairs: Nx 64 292 and 283, 72 317 and 338, 128 234 and 287, 136 301
+// and 316; a box of 4 x 224 x 224: 375 and 170), in both storage types.  Bounded rows,
+// whose ghosts the row form fills and whose pairs straddle 16-byte units, at 3/16 in FP32
+// (Nx 16 964 and 929, 24 639 and 658, 128 307 and 422) and 1/4 with FP16 deviations (24
+// 883 and 433, 32 513 and 546, 128 323 and 348).
 template <typename S> inline bool collide_rows_ok(const Params& p) {
-  return !p.periodic_x || p.Nx % (16 / int(sizeof(typename Store<S>::T))) == 0;   // 4 (FP32) or 8, fields 4
+  constexpr int kA = 16 / int(sizeof(typename Store<S>::T));
+  if (p.periodic_x && p.Nx % kA) return false;
+  const int sixteenths = p.periodic_x ? 9 : (kA == 4 ? 3 : 4);
+  return 16 * p.Nx >= sixteenths * kRowW * collide_segments<S>(p);
 }
 
 __device__ __forceinline__ void bulk_copy(unsigned dst, const void* src, unsigned bytes, unsigned bar) {

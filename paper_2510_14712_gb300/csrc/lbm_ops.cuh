@@ -95,12 +95,12 @@ template <int D, typename S, typename real> struct OpsImpl {
         // registers: blocks per multiprocessor that the shared memory admits (FP32: five
         // of 40 KB, 1013 -> 990 us at 384x128x128 against the bound of 128 registers, which
         // spilled; FP16 deviations: eight of 25 KB, 1234 us at 256^3, with seven 1247)
-        constexpr int W128 = 128, kRowsMinB = sizeof(ST) == 4 ? 5 : 8;
+        constexpr int W128 = kRowW, kRowsMinB = sizeof(ST) == 4 ? 5 : 8;
         using R = RowsLayout<D, S, HD, W128>;
         auto kern = p.periodic_x ? k_collide_rows<D, S, HD, false, W128, kRowsMinB> : k_collide_rows<D, S, HD, true, W128, kRowsMinB>;
         if (p.periodic_x) prepared_blocks<k_collide_rows<D, S, HD, false, W128, kRowsMinB>>(W128 / 2, R::kBytes);
         else prepared_blocks<k_collide_rows<D, S, HD, true, W128, kRowsMinB>>(W128 / 2, R::kBytes);
-        const int nseg = (p.G + p.Nx - R::first(p.G, !p.periodic_x) + W128 - 1) / W128;
+        const int nseg = collide_segments<S>(p);
         launch_overlapped(kern, dim3(unsigned(nseg) * unsigned(p.Ny) * unsigned(p.Nz)), W128 / 2, R::kBytes, h.stream,
             p, nseg, FastDiv(unsigned(nseg)), FastDiv(unsigned(p.Ny)), A, B, M(h), W(h), h.err_dev);
         return p.bc_lo != LBM_BC_WALL && p.bc_hi != LBM_BC_WALL;
