@@ -172,7 +172,14 @@ template <int D, typename S, typename real> struct OpsImpl {
   // 1235 us, 91x75x53 FP32 129 and 67 us, Peng-Robinson 128^3 449 and 275 us, FP64
   // channel 100x24x20 1061 and 128 us, 256x128x96 with a network 1441 and 778 us.
   //
-  // 2-D planes take one tile per block; the default picks the shape.
+  // 2-D planes take one tile per block, the default picks the shape; FP64 planes of
+  // 2^16 nodes and more the split step: a tile evaluates the density on twice its nodes,
+  // which the FP64 units, not the memory, pay for (tiles and split step, us per step:
+  // 128x128 23.9 and 25.5, 256x256 85 and 67, 512x512 256 and 226, 1024x1024 988 and 860,
+  // 2048x2048 3921 and 3415, where the row-marching form before took 3551).
+  static bool plane_splits(const Params& p) {
+    return D == 2 && sizeof(real) == 8 && (long long)p.Nx * p.Ny >= (1 << 16);
+  }
   using LaunchFn = void (*)(Handle&, const void*, void*);
   template <class CL> static int candidates(const LaunchFn** fns) {
     if constexpr (D == 3 && CL::kWarp) {
@@ -197,6 +204,9 @@ template <int D, typename S, typename real> struct OpsImpl {
   template <class CL, class... T> struct TileSet {
     static constexpr int n = int(sizeof...(T));
     static void rule(Handle& h, const void* src, void* dst) {
+      if constexpr (sizeof(real) == 8) {
+        if (plane_splits(h.p)) return split<CL>(h, src, dst);
+      }
       static const LaunchFn fn[] = {&T::launch...};
       const double work[] = {T::work()...};
       const long long tiles[] = {T::tiles(h.p)...};
@@ -243,8 +253,9 @@ template <int D, typename S, typename real> struct OpsImpl {
   template <class CL> static void step_cl(Handle& h, const void* src, void* dst) {
     const LaunchFn* fns;
     const int n = candidates<CL>(&fns);
-    fns[h.tile_cfg < n ? h.tile_cfg : 0](h, src, dst);
-    if (h.p.sc_on && D == 3) {
+    const int cfg = h.tile_cfg < n ? h.tile_cfg : 0;
+    fns[cfg](h, src, dst);
+    if (h.p.sc_on && (D == 3 || (cfg == 0 && plane_splits(h.p)))) {
       shock_capturing(h, M(h), W(h), W(h) + D * h.p.plane);
     } else if (h.p.sc_on) {
       shock_capturing(h, nullptr, nullptr, nullptr);
