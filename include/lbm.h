@@ -216,7 +216,7 @@ int lbm_set_populations(lbm_t h, const void* host, size_t bytes);
 enum { LBM_STEP_FUSED = 0, LBM_STEP_MULTIPASS = 1 };
 
 /* Select how lbm_step runs one time step: LBM_STEP_FUSED (default) is the
- * fastest form of the lattice: D2Q9 one kernel per step (FP64 planes of 2^16
+ * fastest form of the lattice: D2Q9 one kernel per step (FP64 planes of 2^20
  * nodes and more: as D3Q27), D3Q27 moments, primitive fields and collision as
  * three kernels through scratch fields (plus the ghost fill at walls); LBM_STEP_MULTIPASS runs the three kernels in either case.
  * Both compute the same update.

@@ -173,12 +173,14 @@ template <int D, typename S, typename real> struct OpsImpl {
   // channel 100x24x20 1061 and 128 us, 256x128x96 with a network 1441 and 778 us.
   //
   // 2-D planes take one tile per block, the default picks the shape; FP64 planes of
-  // 2^16 nodes and more the split step: a tile evaluates the density on twice its nodes,
+  // 2^20 nodes and more the split step: a tile evaluates the density on twice its nodes,
   // which the FP64 units, not the memory, pay for (tiles and split step, us per step:
-  // 128x128 23.9 and 25.5, 256x256 85 and 67, 512x512 256 and 226, 1024x1024 988 and 860,
-  // 2048x2048 3921 and 3415, where the row-marching form before took 3551).
+  // 256x256 85 and 68, 512x512 256 and 227, 1024x1024 988 and 865, 2048x2048 3921 and
+  // 3423, where the row-marching form before took 3551).  Smaller planes, faster than
+  // that form either way, keep the one launch that their batches share; a batch takes
+  // planes that split in launches of their own, for the bits of a handle.
   static bool plane_splits(const Params& p) {
-    return D == 2 && sizeof(real) == 8 && (long long)p.Nx * p.Ny >= (1 << 16);
+    return D == 2 && sizeof(real) == 8 && (long long)p.Nx * p.Ny >= (1 << 20);
   }
   using LaunchFn = void (*)(Handle&, const void*, void*);
   template <class CL> static int candidates(const LaunchFn** fns) {
@@ -348,6 +350,23 @@ template <int D, typename S, typename real> struct OpsImpl {
   }
 
   // ---- batches -------------------------------------------------------------
+  // 2-D instances that step with launches of their own: planes that a single handle
+  // splits (a batch gives a handle's bits)
+  static bool own_launches(const Batch&, const Params& p) { return plane_splits(p); }
+  static void enqueue_own(Batch& b, int parity) {
+    for (int k = 0; k < b.n; ++k) {
+      Handle& h = *b.inst[k];
+      if (!own_launches(b, h.p)) continue;
+      const Handle saved = h;
+      h.stream = b.stream;
+      h.err_dev = b.d_errs + k;
+      split<ExactClosure<real>>(h, h.pop[parity], h.pop[parity ^ 1]);
+      if (h.p.sc_on && !b.tuning) shock_capturing(h, M(h), W(h), W(h) + D * h.p.plane);
+      b.launches += h.launches - saved.launches;
+      h = saved;
+    }
+  }
+
   // 2-D: one launch over the tiles of every instance
   template <int TX, int TY, int MINB> struct BatchTiles {
     using G = TileGeom<real, Unit<S, real>::N, TX, TY>;
@@ -361,21 +380,23 @@ template <int D, typename S, typename real> struct OpsImpl {
         ti[k].pop[0] = h.pop[0];
         ti[k].pop[1] = h.pop[1];
         order[k] = k;
-        rowstart[k + 1] = rowstart[k] + (h.p.sc_on ? h.p.Ny * h.p.Nz : 0);
+        rowstart[k + 1] = rowstart[k] + (h.p.sc_on && !own_launches(b, h.p) ? h.p.Ny * h.p.Nz : 0);
       }
       std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
         return (long long)ti[a].p.Nx * ti[a].p.Ny > (long long)ti[c].p.Nx * ti[c].p.Ny;
       });
-      for (int k : order)
+      for (int k : order) {
+        if (own_launches(b, ti[k].p)) continue;
         for (int y = 0; y < ti[k].p.Ny; y += TY)
           for (int x = 0; x < ti[k].p.Nx; x += TX) items.push_back({k, x, y});
+      }
       if (b.d_insts) cudaFree(b.d_insts);
       if (b.d_items) cudaFree(b.d_items);
       if (b.d_n1rows) cudaFree(b.d_n1rows);
       b.d_insts = b.d_items = nullptr;
       b.d_n1rows = nullptr;
       if (dev_malloc(&b.d_insts, sizeof(BatchInstance) * b.n) != cudaSuccess) return LBM_ENOMEM;
-      if (dev_malloc(&b.d_items, sizeof(BatchItem) * items.size()) != cudaSuccess) return LBM_ENOMEM;
+      if (dev_malloc(&b.d_items, sizeof(BatchItem) * std::max<size_t>(items.size(), 1)) != cudaSuccess) return LBM_ENOMEM;
       if (dev_malloc(&b.d_n1rows, sizeof(int) * (b.n + 1)) != cudaSuccess) return LBM_ENOMEM;
       cudaMemcpy(b.d_insts, ti.data(), sizeof(BatchInstance) * b.n, cudaMemcpyHostToDevice);
       cudaMemcpy(b.d_items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice);
@@ -385,7 +406,7 @@ template <int D, typename S, typename real> struct OpsImpl {
       // blocks per instance of the wall fill: one item per thread of the instance with the most
       long long ng = 0;
       for (int k = 0; k < b.n; ++k)
-        if (ti[k].p.bc_lo == LBM_BC_WALL || ti[k].p.bc_hi == LBM_BC_WALL)
+        if (!own_launches(b, ti[k].p) && (ti[k].p.bc_lo == LBM_BC_WALL || ti[k].p.bc_hi == LBM_BC_WALL))
           ng = std::max(ng, ghost_items<D>(ti[k].p, true) + ghost_items<D>(ti[k].p, false));
       b.ghost_blocks = unsigned(std::max(1LL, std::min((ng + 255) / 256, 4096LL)));
       cudaFuncSetAttribute(k_step2d_batch<S, real, TX, TY, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(G::kBytes));
@@ -393,15 +414,18 @@ template <int D, typename S, typename real> struct OpsImpl {
     }
     static void enqueue(Batch& b, int parity) {
       const BatchInstance* insts = reinterpret_cast<const BatchInstance*>(b.d_insts);
-      launch_overlapped(k_step2d_batch<S, real, TX, TY, MINB>, dim3(unsigned(b.nitems)), G::NT, G::kBytes, b.stream,
-          insts, reinterpret_cast<const BatchItem*>(b.d_items), parity, b.d_errs);
-      b.launches += 1;
-      for (int k0 = 0; k0 < b.n; k0 += 65535) {
-        launch_overlapped(k_ghosts_batch<D, S>, dim3(b.ghost_blocks, unsigned(b.n - k0 < 65535 ? b.n - k0 : 65535)), 256, 0, b.stream,
-            insts + k0, parity);
+      if (b.nitems > 0) {
+        launch_overlapped(k_step2d_batch<S, real, TX, TY, MINB>, dim3(unsigned(b.nitems)), G::NT, G::kBytes, b.stream,
+            insts, reinterpret_cast<const BatchItem*>(b.d_items), parity, b.d_errs);
         b.launches += 1;
+        for (int k0 = 0; k0 < b.n; k0 += 65535) {
+          launch_overlapped(k_ghosts_batch<D, S>, dim3(b.ghost_blocks, unsigned(b.n - k0 < 65535 ? b.n - k0 : 65535)), 256, 0, b.stream,
+              insts + k0, parity);
+          b.launches += 1;
+        }
       }
       if (b.n1rows > 0 && !b.tuning) b.launches += n1_update_batch<D, real>(insts, b.d_n1rows, b.n, b.n1rows, b.stream);
+      enqueue_own(b, parity);
     }
   };
 

@@ -539,7 +539,7 @@ __global__ void k_ghosts_batch(const BatchInstance* __restrict__ insts, int pari
   using ST = typename Store<S>::T;
   const BatchInstance& bi = insts[blockIdx.y];
   const Params& p = bi.p;
-  if (p.periodic_x || (p.bc_lo != LBM_BC_WALL && p.bc_hi != LBM_BC_WALL)) return;
+  if (p.periodic_x || (p.bc_lo != LBM_BC_WALL && p.bc_hi != LBM_BC_WALL)) return;   // (an instance with launches of its own fills its walls after this)
   ghost_fill<D, S>(p, reinterpret_cast<ST*>(bi.pop[parity ^ 1]), blockIdx.x * (long long)blockDim.x + threadIdx.x,
                    (long long)gridDim.x * blockDim.x);
 }

@@ -119,12 +119,12 @@ def test_shock_capturing_with_fp16_deviations(shape, faces):
         assert node_err(got["u"][a], want["u"][a])[0] <= 4 * ulim
 
 
-PLANES = [((x, 256), f, fl, sc) for x in (255, 256) for f in ("periodic", "walls") for fl in ("vdw", "pr") for sc in (None, (0.3, 0.1, 0.2))]
+PLANES = [((x, 1024), f, fl, sc) for x in (1023, 1024) for f in ("periodic", "walls") for fl in ("vdw", "pr") for sc in (None, (0.3, 0.1, 0.2))]
 
 
 @pytest.mark.parametrize("shape,faces,fluid,coef", PLANES, ids=["%s-%s-%s-%s" % (c[0][0], c[1], c[2], "sc" if c[3] else "") for c in PLANES])
 def test_fp64_planes_on_either_side_of_the_split_step(shape, faces, fluid, coef):
-    """FP64 planes of 2^16 nodes and more take the three passes: one node column less or more
+    """FP64 planes of 2^20 nodes and more take the three passes: one node column less or more
     against the multi-pass step and, in the default form, every tile shape."""
     c = _case(shape, faces, fluid)
     want = run(c, "fp64", 3, step_kernel=P.LBM_STEP_MULTIPASS, sc=coef)
