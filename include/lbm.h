@@ -311,8 +311,8 @@ long long lbm_launch_count(lbm_t h);
  * Many independent instances of one lattice, fluid and precision, each with
  * its own size and x faces, advanced together by one graph launch per step (one
  * graph per buffer parity): D2Q9 one kernel over a work list of (instance, tile)
- * items and one batched ghost fill, D3Q27 the split step of every instance on
- * parallel branches of the graph.  Results are bit-identical to stepping each
+ * items and one batched ghost fill, D3Q27 the three kernels of the split step, each
+ * over the blocks of every instance.  Results are bit-identical to stepping each
  * instance alone.  Instances are numbered 0..n-1; all per-instance calls take
  * that index.  The batch uses its own non-blocking stream unless
  * lbm_batch_set_stream gives one (the default stream cannot be captured). */

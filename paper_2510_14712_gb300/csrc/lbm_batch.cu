@@ -4,7 +4,7 @@
 // instances and one CUDA graph per buffer parity holding a step.  2-D: a work list
 // of (instance, tile) items, one block each, the batched ghost fill and, when any
 // instance has shock capturing on, the batched shock-capturing stencils.  3-D: the
-// split step of every instance on one of four parallel branches of the graph.
+// passes of the split step, each over the blocks of every instance (lbm_batch3d.cuh).
 #include <cstring>
 #include <new>
 #include <string>
@@ -289,11 +289,6 @@ int lbm_batch_destroy(lbm_batch_t b) {
   if (b->d_insts) cudaFree(b->d_insts);
   if (b->d_n1rows) cudaFree(b->d_n1rows);
   if (b->d_items) cudaFree(b->d_items);
-  for (int k = 0; k < kBatchBranches; ++k) {
-    if (b->branch[k]) cudaStreamDestroy(b->branch[k]);
-    if (b->join[k]) cudaEventDestroy(b->join[k]);
-  }
-  if (b->fork) cudaEventDestroy(b->fork);
   if (b->d_errs) cudaFree(b->d_errs);
   if (b->h_errs) cudaFreeHost(b->h_errs);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);

@@ -3,10 +3,12 @@
 // instance and the block of its own launch that a block stands for, the largest instances
 // first; the instances' parameters and geometry are read from a table.
 //
-// Three launches of its own for every instance (on four parallel branches of the step's
-// graph) cost a launch's latency each: 256 boxes of 8^3 FP32 took 1069 us per step, in the
-// one persistent kernel before 140 us, now @A@; 256 of 16^3 1211, 454, @B@; 64 of
-// 32^3 602, 425, @C@; 16 of 48^3 386, 534, @D@; 4 of 64^3 @E@.
+// Three launches of its own for every instance cost a launch's latency each.  us per step
+// with those on four branches of the step's graph, with the persistent kernel before
+// them, and in this form (FP32): 256 boxes of 8^3 1069, 140, 60; 256 of 16^3 1211, 454,
+// 235; 64 of 32^3 602, 425, 316; 16 of 48^3 386, 534, 301; 4 of 64^3 163, 525, 160.  Boxes
+// that fill the device by themselves pay for the parameters being read from memory: 4
+// tubes of 64^3 220, 4266, 249.
 #pragma once
 
 #include "lbm_n1.cuh"

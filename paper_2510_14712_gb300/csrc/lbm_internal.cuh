@@ -156,7 +156,6 @@ template <auto kern> static int prepared_blocks(int threads, size_t smem) {
 }
 
 struct Batch;
-constexpr int kBatchBranches = 4;
 
 // Per (D, precision) kernel set.
 struct Ops {
@@ -183,8 +182,8 @@ struct Ops {
 struct Batch {
   int n, D, Q, precision;
   Handle** inst;              // one handle per instance (own buffers and scratch)
-  void* d_insts;              // device table of BatchInstance
-  void* d_items;              // device work list of BatchItem, largest instances first
+  void* d_insts;              // device table of BatchInstance (2-D) or SplitInstance (3-D)
+  void* d_items;              // device work list of BatchItem or SplitItem, largest instances first
   int nitems;
   int* d_n1rows;              // first global row of each instance's shock capturing (n + 1 entries)
   unsigned ghost_blocks;      // blocks per instance of the batched ghost fill
@@ -192,8 +191,7 @@ struct Batch {
   int graph_launches;         // kernel launches of one step's graph
   int tuning;                 // graphs for timing tile shapes: no shock-capturing stencils (they would
                               // overwrite the coefficients the next real step reads)
-  cudaStream_t branch[kBatchBranches];   // 3-D batches: branches of the step's graph, with their
-  cudaEvent_t fork, join[kBatchBranches];  // fork and join events
+  int group[10];              // 3-D: first work item of each launch of the step, and their end
   unsigned* d_errs;           // status word per instance
   unsigned* h_errs;           // pinned copy
   cudaStream_t stream;

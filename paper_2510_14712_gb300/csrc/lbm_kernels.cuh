@@ -233,7 +233,7 @@ __device__ inline void prim_ext(const Params& p, const double* rho, const double
 // ---------------------------------------------------------------------------
 struct FastDiv {
   unsigned d, m, s;
-  __host__ __device__ FastDiv() : d(1), m(1), s(0) {}
+  __host__ __device__ FastDiv() : d(1), m(1), s(0) {}                     // by one
   __host__ explicit FastDiv(unsigned d_) : d(d_), s(0) {
     while ((1ull << s) < d) ++s;
     m = unsigned(((1ull << 32) * ((1ull << s) - d)) / d + 1);
@@ -246,6 +246,7 @@ struct NodeRange {
   int lo, quad;
   unsigned n;
   FastDiv nx, ny;
+  __host__ NodeRange() : lo(0), quad(1), n(0) {}
   __host__ NodeRange(const Params& p, int lo_, int hi_, int quad_ = 1)
       : lo(lo_), quad(quad_), nx(unsigned((hi_ - lo_ + quad_ - 1) / quad_)), ny(unsigned(p.Ny)) {
     n = nx.d * unsigned(p.Ny) * unsigned(p.Nz);
@@ -414,12 +415,10 @@ __global__ void __launch_bounds__(128) k_init_df(const __grid_constant__ Params 
 // ---------------------------------------------------------------------------
 // FP64: one node per thread
 template <int D>
-__global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params p, const NodeRange range,
-                                                 const double* __restrict__ A, double* __restrict__ M) {
-  wait_previous_launch();
+__device__ __forceinline__ void moments_nodes(const Params& p, const NodeRange& range, const double* __restrict__ A, double* __restrict__ M, const unsigned block) {
   using L = Lattice<D>;
   int xp, y, z;
-  if (!range.decode(blockIdx.x * blockDim.x + threadIdx.x, xp, y, z)) return;
+  if (!range.decode(block * blockDim.x + threadIdx.x, xp, y, z)) return;
   const PullOffsets<D> po(p, xp, y, z);
   auto pulled = [&](const int i, const int ii) {
     const double* Ai = A + (long long)ii * p.plane;
@@ -446,6 +445,12 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params 
   for (int a = 0; a < D; ++a) M[(1 + a) * p.plane + o] = sp[a] - sn[a];
   M[(1 + D) * p.plane + o] = S;
 }
+template <int D>
+__global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params p, const NodeRange range,
+                                                 const double* __restrict__ A, double* __restrict__ M) {
+  wait_previous_launch();
+  moments_nodes<D>(p, range, A, M, blockIdx.x);
+}
 
 // FP32 arithmetic: the nodes of one 16-byte load (4 FP32, 8 FP16-deviation
 // values) per thread, packed sums; a direction with c_x != 0 takes one scalar
@@ -456,15 +461,13 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ Params 
 // loads) FP16-deviation issued as many loads as FP32 for half the bytes: 584 us
 // at 256^3, against FP32's 560 (7 TB/s); with whole groups 314 and 550 us.
 template <int D, typename S, bool RAGGED>
-__global__ void __launch_bounds__(128) k_moments_row(const __grid_constant__ Params p, const NodeRange range,
-                                                     const typename Store<S>::T* __restrict__ A,
-                                                     float* __restrict__ M) {
-  wait_previous_launch();
+__device__ __forceinline__ void moments_groups(const Params& p, const NodeRange& range, const typename Store<S>::T* __restrict__ A,
+                                              float* __restrict__ M, const unsigned block) {
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   constexpr int N = Store<S>::kGroup, H = N / 2, T3 = L::Q / 3;
   int xp, y, z;
-  if (!range.decode(blockIdx.x * blockDim.x + threadIdx.x, xp, y, z)) return;
+  if (!range.decode(block * blockDim.x + threadIdx.x, xp, y, z)) return;
   PullOffsets<D> po;
   po.rows(p, y, z);
   // the node that pulls from right of the group, and the sources left and right
@@ -551,6 +554,13 @@ __global__ void __launch_bounds__(128) k_moments_row(const __grid_constant__ Par
 #pragma unroll
   for (int j = 0; j < H; ++j) rho[j] += F2(p.refsum[1]);
   put(1 + D, rho);
+}
+template <int D, typename S, bool RAGGED>
+__global__ void __launch_bounds__(128) k_moments_row(const __grid_constant__ Params p, const NodeRange range,
+                                                     const typename Store<S>::T* __restrict__ A,
+                                                     float* __restrict__ M) {
+  wait_previous_launch();
+  moments_groups<D, S, RAGGED>(p, range, A, M, blockIdx.x);
 }
 
 // neighbour offset along axis a by s (wrapping periodic axes)
@@ -711,10 +721,8 @@ template <typename real, class CL> struct PrimsSmem {
   real lap[3][(kPrimY + 2) * (kPrimX + 2)];
 };
 template <typename real, class CL, int MINB>
-__global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_constant__ Params p, int lo, int hi, int ncolx,
-                                                           int ncoly, int nseg, const real* __restrict__ M,
-                                                           real* __restrict__ W) {
-  wait_previous_launch();
+__device__ __forceinline__ void prims_column(const Params& p, int lo, int hi, int ncolx, int ncoly, int nseg,
+                                             const real* __restrict__ M, real* __restrict__ W, const unsigned block) {
   constexpr int NT = kPrimX * kPrimY, BX2 = kPrimX + 4, BX1 = kPrimX + 2;
   constexpr int N2 = BX2 * (kPrimY + 4), N1 = BX1 * (kPrimY + 2), K2 = (N2 + NT - 1) / NT, K1 = (N1 + NT - 1) / NT;
   __shared__ PrimsSmem<real, CL> sm;
@@ -723,7 +731,7 @@ __global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_c
   closure.load(p, smem_raw);
   const Model<real> m = model_of<real>(p);
   const int tid = threadIdx.x, lx = tid % kPrimX, ly = tid / kPrimX;
-  int b = blockIdx.x;
+  int b = block;
   const int x0 = lo + (b % ncolx) * kPrimX;
   b /= ncolx;
   const int y0 = (b % ncoly) * kPrimY, seg = b / ncoly;
@@ -814,6 +822,13 @@ __global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_c
     l0 = t;
   }
 }
+template <typename real, class CL, int MINB>
+__global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_constant__ Params p, int lo, int hi, int ncolx,
+                                                           int ncoly, int nseg, const real* __restrict__ M,
+                                                           real* __restrict__ W) {
+  wait_previous_launch();
+  prims_column<real, CL, MINB>(p, lo, hi, ncolx, ncoly, nseg, M, W, blockIdx.x);
+}
 
 // ---------------------------------------------------------------------------
 // split step, pass 3: derivatives and collision of every interior node (Eqs.
@@ -821,16 +836,14 @@ __global__ void __launch_bounds__(kPrimX * kPrimY, MINB) k_prims3(const __grid_c
 // handed on.
 // ---------------------------------------------------------------------------
 template <int D, typename S, typename real, Handed HD, int NTB, int MINB>
-__global__ void __launch_bounds__(NTB, MINB)
-k_collide(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
-          typename Store<S>::T* __restrict__ B, const real* __restrict__ M, const real* __restrict__ W,
-          unsigned* err) {
-  wait_previous_launch();
+__device__ __forceinline__ void collide_nodes(const Params& p, const NodeRange& range, const typename Store<S>::T* __restrict__ A,
+                                              typename Store<S>::T* __restrict__ B, const real* __restrict__ M,
+                                              const real* __restrict__ W, unsigned* err, const unsigned block) {
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   using WP = WPlanes<D>;
   int xp, y, z;
-  if (!range.decode(blockIdx.x * NTB + threadIdx.x, xp, y, z)) return;
+  if (!range.decode(block * NTB + threadIdx.x, xp, y, z)) return;
   const PullOffsets<D> po(p, xp, y, z);
   const unsigned o = po.r[D == 3 ? 4 : 1] + unsigned(xp);
   real v[L::Q];
@@ -892,6 +905,14 @@ k_collide(const __grid_constant__ Params p, const NodeRange range, const typenam
   }
   FactoredRelax<D, real>::g_pass(at, [&](int i) { return v[i]; }, [&](int i, real x) { put(L::Q + i, x); });
 }
+template <int D, typename S, typename real, Handed HD, int NTB, int MINB>
+__global__ void __launch_bounds__(NTB, MINB)
+k_collide(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
+          typename Store<S>::T* __restrict__ B, const real* __restrict__ M, const real* __restrict__ W,
+          unsigned* err) {
+  wait_previous_launch();
+  collide_nodes<D, S, real, HD, NTB, MINB>(p, range, A, B, M, W, err, blockIdx.x);
+}
 
 // ---------------------------------------------------------------------------
 // split step, pass 3 in FP32 arithmetic: two neighbouring nodes per thread
@@ -914,17 +935,15 @@ template <typename T> __device__ __forceinline__ T* at_bytes(T* base, unsigned o
 }
 
 template <int D, typename S, Handed HD, bool ODD, int NTB, int MINB>
-__global__ void __launch_bounds__(NTB, MINB)
-k_collide2(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
-           typename Store<S>::T* __restrict__ B, const float* __restrict__ M, const float* __restrict__ W,
-           unsigned* err) {
-  wait_previous_launch();
+__device__ __forceinline__ void collide_pairs(const Params& p, const NodeRange& range, const typename Store<S>::T* __restrict__ A,
+                                              typename Store<S>::T* __restrict__ B, const float* __restrict__ M,
+                                              const float* __restrict__ W, unsigned* err, const unsigned block) {
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   using WP = WPlanes<D>;
   constexpr unsigned ES = sizeof(ST);
   int xp, y, z;
-  if (!range.decode(blockIdx.x * NTB + threadIdx.x, xp, y, z)) return;
+  if (!range.decode(block * NTB + threadIdx.x, xp, y, z)) return;
   PullOffsets<D> po;                                         // rows in elements, then in bytes
   po.rows(p, y, z);
   const unsigned x = unsigned(xp), xm = unsigned(xpad(p, xp - 1)), x1 = unsigned(xpad(p, xp + 1)),
@@ -1079,6 +1098,14 @@ k_collide2(const __grid_constant__ Params p, const NodeRange range, const typena
   FactoredRelax<D, F2>::g_pass(at, [&](int i) { return Store<S>::value(v[L::Q + i], p.ref[L::Q + i]); },
                                [&](int i, F2 x) { put(L::Q + i, x); });
 }
+template <int D, typename S, Handed HD, bool ODD, int NTB, int MINB>
+__global__ void __launch_bounds__(NTB, MINB)
+k_collide2(const __grid_constant__ Params p, const NodeRange range, const typename Store<S>::T* __restrict__ A,
+           typename Store<S>::T* __restrict__ B, const float* __restrict__ M, const float* __restrict__ W,
+           unsigned* err) {
+  wait_previous_launch();
+  collide_pairs<D, S, HD, ODD, NTB, MINB>(p, range, A, B, M, W, err, blockIdx.x);
+}
 
 // ---------------------------------------------------------------------------
 // ghost fill of the post-collision buffer (non-periodic x only): inflow faces
@@ -1120,8 +1147,10 @@ __device__ __forceinline__ void ghost_store(const Params& p, typename Store<S>::
   }
 }
 
+// (One copy of the code for every kernel that fills walls: inlined, the compiler's choice
+// of multiply-adds in the FP64 equilibrium differed, and a batch's walls with it.)
 template <int D, typename S>
-__device__ inline void ghost_wall_row(const Params& p, typename Store<S>::T* B, bool low, long long row) {
+__device__ __noinline__ void ghost_wall_row(const Params& p, typename Store<S>::T* B, bool low, long long row) {
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   const long long o = row * p.pitch + (low ? 0 : p.Nx + p.G), os = row * p.pitch + (low ? p.G : p.G + p.Nx - 1);
@@ -1325,11 +1354,9 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 template <int D, typename S, Handed HD, bool BOUNDED, int W, int MINB>
-__global__ void __launch_bounds__(W / 2, MINB)
-k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv dny,
-               const typename Store<S>::T* __restrict__ A, typename Store<S>::T* __restrict__ B,
-               const float* __restrict__ M, const float* __restrict__ Wf, unsigned* err) {
-  wait_previous_launch();
+__device__ __forceinline__ void collide_rows(const Params& p, int nseg, FastDiv dseg, FastDiv dny, const typename Store<S>::T* __restrict__ A,
+                                             typename Store<S>::T* __restrict__ B, const float* __restrict__ M,
+                                             const float* __restrict__ Wf, unsigned* err, const unsigned block) {
   using L = Lattice<D>;
   using ST = typename Store<S>::T;
   using WP = WPlanes<D>;
@@ -1339,7 +1366,7 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
   ST* sp = reinterpret_cast<ST*>(smem_raw);
   float* sf = reinterpret_cast<float*>(smem_raw + R::kPopBytes);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + R::kBytes - 16);
-  const unsigned row = dseg.div(blockIdx.x), seg = blockIdx.x - row * unsigned(nseg);
+  const unsigned row = dseg.div(block), seg = block - row * unsigned(nseg);
   const int z = D == 3 ? int(dny.div(row)) : 0, y = int(row) - z * p.Ny;
   const int x0 = R::first(p.G, BOUNDED) + int(seg) * W, xend = BOUNDED ? p.pitch : p.Nx;        // padded x; end of the row's copied part
   const unsigned pitch = unsigned(p.pitch), r0 = row * pitch;
@@ -1552,6 +1579,14 @@ k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv
       for (int i = t; i < 2 * Q; i += W / 2) ghost_row<D, S>(p, B + (long long)i * p.plane + r0, i, first, last);
     }
   }
+}
+template <int D, typename S, Handed HD, bool BOUNDED, int W, int MINB>
+__global__ void __launch_bounds__(W / 2, MINB)
+k_collide_rows(const __grid_constant__ Params p, int nseg, FastDiv dseg, FastDiv dny,
+               const typename Store<S>::T* __restrict__ A, typename Store<S>::T* __restrict__ B,
+               const float* __restrict__ M, const float* __restrict__ Wf, unsigned* err) {
+  wait_previous_launch();
+  collide_rows<D, S, HD, BOUNDED, W, MINB>(p, nseg, dseg, dny, A, B, M, Wf, err, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------

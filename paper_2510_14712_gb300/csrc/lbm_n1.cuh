@@ -190,14 +190,12 @@ template <int D, typename real> struct N1Buffers {
 // arithmetic serve both nodes of an FP32 unit (one node per thread, 64 scalar loads
 // for two nodes: 84 us at 384x128x128, now 53 us).
 template <typename S, typename real>
-__global__ void __launch_bounds__(128)
-k_n1_strain_3d(const __grid_constant__ Params p, unsigned n, FastDiv dnx, FastDiv dny, const real* __restrict__ rho,
-               const real* __restrict__ u, const real* __restrict__ T) {
-  wait_previous_launch();
+__device__ __forceinline__ void n1_strain_units(const Params& p, unsigned n, FastDiv dnx, FastDiv dny, const real* __restrict__ rho,
+                                                 const real* __restrict__ u, const real* __restrict__ T, const unsigned block) {
   using U = Unit<S, real>;
   using V = typename U::V;
   constexpr int N = U::N;
-  const unsigned gid = blockIdx.x * 128u + threadIdx.x;
+  const unsigned gid = block * 128u + threadIdx.x;
   if (gid >= n) return;
   const unsigned row = dnx.div(gid), z = dny.div(row);
   const int y = int(row - z * unsigned(p.Ny)), x = N * int(gid - row * unsigned((p.Nx + N - 1) / N));
@@ -229,6 +227,13 @@ k_n1_strain_3d(const __grid_constant__ Params p, unsigned n, FastDiv dnx, FastDi
   const N1Buffers<3, real> b(p);
   U::store_field(b.w0 + o, Sn, whole);
   U::store_field(b.w0 + p.plane + o, gn, whole);
+}
+template <typename S, typename real>
+__global__ void __launch_bounds__(128)
+k_n1_strain_3d(const __grid_constant__ Params p, unsigned n, FastDiv dnx, FastDiv dny, const real* __restrict__ rho,
+               const real* __restrict__ u, const real* __restrict__ T) {
+  wait_previous_launch();
+  n1_strain_units<S, real>(p, n, dnx, dny, rho, u, T, blockIdx.x);
 }
 
 // ---- 2-D single-instance form: one launch over tiles of the plane ----
@@ -355,12 +360,11 @@ template <typename S, typename real> struct N1Column {
   static constexpr int P4 = TX + 2 * HX, H4 = TY + 8, P2 = TX + 4, H2 = TY + 4, NU = TY * 32 / kN1Threads;
   static constexpr int kPlane = H4 * P4;                         // one field of one plane
   static constexpr size_t kBytes = sizeof(real) * 2 * (5 * kPlane + H2 * P2 + H2 * TX);
+  static constexpr int kMinB = sizeof(real) == 4 ? 3 : 2;        // blocks: what 59 KB admit; FP64 needs 92 registers
 };
 template <typename S, typename real>
-__global__ void __launch_bounds__(kN1Threads)
-k_n1_coef_3d(const __grid_constant__ Params p, const real* __restrict__ rho, const real* __restrict__ T, int ntx, int nty,
-             int nseg) {
-  wait_previous_launch();
+__device__ __forceinline__ void n1_coef_column(const Params& p, const real* __restrict__ rho, const real* __restrict__ T, int ntx,
+                                               int nty, int nseg, const unsigned block) {
   using C = N1Column<S, real>;
   using U = typename C::U;
   using V = typename U::V;
@@ -373,7 +377,7 @@ k_n1_coef_3d(const __grid_constant__ Params p, const real* __restrict__ rho, con
   const N1Buffers<3, real> b(p, rho, nullptr, T);
   const Model<real> m = model_of<real>(p);
   const int tid = threadIdx.x;
-  int blk = blockIdx.x;
+  int blk = block;
   const int x0 = (blk % ntx) * TX;
   blk /= ntx;
   const int y0 = (blk % nty) * C::TY, seg = blk / nty;
@@ -499,6 +503,13 @@ k_n1_coef_3d(const __grid_constant__ Params p, const real* __restrict__ rho, con
     if (pl >= mb + 4) zo += zs;
   }
 }
+template <typename S, typename real>
+__global__ void __launch_bounds__(kN1Threads, N1Column<S, real>::kMinB)
+k_n1_coef_3d(const __grid_constant__ Params p, const real* __restrict__ rho, const real* __restrict__ T, int ntx, int nty,
+             int nseg) {
+  wait_previous_launch();
+  n1_coef_column<S, real>(p, rho, T, ntx, nty, nseg, blockIdx.x);
+}
 
 // S and |grad s| of a plane from its rho, u, T, which also go to sc_prims (the
 // multi-pass step keeps them in its scratch area)
@@ -514,6 +525,22 @@ __global__ void __launch_bounds__(256) k_n1_norms_2d(const __grid_constant__ Par
   n1_store(p, b.w0, o, n1_strain_at<2, real>(p, rho, u, T, x, y, 0, o));
   const_cast<real*>(b.rho)[o] = rho[o];
   const_cast<real*>(b.T)[o] = T[o];
+}
+
+// z-segments of the coefficient columns: whole rounds of resident blocks over all
+// columns of the launch against the eight planes (two thirds of a plane's work) that
+// each segment repeats
+inline int n1_segments(const Params& p, int slots, long long columns) {
+  int nseg = 1;
+  long long least = -1;
+  for (int k = 1; k <= std::min(p.Nz, 32); ++k) {
+    const long long cost = (columns * k + slots - 1) / slots * ((p.Nz + k - 1) / k + 5);
+    if (least < 0 || cost < least) {
+      least = cost;
+      nseg = k;
+    }
+  }
+  return nseg;
 }
 
 // The whole update of a handle's coefficients.  2-D: one launch after a step that
@@ -533,18 +560,7 @@ inline int n1_update(const Params& p, cudaStream_t st, const real* rho, const re
     const unsigned nx = unsigned((p.Nx + C::N - 1) / C::N), n = nx * unsigned(p.Ny) * unsigned(p.Nz);
     launch_overlapped(k_n1_strain_3d<S, real>, dim3((n + 127u) / 128u), 128, 0, st, p, n, FastDiv(nx),
                       FastDiv(unsigned(p.Ny)), rho, u, T);
-    // z-segments: whole rounds of resident blocks against the eight planes (two
-    // thirds of a plane's work) that each segment repeats
-    const int ntx = (p.Nx + C::TX - 1) / C::TX, nty = (p.Ny + C::TY - 1) / C::TY;
-    int nseg = 1;
-    long long least = -1;
-    for (int k = 1; k <= std::min(p.Nz, 32); ++k) {
-      const long long cost = ((long long)ntx * nty * k + slots - 1) / slots * ((p.Nz + k - 1) / k + 5);
-      if (least < 0 || cost < least) {
-        least = cost;
-        nseg = k;
-      }
-    }
+    const int ntx = (p.Nx + C::TX - 1) / C::TX, nty = (p.Ny + C::TY - 1) / C::TY, nseg = n1_segments(p, slots, (long long)ntx * nty);
     launch_overlapped(kern, dim3(unsigned(ntx) * unsigned(nty) * unsigned(nseg)), kN1Threads, C::kBytes, st, p, rho, T, ntx,
                       nty, nseg);
     return 2;

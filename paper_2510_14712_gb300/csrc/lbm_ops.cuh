@@ -7,7 +7,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "lbm_n1.cuh"
+#include "lbm_batch3d.cuh"
 
 namespace lbm {
 
@@ -56,6 +56,13 @@ template <int D, typename S, typename real> struct OpsImpl {
   // blocks of k_prims3 per multiprocessor: 40 registers without a network
   template <class CL> static constexpr int kPrimsMinB = CL::kWarp ? 2 : (sizeof(real) == 8 ? 3 : 6);
 
+  // z-segments of the columns of k_prims3: about one round of resident blocks over all
+  // columns of the launch (a segment repeats four planes of density and two of
+  // Laplacian), at least two planes each
+  static int prim_segments(const Params& p, int slots, long long columns) {
+    return int(std::max(1LL, std::min((long long)(p.Nz / 2), (slots + columns - 1) / columns)));
+  }
+
   // primitive fields from the moments in scratch (3-D: MINB blocks per
   // multiprocessor for the register budget)
   template <class CL, int MINB = kPrimsMinB<CL>> static void prims(Handle& h) {
@@ -66,9 +73,7 @@ template <int D, typename S, typename real> struct OpsImpl {
       auto kern = k_prims3<real, CL, MINB>;
       const int slots = prepared_blocks<k_prims3<real, CL, MINB>>(kPrimX * kPrimY, CL::kSmem);
       const int ncolx = (hi - lo + kPrimX - 1) / kPrimX, ncoly = (p.Ny + kPrimY - 1) / kPrimY;
-      // z-segments: about one round of resident blocks (a segment repeats four
-      // planes of density and two of Laplacian), at least two planes each
-      const int nseg = std::max(1, std::min(p.Nz / 2, (slots + ncolx * ncoly - 1) / (ncolx * ncoly)));
+      const int nseg = prim_segments(p, slots, (long long)ncolx * ncoly);
       launch_overlapped(kern, dim3(unsigned(ncolx * ncoly * nseg)), kPrimX * kPrimY, CL::kSmem, h.stream, p, lo, hi, ncolx, ncoly, nseg,
                                                                                       M(h), W(h));
     } else {
@@ -84,6 +89,12 @@ template <int D, typename S, typename real> struct OpsImpl {
     prims<AnyClosure<real>>(h);
   }
 
+  // registers of the collision by rows: blocks per multiprocessor that the shared memory
+  // admits (FP32: five of 40 KB, 1013 -> 990 us at 384x128x128 against the bound of 128
+  // registers, which spilled; FP16 deviations: eight of 25 KB, 1234 us at 256^3, with
+  // seven 1247); threads and blocks of the other forms
+  static constexpr int kRowsMinB = sizeof(ST) == 4 ? 5 : 8, kColThreads = 128, kColMinB = 2;
+
   // collision of every interior node; whether it filled the ghost layers too
   template <Handed HD> static bool collide(Handle& h, const void* src, void* dst) {
     const Params& p = h.p;
@@ -92,10 +103,7 @@ template <int D, typename S, typename real> struct OpsImpl {
     h.launches += 1;
     if constexpr (sizeof(real) == 4) {
       if (collide_rows_ok<S>(p)) {
-        // registers: blocks per multiprocessor that the shared memory admits (FP32: five
-        // of 40 KB, 1013 -> 990 us at 384x128x128 against the bound of 128 registers, which
-        // spilled; FP16 deviations: eight of 25 KB, 1234 us at 256^3, with seven 1247)
-        constexpr int W128 = kRowW, kRowsMinB = sizeof(ST) == 4 ? 5 : 8;
+        constexpr int W128 = kRowW;
         using R = RowsLayout<D, S, HD, W128>;
         auto kern = p.periodic_x ? k_collide_rows<D, S, HD, false, W128, kRowsMinB> : k_collide_rows<D, S, HD, true, W128, kRowsMinB>;
         if (p.periodic_x) prepared_blocks<k_collide_rows<D, S, HD, false, W128, kRowsMinB>>(W128 / 2, R::kBytes);
@@ -105,12 +113,12 @@ template <int D, typename S, typename real> struct OpsImpl {
             p, nseg, FastDiv(unsigned(nseg)), FastDiv(unsigned(p.Ny)), A, B, M(h), W(h), h.err_dev);
         return p.bc_lo != LBM_BC_WALL && p.bc_hi != LBM_BC_WALL;
       }
-      constexpr int NTB = 128, MINB = 2;
+      constexpr int NTB = kColThreads, MINB = kColMinB;
       const NodeRange r(p, p.G, p.G + p.Nx, 2);
       auto kern = p.Nx % 2 ? k_collide2<D, S, HD, true, NTB, MINB> : k_collide2<D, S, HD, false, NTB, MINB>;
       launch_overlapped(kern, dim3(unsigned((r.n + NTB - 1) / NTB)), NTB, 0, h.stream, p, r, A, B, M(h), W(h), h.err_dev);
     } else {
-      constexpr int NTB = 128, MINB = 2;
+      constexpr int NTB = kColThreads, MINB = kColMinB;
       const NodeRange r(p, p.G, p.G + p.Nx);
       launch_overlapped(k_collide<D, S, real, HD, NTB, MINB>, dim3(unsigned((r.n + NTB - 1) / NTB)), NTB, 0, h.stream, p, r, A, B, M(h),
                                                                                                 W(h), h.err_dev);
@@ -350,9 +358,9 @@ template <int D, typename S, typename real> struct OpsImpl {
   }
 
   // ---- batches -------------------------------------------------------------
-  // 2-D instances that step with launches of their own: planes that a single handle
-  // splits (a batch gives a handle's bits)
-  static bool own_launches(const Batch&, const Params& p) { return plane_splits(p); }
+  // instances that step with launches of their own: planes that a single handle splits
+  // (a batch gives a handle's bits), and a 3-D batch of one
+  static bool own_launches(const Batch& b, const Params& p) { return D == 2 ? plane_splits(p) : b.n == 1; }
   static void enqueue_own(Batch& b, int parity) {
     for (int k = 0; k < b.n; ++k) {
       Handle& h = *b.inst[k];
@@ -429,36 +437,138 @@ template <int D, typename S, typename real> struct OpsImpl {
     }
   };
 
-  // 3-D: the split step of every instance, the instances dealt to branches of
-  // the step's graph that run side by side
+  // 3-D: the passes of the split step, each one launch over the blocks of every instance
+  // (one launch for each kind of instance that a pass distinguishes)
   struct BatchSplit {
+    using Inst = SplitInstance<real>;
+    using CL = ExactClosure<real>;
+    static constexpr int kMinB = kPrimsMinB<CL>;
+    // groups of work items
+    enum { kMoments, kMomentsRagged, kPrims, kRows, kRowsBounded, kNodes, kNodesOdd, kStrain, kCoef };
+    static_assert(kCoef + 2 == sizeof(Batch::group) / sizeof(int), "first items of the groups and their end");
+
     static int prepare(Batch& b) {
-      if (b.fork) return LBM_OK;
-      if (cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming) != cudaSuccess) return LBM_ECUDA;
-      for (int k = 0; k < kBatchBranches; ++k)
-        if (cudaStreamCreateWithFlags(&b.branch[k], cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&b.join[k], cudaEventDisableTiming) != cudaSuccess)
-          return LBM_ECUDA;
-      return LBM_OK;
-    }
-    static void enqueue(Batch& b, int parity) {
-      const int nb = std::min(b.n, kBatchBranches);
-      cudaEventRecord(b.fork, b.stream);
-      for (int k = 0; k < nb; ++k) cudaStreamWaitEvent(b.branch[k], b.fork, 0);
+      std::vector<Inst> ti(b.n);
+      std::vector<int> order;
+      long long columns = 0, n1columns = 0, ng = 0;
+      using N1 = N1Column<S, real>;
       for (int k = 0; k < b.n; ++k) {
         Handle& h = *b.inst[k];
-        const Handle saved = h;
-        h.stream = b.branch[k % nb];
-        h.err_dev = b.d_errs + k;
-        split<ExactClosure<real>>(h, h.pop[parity], h.pop[parity ^ 1]);
-        if (h.p.sc_on && !b.tuning) shock_capturing(h, M(h), W(h), W(h) + D * h.p.plane);
-        b.launches += h.launches - saved.launches;
-        h = saved;
+        const Params& p = h.p;
+        Inst& t = ti[k];
+        t.ghosts = 0;
+        if (own_launches(b, p)) continue;
+        order.push_back(k);
+        t.p = p;
+        t.pop[0] = h.pop[0];
+        t.pop[1] = h.pop[1];
+        t.M = M(h);
+        t.W = W(h);
+        int lo, hi;
+        moment_range(p, 3, lo, hi);
+        if constexpr (sizeof(real) == 4) {
+          t.moments = NodeRange(p, 0, p.Nx + 2 * p.G, Store<S>::kGroup);
+          t.nodes = NodeRange(p, p.G, p.G + p.Nx, 2);
+          t.rowseg = collide_rows_ok<S>(p) ? collide_segments<S>(p) : 0;
+        } else {
+          t.moments = NodeRange(p, lo, hi);
+          t.nodes = NodeRange(p, p.G, p.G + p.Nx);
+          t.rowseg = 0;
+        }
+        t.drowseg = FastDiv(unsigned(std::max(1, t.rowseg)));
+        t.dny = FastDiv(unsigned(p.Ny));
+        const bool wall = p.bc_lo == LBM_BC_WALL || p.bc_hi == LBM_BC_WALL;
+        t.ghosts = !p.periodic_x && (wall || t.rowseg == 0);
+        if (t.ghosts) ng = std::max(ng, ghost_items<D>(p, true) + ghost_items<D>(p, false));
+        moment_range(p, 1, t.lo, t.hi);
+        t.ncolx = (t.hi - t.lo + kPrimX - 1) / kPrimX;
+        t.ncoly = (p.Ny + kPrimY - 1) / kPrimY;
+        columns += (long long)t.ncolx * t.ncoly;
+        const unsigned nx = unsigned((p.Nx + N1::N - 1) / N1::N);
+        t.units = p.sc_on ? nx * unsigned(p.Ny) * unsigned(p.Nz) : 0u;
+        t.dunits = FastDiv(nx);
+        t.n1tx = (p.Nx + N1::TX - 1) / N1::TX;
+        t.n1ty = (p.Ny + N1::TY - 1) / N1::TY;
+        if (p.sc_on) n1columns += (long long)t.n1tx * t.n1ty;
       }
-      for (int k = 0; k < nb; ++k) {
-        cudaEventRecord(b.join[k], b.branch[k]);
-        cudaStreamWaitEvent(b.stream, b.join[k], 0);
+      const int slots = prepared_blocks<k_prims3_batch<real, CL, kMinB>>(kPrimX * kPrimY, CL::kSmem);
+      const int n1slots = prepared_blocks<k_n1_coef_batch3<S, real>>(kN1Threads, N1::kBytes);
+      for (int k : order) {
+        Inst& t = ti[k];
+        t.nseg = prim_segments(t.p, slots, columns);
+        t.n1seg = n1_segments(t.p, n1slots, n1columns);
       }
+      std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return ti[a].p.plane > ti[c].p.plane; });
+      std::vector<SplitItem> items;
+      auto group = [&](int g, auto blocks) {       // blocks(instance): blocks of its own launch, 0 for other kinds
+        b.group[g] = int(items.size());
+        for (int k : order) {
+          const unsigned n = blocks(ti[k]);
+          for (unsigned q = 0; q < n; ++q) items.push_back({k, q});
+        }
+        b.group[g + 1] = int(items.size());
+      };
+      auto over = [](unsigned n, unsigned threads) { return (n + threads - 1) / threads; };
+      constexpr unsigned kMomT = sizeof(real) == 8 ? kBlock : 128;
+      constexpr int kG = sizeof(real) == 8 ? 1 : 16 / int(sizeof(ST));
+      group(kMoments, [&](const Inst& t) { return t.p.Nx % kG ? 0u : over(t.moments.n, kMomT); });
+      group(kMomentsRagged, [&](const Inst& t) { return t.p.Nx % kG ? over(t.moments.n, kMomT) : 0u; });
+      group(kPrims, [&](const Inst& t) { return unsigned(t.ncolx * t.ncoly * t.nseg); });
+      auto rows = [](const Inst& t) { return unsigned(t.rowseg) * unsigned(t.p.Ny) * unsigned(t.p.Nz); };
+      group(kRows, [&](const Inst& t) { return t.p.periodic_x ? rows(t) : 0u; });
+      group(kRowsBounded, [&](const Inst& t) { return t.p.periodic_x ? 0u : rows(t); });
+      constexpr int kPair = sizeof(real) == 8 ? 1 : 2;
+      group(kNodes, [&](const Inst& t) { return t.rowseg || t.p.Nx % kPair ? 0u : over(t.nodes.n, kColThreads); });
+      group(kNodesOdd, [&](const Inst& t) { return t.rowseg || t.p.Nx % kPair == 0 ? 0u : over(t.nodes.n, kColThreads); });
+      group(kStrain, [&](const Inst& t) { return over(t.units, 128); });
+      group(kCoef, [&](const Inst& t) { return t.p.sc_on ? unsigned(t.n1tx * t.n1ty * t.n1seg) : 0u; });
+      b.ghost_blocks = unsigned(std::min((ng + 255) / 256, 4096LL));
+      b.nitems = int(items.size());
+      if (b.d_insts) cudaFree(b.d_insts);
+      if (b.d_items) cudaFree(b.d_items);
+      b.d_insts = b.d_items = nullptr;
+      if (items.empty()) return LBM_OK;
+      if (dev_malloc(&b.d_insts, sizeof(Inst) * ti.size()) != cudaSuccess) return LBM_ENOMEM;
+      if (dev_malloc(&b.d_items, sizeof(SplitItem) * items.size()) != cudaSuccess) return LBM_ENOMEM;
+      cudaMemcpy(b.d_insts, ti.data(), sizeof(Inst) * ti.size(), cudaMemcpyHostToDevice);
+      cudaMemcpy(b.d_items, items.data(), sizeof(SplitItem) * items.size(), cudaMemcpyHostToDevice);
+      if constexpr (sizeof(real) == 4) {
+        constexpr size_t smem = RowsLayout<D, S, kHandNothing, kRowW>::kBytes;
+        prepared_blocks<k_collide_rows_batch<S, false, kRowW, kRowsMinB>>(kRowW / 2, smem);
+        prepared_blocks<k_collide_rows_batch<S, true, kRowW, kRowsMinB>>(kRowW / 2, smem);
+      }
+      return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ECUDA;
+    }
+
+    static void enqueue(Batch& b, int parity) {
+      const Inst* insts = static_cast<const Inst*>(b.d_insts);
+      const SplitItem* items = static_cast<const SplitItem*>(b.d_items);
+      auto launch = [&](int g, auto kern, unsigned threads, size_t smem, auto... args) {
+        const int n = b.group[g + 1] - b.group[g];
+        if (n == 0) return;
+        launch_overlapped(kern, dim3(unsigned(n)), threads, smem, b.stream, insts, items + b.group[g], args...);
+        b.launches += 1;
+      };
+      launch(kMoments, k_moments_batch<S, real, false>, sizeof(real) == 8 ? kBlock : 128, 0, parity);
+      launch(kMomentsRagged, k_moments_batch<S, real, true>, sizeof(real) == 8 ? kBlock : 128, 0, parity);
+      launch(kPrims, k_prims3_batch<real, CL, kMinB>, kPrimX * kPrimY, CL::kSmem);
+      if constexpr (sizeof(real) == 4) {
+        constexpr size_t smem = RowsLayout<D, S, kHandNothing, kRowW>::kBytes;
+        launch(kRows, k_collide_rows_batch<S, false, kRowW, kRowsMinB>, kRowW / 2, smem, parity, b.d_errs);
+        launch(kRowsBounded, k_collide_rows_batch<S, true, kRowW, kRowsMinB>, kRowW / 2, smem, parity, b.d_errs);
+      }
+      launch(kNodes, k_collide_batch<S, real, false, kColThreads, kColMinB>, kColThreads, 0, parity, b.d_errs);
+      launch(kNodesOdd, k_collide_batch<S, real, true, kColThreads, kColMinB>, kColThreads, 0, parity, b.d_errs);
+      for (int k0 = 0; b.ghost_blocks > 0 && k0 < b.n; k0 += 65535) {
+        launch_overlapped(k_ghosts_batch3<S, real>, dim3(b.ghost_blocks, unsigned(std::min(b.n - k0, 65535))), 256, 0, b.stream,
+                          insts + k0, parity);
+        b.launches += 1;
+      }
+      if (!b.tuning) {
+        launch(kStrain, k_n1_strain_batch3<S, real>, 128, 0);
+        launch(kCoef, k_n1_coef_batch3<S, real>, kN1Threads, N1Column<S, real>::kBytes);
+      }
+      enqueue_own(b, parity);
     }
   };
 
