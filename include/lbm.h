@@ -270,8 +270,10 @@ int lbm_set_graphs(lbm_t h, int on);
  * a NULL handle. */
 int lbm_autotune_times(lbm_t h, float* ms_per_step, int n);
 
-/* Number of forms (tile shapes) of the step for this handle's lattice,
+/* Number of form indices (tile shapes) of the step for this handle's lattice,
  * precision and closure (the candidates lbm_autotune times, in its order).
+ * Where a lattice has fewer forms than in earlier versions the indices repeat
+ * them, so that a stored index stays valid; lbm_autotune times each form once.
  * Returns the count (>= 1), or LBM_EINVAL for a NULL handle. */
 int lbm_tile_count(lbm_t h);
 

@@ -260,10 +260,17 @@ template <int D, typename S, typename real> struct OpsImpl {
     h.launches += n1_update<D, S, real>(h.p, h.stream, rho, u, T);
   }
 
+  // Indices of lbm_set_tile: the forms, repeated up to the number of shapes that the
+  // lattice, precision and closure ever had, so that an index that was valid stays valid.
+  template <class CL> static int indices(int n) {
+    constexpr int had = CL::kPr ? 1 : (D == 3 ? (sizeof(real) == 8 ? 1 : (CL::kWarp ? 4 : 5)) : (sizeof(real) == 4 && !CL::kWarp ? 9 : 5));
+    return std::max(n, had);
+  }
+
   template <class CL> static void step_cl(Handle& h, const void* src, void* dst) {
     const LaunchFn* fns;
     const int n = candidates<CL>(&fns);
-    const int cfg = h.tile_cfg < n ? h.tile_cfg : 0;
+    const int cfg = h.tile_cfg < indices<CL>(n) ? h.tile_cfg % n : 0;
     fns[cfg](h, src, dst);
     if (h.p.sc_on && (D == 3 || (cfg == 0 && plane_splits(h.p)))) {
       shock_capturing(h, M(h), W(h), W(h) + D * h.p.plane);
@@ -302,14 +309,15 @@ template <int D, typename S, typename real> struct OpsImpl {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     h.tile_cfg = best;
-    h.tune_n = n < kMaxTiles ? n : kMaxTiles;
+    h.tune_n = std::min(indices<CL>(n), kMaxTiles);
+    for (int c = n; c < h.tune_n; ++c) h.tune_ms[c] = h.tune_ms[c % n];
     if (best_ms) *best_ms = bt / (reps > 0 ? reps : 1);
     return best;
   }
   static int autotune(Handle& h, int reps, float* best_ms) { return autotune_cl<ExactClosure<real>>(h, reps, best_ms); }
   template <class CL> static int ntiles_cl() {
     const LaunchFn* fns;
-    return candidates<CL>(&fns);
+    return indices<CL>(candidates<CL>(&fns));
   }
   static int ntiles() { return ntiles_cl<ExactClosure<real>>(); }
 
