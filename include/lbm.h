@@ -85,7 +85,9 @@ enum {
   LBM_FLAG_NONFINITE = 1u,   /* fatal: rho, u or T not finite                 */
   LBM_FLAG_NEGATIVE = 2u,    /* fatal: rho <= 0 or T <= 0                      */
   LBM_FLAG_THETA = 4u,       /* warning: theta = P/rho >= 1/3 (Sec. 5 bound)   */
-  LBM_FLAG_PRESSURE = 8u     /* warning: P <= 0                                */
+  LBM_FLAG_PRESSURE = 8u,    /* warning: P <= 0                                */
+  LBM_FLAG_INCOMPLETE = 16u  /* fatal: a step gave up its bounded wait for a
+                                copy; part of the new state is not written     */
 };
 
 /* equations of state (lbm_eos.kind) */
@@ -175,9 +177,9 @@ int lbm_init_device(lbm_t h, const double* d_rho, const double* d_u, const doubl
 
 /* Advance n >= 0 time steps.  Returns after enqueuing the work and reading
  * the 4-byte sticky error word once (one stream synchronisation).
- * Errors: LBM_ESTATE (not initialised, or a previous step was unstable),
- * LBM_EINVAL (n < 0), LBM_EUNSTABLE (fatal flag raised; state kept),
- * LBM_ECUDA. */
+ * Errors: LBM_ESTATE (not initialised, or a previous step was unstable or
+ * incomplete), LBM_EINVAL (n < 0), LBM_EUNSTABLE (fatal flag raised; state
+ * kept), LBM_ECUDA (also LBM_FLAG_INCOMPLETE: the state is lost). */
 int lbm_step(lbm_t h, int n);
 
 /* Enqueue n steps without reading the error word (no synchronisation); the
@@ -193,7 +195,8 @@ int lbm_sync(lbm_t h);
  * lbm_temp): rho (Nx*Ny*Nz), u (D planes), T (Nx*Ny*Nz) as FP64 host arrays,
  * and totals[D+2] = (sum rho, sum rho u_1..u_D, sum rho E) over the interior
  * in FP64.  Any pointer may be NULL to skip that output.  Synchronises.
- * Errors: LBM_ESTATE (not initialised), LBM_ECUDA. */
+ * Errors: LBM_ESTATE (not initialised), LBM_ECUDA (also after an incomplete
+ * step, LBM_FLAG_INCOMPLETE, until the next lbm_init or lbm_set_populations). */
 int lbm_moments(lbm_t h, double* rho, double* u, double* T, double* totals);
 
 /* Same outputs as lbm_moments into device pointers (FP64, same layout);
@@ -207,7 +210,7 @@ int lbm_get_flags(lbm_t h, unsigned* flags);
  * last step, ghosts included, library layout) out to / in from a host buffer
  * of lbm_population_bytes() bytes; used for checkpoint and resume.  A resumed
  * run continues bit-identically.  Errors: LBM_EINVAL (size mismatch / NULL),
- * LBM_ESTATE (get before init), LBM_ECUDA. */
+ * LBM_ESTATE (get before init), LBM_ECUDA (get: also as lbm_moments). */
 size_t lbm_population_bytes(lbm_t h);
 int lbm_get_populations(lbm_t h, void* host, size_t bytes);
 int lbm_set_populations(lbm_t h, const void* host, size_t bytes);

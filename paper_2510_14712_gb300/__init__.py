@@ -26,7 +26,7 @@ LBM_CLOSURE_EXACT, LBM_CLOSURE_MLP = 0, 1
 LBM_BC_PERIODIC, LBM_BC_OUTFLOW, LBM_BC_INFLOW, LBM_BC_WALL = 0, 1, 2, 3
 LBM_EOS_VDW, LBM_EOS_PR = 0, 1
 LBM_FACE_XLO, LBM_FACE_XHI = 0, 1
-LBM_FLAG_NONFINITE, LBM_FLAG_NEGATIVE, LBM_FLAG_THETA, LBM_FLAG_PRESSURE = 1, 2, 4, 8
+LBM_FLAG_NONFINITE, LBM_FLAG_NEGATIVE, LBM_FLAG_THETA, LBM_FLAG_PRESSURE, LBM_FLAG_INCOMPLETE = 1, 2, 4, 8, 16
 LBM_STEP_FUSED, LBM_STEP_MULTIPASS = 0, 1
 PRECISIONS = {"fp64": LBM_FP64, "fp32": LBM_FP32, "fp16dev": LBM_FP16DEV}
 

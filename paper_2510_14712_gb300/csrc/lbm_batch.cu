@@ -67,11 +67,21 @@ int ready(Batch& b) {
   return LBM_OK;
 }
 
-int check_errs(Batch& b) {
+int read_errs(Batch& b) {
   BCK(cudaMemcpyAsync(b.h_errs, b.d_errs, sizeof(unsigned) * b.n, cudaMemcpyDeviceToHost, b.stream));
   BCK(cudaStreamSynchronize(b.stream));
+  b.unchecked = 0;
+  return LBM_OK;
+}
+
+int check_errs(Batch& b) {
+  const int rc = read_errs(b);
+  if (rc != LBM_OK) return rc;
   for (int k = 0; k < b.n; ++k)
-    if (b.h_errs[k] & kFlagWait) return bfail(LBM_ECUDA, "a shared-memory copy of the step did not complete");
+    if (b.h_errs[k] & kFlagWait) {
+      b.unstable = 1;
+      return bfail(LBM_ECUDA, "instance " + std::to_string(k) + ": a shared-memory copy of a step did not complete: its state is lost");
+    }
   for (int k = 0; k < b.n; ++k)
     if (b.h_errs[k] & (LBM_FLAG_NONFINITE | LBM_FLAG_NEGATIVE)) {
       b.unstable = 1;
@@ -123,6 +133,7 @@ int lbm_batch_create(lbm_batch_t* out, int lattice, int n, const int* Nx, const 
                        cudaMallocHost(&b->h_errs, sizeof(unsigned) * n) != cudaSuccess))
     rc = LBM_ENOMEM;
   if (rc == LBM_OK && cudaMemset(b->d_errs, 0, sizeof(unsigned) * n) != cudaSuccess) rc = LBM_ECUDA;
+  if (rc == LBM_OK) std::memset(b->h_errs, 0, sizeof(unsigned) * n);
   if (rc != LBM_OK) {
     std::string msg = g_berr.empty() ? "batch creation failed" : g_berr;
     lbm_batch_destroy(b);
@@ -172,6 +183,7 @@ int lbm_batch_init(lbm_batch_t b, int k, const double* rho, const double* u, con
   h.cur = b->cur;
   BCK(cudaMemsetAsync(b->d_errs + k, 0, sizeof(unsigned), b->stream));
   BCK(cudaStreamSynchronize(b->stream));
+  b->h_errs[k] = 0;
   b->unstable = 0;
   for (int j = 0; j < b->n; ++j)
     if (!b->inst[j]->initialized) return LBM_OK;
@@ -186,6 +198,7 @@ int lbm_batch_step_async(lbm_batch_t b, int n) {
   if (b->unstable) return bfail(LBM_ESTATE, "an instance is unstable; re-initialise it");
   int rc = ready(*b);
   if (rc != LBM_OK) return rc;
+  if (n > 0) b->unchecked = 1;
   for (int s = 0; s < n; ++s) {
     BCK(cudaGraphLaunch(b->graph[b->cur], b->stream));
     b->launches += b->graph_launches;
@@ -209,22 +222,30 @@ int lbm_batch_step(lbm_batch_t b, int n) {
 int lbm_batch_moments(lbm_batch_t b, int k, double* rho, double* u, double* T, double* totals) {
   if (!b || k < 0 || k >= b->n) return bfail(LBM_EINVAL, "bad batch or instance index");
   b->inst[k]->cur = b->cur;
+  if (b->unchecked) {
+    const int rc = read_errs(*b);
+    if (rc != LBM_OK) return rc;
+  }
+  if (b->h_errs[k] & kFlagWait) return bfail(LBM_ECUDA, "the instance's last step did not complete: call lbm_batch_init");
   const int rc = lbm_moments(static_cast<lbm_t>(b->inst[k]), rho, u, T, totals);
   return rc == LBM_OK ? rc : bfail(rc, lbm_last_error());
 }
 
 int lbm_batch_flags(lbm_batch_t b, int k, unsigned* flags) {
   if (!b || k < 0 || k >= b->n || !flags) return bfail(LBM_EINVAL, "bad argument");
-  BCK(cudaMemcpyAsync(b->h_errs, b->d_errs, sizeof(unsigned) * b->n, cudaMemcpyDeviceToHost, b->stream));
-  BCK(cudaStreamSynchronize(b->stream));
-  *flags = b->h_errs[k];
-  return LBM_OK;
+  const int rc = read_errs(*b);
+  if (rc == LBM_OK) *flags = b->h_errs[k];
+  return rc;
 }
 
 int lbm_batch_autotune(lbm_batch_t b, int reps, int* chosen, float* ms_per_step) {
   if (!b || reps < 1) return bfail(LBM_EINVAL, "bad argument");
   for (int k = 0; k < b->n; ++k)
     if (!b->inst[k]->initialized) return bfail(LBM_ESTATE, "instance " + std::to_string(k) + " not initialised");
+  const int status = read_errs(*b);
+  if (status != LBM_OK) return status;
+  for (int k = 0; k < b->n; ++k)                             // (the flags of the timing steps are cleared below)
+    if (b->h_errs[k] & kFlagWait) return bfail(LBM_ECUDA, "instance " + std::to_string(k) + " is incomplete: call lbm_batch_init");
   const int ncfg = bops(*b)->batch_ncfg();
   // the timing events and the tuning mode are released on every return path
   struct Guard {
@@ -265,10 +286,23 @@ int lbm_batch_autotune(lbm_batch_t b, int reps, int* chosen, float* ms_per_step)
   if (rc != LBM_OK) return rc;
   BCK(cudaMemsetAsync(b->d_errs, 0, sizeof(unsigned) * b->n, b->stream));
   BCK(cudaStreamSynchronize(b->stream));
+  std::memset(b->h_errs, 0, sizeof(unsigned) * b->n);
   if (chosen) *chosen = best;
   if (ms_per_step) *ms_per_step = bt / reps;
   return LBM_OK;
 }
+
+#ifdef LBM_BOUNDS_CHECK
+// Bounds-check builds, for tests: raise status bits of instance k as a step's kernel would.
+int lbm_debug_raise_batch_flags(lbm_batch_t b, int k, unsigned bits) {
+  const int rc = read_errs(*b);
+  if (rc != LBM_OK) return rc;
+  const unsigned f = b->h_errs[k] | bits;
+  BCK(cudaMemcpy(b->d_errs + k, &f, sizeof(f), cudaMemcpyHostToDevice));
+  b->unchecked = 1;
+  return LBM_OK;
+}
+#endif
 
 long long lbm_batch_nodes(lbm_batch_t b) {
   if (!b) return 0;

@@ -284,12 +284,27 @@ void remember_cfg(const Handle& h) {
 int read_err(Handle& h) {
   CK(cudaMemcpyAsync(h.err_host, h.err_dev, sizeof(unsigned), cudaMemcpyDeviceToHost, h.stream));
   CK(cudaStreamSynchronize(h.stream));
-  if (*h.err_host & kFlagWait) return fail(LBM_ECUDA, "a shared-memory copy of the step did not complete");
+  h.unchecked = 0;
+  if (*h.err_host & kFlagWait) {
+    h.unstable = kIncomplete;
+    return fail(LBM_ECUDA, "a shared-memory copy of a step did not complete: the state is lost");
+  }
   if (*h.err_host & (LBM_FLAG_NONFINITE | LBM_FLAG_NEGATIVE)) {
     h.unstable = 1;
     return fail(LBM_EUNSTABLE, "non-finite or non-positive density/temperature produced");
   }
   return LBM_OK;
+}
+
+// the state is whole: no step since the last look at the status word left part of it
+// unwritten (LBM_EUNSTABLE is the next lbm_step's or lbm_sync's to report)
+int check_complete(Handle& h) {
+  if (h.unchecked) {
+    const int unstable = h.unstable, rc = read_err(h);
+    if (rc == LBM_EUNSTABLE) h.unstable = unstable;
+    else if (rc != LBM_OK) return rc;
+  }
+  return h.unstable == kIncomplete ? fail(LBM_ECUDA, "the last step did not complete: call lbm_init") : LBM_OK;
 }
 
 }  // namespace
@@ -331,6 +346,18 @@ long long lbm_debug_bounds_violations(void) {
   return -1;
 #endif
 }
+
+#ifdef LBM_BOUNDS_CHECK
+// Bounds-check builds, for tests: raise status bits as a step's kernel would.
+int lbm_debug_raise_flags(lbm_t h, unsigned bits) {
+  unsigned f = 0;
+  CK(cudaStreamSynchronize(h->stream));
+  CK(cudaMemcpy(&f, h->err_dev, sizeof(f), cudaMemcpyDeviceToHost));
+  f |= bits;
+  CK(cudaMemcpy(h->err_dev, &f, sizeof(f), cudaMemcpyHostToDevice));
+  return LBM_OK;
+}
+#endif
 
 int lbm_debug_fail_alloc(int k) {
   if (k < 0) return fail(LBM_EINVAL, "k must be >= 0");
@@ -491,7 +518,7 @@ static int init_common(lbm_t h, const double* d_rho, const double* d_u, const do
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(h->stream));
   h->initialized = 1;
-  h->unstable = 0;
+  h->unstable = h->unchecked = 0;
   return LBM_OK;
 }
 
@@ -519,6 +546,7 @@ int lbm_step_async(lbm_t h, int n) {
   if (!h->initialized) return fail(LBM_ESTATE, "lbm_init has not been called");
   if (h->unstable) return fail(LBM_ESTATE, "state is unstable; call lbm_init");
   if (n < 0) return fail(LBM_EINVAL, "n must be >= 0");
+  if (n > 0) h->unchecked = 1;
   const Ops* o = ops_for(*h);
   auto fn = h->step_kernel == LBM_STEP_MULTIPASS ? o->step_multipass : o->step;
   if (!fn) return fail(LBM_EINVAL, "the learned closure runs in the fused step only");
@@ -593,6 +621,8 @@ int lbm_step(lbm_t h, int n) {
 int lbm_moments_device(lbm_t h, double* d_rho, double* d_u, double* d_T, double* totals) {
   if (!h) return fail(LBM_EINVAL, "NULL handle");
   if (!h->initialized) return fail(LBM_ESTATE, "lbm_init has not been called");
+  const int rc = check_complete(*h);
+  if (rc != LBM_OK) return rc;
   ops_for(*h)->macro(*h, h->pop[h->cur], d_rho, d_u, d_T, totals ? h->totals_dev : nullptr);
   CK(cudaGetLastError());
   if (totals)
@@ -632,6 +662,8 @@ int lbm_get_populations(lbm_t h, void* host, size_t bytes) {
   if (!h || !host) return fail(LBM_EINVAL, "NULL argument");
   if (bytes != lbm_population_bytes(h)) return fail(LBM_EINVAL, "size mismatch");
   if (!h->initialized) return fail(LBM_ESTATE, "lbm_init has not been called");
+  const int rc = check_complete(*h);
+  if (rc != LBM_OK) return rc;
   CK(cudaMemcpyAsync(host, h->pop[h->cur], bytes, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   return LBM_OK;
@@ -646,7 +678,7 @@ int lbm_set_populations(lbm_t h, const void* host, size_t bytes) {
   CK(cudaMemsetAsync(h->err_dev, 0, sizeof(unsigned), h->stream));
   CK(cudaStreamSynchronize(h->stream));
   h->initialized = 1;
-  h->unstable = 0;
+  h->unstable = h->unchecked = 0;
   return LBM_OK;
 }
 

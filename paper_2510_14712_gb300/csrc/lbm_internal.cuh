@@ -15,7 +15,7 @@ namespace lbm {
 
 constexpr int kGhost = 4;         // ghost layers per non-periodic x face
 constexpr int kMaxPartials = 1024;
-constexpr unsigned kFlagWait = 16u;   // status bit: a bounded wait for an asynchronous copy ran out
+constexpr unsigned kFlagWait = LBM_FLAG_INCOMPLETE;   // a bounded wait for an asynchronous copy ran out
 constexpr int kMaxTiles = 16;     // tile candidates whose autotune times are kept
 
 // Everything a kernel needs, passed by value.
@@ -76,6 +76,8 @@ template <typename real> __host__ __device__ inline Model<real> model_of(const P
 // fill Params::mf from the FP64 constants (after every change of them)
 inline void set_model_fp32(Params& p) { p.mf = model_convert<float>(p); }
 
+constexpr int kIncomplete = 2;
+
 // One solver instance.
 struct Handle {
   int D, Q, Nx, Ny, Nz;
@@ -95,7 +97,8 @@ struct Handle {
   double* io_dev;             // staging for host <-> device field copies
   size_t io_bytes;
   cudaStream_t stream;
-  int initialized, unstable;
+  int initialized, unstable;  // unstable: 1 a fatal flag, kIncomplete the state is lost
+  int unchecked;              // steps enqueued since the status word was last read
   int step_kernel;            // LBM_STEP_FUSED | LBM_STEP_MULTIPASS
   int tile_cfg;               // index of the step's candidate (lbm_autotune)
   long long launches;
@@ -201,6 +204,7 @@ struct Batch {
   cudaGraphExec_t graph[2];   // one step from parity 0 / 1
   int graph_ready;
   int unstable;
+  int unchecked;              // steps enqueued since the status words were last read
   long long launches;
 };
 
