@@ -349,6 +349,13 @@ long long lbm_debug_bounds_violations(void) {
 
 #ifdef LBM_BOUNDS_CHECK
 // Bounds-check builds, for tests: raise status bits as a step's kernel would.
+// elements [lo, hi) of both population buffers count as outside (lo == hi: none)
+int lbm_debug_hide_populations(lbm_t h, long long lo, long long hi) {
+  CK(cudaStreamSynchronize(h->stream));
+  h->p.hide_lo = lo;
+  h->p.hide_hi = hi;
+  return LBM_OK;
+}
 int lbm_debug_raise_flags(lbm_t h, unsigned bits) {
   unsigned f = 0;
   CK(cudaStreamSynchronize(h->stream));

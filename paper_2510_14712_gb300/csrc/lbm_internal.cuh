@@ -52,6 +52,10 @@ struct Params {
   // the handle's two population buffers (2 Q plane elements each): the
   // bounds of every population access in bounds-check builds
   const void* pop[2];
+#ifdef LBM_BOUNDS_CHECK
+  // elements [hide_lo, hide_hi) of both buffers that count as outside (for tests)
+  long long hide_lo, hide_hi;
+#endif
   // the model constants above rounded to FP32 once on the host (set_model_fp32),
   // so that FP32 kernels read them as they are instead of converting the FP64
   // copies (a conversion the compiler may repeat inside loops, on the FP64 pipe)

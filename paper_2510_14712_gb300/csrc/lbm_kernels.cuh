@@ -47,6 +47,7 @@ template <> struct Store<float> {
   __device__ static Raw raw2(const T* p) { return f2_of(__ldcs(reinterpret_cast<const float2*>(p))); }
   __device__ static Raw raw2g(const T* p) { return f2_of(__ldg(reinterpret_cast<const float2*>(p))); }
   __device__ static Raw raw11(const T* a, const T* b) { return F2(__ldg(a), __ldg(b)); }
+  __device__ static Raw raw_of(T a, T b) { return F2(a, b); }
   __device__ static F2 value(Raw v, float) { return v; }
   __device__ static void st2_stream(T* p, F2 v, float) { __stcs(reinterpret_cast<float2*>(p), f2_in(v)); }
   // the same from shared memory, the rounded pair and its halves
@@ -89,6 +90,7 @@ template <> struct Store<Fp16Dev> {
     return *reinterpret_cast<const __half2*>(&q);
   }
   __device__ static Raw raw11(const T* a, const T* b) { return __halves2half2(__ldg(a), __ldg(b)); }
+  __device__ static Raw raw_of(T a, T b) { return __halves2half2(a, b); }
   __device__ static F2 value(Raw v, float ref) { return f2_of(__half22float2(v)) + F2(ref); }
   __device__ static void st2_stream(T* p, F2 v, float ref) {
     st2_raw(p, pack(v, ref));
@@ -124,8 +126,9 @@ template <> struct Store<Fp16Dev> {
 // ---------------------------------------------------------------------------
 // bounds-check builds (-DLBM_BOUNDS_CHECK): every population access of the
 // step kernels must lie inside one of the handle's two population buffers;
-// one outside is skipped (a load gives 0) and counted.  Other builds compile
-// the check away.
+// one outside is skipped (a load gives 0) and counted: every element of a pull and of
+// a bulk copy with its side units, the elements of a vector load or store together.
+// Other builds compile the check away.
 // ---------------------------------------------------------------------------
 #ifdef LBM_BOUNDS_CHECK
 namespace {
@@ -141,21 +144,36 @@ struct OobReaderRegistration {
 }  // namespace
 #endif
 
-// access to the n elements ptr[off .. off + n) is inside a population buffer of p
+// the n elements ptr[off .. off + n) are inside a population buffer of p (not counted)
 template <typename T>
-__device__ __forceinline__ bool pop_ok(const Params& p, const T* ptr, long long off, int n = 1) {
+__device__ __forceinline__ bool pop_inside(const Params& p, const T* ptr, long long off, int n) {
 #ifdef LBM_BOUNDS_CHECK
   const T* a = ptr + off;
   const long long len = 2LL * p.Q * p.plane;
   for (int k = 0; k < 2; ++k) {
     const T* lo = static_cast<const T*>(p.pop[k]);
-    if (lo && a >= lo && a + n <= lo + len) return true;
+    if (lo && a >= lo && a + n <= lo + len) return a + n <= lo + p.hide_lo || a >= lo + p.hide_hi;
   }
+  return false;
+#else
+  return true;
+#endif
+}
+// the same, an access outside counted
+template <typename T>
+__device__ __forceinline__ bool pop_ok(const Params& p, const T* ptr, long long off, int n = 1) {
+#ifdef LBM_BOUNDS_CHECK
+  if (pop_inside(p, ptr, off, n)) return true;
   atomicAdd(&g_oob, 1ULL);
   return false;
 #else
   return true;
 #endif
+}
+
+// one population value as stored, checked; 0 outside
+template <typename T> __device__ __forceinline__ T pop_value(const Params& p, const T* a) {
+  return pop_ok(p, a, 0) ? __ldg(a) : T(0.f);
 }
 
 // ---------------------------------------------------------------------------
@@ -965,9 +983,11 @@ __device__ __forceinline__ void collide_pairs(const Params& p, const NodeRange& 
     const ST* Ai = A + (long long)ii * p.plane;
     const int cx = L::c(i, 0);
     const unsigned r = po.row(i);
-    if (cx == 0) return pop_ok(p, at_bytes(Ai, r + bx), 0, 2) ? Store<S>::raw2(at_bytes(Ai, r + bx)) : typename Store<S>::Raw();
-    const ST *a = at_bytes(Ai, r + (cx > 0 ? bm : b1)), *b = at_bytes(Ai, r + (cx > 0 ? bx : b2));
-    return pop_ok(p, a, 0) && pop_ok(p, b, 0) ? Store<S>::raw11(a, b) : typename Store<S>::Raw();
+    const ST *a = at_bytes(Ai, r + (cx > 0 ? bm : (cx < 0 ? b1 : bx))), *b = cx == 0 ? a + 1 : at_bytes(Ai, r + (cx > 0 ? bx : b2));
+#ifdef LBM_BOUNDS_CHECK
+    return Store<S>::raw_of(pop_value(p, a), pop_value(p, b));
+#endif
+    return cx == 0 ? Store<S>::raw2(a) : Store<S>::raw11(a, b);
   };
   typename Store<S>::Raw v[2 * L::Q];
 #pragma unroll
@@ -1388,13 +1408,27 @@ __device__ __forceinline__ void collide_rows(const Params& p, int nseg, FastDiv 
     // addresses are uniform, so a request costs a few instructions
     const unsigned s0 = tc::smem_addr(smem_raw), b0 = tc::smem_addr(bar);
     const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);
-    auto segment = [&](const void* rowp, const unsigned es, const unsigned dst, const bool left, const bool right) {
+    // (pop: a row of populations, checked)
+    auto copy = [&](const bool pop, const unsigned d, const char* src, const unsigned bytes) {
+#ifdef LBM_BOUNDS_CHECK
+      const ST* e = reinterpret_cast<const ST*>(src);
+      const int ne = int(bytes / sizeof(ST));
+      if (pop && !pop_inside(p, e, 0, ne)) {
+        ST* to = reinterpret_cast<ST*>(smem_raw + (d - s0));
+        for (int k = 0; k < ne; ++k) to[k] = pop_value(p, e + k);
+        asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(b0), "r"(bytes) : "memory");
+        return;
+      }
+#endif
+      bulk_copy(d, src, bytes, b0);
+    };
+    auto segment = [&](const bool pop, const void* rowp, const unsigned es, const unsigned dst, const bool left, const bool right) {
       const char* src = static_cast<const char*>(rowp) + (long long)x0 * es;
       const unsigned d = s0 + dst, nb = unsigned(n) * es;
       const unsigned l = left && lside ? 16u : 0u, r = right && rside ? 16u : 0u;
-      bulk_copy(d - l, src - l, nb + l + r, b0);
-      if (left && lseam) bulk_copy(d - 16, static_cast<const char*>(rowp) + (long long)p.Nx * es - 16, 16, b0);
-      if (right && rseam) bulk_copy(d + nb, rowp, 16, b0);
+      copy(pop, d - l, src - l, nb + l + r);
+      if (left && lseam) copy(pop, d - 16, static_cast<const char*>(rowp) + (long long)p.Nx * es - 16, 16);
+      if (right && rseam) copy(pop, d + nb, static_cast<const char*>(rowp), 16);
     };
     if (elect_one()) {
       constexpr int NW = W / 64;
@@ -1411,8 +1445,7 @@ __device__ __forceinline__ void collide_rows(const Params& p, int nseg, FastDiv 
           if (k < 2 * Q) {
             const int i = k < Q ? k : k - Q, cx = L::c(i, 0);
             const ST* rowp = A + (long long)k * p.plane + rowof(-L::c(i, 1), D == 3 ? -L::c(i, D - 1) : 0);
-            if (!pop_ok(p, rowp, x0, n)) rowp = A;                     // (bounds-check builds) counted, not read
-            segment(rowp, sizeof(ST), unsigned((k < Q ? 0 : R::kSet) + R::row(i) + R::lead(i)) * unsigned(sizeof(ST)), cx > 0, cx < 0);
+            segment(true, rowp, sizeof(ST), unsigned((k < Q ? 0 : R::kSet) + R::row(i) + R::lead(i)) * unsigned(sizeof(ST)), cx > 0, cx < 0);
           } else {
             int c = k - 2 * Q, f = 0, dst = 0, dy = 0, dz = 0;
             const bool wide = c < R::nWide;
@@ -1429,13 +1462,16 @@ __device__ __forceinline__ void collide_rows(const Params& p, int nseg, FastDiv 
               f = R::field(bb, q);
               (bb == 1 ? dy : dz) = side ? 1 : -1;
             }
-            segment((f < 0 ? M : Wf + (long long)f * p.plane) + rowof(dy, dz), sizeof(float), unsigned(R::kPopBytes) + unsigned(dst) * 4u, wide, wide);
+            segment(false, (f < 0 ? M : Wf + (long long)f * p.plane) + rowof(dy, dz), sizeof(float), unsigned(R::kPopBytes) + unsigned(dst) * 4u, wide, wide);
           }
         }
       }
     }
     __syncwarp();
   }
+#ifdef LBM_BOUNDS_CHECK
+  __syncthreads();                                                     // the elements copied by plain stores
+#endif
   const int t = threadIdx.x, xp = x0 + 2 * t, xhi = p.G + p.Nx;
   const bool act = xp >= p.G && xp < xhi, two = xp + 1 < xhi;
   const unsigned o = r0 + unsigned(xp);

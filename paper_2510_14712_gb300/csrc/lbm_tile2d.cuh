@@ -71,6 +71,11 @@ template <typename S> struct Unit<S, float> {          // two nodes, packed
     if (cx < 0) return Store<S>::raw11(at_bytes(row, x.p), at_bytes(row, x.q));
     return x.vec ? Store<S>::raw2g(at_bytes(row, x.c)) : Store<S>::raw11(at_bytes(row, x.c), at_bytes(row, x.p));
   }
+  // the same with every element checked
+  __device__ static Raw pull_checked(const Params& p, const ST* row, int cx, const X& x) {
+    const unsigned a = cx > 0 ? x.m : (cx < 0 ? x.p : x.c), b = cx > 0 ? x.c : (cx < 0 ? x.q : x.p);
+    return Store<S>::raw_of(pop_value(p, at_bytes(row, a)), pop_value(p, at_bytes(row, b)));
+  }
   __device__ static V value(Raw r, float ref) { return Store<S>::value(r, ref); }
   __device__ static V ld(const float* s) { return f2_of(*reinterpret_cast<const float2*>(s)); }
   __device__ static void st(float* s, V v) { *reinterpret_cast<float2*>(s) = f2_in(v); }
@@ -109,6 +114,9 @@ template <typename S> struct Unit<S, double> {         // one node
   }
   __device__ static Raw pull(const ST* row, int cx, const X& x) {
     return double(__ldg(at_bytes(row, cx > 0 ? x.m : (cx < 0 ? x.p : x.c))));
+  }
+  __device__ static Raw pull_checked(const Params& p, const ST* row, int cx, const X& x) {
+    return double(pop_value(p, at_bytes(row, cx > 0 ? x.m : (cx < 0 ? x.p : x.c))));
   }
   __device__ static V value(Raw r, float) { return r; }
   __device__ static V ld(const double* s) { return *s; }
@@ -213,8 +221,11 @@ __device__ __forceinline__ void tile2d(const Params& p, const typename Store<S>:
     for (int i = 0; i < Q; ++i) {
       const ST* Ai = A + (long long)(set + i) * p.plane;
       const ST* rp = at_bytes(Ai, r[L::c(i, 1) + 1]);
-      if (!pop_ok(p, at_bytes(rp, x.c), 0)) rp = A;
+#ifdef LBM_BOUNDS_CHECK
+      v[i] = U::pull_checked(p, rp, L::c(i, 0), x);
+#else
       v[i] = U::pull(rp, L::c(i, 0), x);
+#endif
     }
   };
   auto rows3 = [&](int gy, unsigned (&r)[3]) {
