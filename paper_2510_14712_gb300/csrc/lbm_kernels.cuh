@@ -1684,27 +1684,41 @@ __global__ void k_totals(Params p, const real* M, const real* W, double* partial
 }
 
 // The same of FP32 fields, bound by the FP64 units when every value is converted and
-// added in FP64 (28 such instructions per node).  A thread takes
-// four nodes of a row at a time and sums them without rounding in FP32: two-sums
-// (Knuth, The Art of Computer Programming 2, 4.2.2) leave a sum and its error, products
-// a value and a remainder; FP64 takes the sum and the small errors' sum of the four,
-// 2.5 pairs per node.  Errors relative to the sum of the magnitudes are the last
-// rounding of FP64 either way (4 million random values, 1e-16).
-// 384x128x128: 296 -> 58 us; 800x800: 35 -> 16 us.
-template <typename V> __device__ __forceinline__ V two_sum(V a, V b, V& err) {
-  const V s = a + b, t = s - a;
-  err = (a - (s - t)) + (b - t);
-  return s;
-}
+// added in FP64 (28 such instructions per node).  A thread takes four nodes of a row at a
+// time and sums them in FP32 without loss: the sum's rounding errors (two-sums, Knuth, The
+// Art of Computer Programming 2, 4.2.2; products leave a remainder) are summed next to it,
+// and their rounding errors in turn (the second-order form of Klein, "A generalized
+// Kahan-Babuska-Summation-Algorithm", 2006); what is dropped is 2^-72 of the sum.  FP64
+// joins the three once per thread.  A thread that met an infinity, a NaN or FP32's range
+// (its sums are then not finite) adds its nodes again in FP64.
+// 384x128x128: 77 us, 800x800 18 us; all in FP64 296 and 35; with FP64 additions for each
+// group of four and the errors in FP32 alone (2^-48) 58 and 16.
+struct Sum3 {                                                    // two lanes
+  F2 s = F2(0.f), e = F2(0.f), r = F2(0.f);
+  __device__ __forceinline__ void error(F2 v) {
+    F2 b;
+    e = two_sum(e, v, b);
+    r = r + b;
+  }
+  __device__ __forceinline__ void add(F2 v) {
+    F2 a;
+    s = two_sum(s, v, a);
+    error(a);
+  }
+  __device__ __forceinline__ bool finite() const { return isfinite((s.x + s.y) + (e.x + e.y)); }
+  __device__ __forceinline__ double value() const {
+    float a, b, c;                                               // the lanes joined without loss first
+    const float t = two_sum(s.x, s.y, a), u = two_sum(e.x, e.y, b), w = two_sum(u, a, c);
+    return double(t) + (double(w) + double((r.x + r.y) + (b + c)));
+  }
+};
 template <int D>
 __global__ void __launch_bounds__(256) k_totals_row(const __grid_constant__ Params p, const NodeRange range,
                                                     const float* __restrict__ M, const float* __restrict__ W,
                                                     double* partials) {
   using WP = WPlanes<D>;
   constexpr int K = D + 2;
-  double acc[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) acc[k] = 0.0;
+  Sum3 sum[K];
   for (unsigned gid = blockIdx.x * 256u + threadIdx.x; gid < range.n; gid += gridDim.x * 256u) {
     int xp, y, z;
     range.decode(gid, xp, y, z);
@@ -1717,36 +1731,55 @@ __global__ void __launch_bounds__(256) k_totals_row(const __grid_constant__ Para
       v[0] = F2(in[0] ? q.x : 0.f, in[1] ? q.y : 0.f);
       v[1] = F2(in[2] ? q.z : 0.f, in[3] ? q.w : 0.f);
     };
-    auto add = [&](const int k, const F2 (&v)[2], F2 err) {      // four values and the sum of their errors
-      F2 e;
-      const F2 s = two_sum(v[0], v[1], e);
-      err = err + e;
-      float e1;
-      const float t = two_sum(s.x, s.y, e1);
-      acc[k] += double(t) + double((err.x + err.y) + e1);
-    };
-    F2 v[2], u[2], F[2], e;
+    F2 v[2], w[2], u[2], F[2];
     load(M, v);
-    add(0, v, F2(0.f));
-    F2 w[2], ew(0.f);                                            // S + u . F / 2
     load(M + (1 + D) * p.plane, w);
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
+    for (int q = 0; q < 2; ++q) {
+      sum[0].add(v[q]);
+      sum[1 + D].add(w[q]);
+    }
+#pragma unroll
+    for (int a = 0; a < D; ++a) {                                // j + F / 2; S + u . F / 2
       load(M + (1 + a) * p.plane, v);
       load(W + (WP::F + a) * p.plane, F);
       load(W + (WP::U + a) * p.plane, u);
-      F2 ev(0.f);
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const F2 h = F2(0.5f) * F[q], m = u[q] * h;
-        v[q] = two_sum(v[q], h, e);
-        ev = ev + e;
-        w[q] = two_sum(w[q], m, e);
-        ew = ew + (e + mad(u[q], h, F2(-1.f) * m));
+        sum[1 + a].add(v[q]);
+        sum[1 + a].add(h);
+        sum[1 + D].add(m);
+        sum[1 + D].error(mad(u[q], h, F2(-1.f) * m));
       }
-      add(1 + a, v, ev);
     }
-    add(1 + D, w, ew);
+  }
+  double acc[K];
+  bool finite = true;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    acc[k] = sum[k].value();
+    finite = finite && sum[k].finite();
+  }
+  if (!finite) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k] = 0.0;
+    for (unsigned gid = blockIdx.x * 256u + threadIdx.x; gid < range.n; gid += gridDim.x * 256u) {
+      int xp, y, z;
+      range.decode(gid, xp, y, z);
+      const unsigned o = (unsigned(z) * unsigned(p.Ny) + unsigned(y)) * unsigned(p.pitch);
+      for (int x = max(xp, p.G); x < min(xp + 4, p.G + p.Nx); ++x) {
+        double uF = 0.0;
+        acc[0] += double(M[o + x]);
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+          const double f = double(W[(WP::F + a) * p.plane + o + x]);
+          acc[1 + a] += double(M[(1 + a) * p.plane + o + x]) + 0.5 * f;
+          uF += double(W[(WP::U + a) * p.plane + o + x]) * f;
+        }
+        acc[1 + D] += double(M[(1 + D) * p.plane + o + x]) + 0.5 * uF;
+      }
+    }
   }
   block_partials<K>(acc, partials);
 }
