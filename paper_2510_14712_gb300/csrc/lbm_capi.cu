@@ -173,10 +173,14 @@ void free_state(Handle& h) {
   h.io_dev = nullptr;
 }
 
-// shock-capturing fields: rho, u, T of the last step (D+2 planes), the
-// numerical mu, eta, k (3 planes), work (4 planes), in compute precision
+// shock-capturing fields in compute precision.  2-D: rho, u, T of the last step (D+2
+// planes; a single handle writes rho and T, the batched stencils read u too), the
+// numerical mu, eta, k (3 planes), work (4 planes).  3-D, whose step leaves its fields in
+// the scratch planes: mu, eta, k and two work planes.
+int sc_prims_planes(const Handle& h) { return h.D == 2 ? h.D + 2 : 0; }
 size_t sc_bytes(const Handle& h) {
-  return size_t(h.D + 9) * size_t(h.p.plane) * (h.precision == LBM_FP64 ? 8 : 4);
+  const int planes = sc_prims_planes(h) + 3 + (h.D == 2 ? 4 : 2);
+  return size_t(planes) * size_t(h.p.plane) * (h.precision == LBM_FP64 ? 8 : 4);
 }
 
 int sc_alloc(Handle& h) {
@@ -189,7 +193,7 @@ int sc_alloc(Handle& h) {
   CK(cudaMemsetAsync(h.sc_buf, 0, sc_bytes(h), h.stream));
   const size_t es = h.precision == LBM_FP64 ? 8 : 4;
   h.p.sc_prims = h.sc_buf;
-  h.p.sc_visc = static_cast<char*>(h.sc_buf) + size_t(h.D + 2) * size_t(h.p.plane) * es;
+  h.p.sc_visc = static_cast<char*>(h.sc_buf) + size_t(sc_prims_planes(h)) * size_t(h.p.plane) * es;
   return LBM_OK;
 }
 

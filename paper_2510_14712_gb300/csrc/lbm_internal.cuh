@@ -39,9 +39,9 @@ struct Params {
   // learned closure: device inference image (mlp::Image), NULL for the exact closure
   const void* mlp;
   // shock capturing (Sec. 4.4): on/off, coefficients C_mu, C_eta, C_k; the step
-  // writes rho, u[D], T of every interior node to sc_prims (D+2 planes) and
-  // reads the numerical mu, eta, k of the node from sc_visc (3 planes), both in
-  // compute precision on the padded plane layout
+  // reads the numerical mu, eta, k of the node from sc_visc (3 planes, work planes
+  // after them); the 2-D step writes rho and T (batches: u too) to sc_prims (4
+  // planes), all in compute precision on the padded plane layout
   int sc_on;
   double sc_c[3];
   void* sc_prims;
@@ -112,7 +112,7 @@ struct Handle {
   int tune_n;
   int use_graphs;             // lbm_set_graphs: replay captured two-step graphs
   void* graphs;               // StepGraphs (lbm_capi.cu), created on first use
-  void* sc_buf;               // shock capturing: prims (D+2), visc (3), work (4) planes
+  void* sc_buf;               // shock capturing: prims (2-D), visc, work planes
   int t64;                    // FP64 temperature inversion in the FP32 / FP16-deviation kernels
 };
 

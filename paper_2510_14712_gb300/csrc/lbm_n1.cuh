@@ -15,7 +15,8 @@
 // share the per-node arithmetic: in 2-D the step itself leaves S and |grad s|
 // (its block holds the neighbours' u, T and rho) and one launch over tiles does
 // the rest; in 3-D one launch for S and |grad s| and one over columns of
-// the box; one block per row for the 2-D batches.
+// the box (3-D batches: the same over the blocks of every instance); one block per row
+// for the 2-D batches.
 #pragma once
 
 #include "lbm_tile2d.cuh"
@@ -106,17 +107,16 @@ __device__ __forceinline__ N1Vals<real, 2> n1_strain_at(const Params& p, const r
   return v;
 }
 
-// norm of the per-axis fourth differences of the two fields of `in` at the node
-template <int D, typename real>
-__device__ __forceinline__ N1Vals<real, 2> n1_d4_at(const Params& p, const real* __restrict__ in, int x, int y, int z,
-                                                    unsigned o) {
-  unsigned nb[D][4];                               // offsets of the -2, -1, +1, +2 neighbours along a
+// norm of the per-axis fourth differences of the two fields of `in` at the node (2-D)
+template <typename real>
+__device__ __forceinline__ N1Vals<real, 2> n1_d4_at(const Params& p, const real* __restrict__ in, int x, int y, unsigned o) {
+  unsigned nb[2][4];                               // offsets of the -2, -1, +1, +2 neighbours along a
 #pragma unroll
-  for (int a = 0; a < D; ++a) {
-    nb[a][0] = n1_nb(p, x, y, z, o, a, -2);
-    nb[a][1] = n1_nb(p, x, y, z, o, a, -1);
-    nb[a][2] = n1_nb(p, x, y, z, o, a, 1);
-    nb[a][3] = n1_nb(p, x, y, z, o, a, 2);
+  for (int a = 0; a < 2; ++a) {
+    nb[a][0] = n1_nb(p, x, y, 0, o, a, -2);
+    nb[a][1] = n1_nb(p, x, y, 0, o, a, -1);
+    nb[a][2] = n1_nb(p, x, y, 0, o, a, 1);
+    nb[a][3] = n1_nb(p, x, y, 0, o, a, 2);
   }
   N1Vals<real, 2> res;
 #pragma unroll
@@ -124,7 +124,7 @@ __device__ __forceinline__ N1Vals<real, 2> n1_d4_at(const Params& p, const real*
     const real* v = in + f * p.plane;
     real acc = real(0);
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
+    for (int a = 0; a < 2; ++a) {
       const real d4 = n1_fourth(n1_ld(v + nb[a][0]), n1_ld(v + nb[a][1]), n1_ld(v + o), n1_ld(v + nb[a][2]),
                                 n1_ld(v + nb[a][3]));
       acc = mad(d4, d4, acc);
@@ -134,39 +134,26 @@ __device__ __forceinline__ N1Vals<real, 2> n1_d4_at(const Params& p, const real*
   return res;
 }
 
-// binomial (1, 4, 6, 4, 1)/16 along axis a of field f of `in` at the node
+// binomial (1, 4, 6, 4, 1)/16 along axis a of both fields of `in` at the node (2-D)
 template <typename real>
-__device__ __forceinline__ real n1_binomial(const Params& p, const real* __restrict__ in, int f, int a, int x, int y,
-                                            int z, unsigned o) {
-  const unsigned m2 = n1_nb(p, x, y, z, o, a, -2), m1 = n1_nb(p, x, y, z, o, a, -1);
-  const unsigned p1 = n1_nb(p, x, y, z, o, a, 1), p2 = n1_nb(p, x, y, z, o, a, 2);
-  const real* v = in + f * p.plane;
-  return n1_binom5(n1_ld(v + m2), n1_ld(v + m1), n1_ld(v + o), n1_ld(v + p1), n1_ld(v + p2));
-}
-
-template <typename real>
-__device__ __forceinline__ N1Vals<real, 2> n1_filter_at(const Params& p, int a, const real* __restrict__ in, int x,
-                                                        int y, int z, unsigned o) {
-  return {{n1_binomial(p, in, 0, a, x, y, z, o), n1_binomial(p, in, 1, a, x, y, z, o)}};
-}
-
-// the last filter pass (along axis D-1) and the coefficients from the filtered
-// norms: mu, eta, k numerical (the three planes of visc)
-template <int D, typename real>
-__device__ __forceinline__ N1Vals<real, 3> n1_filter_coef_at(const Params& p, const Model<real>& m,
-                                                             const real* __restrict__ in, const real* __restrict__ rho,
-                                                             const real* __restrict__ T, int x, int y, int z,
-                                                             unsigned o) {
-  const real s4 = n1_binomial(p, in, 0, D - 1, x, y, z, o), g4 = n1_binomial(p, in, 1, D - 1, x, y, z, o);
-  return n1_coefs(p, m, n1_ld(rho + o), n1_ld(T + o), s4, g4);
+__device__ __forceinline__ N1Vals<real, 2> n1_filter_at(const Params& p, int a, const real* __restrict__ in, int x, int y,
+                                                        unsigned o) {
+  const unsigned m2 = n1_nb(p, x, y, 0, o, a, -2), m1 = n1_nb(p, x, y, 0, o, a, -1);
+  const unsigned p1 = n1_nb(p, x, y, 0, o, a, 1), p2 = n1_nb(p, x, y, 0, o, a, 2);
+  N1Vals<real, 2> res;
+#pragma unroll
+  for (int f = 0; f < 2; ++f) {
+    const real* v = in + f * p.plane;
+    res.v[f] = n1_binom5(n1_ld(v + m2), n1_ld(v + m1), n1_ld(v + o), n1_ld(v + p1), n1_ld(v + p2));
+  }
+  return res;
 }
 
 // Buffers of one handle's shock capturing: the step's rho, u (D planes), T (by
 // default the 2-D step's copy in sc_prims), the coefficients (3 planes) followed by
-// the work planes w0, w1 (2 each).  S and |grad s| go to w0; the single-instance
-// forms go from there to the coefficients, the batched stages run fourth differences
-// w0 -> w1, filter passes alternating w1 -> w0 -> w1 ..., the last pass with the
-// coefficients.
+// the work planes w0, w1 (2 each; w1 in 2-D only).  S and |grad s| go to w0; the tiled
+// and column forms go from there to the coefficients, the 2-D batched stages run fourth
+// differences w0 -> w1, the x pass w1 -> w0, the y pass with the coefficients.
 template <int D, typename real> struct N1Buffers {
   const real *rho, *u, *T;
   real *visc, *w0, *w1;
@@ -179,9 +166,6 @@ template <int D, typename real> struct N1Buffers {
   __host__ __device__ explicit N1Buffers(const Params& p)
       : N1Buffers(p, static_cast<const real*>(p.sc_prims), static_cast<const real*>(p.sc_prims) + p.plane,
                   static_cast<const real*>(p.sc_prims) + (1 + D) * p.plane) {}
-  // input of filter pass a (a = D - 1: the pass with the coefficients)
-  __host__ __device__ const real* filter_in(int a) const { return a % 2 == 0 ? w1 : w0; }
-  __host__ __device__ real* filter_out(int a) const { return a % 2 == 0 ? w0 : w1; }
 };
 
 // ---- single-instance kernels ----
@@ -356,7 +340,7 @@ __global__ void __launch_bounds__(kN1Threads) k_n1_coef_2d(const __grid_constant
 // launch 151.
 template <typename S, typename real> struct N1Column {
   using U = Unit<S, real>;
-  static constexpr int N = U::N, TX = 32 * N, TY = sizeof(real) == 4 ? 8 : 8, HX = 4;
+  static constexpr int N = U::N, TX = 32 * N, TY = 8, HX = 4;
   static constexpr int P4 = TX + 2 * HX, H4 = TY + 8, P2 = TX + 4, H2 = TY + 4, NU = TY * 32 / kN1Threads;
   static constexpr int kPlane = H4 * P4;                         // one field of one plane
   static constexpr size_t kBytes = sizeof(real) * 2 * (5 * kPlane + H2 * P2 + H2 * TX);
@@ -581,35 +565,36 @@ __device__ __forceinline__ int n1_instance(const int* __restrict__ rowstart, int
   return lo;
 }
 
-// stage 0: strain, 1: fourth differences, 2: filter pass a, 3: last pass + coefficients
-template <int D, typename real, int STAGE>
-__global__ void k_n1_batch(const BatchInstance* __restrict__ insts, const int* __restrict__ rowstart, int n, int a) {
+// stage 0: S and |grad s|, 1: fourth differences, 2: x pass, 3: y pass and coefficients
+template <typename real, int STAGE>
+__global__ void k_n1_batch(const BatchInstance* __restrict__ insts, const int* __restrict__ rowstart, int n) {
   wait_previous_launch();
   const int k = n1_instance(rowstart, n, blockIdx.x);
   const Params& p = insts[k].p;
-  const N1Buffers<D, real> b(p);
-  const int row = blockIdx.x - rowstart[k];
-  const int y = row % p.Ny, z = row / p.Ny;
+  const N1Buffers<2, real> b(p);
+  const int y = blockIdx.x - rowstart[k];
   const Model<real> m = model_of<real>(p);
   for (int x = threadIdx.x; x < p.Nx; x += blockDim.x) {
-    const unsigned o = unsigned(row) * unsigned(p.pitch) + unsigned(x + p.G);
-    if constexpr (STAGE == 0) n1_store(p, b.w0, o, n1_strain_at<D, real>(p, b.rho, b.u, b.T, x, y, z, o));
-    else if constexpr (STAGE == 1) n1_store(p, b.w1, o, n1_d4_at<D, real>(p, b.w0, x, y, z, o));
-    else if constexpr (STAGE == 2)
-      n1_store(p, b.filter_out(a), o, n1_filter_at<real>(p, a, b.filter_in(a), x, y, z, o));
-    else n1_store(p, b.visc, o, n1_filter_coef_at<D, real>(p, m, b.filter_in(D - 1), b.rho, b.T, x, y, z, o));
+    const unsigned o = unsigned(y) * unsigned(p.pitch) + unsigned(x + p.G);
+    if constexpr (STAGE == 0) n1_store(p, b.w0, o, n1_strain_at<2, real>(p, b.rho, b.u, b.T, x, y, 0, o));
+    else if constexpr (STAGE == 1) n1_store(p, b.w1, o, n1_d4_at(p, static_cast<const real*>(b.w0), x, y, o));
+    else if constexpr (STAGE == 2) n1_store(p, b.w0, o, n1_filter_at(p, 0, static_cast<const real*>(b.w1), x, y, o));
+    else {
+      const N1Vals<real, 2> q = n1_filter_at(p, 1, static_cast<const real*>(b.w0), x, y, o);
+      n1_store(p, b.visc, o, n1_coefs(p, m, n1_ld(b.rho + o), n1_ld(b.T + o), q.v[0], q.v[1]));
+    }
   }
 }
 
-// the update of every instance with shock capturing on: D + 2 launches over
-// `rows` global rows
-template <int D, typename real>
+// the update of every 2-D instance with shock capturing on: four launches over `rows`
+// global rows
+template <typename real>
 inline int n1_update_batch(const BatchInstance* insts, const int* rowstart, int n, int rows, cudaStream_t st) {
-  launch_overlapped(k_n1_batch<D, real, 0>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, 0);
-  launch_overlapped(k_n1_batch<D, real, 1>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, 0);
-  for (int a = 0; a + 1 < D; ++a) launch_overlapped(k_n1_batch<D, real, 2>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, a);
-  launch_overlapped(k_n1_batch<D, real, 3>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n, D - 1);
-  return D + 2;
+  launch_overlapped(k_n1_batch<real, 0>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n);
+  launch_overlapped(k_n1_batch<real, 1>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n);
+  launch_overlapped(k_n1_batch<real, 2>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n);
+  launch_overlapped(k_n1_batch<real, 3>, dim3(unsigned(rows)), 128u, 0, st, insts, rowstart, n);
+  return 4;
 }
 
 }  // namespace lbm

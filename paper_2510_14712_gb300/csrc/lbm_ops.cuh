@@ -440,7 +440,7 @@ template <int D, typename S, typename real> struct OpsImpl {
           b.launches += 1;
         }
       }
-      if (b.n1rows > 0 && !b.tuning) b.launches += n1_update_batch<D, real>(insts, b.d_n1rows, b.n, b.n1rows, b.stream);
+      if (b.n1rows > 0 && !b.tuning) b.launches += n1_update_batch<real>(insts, b.d_n1rows, b.n, b.n1rows, b.stream);
       enqueue_own(b, parity);
     }
   };
