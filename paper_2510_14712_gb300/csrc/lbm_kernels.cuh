@@ -1354,10 +1354,13 @@ template <typename S> inline int collide_segments(const Params& p) {
 // and 316; a box of 4 x 224 x 224: 375 and 170), in both storage types.  Bounded rows,
 // whose ghosts the row form fills and whose pairs straddle 16-byte units, at 3/16 in FP32
 // (Nx 16 964 and 929, 24 639 and 658, 128 307 and 422) and 1/4 with FP16 deviations (24
-// 883 and 433, 32 513 and 546, 128 323 and 348).
+// 883 and 433, 32 513 and 546, 128 323 and 348); and whatever the fill while the segments
+// are one round of blocks, for the launch that the ghosts take otherwise (17 x 16 x 16
+// FP32: 16.6 and 19.0; 1225 segments of 16 nodes 18 and 17).
 template <typename S> inline bool collide_rows_ok(const Params& p) {
   constexpr int kA = 16 / int(sizeof(typename Store<S>::T));
   if (p.periodic_x && p.Nx % kA) return false;
+  if (!p.periodic_x && (long long)collide_segments<S>(p) * p.Ny * p.Nz <= 512) return true;
   const int sixteenths = p.periodic_x ? 9 : (kA == 4 ? 3 : 4);
   return 16 * p.Nx >= sixteenths * kRowW * collide_segments<S>(p);
 }
