@@ -91,14 +91,16 @@ k_n1_strain_batch3(const SplitInstance<real>* __restrict__ insts, const SplitIte
   n1_strain_units<S, real>(in.p, in.units, in.dunits, in.dny, in.M, in.W, in.W + 3 * in.p.plane, it.block);
 }
 
-template <typename S, typename real>
-__global__ void __launch_bounds__(kN1Threads, N1Column<S, real>::kMinB)
-k_n1_coef_batch3(const SplitInstance<real>* __restrict__ insts, const SplitItem* __restrict__ items) {
-  wait_previous_launch();
-  const SplitItem it = items[blockIdx.x];
-  const SplitInstance<real>& in = insts[it.inst];
-  n1_coef_column<S, real>(in.p, in.M, in.W + 3 * in.p.plane, in.n1tx, in.n1ty, in.n1seg, it.block);
-}
+// the columns of the coefficients of a batch's instances (k_n1_coef_3d)
+template <typename real> struct N1CoefBatch {
+  const SplitInstance<real>* insts;
+  const SplitItem* items;
+  __device__ __forceinline__ N1CoefArgs<real> args() const {
+    const SplitItem it = items[blockIdx.x];
+    const SplitInstance<real>& in = insts[it.inst];
+    return {in.p, in.M, in.W + 3 * in.p.plane, in.n1tx, in.n1ty, in.n1seg, it.block};
+  }
+};
 
 // the ghost layers of the instances whose collision leaves them
 template <typename S, typename real>

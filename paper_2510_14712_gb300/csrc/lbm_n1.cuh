@@ -344,11 +344,28 @@ template <typename S, typename real> struct N1Column {
   static constexpr int P4 = TX + 2 * HX, H4 = TY + 8, P2 = TX + 4, H2 = TY + 4, NU = TY * 32 / kN1Threads;
   static constexpr int kPlane = H4 * P4;                         // one field of one plane
   static constexpr size_t kBytes = sizeof(real) * 2 * (5 * kPlane + H2 * P2 + H2 * TX);
-  static constexpr int kMinB = sizeof(real) == 4 ? 3 : 2;        // blocks: what 59 KB admit; FP64 needs 92 registers
 };
-template <typename S, typename real>
-__device__ __forceinline__ void n1_coef_column(const Params& p, const real* __restrict__ rho, const real* __restrict__ T, int ntx,
-                                               int nty, int nseg, const unsigned block) {
+// the arguments of one column: of a handle, here, or of an instance of a batch
+template <typename real> struct N1CoefArgs {
+  const Params& p;
+  const real *rho, *T;
+  int ntx, nty, nseg;
+  unsigned block;
+};
+template <typename real> struct N1CoefHandle {
+  Params p;
+  const real *rho, *T;
+  int ntx, nty, nseg;
+  __device__ __forceinline__ N1CoefArgs<real> args() const { return {p, rho, T, ntx, nty, nseg, blockIdx.x}; }
+};
+// (the body stands in the kernel: in a function that a kernel of each calls the compiler
+// took 114 registers instead of 80, and bounded to 85 the column took 158 us for 152)
+template <typename S, typename real, class Src>
+__global__ void __launch_bounds__(kN1Threads) k_n1_coef_3d(const __grid_constant__ Src from) {
+  wait_previous_launch();
+  const N1CoefArgs<real> arg = from.args();
+  const Params& p = arg.p;
+  const int ntx = arg.ntx, nty = arg.nty, nseg = arg.nseg;
   using C = N1Column<S, real>;
   using U = typename C::U;
   using V = typename U::V;
@@ -358,10 +375,10 @@ __device__ __forceinline__ void n1_coef_column(const Params& p, const real* __re
   real* ring = reinterpret_cast<real*>(smem_raw);
   real* s2 = ring + 10 * C::kPlane;                              // norms of the fourth differences
   real* sx = s2 + 2 * H2 * P2;                                   // the same after the x pass
-  const N1Buffers<3, real> b(p, rho, nullptr, T);
+  const N1Buffers<3, real> b(p, arg.rho, nullptr, arg.T);
   const Model<real> m = model_of<real>(p);
   const int tid = threadIdx.x;
-  int blk = block;
+  int blk = int(arg.block);
   const int x0 = (blk % ntx) * TX;
   blk /= ntx;
   const int y0 = (blk % nty) * C::TY, seg = blk / nty;
@@ -487,13 +504,6 @@ __device__ __forceinline__ void n1_coef_column(const Params& p, const real* __re
     if (pl >= mb + 4) zo += zs;
   }
 }
-template <typename S, typename real>
-__global__ void __launch_bounds__(kN1Threads, N1Column<S, real>::kMinB)
-k_n1_coef_3d(const __grid_constant__ Params p, const real* __restrict__ rho, const real* __restrict__ T, int ntx, int nty,
-             int nseg) {
-  wait_previous_launch();
-  n1_coef_column<S, real>(p, rho, T, ntx, nty, nseg, blockIdx.x);
-}
 
 // S and |grad s| of a plane from its rho, u, T, which also go to sc_prims (the
 // multi-pass step keeps them in its scratch area)
@@ -539,14 +549,14 @@ inline int n1_update(const Params& p, cudaStream_t st, const real* rho, const re
     return rho ? 2 : 1;
   } else {
     using C = N1Column<S, real>;
-    auto kern = k_n1_coef_3d<S, real>;
-    const int slots = prepared_blocks<k_n1_coef_3d<S, real>>(kN1Threads, C::kBytes);
+    using Src = N1CoefHandle<real>;
+    const int slots = prepared_blocks<k_n1_coef_3d<S, real, Src>>(kN1Threads, C::kBytes);
     const unsigned nx = unsigned((p.Nx + C::N - 1) / C::N), n = nx * unsigned(p.Ny) * unsigned(p.Nz);
     launch_overlapped(k_n1_strain_3d<S, real>, dim3((n + 127u) / 128u), 128, 0, st, p, n, FastDiv(nx),
                       FastDiv(unsigned(p.Ny)), rho, u, T);
     const int ntx = (p.Nx + C::TX - 1) / C::TX, nty = (p.Ny + C::TY - 1) / C::TY, nseg = n1_segments(p, slots, (long long)ntx * nty);
-    launch_overlapped(kern, dim3(unsigned(ntx) * unsigned(nty) * unsigned(nseg)), kN1Threads, C::kBytes, st, p, rho, T, ntx,
-                      nty, nseg);
+    launch_overlapped(k_n1_coef_3d<S, real, Src>, dim3(unsigned(ntx) * unsigned(nty) * unsigned(nseg)), kN1Threads, C::kBytes,
+                      st, Src{p, rho, T, ntx, nty, nseg});
     return 2;
   }
 }

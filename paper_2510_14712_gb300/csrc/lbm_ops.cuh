@@ -500,7 +500,7 @@ template <int D, typename S, typename real> struct OpsImpl {
         if (p.sc_on) n1columns += (long long)t.n1tx * t.n1ty;
       }
       const int slots = prepared_blocks<k_prims3_batch<real, CL, kMinB>>(kPrimX * kPrimY, CL::kSmem);
-      const int n1slots = prepared_blocks<k_n1_coef_batch3<S, real>>(kN1Threads, N1::kBytes);
+      const int n1slots = prepared_blocks<k_n1_coef_3d<S, real, N1CoefBatch<real>>>(kN1Threads, N1::kBytes);
       for (int k : order) {
         Inst& t = ti[k];
         t.nseg = prim_segments(t.p, slots, columns);
@@ -574,7 +574,12 @@ template <int D, typename S, typename real> struct OpsImpl {
       }
       if (!b.tuning) {
         launch(kStrain, k_n1_strain_batch3<S, real>, 128, 0);
-        launch(kCoef, k_n1_coef_batch3<S, real>, kN1Threads, N1Column<S, real>::kBytes);
+        const int n = b.group[kCoef + 1] - b.group[kCoef];
+        if (n > 0) {
+          launch_overlapped(k_n1_coef_3d<S, real, N1CoefBatch<real>>, dim3(unsigned(n)), kN1Threads, N1Column<S, real>::kBytes,
+                            b.stream, N1CoefBatch<real>{insts, items + b.group[kCoef]});
+          b.launches += 1;
+        }
       }
       enqueue_own(b, parity);
     }
