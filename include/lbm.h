@@ -286,12 +286,13 @@ int lbm_tile_count(lbm_t h);
  * in FP64 from the FP32 moments E = (S + u.F/2)/rho and u, and rounded once to
  * FP32; for the Peng-Robinson fluid (Sec. 2: T from the non-linear caloric
  * relation) e = E - |u|^2/2 and the root's argument e - B0 are formed in FP64.
- * Off (the default): the whole step in FP32.  The FP64 form costs about 6% of
- * the 256^3 D3Q27 step.  Its effect on the error against the FP64 oracle
- * depends on the flow: on Ma 1.2 shock tubes it lowers it (T about threefold),
- * on a drifting Taylor-Green vortex it raises it (rho about twofold); the
- * trajectory error of FP32 runs is set by rounding throughout the step, not
- * by the inversion alone.  FP64 handles ignore the setting (their arithmetic
+ * The collision takes e and h = e + P / rho from e as so formed, not from the
+ * rounded T.  Off (the default): the whole step in FP32.  The FP64 form costs 9%
+ * of a 128^3 D3Q27 step in FP32, 20% with FP16 deviations.  Its effect on the
+ * error against FP64 depends on the flow: 0.8 to 1.2 times the plain FP32 error
+ * on Taylor-Green vortices, channels and shock tubes; past the impact of a shock
+ * on a liquid column rounding at the stagnation point decides either.
+ * FP64 handles ignore the setting (their arithmetic
  * is FP64), and so do the learned closure (its network replaces the
  * inversion) and the batched step (FP32 inversion).  Applies to both
  * step kernels from the next step on; does not synchronise.
@@ -316,8 +317,9 @@ long long lbm_launch_count(lbm_t h);
  * Many independent instances of one lattice, fluid and precision, each with
  * its own size and x faces, advanced together by one graph launch per step (one
  * graph per buffer parity): D2Q9 one kernel over a work list of (instance, tile)
- * items and one batched ghost fill, D3Q27 the three kernels of the split step, each
- * over the blocks of every instance.  Results are bit-identical to stepping each
+ * items and one batched ghost fill (FP64 planes of 2^20 nodes and more: kernels of
+ * their own), D3Q27 the three kernels of the split step, each over the blocks of
+ * every instance.  Results are bit-identical to stepping each
  * instance alone.  Instances are numbered 0..n-1; all per-instance calls take
  * that index.  The batch uses its own non-blocking stream unless
  * lbm_batch_set_stream gives one (the default stream cannot be captured). */
